@@ -376,7 +376,8 @@ int pqhsa_debug_predicate(int which, long long value, long long lo, long long hi
  * tests and tools); (size_t)-1 on error. */
 size_t pqhsa_decode_buffer_offset(const pqhsa_params* params, int which);
 
-/* Number of kernels (memsets included) pqhsa_decode enqueues for these params. */
+/* Number of kernels (memsets included) that pqhsa_decode enqueues at most for these params (with few or
+ * short score rows the top-k and the background preparation are one kernel instead of three). */
 int pqhsa_decode_launch_count(const pqhsa_params* params);
 
 const char* pqhsa_status_string(int status);

@@ -11,7 +11,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libpqhsa.so")
-SOURCES = ["api.cu", "lut.cu", "scan.cu", "scan4.cu", "select.cu", "attend.cu", "select_static.cu", "dense.cu",
+SOURCES = ["api.cu", "lut.cu", "scan.cu", "scan4.cu", "select.cu", "select_cluster.cu",
+           "attend.cu", "select_static.cu", "dense.cu",
            "update.cu", "build.cu", "rescore.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),

@@ -145,8 +145,12 @@ int make_plan(const pqhsa_params* p, Plan* pl) {
   // background preparation: CTAs per row
   o.bg_ctas = ceil_div(2LL * o.num_sms, o.rows);
   if (o.bg_ctas > 8) o.bg_ctas = 8;
+  if (o.bg_ctas < o.n_list / 256 && o.rows * (o.n_list / 256) <= 4 * o.num_sms)
+    o.bg_ctas = o.n_list / 256;                           // 2 lists per thread
   if (o.bg_ctas < ceil_div(o.k_max, 768)) o.bg_ctas = ceil_div(o.k_max, 768);   // 6 tokens per thread
   if (o.bg_ctas < 1) o.bg_ctas = 1;
+  o.bg_in_select = 0;
+  plan_select_cluster(&o);
   return PQHSA_OK;
 }
 
@@ -423,6 +427,7 @@ static int decode_impl(const pqhsa_params* params, const void* q, const pqhsa_in
     return ev == nullptr ? cudaSuccess : cudaEventRecord(static_cast<cudaEvent_t>(ev[i]), st);
   };
   cudaError_t e = mark(0);
+  pl.bg_in_select = pl.sel_cluster > 0 && pl.variant == PQHSA_VARIANT_B ? 1 : 0;
   // the LUT kernel also clears the status word, histograms, counters and tickets
   if (e == cudaSuccess)
     e = launch_build_lut(pl, q, *index, lut, coarse, w + L.zero_begin, L.zero_bytes, st);
@@ -432,7 +437,13 @@ static int decode_impl(const pqhsa_params* params, const void* q, const pqhsa_in
     e = launch_scan(pl, *index, lut, coarse, seq_lens, scores, partials,
                     reinterpret_cast<int*>(w + L.status), st);
   if (e == cudaSuccess) e = mark(2);
-  if (e == cudaSuccess) e = launch_select(pl, L, w, scores, seq_lens, sel_idx, sel_count, kth, st);
+  if (e == cudaSuccess)
+    e = pl.bg_in_select
+            ? launch_select_cluster_bg(pl, scores, seq_lens, sel_idx, sel_count, kth,
+                                       reinterpret_cast<int*>(w + L.status), partials, index->list_ids,
+                                       reinterpret_cast<float*>(w + L.bg_mass),
+                                       reinterpret_cast<float*>(w + L.bg_max), st)
+            : launch_select(pl, L, w, scores, seq_lens, sel_idx, sel_count, kth, st);
   if (e == cudaSuccess && pl.rescore)
     e = launch_rescore(pl, L, w, *index, lut, coarse, scores, seq_lens, sel_idx, sel_count, kth, st);
   if (e == cudaSuccess) e = mark(3);

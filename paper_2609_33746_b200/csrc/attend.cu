@@ -24,8 +24,8 @@
 // what the top-k wrote, to skip their own griddepcontrol.wait and run beside the background
 // preparation.  Nothing may be added above those waits that returns early.
 #include "attn_common.cuh"
+#include "background.cuh"
 #include "common.cuh"
-#include "scan_common.cuh"
 
 namespace pqhsa {
 
@@ -47,11 +47,10 @@ bg_prep_kernel(Plan pl, const float* __restrict__ scores, const float* __restric
                const uint16_t* __restrict__ lids, const int32_t* __restrict__ seq_lens,
                float* __restrict__ bg_mass, float* __restrict__ bg_max,
                float* __restrict__ bg_aux, int32_t* __restrict__ bg_tcount) {
-  __shared__ float s_scale[kMaxSeg], s_ref2[kMaxSeg];
-  __shared__ int s_segend[kMaxSeg];      // first tile of the row (32-token units) past segment sg
+  __shared__ SegTables seg;
   const int row = blockIdx.y, c = blockIdx.x, C = gridDim.x, tid = threadIdx.x;
   const int b = row / pl.Hq, h = row % pl.Hq;
-  const int kv = h / pl.G, hg = (h % pl.G) / pl.Gc;
+  const int kv = h / pl.G;
   const int n_list = pl.n_list;
   pdl_wait();               // (nothing above this line may return: see the file header)
   pdl_launch_dependents();
@@ -106,71 +105,37 @@ bg_prep_kernel(Plan pl, const float* __restrict__ scores, const float* __restric
     return;
   }
 
-  // which scan segments cover this row's unit
-  const ScanSplit sp = scan_split(seq_lens, pl.B, pl.N_max, pl.upb, pl.scan_ctas);
-  long long base = 0;
-  for (int bb = 0; bb < b; ++bb) base += (long long)seq_tiles(seq_lens, bb, pl.N_max) * pl.upb;
-  const int tb = seq_tiles(seq_lens, b, pl.N_max);
-  const long long s_u = base + (long long)(kv * pl.n_hg + hg) * tb;
-  const int c_first = split_cta_of(sp, s_u);
-  const int nseg = min(kMaxSeg, split_cta_of(sp, s_u + tb - 1) - c_first + 1);
-  // the unit's partials: per segment a header [2 Gc] (reference, maximum per head) and the sums
-  // [n_list][Gc] relative to the reference
-  const int Gc = pl.Gc, g = (h % pl.G) % Gc;
-  const size_t seg_stride = (size_t)Gc * (n_list + 2);
-  const float* pr = partials + (((size_t)b * pl.Hkv + kv) * pl.n_hg + hg) * pl.n_part * seg_stride;
-
-  float m = -CUDART_INF_F;
-  for (int sg = tid; sg < nseg; sg += kBgThreads) {                    // segment maxima
-    const float v = pr[(size_t)sg * seg_stride + Gc + g];
-    s_scale[sg] = v;
-  }
-  __syncthreads();
-  for (int s = 0; s < nseg; ++s) m = fmaxf(m, s_scale[s]);
-  if (!(m > -CUDART_INF_F)) {            // no token of R in this row: no background at all
+  BgRow bg = bg_row_plan(pl, row, seq_lens, partials);
+  bg_segment_ends(bg, seg, kBgThreads);
+  bg_row_begin(pl, bg, seg, kBgThreads);
+  if (!(bg.m > -CUDART_INF_F)) {         // no token of R in this row: no background at all
     if (c == 0 && tid == 0) bg_max[row] = -CUDART_INF_F;
     return;
   }
-  const float m2 = m * kLog2e;
-  __syncthreads();
-  for (int sg = tid; sg < nseg; sg += kBgThreads) {
-    // a segment's sums are relative to its reference: exp2(l~ log2 e - ref log2 e)
-    const float ref = pr[(size_t)sg * seg_stride + g];
-    s_scale[sg] = s_scale[sg] > -CUDART_INF_F ? fast_exp2(ref * kLog2e - m2) : 0.f;
-    s_ref2[sg] = __fmul_rn(ref, kLog2e);           // the scan's own product, rounded as there
-    s_segend[sg] = sg + 1 < nseg ? (int)(split_start(sp, c_first + sg + 1) - s_u) : 0x7fffffff;
-  }
-  __syncthreads();
   const int jl = (int)((long long)c * n_list / C), jh = (int)((long long)(c + 1) * n_list / C);
-  const float* sums = pr + 2 * Gc + g;
-  for (int j = jl + tid; j < jh; j += kBgThreads) {
-    float acc = 0.f;
-    for (int s0 = 0; s0 < nseg; s0 += 8) {
-      float v[8];
+  for (int j = jl + tid; j < jh; j += 2 * kBgThreads) {          // two lists, 16 reads in flight
+    float acc0 = 0.f, acc1 = 0.f;
+    const bool two = j + kBgThreads < jh;
+    for (int s0 = 0; s0 < bg.nseg; s0 += 8) {
+      float v0[8], v1[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        v[u] = (s0 + u < nseg) ? sums[(size_t)(s0 + u) * seg_stride + (size_t)j * Gc] : 0.f;
+      for (int u = 0; u < 8; ++u) {
+        const float* at = bg.sums + (size_t)(s0 + u) * bg.seg_stride + (size_t)j * pl.Gc;
+        v0[u] = s0 + u < bg.nseg ? __ldg(at) : 0.f;
+        v1[u] = s0 + u < bg.nseg && two ? __ldg(at + kBgThreads * pl.Gc) : 0.f;
+      }
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (s0 + u < nseg) acc = fmaf(v[u], s_scale[s0 + u], acc);
+      for (int u = 0; u < 8; ++u) {
+        const float sc_u = s0 + u < bg.nseg ? seg.scale[s0 + u] : 0.f;
+        acc0 = fmaf(v0[u], sc_u, acc0);
+        acc1 = fmaf(v1[u], sc_u, acc1);
+      }
     }
-    if (acc != 0.f) atomicAdd(&mass[j], acc);
+    if (acc0 != 0.f) atomicAdd(&mass[j], acc0);
+    if (two && acc1 != 0.f) atomicAdd(&mass[j + kBgThreads], acc1);
   }
-  // Take the selected tokens out of their lists' sums.  A selected token can hold nearly all of
-  // its list's mass, and what is left after the subtraction is multiplied by the list's mean
-  // value, so the term taken out is formed exactly as the scan formed the term it put in (the
-  // exponent against the reference of the token's own segment, the same instructions) and
-  // scaled like that segment's sums: what remains is the rounding of the additions alone.
-  const float inv_seg_tiles = (float)sp.P_eff / (float)sp.T;          // segments per tile
-  const float tile_off = (float)(s_u - split_start(sp, c_first));     // tiles of segment 0 before this unit
   auto take_out = [&](int i, float s, uint32_t lid) {
-    // segments are equally long up to one tile: estimate, then settle against the boundaries
-    const int tile = i / kTile;
-    int sg = min(nseg - 1, max(0, (int)(((float)tile + tile_off) * inv_seg_tiles)));
-    while (sg > 0 && tile < s_segend[sg - 1]) --sg;
-    while (tile >= s_segend[sg]) ++sg;             // (the last entry is INT_MAX)
-    const float x = fmaf(s, kLog2e, -s_ref2[sg]);
-    if (x > kScanNegligibleLog2) atomicAdd(&mass[lid], -(fast_exp2(x) * s_scale[sg]));
+    bg_take_out(bg, seg, i, s, lid, mass);
     if (bg_tcount != nullptr) atomicAdd(&bg_tcount[(size_t)row * n_list + lid], 1);
   };
 #pragma unroll
@@ -181,7 +146,7 @@ bg_prep_kernel(Plan pl, const float* __restrict__ scores, const float* __restric
     if ((unsigned)i >= (unsigned)n) continue;
     take_out(i, rs[i], min((uint32_t)rl[i], (uint32_t)(n_list - 1)));
   }
-  if (c == 0 && tid == 0) bg_max[row] = m;
+  if (c == 0 && tid == 0) bg_max[row] = bg.m;
 }
 
 // One grid, two kinds of CTA.
@@ -349,9 +314,9 @@ attend_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc, const 
   // ================= exact (selected-token) CTA =================
   const int row = (int)blockIdx.x / S, split = (int)blockIdx.x % S;
   const int b = row / pl.Hq, h = row % pl.Hq, kv = h / pl.G;
-  // (variant Bx: the CTA that merges a row also reads the correction partials of the kernel
-  // right before this one, so it cannot skip the wait)
-  if (variant == PQHSA_VARIANT_BX) pdl_wait();
+  // (the wait cannot be skipped where the kernel right before this one is the top-k itself, or,
+  // with variant Bx, leaves correction partials that the CTA which merges a row reads)
+  if (pl.bg_in_select || variant == PQHSA_VARIANT_BX) pdl_wait();
   pdl_launch_dependents();
   // the exact set E = T u S u L (Sec. 3.2), as one index space: the selected tokens first,
   // then the sink prefix, then the local window
@@ -579,7 +544,9 @@ cudaError_t launch_attend(const Plan& pl_in, const WsLayout& L, char* ws, const 
   float* split_part = reinterpret_cast<float*>(ws + L.split_part);
   uint32_t* tickets = reinterpret_cast<uint32_t*>(ws + L.attend_tickets);
   if (attend_parts(pl) > kMaxParts) return cudaErrorInvalidValue;
-  cudaError_t e = launch_pdl(bg_prep_kernel, dim3(pl.bg_ctas, pl.rows), dim3(kBgThreads), 0, st, pl,
+  cudaError_t e = cudaSuccess;
+  if (!pl.bg_in_select)
+    e = launch_pdl(bg_prep_kernel, dim3(pl.bg_ctas, pl.rows), dim3(kBgThreads), 0, st, pl,
                              scores, list_partials, sel_idx, sel_count, ix.list_ids, seq_lens,
                              bg_mass, bg_max, bg_aux, bg_tcount);
   if (e != cudaSuccess) return e;

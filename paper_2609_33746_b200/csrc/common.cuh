@@ -56,6 +56,8 @@ struct Plan {
                                      // one conflict-free 128-byte row per list)
   int scan_stages;                   // stages per warp in the scan's code ring (3 or 2)
   int num_sms;
+  int sel_cluster;                   // > 0: top-k by a cluster of that many CTAs per row (select_cluster.cu)
+  int bg_in_select;                  // fused call: the background is prepared by the top-k kernel
 };
 
 // Workspace carve-up (byte offsets from a 256-byte aligned base).
@@ -277,6 +279,16 @@ cudaError_t launch_rescore(const Plan& pl, const WsLayout& L, char* ws, const pq
 cudaError_t launch_select(const Plan& pl, const WsLayout& L, char* ws, const float* scores,
                           const int32_t* seq_lens, int32_t* sel_idx, int32_t* sel_count,
                           float* kth, cudaStream_t st);
+// The same result from one cluster of CTAs per row, for few or short rows (plan_select_cluster decides);
+// the _bg form also leaves the row's background mass and maximum, as bg_prep_kernel does.
+void plan_select_cluster(Plan* pl);
+cudaError_t launch_select_cluster(const Plan& pl, const float* scores, const int32_t* seq_lens,
+                                  int32_t* sel_idx, int32_t* sel_count, float* kth, int* status,
+                                  cudaStream_t st);
+cudaError_t launch_select_cluster_bg(const Plan& pl, const float* scores, const int32_t* seq_lens,
+                                     int32_t* sel_idx, int32_t* sel_count, float* kth, int* status,
+                                     const float* partials, const uint16_t* lids, float* bg_mass,
+                                     float* bg_max, cudaStream_t st);
 cudaError_t launch_attend(const Plan& pl, const WsLayout& L, char* ws, const void* q,
                           const pqhsa_paged_kv& kv, const pqhsa_index& ix, const float* scores,
                           const float* list_partials, const int32_t* sel_idx,
