@@ -33,6 +33,15 @@ template <> struct Unpack<__half> {
   static __device__ __forceinline__ __half pack(float v) { return __float2half_rn(v); }
 };
 
+// Four consecutive cache elements (rows are 16-byte aligned: one 8-byte load).
+template <typename T> __device__ __forceinline__ void load4(const T* p, float (&x)[4]) {
+  const uint2 w = __ldg(reinterpret_cast<const uint2*>(p));
+  float f[8];
+  Unpack<T>::run(make_uint4(w.x, w.y, 0u, 0u), f);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = f[i];
+}
+
 // Online-softmax state of a lane group: running max m (log2 units), normaliser Z and the 16
 // output dims the lane owns.
 struct GroupState {

@@ -1,0 +1,220 @@
+// Fifth-generation tensor core blocks (tcgen05, accumulators in TMEM) for the nearest-centre
+// searches of the index: fp16 operands split in two, fp32 accumulation.
+//
+// A nearest-centre search needs argmin_c (|c|^2 - 2 x.c) with fp32-grade products.  Every fp32
+// factor is split as hi + lo in fp16 (22 bits together; scaled by 2^8 so that lo keeps an absolute
+// resolution of 2^-32), and x.c is taken as hi.hi + hi.lo + lo.hi, the dropped lo.lo term being
+// 2^-22 of the product.  The centre side carries the factor -2, and |c|^2 rides along as three more
+// fp16 terms against the constant 256, so the accumulator holds 2^16 (|c|^2 - 2 x.c) itself.
+//
+// Operand tiles in shared memory use the K-major layout without swizzle: 8 x 16-byte core matrices;
+// 8 consecutive k of all R rows form one block ("chunk") of R * 16 bytes, row r at r * 16, so that
+// threads that own rows store 16 bytes each without bank conflicts.
+#pragma once
+
+#include "common.cuh"
+#include "scan_common.cuh"
+
+namespace pqhsa {
+namespace {
+
+constexpr float kTcScale = 256.f;              // 2^8 on each side of a product
+constexpr float kTcUnscale = 1.f / (kTcScale * kTcScale);
+constexpr float kTcFar = 60000.f;              // |c|^2 term of a padding row: farther than any centre
+
+// ---- descriptors (PTX ISA, tcgen05 matrix and instruction descriptors)
+// K-major, no swizzle: chunk stride (between core matrices along k) and 8-row stride, in bytes.
+__device__ __forceinline__ uint64_t tc_desc(uint32_t saddr, uint32_t chunk_stride) {
+  return (uint64_t)((saddr & 0x3ffffu) >> 4) | ((uint64_t)(chunk_stride >> 4) << 16) |
+         ((uint64_t)(128u >> 4) << 32) | (1ull << 46);
+}
+// fp16 x fp16 -> fp32, both K-major, M = 128
+__device__ __forceinline__ constexpr uint32_t tc_idesc(uint32_t n) {
+  return (1u << 4) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+}
+// D[tmem] (+)= A B^T for one K = 16 step; one thread
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory");
+}
+// the mbarrier gets one arrival when all MMAs issued by this thread so far are complete
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+               ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// generic shared-memory stores become visible to the tensor core
+__device__ __forceinline__ void tc_fence_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// one whole warp; the address lands in *slot.  n_cols: power of two, 32 .. 512
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t n_cols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(n_cols) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tmem_free(uint32_t addr, uint32_t n_cols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(n_cols));
+}
+// 32 (16) consecutive columns of this thread's TMEM lane (lane = row of the tile); whole warp
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void group_sync(int id) {      // the 128 threads of a warpgroup
+  asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory");
+}
+
+// bounded wait for a commit (see mbar_wait; an MMA takes microseconds at most)
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity) {
+  for (int it = 0; it < (1 << 16); ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+// ---- fp16 split
+__device__ __forceinline__ void split16(float v, __half& hi, __half& lo) {
+  hi = __float2half_rn(v);
+  lo = __float2half_rn(v - __half2float(hi));
+}
+__device__ __forceinline__ uint32_t pack16(__half a, __half b) {
+  const __half2 h = __halves2half2(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+// 8 values, scaled, as a chunk of hi and a chunk of lo
+__device__ __forceinline__ void split_chunk(const float (&v)[8], float scale, uint4& hi, uint4& lo) {
+  __half h[8], l[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) split16(scale * v[i], h[i], l[i]);
+  hi = make_uint4(pack16(h[0], h[1]), pack16(h[2], h[3]), pack16(h[4], h[5]), pack16(h[6], h[7]));
+  lo = make_uint4(pack16(l[0], l[1]), pack16(l[2], l[3]), pack16(l[4], l[5]), pack16(l[6], l[7]));
+}
+// |c|^2 as three fp16 terms (33 bits) against the constant 256 on the other side
+__device__ __forceinline__ void split_norm(float n2, __half (&h)[3]) {
+  const float v = kTcScale * n2;
+  h[0] = __float2half_rn(v);
+  const float r1 = v - __half2float(h[0]);
+  h[1] = __float2half_rn(r1);
+  h[2] = __float2half_rn(r1 - __half2float(h[1]));
+}
+
+// ---- coarse search: 128-dim rows; chunks 0-15 hi, 16-31 lo, 32 the |c|^2 terms, 33 zero
+constexpr int kCoarseChunks = 34;
+// the 25 K-steps of one tile (the cross terms first: they are 2^-11 of the rest, so that only nine
+// accumulations round at full magnitude)
+__device__ __forceinline__ void tc_coarse_tile(uint32_t d, uint32_t sa, uint32_t rows_a, uint32_t sb, uint32_t rows_b) {
+  const uint32_t idesc = tc_idesc(rows_b), ca = rows_a * 16u, cb = rows_b * 16u;
+#pragma unroll 1
+  for (uint32_t s = 0; s < 16; s += 2) {
+    tc_mma(d, tc_desc(sa + s * ca, ca), tc_desc(sb + (16u + s) * cb, cb), idesc, s != 0);
+    tc_mma(d, tc_desc(sa + (16u + s) * ca, ca), tc_desc(sb + s * cb, cb), idesc, true);
+  }
+#pragma unroll 1
+  for (uint32_t s = 0; s < 16; s += 2) tc_mma(d, tc_desc(sa + s * ca, ca), tc_desc(sb + s * cb, cb), idesc, true);
+  tc_mma(d, tc_desc(sa + 32u * ca, ca), tc_desc(sb + 32u * cb, cb), idesc, true);
+}
+__device__ __forceinline__ uint4 coarse_ext_row() {       // the row side of chunk 32
+  const __half c = __float2half_rn(kTcScale), z = __float2half_rn(0.f);
+  return make_uint4(pack16(c, c), pack16(c, z), 0u, 0u);
+}
+__device__ __forceinline__ uint4 coarse_ext_centre(float n2, bool real) {
+  __half h[3];
+  split_norm(real ? n2 : 0.f, h);
+  if (!real) h[0] = __float2half_rn(kTcFar);
+  return make_uint4(pack16(h[0], h[1]), pack16(h[2], __float2half_rn(0.f)), 0u, 0u);
+}
+
+// ---- codeword search: DSUB dims; one row is [hi | hi | lo | 256 256 256 | 0 ..] on the token side
+// and [hi | lo | hi | |p|^2 terms | 0 ..] on the codeword side, K padded to 16
+template <int DSUB> struct PqTile {
+  static constexpr int kK = (3 * DSUB + 3 + 15) / 16 * 16;
+  static constexpr int kChunks = kK / 8;
+  static __device__ __forceinline__ void token_row(const float (&e)[DSUB], uint4 (&c)[kChunks]) {
+    __half k[kK];
+#pragma unroll
+    for (int i = 0; i < kK; ++i) k[i] = __float2half_rn(0.f);
+#pragma unroll
+    for (int t = 0; t < DSUB; ++t) {
+      split16(kTcScale * e[t], k[t], k[2 * DSUB + t]);
+      k[DSUB + t] = k[t];
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) k[3 * DSUB + t] = __float2half_rn(kTcScale);
+    pack(k, c);
+  }
+  static __device__ __forceinline__ void code_row(const float (&p)[DSUB], uint4 (&c)[kChunks]) {
+    __half k[kK];
+#pragma unroll
+    for (int i = 0; i < kK; ++i) k[i] = __float2half_rn(0.f);
+    float n2 = 0.f;
+#pragma unroll
+    for (int t = 0; t < DSUB; ++t) {
+      split16(-2.f * kTcScale * p[t], k[t], k[DSUB + t]);
+      k[2 * DSUB + t] = k[t];
+      n2 = fmaf(p[t], p[t], n2);
+    }
+    __half h[3];
+    split_norm(n2, h);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) k[3 * DSUB + t] = h[t];
+    pack(k, c);
+  }
+  static __device__ __forceinline__ void pack(const __half (&k)[kK], uint4 (&c)[kChunks]) {
+#pragma unroll
+    for (int i = 0; i < kChunks; ++i)
+      c[i] = make_uint4(pack16(k[8 * i], k[8 * i + 1]), pack16(k[8 * i + 2], k[8 * i + 3]),
+                        pack16(k[8 * i + 4], k[8 * i + 5]), pack16(k[8 * i + 6], k[8 * i + 7]));
+  }
+  // 128 tokens x n codewords
+  static __device__ __forceinline__ void mma(uint32_t d, uint32_t sa, uint32_t sb, uint32_t n_rows_b, uint32_t n) {
+    const uint32_t ca = 128u * 16u, cb = n_rows_b * 16u;
+#pragma unroll
+    for (int s = 0; s < kChunks; s += 2)
+      tc_mma(d, tc_desc(sa + s * ca, ca), tc_desc(sb + s * cb, cb), tc_idesc(n), s != 0);
+  }
+};
+
+// Smallest of groups of 8 accumulators; `best` / `grp` keep the smallest group and the first one
+// that has it.  The codeword inside the group is found by the caller in fp32: two instructions less
+// per accumulator than carrying an index.
+__device__ __forceinline__ float min3(float a, float b, float c) { return fminf(fminf(a, b), c); }
+template <int N> __device__ __forceinline__ void group_minima(const float (&v)[N], int grp0, float& best, int& grp) {
+#pragma unroll
+  for (int g = 0; g < N / 8; ++g) {
+    const float* w = v + 8 * g;
+    const float m = min3(min3(w[0], w[1], w[2]), min3(w[3], w[4], w[5]), fminf(w[6], w[7]));
+    if (m < best) { best = m; grp = grp0 + g; }
+  }
+}
+
+}  // namespace
+}  // namespace pqhsa

@@ -4,25 +4,43 @@
 // a_i = the list whose centroid is nearest to u_i (squared Euclidean distance, lower index on
 // ties), z_im = the codeword nearest to the m-th sub-vector of the residual u_i - c_{a_i}.
 //
-//   index_encode_kernel         8 new tokens per CTA.  Centroids pass through shared memory
-//       in tiles of 32 rows (a lane owns a centroid, a warp a token); for the codes a warp owns
-//       a subspace and a lane a codeword, so a codebook row is read once, coalesced, for all 8
-//       tokens.  Writes codes, list ids and norms at the tokens' positions.
-//   index_refresh_means_kernel  one CTA per (sequence, KV head).  Groups the new tokens by list
-//       (first occurrence = leader), sums each group's value rows in token order and sets
-//       vbar_j = (n_j vbar_j + sum) / (n_j + new_j), n_j += new_j.
+//   index_encode_kernel         128 new tokens of one (sequence, KV head) per CTA.  Both searches
+//       are contractions and run on the tensor cores with split fp16 operands (tc.cuh): tiles of 128
+//       centroids, then every warpgroup takes every fourth subspace.
+//       The codeword is decided in fp32 among the 8 of the winning group.
+//   index_refresh_means_kernel  groups the new tokens by list (first occurrence = leader), sums
+//       each group's value rows in token order and sets vbar_j = (n_j vbar_j + sum) / (n_j + new_j),
+//       n_j += new_j; a warp per leader.
+// What bounds the encoding: per CTA the centroids (512 KB at 1024 lists) pass through registers once
+// to be split, and the tensor core re-reads the token tile for every 32 centroids.
 #include "attn_common.cuh"
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace pqhsa {
 
 namespace {
 
-constexpr int kUpdTok = 8;              // tokens per CTA = warps per CTA
-constexpr int kUpdThreads = 32 * kUpdTok;
-constexpr int kCTile = 32;              // centroid rows per shared-memory tile
-constexpr int kCStride = kHeadDim + 1;  // padded row: lane j reads row j without conflicts
+constexpr int kUpdTok = 128;            // tokens per CTA: rows of the tensor-core tile
+constexpr int kUpdGroups = 4;           // warpgroups
+constexpr int kUpdThreads = 128 * kUpdGroups;
+constexpr int kUpdWarps = kUpdThreads / 32;
+constexpr int kUpdCen = 128;            // centroids per tile, 32 columns per warpgroup
+constexpr int kUpdWords = 128;          // codewords per tile of a warpgroup
+constexpr int kUStride = kHeadDim + 4;  // floats per row of the directions in shared memory
 constexpr int kMaxNew = 1024;           // new tokens per sequence and call
+constexpr int kMeanTok = 16;            // positions per CTA of the means kernel: one per warp
+constexpr int kMeanThreads = 512;
+
+// dynamic shared memory: token tile and two centroid tiles; the residuals and the tiles of the
+// codeword search (token rows and codeword rows per warpgroup) take their place afterwards
+constexpr int kUpdU = kUpdTok * kUStride * 4;
+constexpr int kUpdA = kCoarseChunks * kUpdTok * 16;
+constexpr int kUpdB = kCoarseChunks * kUpdCen * 16;
+constexpr int kUpdSmem = kUpdA + 2 * kUpdB;
+constexpr int kUpdPq = (kUpdSmem - kUpdU) / kUpdGroups;     // codeword search, per warpgroup
+static_assert(kUpdU <= kUpdB, "the directions pass through a centroid tile's place");
+static_assert(2 * 8 * 128 * 16 <= kUpdPq && kUpdPq % 128 == 0, "codeword tiles of the widest subspace");
 
 // cache row of token `pos` of (sequence b, KV head kv), in elements
 __device__ __forceinline__ long long row_offset(const Plan& pl, const int32_t* __restrict__ bt,
@@ -34,19 +52,25 @@ __device__ __forceinline__ long long row_offset(const Plan& pl, const int32_t* _
 }
 
 template <typename T, int DSUB>
-__global__ void __launch_bounds__(kUpdThreads)
+__global__ void __launch_bounds__(kUpdThreads, 1)
 index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, long long stride_token,
                     long long stride_head, const int32_t* __restrict__ block_table,
                     const int32_t* __restrict__ first_pos, const int32_t* __restrict__ n_new,
                     int max_new, const float* __restrict__ centroids,
                     const float* __restrict__ codebooks, uint8_t* __restrict__ codes,
                     uint16_t* __restrict__ list_ids, float* __restrict__ key_norms) {
-  __shared__ float s_u[kUpdTok][kHeadDim];          // direction, later the residual
-  __shared__ float s_c[kCTile][kCStride];
-  __shared__ int s_a[kUpdTok];
-  __shared__ uint8_t s_code[kUpdTok][64];
+  extern __shared__ __align__(128) unsigned char s_dyn[];
+  unsigned char* s_a = s_dyn;
+  unsigned char* s_b = s_a + kUpdA;
+  __shared__ float s_inv[kUpdTok];
+  __shared__ float s_best[kUpdGroups][kUpdTok];
+  __shared__ uint16_t s_near[kUpdGroups][kUpdTok];
+  __shared__ __align__(16) uint8_t s_code[kUpdTok][64];
+  __shared__ uint32_t s_tmem;
+  __shared__ __align__(8) uint64_t s_bar[2 + kUpdGroups];        // centroid tiles, codeword tiles
   const int kv = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wg = tid >> 7, row = tid & 127, wq = warp & 3;  // warpgroup, tile row, warp in the group
   const size_t ukv = (size_t)b * pl.Hkv + kv;
   pdl_wait();
   pdl_launch_dependents();
@@ -57,110 +81,264 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
   const int p0 = first_pos[b] + t0;                 // position of this CTA's first token
   const int32_t* bt = block_table + (size_t)b * pl.max_pages;
   // tokens whose position falls outside the index rows are left alone
-  const bool mine_ok = warp < ntok && p0 + warp >= 0 && p0 + warp < pl.N_max;
+  auto ok = [&](int t) { return t < ntok && p0 + t >= 0 && p0 + t < pl.N_max; };
 
-  // ---- norm and direction: warp w <-> token w, a lane holds 4 of the 128 dims
-  {
-    float x[4] = {0.f, 0.f, 0.f, 0.f};
-    if (mine_ok) {
-      const T* row = kc + row_offset(pl, bt, p0 + warp, kv, stride_page, stride_token, stride_head);
+  if (warp == 0) tmem_alloc(&s_tmem, 512);
+  if (tid < 2 + kUpdGroups) mbar_init(&s_bar[tid], 1);
+  if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+
+  // ---- norms and directions: a warp per token, a lane holds 4 of the 128 dims
+  constexpr int kPer = kUpdTok / kUpdWarps;
+  auto load_rows = [&](float (&x)[kPer][4]) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) x[i] = Unpack<T>::one(row[4 * lane + i]);
+    for (int r = 0; r < kPer; ++r) {
+      const int t = r * kUpdWarps + warp;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[r][i] = 0.f;
+      if (ok(t)) load4<T>(kc + row_offset(pl, bt, p0 + t, kv, stride_page, stride_token, stride_head) + 4 * lane, x[r]);
     }
-    const float ss = warp_sum(x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3]);
-    const float r = sqrtf(ss);
-    const float inv = r > 0.f ? 1.f / r : 0.f;
+  };
+  {
+    float x[kPer][4];
+    load_rows(x);
+    float* s_u = reinterpret_cast<float*>(s_b);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) s_u[warp][4 * lane + i] = x[i] * inv;
-    if (mine_ok && lane == 0) key_norms[ukv * pl.N_max + p0 + warp] = r;
+    for (int r = 0; r < kPer; ++r) {
+      const int t = r * kUpdWarps + warp;
+      const float ss = warp_sum(x[r][0] * x[r][0] + x[r][1] * x[r][1] + x[r][2] * x[r][2] + x[r][3] * x[r][3]);
+      const float nr = sqrtf(ss);
+      const float inv = nr > 0.f ? 1.f / nr : 0.f;
+      *reinterpret_cast<float4*>(s_u + t * kUStride + 4 * lane) =
+          make_float4(x[r][0] * inv, x[r][1] * inv, x[r][2] * inv, x[r][3] * inv);
+      if (lane == 0) {
+        s_inv[t] = inv;
+        if (ok(t)) key_norms[ukv * pl.N_max + p0 + t] = nr;
+      }
+    }
   }
-
-  // ---- nearest centroid: |u - c|^2 = |u|^2 - 2 u.c + |c|^2, the first term is common
-  float best_d = CUDART_INF_F;
-  int best_j = 0;
+  // A warp splits 8 rows of a centroid tile: lane l holds row l & 7 and the chunks (l >> 3) + 4 i, so
+  // that loads take whole 128-byte lines and stores have no conflicts.  Fetched one tile ahead.
   const float* cbase = centroids + ukv * (size_t)pl.n_list * kHeadDim;
-  for (int c0 = 0; c0 < pl.n_list; c0 += kCTile) {
-    __syncthreads();                                // previous tile consumed, s_u complete
-    for (int i = tid; i < kCTile * (kHeadDim / 4); i += kUpdThreads) {
-      const int rr = i / (kHeadDim / 4), c4 = i % (kHeadDim / 4);
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c0 + rr < pl.n_list)
-        v = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)(c0 + rr) * kHeadDim) + c4);
-      s_c[rr][4 * c4] = v.x; s_c[rr][4 * c4 + 1] = v.y;
-      s_c[rr][4 * c4 + 2] = v.z; s_c[rr][4 * c4 + 3] = v.w;
-    }
-    __syncthreads();
-    float dot = 0.f, cn = 0.f;
-#pragma unroll 8
-    for (int d = 0; d < kHeadDim; ++d) {
-      const float c = s_c[lane][d];
-      dot = fmaf(s_u[warp][d], c, dot);
-      cn = fmaf(c, c, cn);
-    }
-    const float dist = fmaf(-2.f, dot, cn);
-    if (c0 + lane < pl.n_list && dist < best_d) { best_d = dist; best_j = c0 + lane; }
-  }
+  const int br = 8 * warp + (lane & 7), bc = lane >> 3;
+  float v[4][8];
+  auto fetch = [&](int c0) {
+    const bool real = c0 + br < pl.n_list;
+    const float4* src = reinterpret_cast<const float4*>(cbase + (size_t)(real ? c0 + br : 0) * kHeadDim);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float od = __shfl_xor_sync(0xffffffffu, best_d, o);
-    const int oj = __shfl_xor_sync(0xffffffffu, best_j, o);
-    if (od < best_d || (od == best_d && oj < best_j)) { best_d = od; best_j = oj; }
+    for (int i = 0; i < 4; ++i) {
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+      if (real) { x = __ldg(src + 2 * (bc + 4 * i)); y = __ldg(src + 2 * (bc + 4 * i) + 1); }
+      *reinterpret_cast<float4*>(v[i]) = x;
+      *reinterpret_cast<float4*>(v[i] + 4) = y;
+    }
+  };
+  fetch(0);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;
+  // ---- token tile: thread = row, a quarter of the dims each
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int c = 4 * wg + q;
+    const float* src = reinterpret_cast<const float*>(s_b) + row * kUStride + 8 * c;
+    float x[8];
+    *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(src);
+    *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(src + 4);
+    uint4 hi, lo;
+    split_chunk(x, kTcScale, hi, lo);
+    *reinterpret_cast<uint4*>(s_a + (c * kUpdTok + row) * 16) = hi;
+    *reinterpret_cast<uint4*>(s_a + ((16 + c) * kUpdTok + row) * 16) = lo;
   }
-  if (lane == 0) {
-    s_a[warp] = best_j;
-    if (mine_ok) list_ids[ukv * pl.N_max + p0 + warp] = (uint16_t)best_j;
+  if (wg == 0) *reinterpret_cast<uint4*>(s_a + (32 * kUpdTok + row) * 16) = coarse_ext_row();
+  if (wg == 1) *reinterpret_cast<uint4*>(s_a + (33 * kUpdTok + row) * 16) = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();                                          // the directions have been read
+
+  // ---- nearest centroid: tile i + 1 is split and its MMAs issued before tile i is looked at
+  auto put_tile = [&](int c0, unsigned char* dst) {
+    float n2 = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint4 hi, lo;
+      split_chunk(v[i], -2.f * kTcScale, hi, lo);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) n2 = fmaf(v[i][t], v[i][t], n2);
+      *reinterpret_cast<uint4*>(dst + ((bc + 4 * i) * kUpdCen + br) * 16) = hi;
+      *reinterpret_cast<uint4*>(dst + ((16 + bc + 4 * i) * kUpdCen + br) * 16) = lo;
+    }
+    n2 += __shfl_xor_sync(0xffffffffu, n2, 8);
+    n2 += __shfl_xor_sync(0xffffffffu, n2, 16);
+    if (bc == 0) *reinterpret_cast<uint4*>(dst + (32 * kUpdCen + br) * 16) = coarse_ext_centre(n2, c0 + br < pl.n_list);
+    if (bc == 1) *reinterpret_cast<uint4*>(dst + (33 * kUpdCen + br) * 16) = make_uint4(0u, 0u, 0u, 0u);
+  };
+  const uint32_t my_lanes = (uint32_t)(wq * 32) << 16;      // this warp's TMEM lanes
+  const int n_tiles = (pl.n_list + kUpdCen - 1) / kUpdCen;
+  float best = CUDART_INF_F;
+  int near = 0;
+  bool late = false;
+  for (int i = -1; i < n_tiles; ++i) {
+    if (i + 1 < n_tiles) {
+      unsigned char* dst = s_b + ((i + 1) & 1) * kUpdB;
+      put_tile((i + 1) * kUpdCen, dst);
+      if (i + 2 < n_tiles) fetch((i + 2) * kUpdCen);
+      tc_fence_smem();
+      tc_fence_before();
+      __syncthreads();
+      if (tid == 0) {
+        tc_fence_after();
+        tc_coarse_tile(tmem + ((i + 1) & 1) * kUpdCen, smem_u32(s_a), kUpdTok, smem_u32(dst), kUpdCen);
+        tc_commit(&s_bar[(i + 1) & 1]);
+      }
+      __syncwarp();
+    }
+    if (i < 0) continue;
+    late |= !tc_wait(&s_bar[i & 1], (uint32_t)(i >> 1) & 1u);
+    tc_fence_after();
+    float acc[32];
+    tmem_ld32(tmem + (i & 1) * kUpdCen + 32 * wg + my_lanes, acc);
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (acc[j] < best) { best = acc[j]; near = i * kUpdCen + 32 * wg + j; }     // ascending: the first minimum stays
   }
-  // ---- residual, in place
+  s_best[wg][row] = best;
+  s_near[wg][row] = (uint16_t)min(near, pl.n_list - 1);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
   {
-    const float4 c = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)best_j * kHeadDim) + lane);
-    s_u[warp][4 * lane] -= c.x; s_u[warp][4 * lane + 1] -= c.y;
-    s_u[warp][4 * lane + 2] -= c.z; s_u[warp][4 * lane + 3] -= c.w;
+    // the groups' minima (equal distances: lower index)
+    float d = s_best[0][row];
+    int j = s_near[0][row];
+#pragma unroll
+    for (int g = 1; g < kUpdGroups; ++g) {
+      const float od = s_best[g][row];
+      const int oj = s_near[g][row];
+      if (od < d || (od == d && oj < j)) { d = od; j = oj; }
+    }
+    near = j;
+  }
+  __syncthreads();
+  if (wg == 0) {
+    s_near[0][row] = (uint16_t)near;
+    if (ok(row)) list_ids[ukv * pl.N_max + p0 + row] = (uint16_t)near;
+  }
+  __syncthreads();
+  // ---- residuals, from the cache rows again (L2)
+  float* s_u = reinterpret_cast<float*>(s_dyn);
+  {
+    float x[kPer][4];
+    load_rows(x);
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+      const int t = r * kUpdWarps + warp;
+      const float inv = s_inv[t];
+      const float4 c = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)s_near[0][t] * kHeadDim) + lane);
+      *reinterpret_cast<float4*>(s_u + t * kUStride + 4 * lane) =
+          make_float4(__fmul_rn(x[r][0], inv) - c.x, __fmul_rn(x[r][1], inv) - c.y, __fmul_rn(x[r][2], inv) - c.z,
+                      __fmul_rn(x[r][3], inv) - c.w);
+    }
   }
   __syncthreads();
 
-  // ---- codes: warp <-> subspaces m = warp, warp + 8, ...; lane <-> codewords lane + 32 i
-  for (int m = warp; m < pl.M; m += kUpdTok) {
-    float bd[kUpdTok];
-    int bz[kUpdTok];
+  // ---- codes: group <-> subspaces wg, wg + 4, ..; thread = token, and codeword while a tile is made
+  using Tile = PqTile<DSUB>;
+  const uint32_t d_tmem = tmem + (uint32_t)wg * 128u;       // this group's accumulator columns
+  const uint32_t my_tmem = d_tmem + my_lanes;
+  uint32_t parity = 0u;
+  unsigned char* pa = s_dyn + kUpdU + wg * kUpdPq;
+  unsigned char* pb = pa + Tile::kChunks * 2048;
+  // the subspace's codewords in fp32 for the final decision, where they fit
+  float* s_word = reinterpret_cast<float*>(pb + Tile::kChunks * 2048);
+  const bool staged = 2 * Tile::kChunks * 2048 + pl.n_code * DSUB * 4 <= kUpdPq;
+  auto load_sub = [](const float* src, float (&x)[DSUB]) {
+    if constexpr (DSUB == 2) {
+      *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(src);
+    } else {
 #pragma unroll
-    for (int t = 0; t < kUpdTok; ++t) { bd[t] = CUDART_INF_F; bz[t] = 0; }
+      for (int c4 = 0; c4 < DSUB / 4; ++c4)
+        *reinterpret_cast<float4*>(x + 4 * c4) = *reinterpret_cast<const float4*>(src + 4 * c4);
+    }
+  };
+  const int words = min(kUpdWords, pl.n_code);
+  float p[DSUB];                                            // this thread's codeword, one tile ahead
+  auto fetch_word = [&](int m, int z0) {
+    if (row < words && m < pl.M) load_sub(codebooks + ((ukv * pl.M + m) * (size_t)pl.n_code + z0 + row) * DSUB, p);
+  };
+  fetch_word(wg, 0);
+  for (int m = wg; m < pl.M; m += kUpdGroups) {
     const float* cb = codebooks + (ukv * pl.M + m) * (size_t)pl.n_code * DSUB;
-    for (int z0 = 0; z0 < pl.n_code; z0 += 32) {
-      const int z = min(z0 + lane, pl.n_code - 1);      // lanes past the codebook repeat its last word
-      float p[DSUB];
-      if constexpr (DSUB == 2) {
-        const float2 v = __ldg(reinterpret_cast<const float2*>(cb + (size_t)z * DSUB));
-        p[0] = v.x; p[1] = v.y;
+    float e[DSUB];
+    load_sub(s_u + row * kUStride + m * DSUB, e);
+    uint4 ch[Tile::kChunks];
+    Tile::token_row(e, ch);
+#pragma unroll
+    for (int i = 0; i < Tile::kChunks; ++i) *reinterpret_cast<uint4*>(pa + (i * 128 + row) * 16) = ch[i];
+    float bd = CUDART_INF_F;
+    int grp = 0;
+    for (int z0 = 0; z0 < pl.n_code; z0 += kUpdWords) {
+      if (row < words) {
+        Tile::code_row(p, ch);
+        if (staged) {
+#pragma unroll
+          for (int t = 0; t < DSUB; ++t) s_word[(z0 + row) * DSUB + t] = p[t];
+        }
+#pragma unroll
+        for (int i = 0; i < Tile::kChunks; ++i) *reinterpret_cast<uint4*>(pb + (i * 128 + row) * 16) = ch[i];
+      }
+      tc_fence_smem();
+      tc_fence_before();
+      group_sync(1 + wg);
+      if (row == 0) {
+        tc_fence_after();
+        Tile::mma(d_tmem, smem_u32(pa), smem_u32(pb), 128u, (uint32_t)words);
+        tc_commit(&s_bar[2 + wg]);
+      }
+      if (z0 + kUpdWords < pl.n_code) fetch_word(m, z0 + kUpdWords);
+      else fetch_word(m + kUpdGroups, 0);
+      late |= !tc_wait(&s_bar[2 + wg], parity);
+      parity ^= 1u;
+      tc_fence_after();
+      if (pl.n_code == 16) {
+        float acc[16];
+        tmem_ld16(my_tmem, acc);
+        group_minima(acc, 0, bd, grp);
       } else {
 #pragma unroll
-        for (int c4 = 0; c4 < DSUB / 4; ++c4) {
-          const float4 v = __ldg(reinterpret_cast<const float4*>(cb + (size_t)z * DSUB) + c4);
-          p[4 * c4] = v.x; p[4 * c4 + 1] = v.y; p[4 * c4 + 2] = v.z; p[4 * c4 + 3] = v.w;
+        for (int c = 0; c < kUpdWords; c += 32) {
+          float acc[32];
+          tmem_ld32(my_tmem + c, acc);
+          group_minima(acc, (z0 + c) / 8, bd, grp);
         }
       }
+    }
+    // the winning group's codewords in fp32, first minimum.  The lanes start at different codewords:
+    // at 16 bytes a codeword the eight lanes of an access then hit eight different bank groups
+    float dm = CUDART_INF_F;
+    int bz = 0;
+    auto decide = [&](const float* words_of_m) {
 #pragma unroll
-      for (int t = 0; t < kUpdTok; ++t) {
+      for (int i = 0; i < 8; ++i) {
+        const int z = 8 * grp + ((i + lane) & 7);
+        float w[DSUB];
+        load_sub(words_of_m + z * DSUB, w);
         float dist = 0.f;
 #pragma unroll
         for (int dd = 0; dd < DSUB; ++dd) {
-          const float e = s_u[t][m * DSUB + dd] - p[dd];
-          dist = fmaf(e, e, dist);
+          const float x = e[dd] - w[dd];
+          dist = fmaf(x, x, dist);
         }
-        if (dist < bd[t]) { bd[t] = dist; bz[t] = z; }      // z ascends: first minimum stays
+        if (dist < dm || (dist == dm && z < bz)) { dm = dist; bz = z; }
       }
-    }
-#pragma unroll
-    for (int t = 0; t < kUpdTok; ++t) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float od = __shfl_xor_sync(0xffffffffu, bd[t], o);
-        const int oz = __shfl_xor_sync(0xffffffffu, bz[t], o);
-        if (od < bd[t] || (od == bd[t] && oz < bz[t])) { bd[t] = od; bz[t] = oz; }
-      }
-      if (lane == 0) s_code[t][m] = (uint8_t)bz[t];
-    }
+    };
+    if (staged) decide(s_word); else decide(cb);
+    group_sync(1 + wg);                              // (the codewords are overwritten next)
+    s_code[row][m] = (uint8_t)bz;
   }
+  tc_fence_before();
   __syncthreads();
+  if (warp == 0) { tc_fence_after(); tmem_free(tmem, 512); }
+  // a bounded wait ran out (no status word here): the tokens' norms say so
+  if (late && ok(row)) key_norms[ukv * pl.N_max + p0 + row] = CUDART_NAN_F;
   // one byte per code, or two 4-bit codes per byte (subspace 2j in the low nibble of byte j)
   for (int i = tid; i < ntok * pl.code_bytes; i += kUpdThreads) {
     const int t = i / pl.code_bytes, j = i - t * pl.code_bytes;
@@ -172,55 +350,56 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kUpdThreads)
+__global__ void __launch_bounds__(kMeanThreads)
 index_refresh_means_kernel(Plan pl, const T* __restrict__ vc, long long stride_page,
                            long long stride_token, long long stride_head,
                            const int32_t* __restrict__ block_table,
                            const int32_t* __restrict__ first_pos, const int32_t* __restrict__ n_new,
                            int max_new, const uint16_t* __restrict__ list_ids,
                            float* __restrict__ list_vmeans, int32_t* __restrict__ list_counts) {
+  extern __shared__ int s_first[];                   // [n_list] first new token of every list
   __shared__ uint16_t s_lid[kMaxNew];
-  __shared__ int s_lead[kMaxNew];
-  __shared__ uint32_t s_nlead;
-  const int kv = blockIdx.x, b = blockIdx.y;
+  const int kv = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const size_t ukv = (size_t)b * pl.Hkv + kv;
-  pdl_wait();                                        // the list ids come from the encode kernel
-  pdl_launch_dependents();
+  for (int j = tid; j < pl.n_list; j += kMeanThreads) s_first[j] = kMaxNew;
   const int p0 = first_pos[b];
   int nb = min(max(n_new[b], 0), max_new);
   if (p0 < 0) nb = 0;
   nb = min(nb, pl.N_max - p0);                       // same positions as the encode kernel
-  if (nb <= 0) return;
+  const int t_begin = blockIdx.x * kMeanTok, t_end = min(nb, t_begin + kMeanTok);
+  pdl_wait();                                        // the list ids come from the encode kernel
+  pdl_launch_dependents();
+  if (t_begin >= nb) return;
   const int32_t* bt = block_table + (size_t)b * pl.max_pages;
-  for (int t = tid; t < nb; t += kUpdThreads) s_lid[t] = list_ids[ukv * pl.N_max + p0 + t];
-  if (tid == 0) s_nlead = 0u;
   __syncthreads();
-  // leaders: the first new token of every list that received one
-  for (int t = tid; t < nb; t += kUpdThreads) {
-    const uint16_t j = s_lid[t];
-    bool first = true;
-    for (int e = 0; e < t; ++e) first = first && (s_lid[e] != j);
-    if (first) s_lead[atomicAdd(&s_nlead, 1u)] = t;
+  for (int t = tid; t < nb; t += kMeanThreads) {
+    const uint16_t j = (uint16_t)min((int)list_ids[ukv * pl.N_max + p0 + t], pl.n_list - 1);
+    s_lid[t] = j;
+    atomicMin(&s_first[j], t);
   }
   __syncthreads();
-  const int n_lead = (int)s_nlead;
-  for (int l = warp; l < n_lead; l += kUpdTok) {
-    const int t_first = s_lead[l];
-    const int j = s_lid[t_first];
+  for (int t1 = t_begin + warp; t1 < t_end; t1 += kMeanThreads / 32) {
+    const int j = s_lid[t1];
+    if (s_first[j] != t1) continue;                  // not a leader (warp-uniform)
+    float4* mean = reinterpret_cast<float4*>(list_vmeans + (ukv * pl.n_list + j) * kHeadDim) + lane;
+    float4 v = *mean;
+    const int n_old = list_counts[ukv * pl.n_list + j];
     float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
     int cnt = 0;
-    for (int t = t_first; t < nb; ++t) {             // token order: the sum is deterministic
-      if (s_lid[t] != j) continue;                   // warp-uniform
-      const T* row = vc + row_offset(pl, bt, p0 + t, kv, stride_page, stride_token, stride_head);
-      sum.x += Unpack<T>::one(row[4 * lane]);     sum.y += Unpack<T>::one(row[4 * lane + 1]);
-      sum.z += Unpack<T>::one(row[4 * lane + 2]); sum.w += Unpack<T>::one(row[4 * lane + 3]);
-      ++cnt;
+    for (int base = t1; base < nb; base += 32) {     // token order: the sum is deterministic
+      unsigned hit = __ballot_sync(0xffffffffu, base + lane < nb && s_lid[min(base + lane, nb - 1)] == j);
+      while (hit) {
+        const int t = base + __ffs(hit) - 1;
+        hit &= hit - 1u;
+        const T* src = vc + row_offset(pl, bt, p0 + t, kv, stride_page, stride_token, stride_head);
+        float x[4];
+        load4<T>(src + 4 * lane, x);
+        sum.x += x[0]; sum.y += x[1]; sum.z += x[2]; sum.w += x[3];
+        ++cnt;
+      }
     }
-    float4* mean = reinterpret_cast<float4*>(list_vmeans + (ukv * pl.n_list + j) * kHeadDim) + lane;
-    const int n_old = list_counts[ukv * pl.n_list + j];
     const float w_old = (float)n_old, inv = 1.f / (float)(n_old + cnt);
-    float4 v = *mean;
     v.x = (w_old * v.x + sum.x) * inv; v.y = (w_old * v.y + sum.y) * inv;
     v.z = (w_old * v.z + sum.z) * inv; v.w = (w_old * v.w + sum.w) * inv;
     *mean = v;
@@ -239,7 +418,10 @@ cudaError_t launch_update_t(const Plan& pl, const pqhsa_index_rw& ix, const pqhs
   cudaError_t e;
 #define PQHSA_UPD_CASE(D)                                                                       \
   case D:                                                                                       \
-    e = launch_pdl(index_encode_kernel<T, D>, grid, block, 0, st, pl, kc,                       \
+    e = cudaFuncSetAttribute(index_encode_kernel<T, D>,                                         \
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kUpdSmem);            \
+    if (e != cudaSuccess) return e;                                                             \
+    e = launch_pdl(index_encode_kernel<T, D>, grid, block, kUpdSmem, st, pl, kc,                \
                    (long long)kv.stride_page, (long long)kv.stride_token,                       \
                    (long long)kv.stride_head, kv.block_table, first_pos, n_new, max_new,        \
                    ix.centroids, ix.codebooks, ix.codes, ix.list_ids, ix.key_norms);            \
@@ -250,7 +432,8 @@ cudaError_t launch_update_t(const Plan& pl, const pqhsa_index_rw& ix, const pqhs
   }
 #undef PQHSA_UPD_CASE
   if (e != cudaSuccess) return e;
-  return launch_pdl(index_refresh_means_kernel<T>, dim3(pl.Hkv, pl.B), block, 0, st, pl, vc,
+  return launch_pdl(index_refresh_means_kernel<T>, dim3((max_new + kMeanTok - 1) / kMeanTok, pl.Hkv, pl.B),
+                    dim3(kMeanThreads), (size_t)pl.n_list * 4, st, pl, vc,
                     (long long)kv.stride_page, (long long)kv.stride_token,
                     (long long)kv.stride_head, kv.block_table, first_pos, n_new, max_new,
                     static_cast<const uint16_t*>(ix.list_ids), ix.list_vmeans, ix.list_counts);
