@@ -101,56 +101,57 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-// ---- fp16 split
-__device__ __forceinline__ void split16(float v, __half& hi, __half& lo) {
-  hi = __float2half_rn(v);
-  lo = __float2half_rn(v - __half2float(hi));
-}
-__device__ __forceinline__ uint32_t pack16(__half a, __half b) {
-  const __half2 h = __halves2half2(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
+// ---- fp16 split.  Always two values at a time: the packed conversion runs on the integer pipe, the
+// single one on the transcendental unit at an eighth of the rate.
+__device__ __forceinline__ uint32_t bits16(__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); }
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  hi = bits16(h);
+  lo = bits16(__floats2half2_rn(a - f.x, b - f.y));
 }
 // 8 values, scaled, as a chunk of hi and a chunk of lo
 __device__ __forceinline__ void split_chunk(const float (&v)[8], float scale, uint4& hi, uint4& lo) {
-  __half h[8], l[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) split16(scale * v[i], h[i], l[i]);
-  hi = make_uint4(pack16(h[0], h[1]), pack16(h[2], h[3]), pack16(h[4], h[5]), pack16(h[6], h[7]));
-  lo = make_uint4(pack16(l[0], l[1]), pack16(l[2], l[3]), pack16(l[4], l[5]), pack16(l[6], l[7]));
+  split2(scale * v[0], scale * v[1], hi.x, lo.x);
+  split2(scale * v[2], scale * v[3], hi.y, lo.y);
+  split2(scale * v[4], scale * v[5], hi.z, lo.z);
+  split2(scale * v[6], scale * v[7], hi.w, lo.w);
 }
-// |c|^2 as three fp16 terms (33 bits) against the constant 256 on the other side
-__device__ __forceinline__ void split_norm(float n2, __half (&h)[3]) {
+// |c|^2 as three fp16 terms (33 bits) against the constant 256 on the other side: the first two in
+// one word, the third in the low half of the next
+__device__ __forceinline__ void split_norm(float n2, uint32_t& w0, uint32_t& w1) {
   const float v = kTcScale * n2;
-  h[0] = __float2half_rn(v);
-  const float r1 = v - __half2float(h[0]);
-  h[1] = __float2half_rn(r1);
-  h[2] = __float2half_rn(r1 - __half2float(h[1]));
+  const float r1 = v - __low2float(__floats2half2_rn(v, 0.f));
+  const __half2 h = __floats2half2_rn(v, r1);
+  w0 = bits16(h);
+  w1 = bits16(__floats2half2_rn(r1 - __high2float(h), 0.f));
 }
 
 // ---- coarse search: 128-dim rows; chunks 0-15 hi, 16-31 lo, 32 the |c|^2 terms, 33 zero
 constexpr int kCoarseChunks = 34;
-// the 25 K-steps of one tile (the cross terms first: they are 2^-11 of the rest, so that only nine
-// accumulations round at full magnitude)
-__device__ __forceinline__ void tc_coarse_tile(uint32_t d, uint32_t sa, uint32_t rows_a, uint32_t sb, uint32_t rows_b) {
-  const uint32_t idesc = tc_idesc(rows_b), ca = rows_a * 16u, cb = rows_b * 16u;
-#pragma unroll 1
+// The 25 K-steps of one tile (the cross terms first: they are 2^-11 of the rest, so that only nine
+// accumulations round at full magnitude).  Unrolled over constant descriptor offsets: an MMA then
+// costs its 64 clocks at 128 x 128; with descriptors formed in a loop the issue alone took 148.
+template <uint32_t kRowsA, uint32_t kRowsB>
+__device__ __forceinline__ void tc_coarse_tile(uint32_t d, uint32_t sa, uint32_t sb) {
+  constexpr uint32_t idesc = tc_idesc(kRowsB);
+  const uint64_t a = tc_desc(sa, kRowsA * 16u), b = tc_desc(sb, kRowsB * 16u);
+#pragma unroll
   for (uint32_t s = 0; s < 16; s += 2) {
-    tc_mma(d, tc_desc(sa + s * ca, ca), tc_desc(sb + (16u + s) * cb, cb), idesc, s != 0);
-    tc_mma(d, tc_desc(sa + (16u + s) * ca, ca), tc_desc(sb + s * cb, cb), idesc, true);
+    tc_mma(d, a + s * kRowsA, b + (16u + s) * kRowsB, idesc, s != 0);     // (offsets in 16-byte units)
+    tc_mma(d, a + (16u + s) * kRowsA, b + s * kRowsB, idesc, true);
   }
-#pragma unroll 1
-  for (uint32_t s = 0; s < 16; s += 2) tc_mma(d, tc_desc(sa + s * ca, ca), tc_desc(sb + s * cb, cb), idesc, true);
-  tc_mma(d, tc_desc(sa + 32u * ca, ca), tc_desc(sb + 32u * cb, cb), idesc, true);
+#pragma unroll
+  for (uint32_t s = 0; s < 16; s += 2) tc_mma(d, a + s * kRowsA, b + s * kRowsB, idesc, true);
+  tc_mma(d, a + 32u * kRowsA, b + 32u * kRowsB, idesc, true);
 }
 __device__ __forceinline__ uint4 coarse_ext_row() {       // the row side of chunk 32
-  const __half c = __float2half_rn(kTcScale), z = __float2half_rn(0.f);
-  return make_uint4(pack16(c, c), pack16(c, z), 0u, 0u);
+  return make_uint4(bits16(__floats2half2_rn(kTcScale, kTcScale)), bits16(__floats2half2_rn(kTcScale, 0.f)), 0u, 0u);
 }
 __device__ __forceinline__ uint4 coarse_ext_centre(float n2, bool real) {
-  __half h[3];
-  split_norm(real ? n2 : 0.f, h);
-  if (!real) h[0] = __float2half_rn(kTcFar);
-  return make_uint4(pack16(h[0], h[1]), pack16(h[2], __float2half_rn(0.f)), 0u, 0u);
+  uint32_t w0, w1;
+  split_norm(n2, w0, w1);
+  return real ? make_uint4(w0, w1, 0u, 0u) : make_uint4(bits16(__floats2half2_rn(kTcFar, 0.f)), 0u, 0u, 0u);
 }
 
 // ---- codeword search: DSUB dims; one row is [hi | hi | lo | 256 256 256 | 0 ..] on the token side
@@ -158,48 +159,46 @@ __device__ __forceinline__ uint4 coarse_ext_centre(float n2, bool real) {
 template <int DSUB> struct PqTile {
   static constexpr int kK = (3 * DSUB + 3 + 15) / 16 * 16;
   static constexpr int kChunks = kK / 8;
+  // (DSUB is even, so whole words of two: DSUB / 2 words per copy, the norm's words behind them)
   static __device__ __forceinline__ void token_row(const float (&e)[DSUB], uint4 (&c)[kChunks]) {
-    __half k[kK];
+    uint32_t w[kK / 2];
 #pragma unroll
-    for (int i = 0; i < kK; ++i) k[i] = __float2half_rn(0.f);
+    for (int i = 0; i < kK / 2; ++i) w[i] = 0u;
 #pragma unroll
-    for (int t = 0; t < DSUB; ++t) {
-      split16(kTcScale * e[t], k[t], k[2 * DSUB + t]);
-      k[DSUB + t] = k[t];
+    for (int t = 0; t < DSUB / 2; ++t) {
+      split2(kTcScale * e[2 * t], kTcScale * e[2 * t + 1], w[t], w[DSUB + t]);
+      w[DSUB / 2 + t] = w[t];
     }
-#pragma unroll
-    for (int t = 0; t < 3; ++t) k[3 * DSUB + t] = __float2half_rn(kTcScale);
-    pack(k, c);
+    w[3 * DSUB / 2] = bits16(__floats2half2_rn(kTcScale, kTcScale));
+    w[3 * DSUB / 2 + 1] = bits16(__floats2half2_rn(kTcScale, 0.f));
+    pack(w, c);
   }
   static __device__ __forceinline__ void code_row(const float (&p)[DSUB], uint4 (&c)[kChunks]) {
-    __half k[kK];
+    uint32_t w[kK / 2];
 #pragma unroll
-    for (int i = 0; i < kK; ++i) k[i] = __float2half_rn(0.f);
+    for (int i = 0; i < kK / 2; ++i) w[i] = 0u;
     float n2 = 0.f;
 #pragma unroll
-    for (int t = 0; t < DSUB; ++t) {
-      split16(-2.f * kTcScale * p[t], k[t], k[DSUB + t]);
-      k[2 * DSUB + t] = k[t];
-      n2 = fmaf(p[t], p[t], n2);
+    for (int t = 0; t < DSUB / 2; ++t) {
+      split2(-2.f * kTcScale * p[2 * t], -2.f * kTcScale * p[2 * t + 1], w[t], w[DSUB / 2 + t]);
+      w[DSUB + t] = w[t];
     }
-    __half h[3];
-    split_norm(n2, h);
 #pragma unroll
-    for (int t = 0; t < 3; ++t) k[3 * DSUB + t] = h[t];
-    pack(k, c);
+    for (int t = 0; t < DSUB; ++t) n2 = fmaf(p[t], p[t], n2);
+    split_norm(n2, w[3 * DSUB / 2], w[3 * DSUB / 2 + 1]);
+    pack(w, c);
   }
-  static __device__ __forceinline__ void pack(const __half (&k)[kK], uint4 (&c)[kChunks]) {
+  static __device__ __forceinline__ void pack(const uint32_t (&w)[kK / 2], uint4 (&c)[kChunks]) {
 #pragma unroll
-    for (int i = 0; i < kChunks; ++i)
-      c[i] = make_uint4(pack16(k[8 * i], k[8 * i + 1]), pack16(k[8 * i + 2], k[8 * i + 3]),
-                        pack16(k[8 * i + 4], k[8 * i + 5]), pack16(k[8 * i + 6], k[8 * i + 7]));
+    for (int i = 0; i < kChunks; ++i) c[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
   }
-  // 128 tokens x n codewords
-  static __device__ __forceinline__ void mma(uint32_t d, uint32_t sa, uint32_t sb, uint32_t n_rows_b, uint32_t n) {
-    const uint32_t ca = 128u * 16u, cb = n_rows_b * 16u;
+  // 128 tokens x n codewords (chunks of kRowsB rows)
+  template <uint32_t kRowsB>
+  static __device__ __forceinline__ void mma(uint32_t d, uint32_t sa, uint32_t sb, uint32_t n) {
+    const uint64_t a = tc_desc(sa, 128u * 16u), b = tc_desc(sb, kRowsB * 16u);
+    const uint32_t idesc = tc_idesc(n);
 #pragma unroll
-    for (int s = 0; s < kChunks; s += 2)
-      tc_mma(d, tc_desc(sa + s * ca, ca), tc_desc(sb + s * cb, cb), tc_idesc(n), s != 0);
+    for (uint32_t s = 0; s < kChunks; s += 2) tc_mma(d, a + s * 128u, b + s * kRowsB, idesc, s != 0);
   }
 };
 

@@ -62,7 +62,6 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
   extern __shared__ __align__(128) unsigned char s_dyn[];
   unsigned char* s_a = s_dyn;
   unsigned char* s_b = s_a + kUpdA;
-  __shared__ float s_inv[kUpdTok];
   __shared__ float s_best[kUpdGroups][kUpdTok];
   __shared__ uint16_t s_near[kUpdGroups][kUpdTok];
   __shared__ __align__(16) uint8_t s_code[kUpdTok][64];
@@ -89,31 +88,35 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
 
   // ---- norms and directions: a warp per token, a lane holds 4 of the 128 dims
   constexpr int kPer = kUpdTok / kUpdWarps;
-  auto load_rows = [&](float (&x)[kPer][4]) {
+  uint2 raw[kPer];                                          // (kept for the residuals)
+  float inv[kPer];
 #pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-      const int t = r * kUpdWarps + warp;
+  for (int r = 0; r < kPer; ++r) {
+    const int t = r * kUpdWarps + warp;
+    raw[r] = make_uint2(0u, 0u);
+    if (ok(t))
+      raw[r] = __ldg(reinterpret_cast<const uint2*>(kc + row_offset(pl, bt, p0 + t, kv, stride_page, stride_token, stride_head)) + lane);
+  }
+  auto direction = [&](int r, float (&x)[4]) {
+    float f[8];
+    Unpack<T>::run(make_uint4(raw[r].x, raw[r].y, 0u, 0u), f);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) x[r][i] = 0.f;
-      if (ok(t)) load4<T>(kc + row_offset(pl, bt, p0 + t, kv, stride_page, stride_token, stride_head) + 4 * lane, x[r]);
-    }
+    for (int i = 0; i < 4; ++i) x[i] = __fmul_rn(f[i], inv[r]);      // (not contracted into what follows)
   };
   {
-    float x[kPer][4];
-    load_rows(x);
     float* s_u = reinterpret_cast<float*>(s_b);
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
       const int t = r * kUpdWarps + warp;
-      const float ss = warp_sum(x[r][0] * x[r][0] + x[r][1] * x[r][1] + x[r][2] * x[r][2] + x[r][3] * x[r][3]);
+      float x[4];
+      inv[r] = 1.f;
+      direction(r, x);
+      const float ss = warp_sum(x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3]);
       const float nr = sqrtf(ss);
-      const float inv = nr > 0.f ? 1.f / nr : 0.f;
-      *reinterpret_cast<float4*>(s_u + t * kUStride + 4 * lane) =
-          make_float4(x[r][0] * inv, x[r][1] * inv, x[r][2] * inv, x[r][3] * inv);
-      if (lane == 0) {
-        s_inv[t] = inv;
-        if (ok(t)) key_norms[ukv * pl.N_max + p0 + t] = nr;
-      }
+      inv[r] = nr > 0.f ? 1.f / nr : 0.f;
+      direction(r, x);
+      *reinterpret_cast<float4*>(s_u + t * kUStride + 4 * lane) = make_float4(x[0], x[1], x[2], x[3]);
+      if (lane == 0 && ok(t)) key_norms[ukv * pl.N_max + p0 + t] = nr;
     }
   }
   // A warp splits 8 rows of a centroid tile: lane l holds row l & 7 and the chunks (l >> 3) + 4 i, so
@@ -186,7 +189,7 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
       __syncthreads();
       if (tid == 0) {
         tc_fence_after();
-        tc_coarse_tile(tmem + ((i + 1) & 1) * kUpdCen, smem_u32(s_a), kUpdTok, smem_u32(dst), kUpdCen);
+        tc_coarse_tile<kUpdTok, kUpdCen>(tmem + ((i + 1) & 1) * kUpdCen, smem_u32(s_a), smem_u32(dst));
         tc_commit(&s_bar[(i + 1) & 1]);
       }
       __syncwarp();
@@ -223,19 +226,19 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
     if (ok(row)) list_ids[ukv * pl.N_max + p0 + row] = (uint16_t)near;
   }
   __syncthreads();
-  // ---- residuals, from the cache rows again (L2)
+  // ---- residuals
   float* s_u = reinterpret_cast<float*>(s_dyn);
   {
-    float x[kPer][4];
-    load_rows(x);
+    float4 c[kPer];
+#pragma unroll
+    for (int r = 0; r < kPer; ++r)
+      c[r] = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)s_near[0][r * kUpdWarps + warp] * kHeadDim) + lane);
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
-      const int t = r * kUpdWarps + warp;
-      const float inv = s_inv[t];
-      const float4 c = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)s_near[0][t] * kHeadDim) + lane);
-      *reinterpret_cast<float4*>(s_u + t * kUStride + 4 * lane) =
-          make_float4(__fmul_rn(x[r][0], inv) - c.x, __fmul_rn(x[r][1], inv) - c.y, __fmul_rn(x[r][2], inv) - c.z,
-                      __fmul_rn(x[r][3], inv) - c.w);
+      float x[4];
+      direction(r, x);
+      *reinterpret_cast<float4*>(s_u + (r * kUpdWarps + warp) * kUStride + 4 * lane) =
+          make_float4(x[0] - c[r].x, x[1] - c[r].y, x[2] - c[r].z, x[3] - c[r].w);
     }
   }
   __syncthreads();
@@ -290,7 +293,7 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
       group_sync(1 + wg);
       if (row == 0) {
         tc_fence_after();
-        Tile::mma(d_tmem, smem_u32(pa), smem_u32(pb), 128u, (uint32_t)words);
+        Tile::template mma<128>(d_tmem, smem_u32(pa), smem_u32(pb), (uint32_t)words);
         tc_commit(&s_bar[2 + wg]);
       }
       if (z0 + kUpdWords < pl.n_code) fetch_word(m, z0 + kUpdWords);
