@@ -10,22 +10,20 @@
 //
 //   build_prepare_kernel     norms and unit directions U (fp32, workspace) from the paged cache
 //   build_seed_kernel        centroids <- U rows at the given positions
-//   build_assign_kernel      nearest centroid of every token: a register-tiled fp32 product
-//                            U (128 tokens) x C^T (64 centroids at a time) with the argmin fused
-//                            into its epilogue; distance = (|u|^2 - 2 u.c) + |c|^2, the form the
-//                            reference builder uses.  No tensor cores: the argmin flips under
-//                            tf32 / bf16 rounding, and a split-precision tensor-core product
-//                            with an exact re-check of near-ties is future work.  This kernel
-//                            is bound by the fp32 FMA pipe (2 * 128 * n_list flops per token
-//                            against 512 bytes), not by memory.
-//   build_accumulate_kernel  per-list sums of the member directions (64-bit fixed point, so the
-//                            result does not depend on the order of the atomics) and member
-//                            counts; build_update_centroids_kernel takes the mean
-//   build_reseed_kernel      empty lists take the farthest points (rare)
-//   build_pq_* kernels       the same three steps for the residual sub-vectors
-//   build_value_* kernels    list value means and member counts from the paged values
+//   build_split_kernel       centroids as split fp16 tensor-core tiles (tc.cuh), once per iteration
+//   build_assign_kernel      nearest centroid of 256 tokens per CTA on the tensor cores
+//   build_hist / _offsets / _scatter   the tokens of a unit grouped by list (counting sort)
+//   build_dir_sums_kernel    per-list sums of the member directions (64-bit fixed point, so the
+//                            result does not depend on the order of the atomics): a warp sums the
+//                            rows of consecutive grouped tokens and adds once per list it meets
+//   build_update_centroids_kernel   takes the mean; build_reseed_kernel: empty lists take the
+//                            farthest points (rare)
+//   build_residual_kernel    U <- U - c_a, in place
+//   build_pq_* kernels       the same steps for the residual sub-vectors, also on the tensor cores
+//   build_value_* kernels    list value means and member counts from the paged values, in list order
 #include "attn_common.cuh"
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace pqhsa {
 
@@ -41,9 +39,6 @@ constexpr int kPrepThreads = 256;
 // 2^58); values are cache-dtype numbers (scale 2^24, exact for bf16 / fp16 inputs up to 2^15).
 constexpr float kFixDir = 1099511627776.0f;      // 2^40
 constexpr float kFixVal = 16777216.0f;           // 2^24
-__device__ __forceinline__ void fix_add(long long* dst, float v, float scale) {
-  atomicAdd(reinterpret_cast<unsigned long long*>(dst), (unsigned long long)__float2ll_rn(v * scale));
-}
 __device__ __forceinline__ float fix_mean(long long s, int count, float scale) {
   return (float)(((double)s / (double)scale) / (double)count);
 }
@@ -68,8 +63,7 @@ build_prepare_kernel(Plan pl, const T* __restrict__ kc, long long sp, long long 
   for (int i = blockIdx.x * (kPrepThreads / 32) + warp; i < n; i += gridDim.x * (kPrepThreads / 32)) {
     const T* row = kc + kv_row(pl, bt, i, kv, sp, st, sh);
     float x[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) x[t] = Unpack<T>::one(row[4 * lane + t]);
+    load4<T>(row + 4 * lane, x);
     const float ss = warp_sum(x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3]);
     const float r = sqrtf(ss);
     const float inv = r > 0.f ? 1.f / r : 0.f;
@@ -92,135 +86,344 @@ __global__ void build_seed_kernel(Plan pl, const float* __restrict__ U,
   *reinterpret_cast<float4*>(dst + (unit * n_rows + j) * kD + 4 * lane) = v;
 }
 
-// ---- nearest centroid.  CTA: 128 tokens of one unit; 256 threads as 16 x 16; thread (ty, tx)
-// owns tokens ty + 16 i (i < 8) and, of every 64-centroid tile, centroids tx + 16 j (j < 4).
-// Both tiles sit in shared memory row-major with a stride of 132 floats, so that the float4
-// reads along the dims are conflict free (the rows a quarter warp reads start 4 banks apart).
-constexpr int kAsgTok = 128, kAsgCen = 64, kAsgThreads = 256, kAsgStride = kD + 4;
-constexpr int kAsgSmemBytes = (kAsgTok + kAsgCen) * kAsgStride * 4 + kAsgCen * 4;
+// ---- centroids as tensor-core tiles: 64 rows in the layout of the coarse search, the factor -2 and
+// |c|^2 included; rows past n_list are farther than any centroid
+constexpr int kAsgTok = 256, kAsgCen = 64, kAsgThreads = 288;
+constexpr int kCenTileBytes = kCoarseChunks * kAsgCen * 16;       // 34816
+constexpr int kTokTileBytes = kCoarseChunks * 128 * 16;           // 69632
+constexpr float kNearTie = 4e-6f * kTcScale * kTcScale;          // 4e-6 of a squared distance
+constexpr int kAsgSmemBytes = 2 * kTokTileBytes + 2 * kCenTileBytes;
 
-__global__ void __launch_bounds__(kAsgThreads, 2)
-build_assign_kernel(Plan pl, const float* __restrict__ U, const float* __restrict__ centroids,
-                    const int32_t* __restrict__ seq_lens, uint16_t* __restrict__ list_ids,
-                    float* __restrict__ dmin) {
-  extern __shared__ __align__(16) float s_asg[];
-  float* s_u = s_asg;                                   // [128][132]
-  float* s_c = s_u + kAsgTok * kAsgStride;              // [64][132]
-  float* s_cn = s_c + kAsgCen * kAsgStride;             // [64] |c|^2
-  const int kv = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
+// 8 rows of 128 fp32 into a tile: lane l holds row l & 7 and the chunks (l >> 3) + 4 i, so that loads
+// take whole 128-byte lines and stores have no conflicts.  Returns |row|^2 (all lanes of the row).
+__device__ __forceinline__ float split_rows(const float* __restrict__ src, bool real, float scale,
+                                            unsigned char* dst, int rows, int r, int lane) {
+  const int c0 = lane >> 3;
+  float n2 = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (real) {
+      *reinterpret_cast<float4*>(v) = __ldcg(reinterpret_cast<const float4*>(src) + 2 * (c0 + 4 * i));
+      *reinterpret_cast<float4*>(v + 4) = __ldcg(reinterpret_cast<const float4*>(src) + 2 * (c0 + 4 * i) + 1);
+    }
+    uint4 hi, lo;
+    split_chunk(v, scale, hi, lo);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) n2 = fmaf(v[t], v[t], n2);
+    *reinterpret_cast<uint4*>(dst + ((c0 + 4 * i) * rows + r) * 16) = hi;
+    *reinterpret_cast<uint4*>(dst + ((16 + c0 + 4 * i) * rows + r) * 16) = lo;
+  }
+  n2 += __shfl_xor_sync(0xffffffffu, n2, 8);
+  n2 += __shfl_xor_sync(0xffffffffu, n2, 16);
+  return n2;
+}
+
+__global__ void __launch_bounds__(256)
+build_split_kernel(Plan pl, const float* __restrict__ centroids, unsigned char* __restrict__ images) {
+  const size_t unit = blockIdx.y;
+  const int lane = threadIdx.x & 31, r = (threadIdx.x >> 5) * 8 + (lane & 7);
+  const int j = blockIdx.x * kAsgCen + r;
+  unsigned char* dst = images + (unit * gridDim.x + blockIdx.x) * (size_t)kCenTileBytes;
+  const bool real = j < pl.n_list;
+  const float n2 = split_rows(centroids + (unit * pl.n_list + (real ? j : 0)) * kD, real, -2.f * kTcScale, dst,
+                              kAsgCen, r, lane);
+  if (lane < 8) *reinterpret_cast<uint4*>(dst + (32 * kAsgCen + r) * 16) = coarse_ext_centre(n2, real);
+  else if (lane < 16) *reinterpret_cast<uint4*>(dst + (33 * kAsgCen + r) * 16) = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// ---- nearest centroid.  CTA: 256 tokens of one unit as two 128-row tiles that stay in shared
+// memory, while the centroid tiles (64 rows, 34 KB, already in the tensor core's layout) stream
+// through two stages by bulk copies: 256 tokens per stage keep the L2 reads at 15 bytes per clock
+// and SM.  Warp 8 copies and issues; warpgroup w reads the accumulators of token tile w (64 columns,
+// double buffered) and keeps the minimum.  What bounds it: the MMAs (25 K-steps per tile pair at 48
+// clocks: shared-memory operand reads), then the split of the token tile at the start.
+__global__ void __launch_bounds__(kAsgThreads, 1)
+build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* __restrict__ images,
+                    const float* __restrict__ centroids, const int32_t* __restrict__ seq_lens,
+                    uint16_t* __restrict__ list_ids, float* __restrict__ dmin, float* __restrict__ key_norms) {
+  extern __shared__ __align__(128) unsigned char s_asg[];
+  unsigned char* s_tok = s_asg;                             // two token tiles
+  unsigned char* s_cen = s_asg + 2 * kTokTileBytes;         // two centroid stages
+  __shared__ float s_x2[kAsgTok];
+  __shared__ uint32_t s_tmem;
+  __shared__ __align__(8) uint64_t s_full[2], s_done[2], s_free[2];
+  const int kv = blockIdx.y, b = blockIdx.z;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = clamp_len(seq_lens[b], pl.N_max);
   const int t0 = blockIdx.x * kAsgTok;
   if (t0 >= n) return;
   const size_t ukv = (size_t)b * pl.Hkv + kv;
-  const float* Ub = U + (ukv * pl.N_max + t0) * kD;
-  const float* Cb = centroids + ukv * (size_t)pl.n_list * kD;
-  const int n_tok = min(kAsgTok, n - t0);
-  for (int i = tid; i < kAsgTok * (kD / 4); i += kAsgThreads) {
-    const int r = i / (kD / 4), c4 = i % (kD / 4);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < n_tok) v = __ldg(reinterpret_cast<const float4*>(Ub + (size_t)r * kD) + c4);
-    *reinterpret_cast<float4*>(s_u + r * kAsgStride + 4 * c4) = v;
+  const int n_tiles = (pl.n_list + kAsgCen - 1) / kAsgCen;
+  const unsigned char* img = images + ukv * (size_t)n_tiles * kCenTileBytes;
+  if (warp == 8) tmem_alloc(&s_tmem, 256);
+  if (tid < 2) { mbar_init(&s_full[tid], 1); mbar_init(&s_done[tid], 1); mbar_init(&s_free[tid], 8); }
+  if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  // the token tiles
+  if (warp < 8) {
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+      const int r = q * 64 + warp * 8 + (lane & 7);
+      const bool real = t0 + r < n;
+      unsigned char* dst = s_tok + (r >> 7) * kTokTileBytes;
+      const float x2 = split_rows(U + (ukv * pl.N_max + t0 + (real ? r : 0)) * kD, real, kTcScale, dst, 128, r & 127, lane);
+      if (lane < 8) {
+        s_x2[r] = x2;
+        *reinterpret_cast<uint4*>(dst + (32 * 128 + (r & 127)) * 16) = coarse_ext_row();
+      } else if (lane < 16) {
+        *reinterpret_cast<uint4*>(dst + (33 * 128 + (r & 127)) * 16) = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+    tc_fence_smem();
   }
+  tc_fence_before();
   __syncthreads();
-  float xs2[8];                                         // |u|^2 of my tokens
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float* ur = s_u + (ty + 16 * i) * kAsgStride;
-    float a = 0.f;
-    for (int k = 0; k < kD; ++k) a = fmaf(ur[k], ur[k], a);
-    xs2[i] = a;
-  }
-  float best_d[8];
-  int best_j[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { best_d[i] = CUDART_INF_F; best_j[i] = 0; }
-
-  for (int c0 = 0; c0 < pl.n_list; c0 += kAsgCen) {
-    __syncthreads();                                    // previous tile consumed
-    for (int i = tid; i < kAsgCen * (kD / 4); i += kAsgThreads) {
-      const int r = i / (kD / 4), c4 = i % (kD / 4);
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c0 + r < pl.n_list) v = __ldg(reinterpret_cast<const float4*>(Cb + (size_t)(c0 + r) * kD) + c4);
-      *reinterpret_cast<float4*>(s_c + r * kAsgStride + 4 * c4) = v;
-    }
-    __syncthreads();
-    if (tid < kAsgCen) {
-      const float* cr = s_c + tid * kAsgStride;
-      float a = 0.f;
-      for (int k = 0; k < kD; ++k) a = fmaf(cr[k], cr[k], a);
-      s_cn[tid] = a;
-    }
-    float acc[8][4];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 2
-    for (int k = 0; k < kD; k += 4) {
-      float4 uv[8], cv[4];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) uv[i] = *reinterpret_cast<const float4*>(s_u + (ty + 16 * i) * kAsgStride + k);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) cv[j] = *reinterpret_cast<const float4*>(s_c + (tx + 16 * j) * kAsgStride + k);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[i][j] = fmaf(uv[i].x, cv[j].x, acc[i][j]);
-          acc[i][j] = fmaf(uv[i].y, cv[j].y, acc[i][j]);
-          acc[i][j] = fmaf(uv[i].z, cv[j].z, acc[i][j]);
-          acc[i][j] = fmaf(uv[i].w, cv[j].w, acc[i][j]);
-        }
-    }
-    __syncthreads();                                    // s_cn written
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int cj = c0 + tx + 16 * j;
-      if (cj < pl.n_list) {
-        const float cn = s_cn[tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float d = (xs2[i] - 2.0f * acc[i][j]) + cn;
-          if (d < best_d[i] || (d == best_d[i] && cj < best_j[i])) { best_d[i] = d; best_j[i] = cj; }
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;
+  bool late = false;
+  if (warp == 8) {
+    if (lane == 0) {
+      auto copy = [&](int i) {
+        mbar_expect_tx(&s_full[i & 1], kCenTileBytes);
+        bulk_g2s(s_cen + (i & 1) * kCenTileBytes, img + (size_t)i * kCenTileBytes, kCenTileBytes, &s_full[i & 1]);
+      };
+      copy(0);
+      if (n_tiles > 1) copy(1);
+      const uint32_t sa = smem_u32(s_tok);
+      for (int i = 0; i < n_tiles; ++i) {
+        const uint32_t st = i & 1, ph = (uint32_t)(i >> 1) & 1u;
+        late |= !tc_wait(&s_full[st], ph);
+        if (i >= 2) late |= !tc_wait(&s_free[st], ph ^ 1u);          // tile i - 2 has been read
+        tc_fence_after();
+        const uint32_t sb = smem_u32(s_cen + st * kCenTileBytes);
+        tc_coarse_tile<128, kAsgCen>(tmem + st * 128u, sa, sb);
+        tc_coarse_tile<128, kAsgCen>(tmem + st * 128u + 64u, sa + kTokTileBytes, sb);
+        tc_commit(&s_done[st]);
+        if (i >= 1 && i + 1 < n_tiles) {                             // the stage of tile i - 1 is free
+          late |= !tc_wait(&s_done[st ^ 1u], (uint32_t)((i - 1) >> 1) & 1u);
+          copy(i + 1);
         }
       }
     }
+    __syncwarp();
+  } else {
+    const int wg = warp >> 2;
+    const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+    float best = CUDART_INF_F, second = CUDART_INF_F;
+    int near = 0, next = 0;                                 // nearest and second nearest so far
+    for (int i = 0; i < n_tiles; ++i) {
+      const uint32_t st = i & 1;
+      late |= !tc_wait(&s_done[st], (uint32_t)(i >> 1) & 1u);
+      tc_fence_after();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float acc[32];
+        tmem_ld32(tmem + st * 128u + wg * 64u + h * 32u + lanes, acc);
+        if (h == 1) {
+          tc_fence_before();
+          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&s_free[st])) : "memory");
+        }
+        // the minimum of the 32 first (three inputs per instruction); one by one only where it could
+        // become the nearest or a near-tie of it
+        const float m = min32(acc);
+        if (m < best + kNearTie) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {                             // ascending: the first minimum stays
+            const int cj = i * kAsgCen + h * 32 + j;
+            const bool first = acc[j] < best;
+            const float other = fmaxf(acc[j], best);
+            if (other < second) next = first ? near : cj;
+            second = fminf(second, other);
+            if (first) near = cj;
+            best = fminf(best, acc[j]);
+          }
+        }
+      }
+    }
+    const int r = wg * 128 + (warp & 3) * 32 + lane;
+    if (t0 + r < n) {
+      const size_t at = ukv * pl.N_max + t0 + r;
+      float d = s_x2[r] + best * kTcUnscale;
+      if (second < best + kNearTie && max(near, next) < pl.n_list) {
+        // the two are within the rounding of either arithmetic: decided in plain fp32, every sum one
+        // chain over the dims (a few tokens in a thousand)
+        const float4* u = reinterpret_cast<const float4*>(U + at * kD);
+        const float4* c0 = reinterpret_cast<const float4*>(centroids + (ukv * pl.n_list + min(near, next)) * kD);
+        const float4* c1 = reinterpret_cast<const float4*>(centroids + (ukv * pl.n_list + max(near, next)) * kD);
+        float xx = 0.f, a0 = 0.f, a1 = 0.f, n0 = 0.f, n1 = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < kD / 4; ++k) {
+          const float4 x = __ldcg(u + k), y = __ldcg(c0 + k), z = __ldcg(c1 + k);
+          xx = fmaf(x.x, x.x, xx); xx = fmaf(x.y, x.y, xx); xx = fmaf(x.z, x.z, xx); xx = fmaf(x.w, x.w, xx);
+          a0 = fmaf(x.x, y.x, a0); a0 = fmaf(x.y, y.y, a0); a0 = fmaf(x.z, y.z, a0); a0 = fmaf(x.w, y.w, a0);
+          n0 = fmaf(y.x, y.x, n0); n0 = fmaf(y.y, y.y, n0); n0 = fmaf(y.z, y.z, n0); n0 = fmaf(y.w, y.w, n0);
+          a1 = fmaf(x.x, z.x, a1); a1 = fmaf(x.y, z.y, a1); a1 = fmaf(x.z, z.z, a1); a1 = fmaf(x.w, z.w, a1);
+          n1 = fmaf(z.x, z.x, n1); n1 = fmaf(z.y, z.y, n1); n1 = fmaf(z.z, z.z, n1); n1 = fmaf(z.w, z.w, n1);
+        }
+        const float d0 = (xx - 2.0f * a0) + n0, d1 = (xx - 2.0f * a1) + n1;
+        near = d1 < d0 ? max(near, next) : min(near, next);
+        d = fminf(d0, d1);
+      }
+      list_ids[at] = (uint16_t)min(near, pl.n_list - 1);
+      dmin[at] = d;
+      if (late) key_norms[at] = CUDART_NAN_F;              // a bounded wait ran out: the norms say so
+    }
   }
-  // the 16 threads of a row (same ty: consecutive lanes of a half warp) join their minima
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) { tc_fence_after(); tmem_free(tmem, 256); }
+}
+
+// ---- tokens grouped by list.  hist: members per list; offsets: exclusive prefix (and a running
+// copy); scatter: every token to its list's next slot (the order inside a list does not matter: all
+// sums over it are integers).  Only tokens of [lo, hi) take part: the whole sequence for the
+// centroids, the indexed region for the value means.
+constexpr int kSortThreads = 512;
+constexpr int kSortChunk = 4096;         // tokens per CTA
+template <bool kRegion> __device__ __forceinline__ Region sort_range(const Plan& pl, int n, int b) {
+  if (kRegion) return region_of(pl, n, b);
+  return Region{0, n};
+}
+
+template <bool kRegion>
+__global__ void __launch_bounds__(kSortThreads)
+build_hist_kernel(Plan pl, const uint16_t* __restrict__ list_ids, const int32_t* __restrict__ seq_lens,
+                  int32_t* __restrict__ counts) {
+  extern __shared__ int s_cnt[];                            // [n_list]
+  const int kv = blockIdx.y, b = blockIdx.z;
+  const int n = clamp_len(seq_lens[b], pl.N_max);
+  const Region rg = sort_range<kRegion>(pl, n, b);
+  const int lo = rg.r_begin + blockIdx.x * kSortChunk, hi = min(rg.r_end, lo + kSortChunk);
+  if (lo >= hi) return;
+  const size_t ukv = (size_t)b * pl.Hkv + kv;
+  for (int j = threadIdx.x; j < pl.n_list; j += kSortThreads) s_cnt[j] = 0;
+  __syncthreads();
+  for (int i = lo + threadIdx.x; i < hi; i += kSortThreads)
+    atomicAdd(&s_cnt[min((int)list_ids[ukv * pl.N_max + i], pl.n_list - 1)], 1);
+  __syncthreads();
+  for (int j = threadIdx.x; j < pl.n_list; j += kSortThreads)
+    if (s_cnt[j]) atomicAdd(&counts[ukv * pl.n_list + j], s_cnt[j]);
+}
+
+__global__ void __launch_bounds__(1024)
+build_offsets_kernel(Plan pl, const int32_t* __restrict__ counts, int32_t* __restrict__ cursor) {
+  __shared__ int s_warp[32];
+  const size_t unit = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int v[4], local = 0;                                      // n_list <= 4096: 4 lists per thread
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int u = 0; u < 4; ++u) {
+    const int j = 4 * tid + u;
+    v[u] = j < pl.n_list ? counts[unit * pl.n_list + j] : 0;
+    local += v[u];
+  }
+  int inc = local;
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-      const float od = __shfl_xor_sync(0xffffffffu, best_d[i], o);
-      const int oj = __shfl_xor_sync(0xffffffffu, best_j[i], o);
-      if (od < best_d[i] || (od == best_d[i] && oj < best_j[i])) { best_d[i] = od; best_j[i] = oj; }
-    }
-    const int r = ty + 16 * i;
-    if (tx == 0 && r < n_tok) {
-      list_ids[ukv * pl.N_max + t0 + r] = (uint16_t)best_j[i];
-      dmin[ukv * pl.N_max + t0 + r] = best_d[i];
-    }
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
+  }
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  int run = inc - local;
+  for (int w = 0; w < warp; ++w) run += s_warp[w];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int j = 4 * tid + u;
+    if (j < pl.n_list) cursor[unit * pl.n_list + j] = run;
+    run += v[u];
   }
 }
 
-// ---- per-list sums of member directions: a warp per token, one 16-byte reduction per lane
+template <bool kRegion>
+__global__ void __launch_bounds__(kSortThreads)
+build_scatter_kernel(Plan pl, const uint16_t* __restrict__ list_ids, const int32_t* __restrict__ seq_lens,
+                     int32_t* __restrict__ cursor, int32_t* __restrict__ order) {
+  extern __shared__ int s_cnt[];                            // [n_list] members here, then next slot
+  const int kv = blockIdx.y, b = blockIdx.z;
+  const int n = clamp_len(seq_lens[b], pl.N_max);
+  const Region rg = sort_range<kRegion>(pl, n, b);
+  const int lo = rg.r_begin + blockIdx.x * kSortChunk, hi = min(rg.r_end, lo + kSortChunk);
+  if (lo >= hi) return;
+  const size_t ukv = (size_t)b * pl.Hkv + kv;
+  constexpr int kPer = kSortChunk / kSortThreads;
+  int lid[kPer], rank[kPer];
+  for (int j = threadIdx.x; j < pl.n_list; j += kSortThreads) s_cnt[j] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int i = lo + u * kSortThreads + threadIdx.x;
+    lid[u] = i < hi ? min((int)list_ids[ukv * pl.N_max + i], pl.n_list - 1) : -1;
+    if (lid[u] >= 0) rank[u] = atomicAdd(&s_cnt[lid[u]], 1);
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < pl.n_list; j += kSortThreads)
+    if (s_cnt[j]) s_cnt[j] = atomicAdd(&cursor[ukv * pl.n_list + j], s_cnt[j]);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kPer; ++u)
+    if (lid[u] >= 0) order[ukv * pl.N_max + s_cnt[lid[u]] + rank[u]] = lo + u * kSortThreads + threadIdx.x;
+}
+
+// ---- sums over grouped tokens: a warp takes kRun consecutive entries of `order`, a lane 4 dims; the
+// sum goes out when the list changes.  row(i, x) reads token i's 4 dims.
+constexpr int kRun = 64, kRunBatch = 8;
+template <class Row>
+__device__ __forceinline__ void run_sums(const Plan& pl, const uint16_t* __restrict__ lids_u,
+                                         const int32_t* __restrict__ order_u, int first, int last,
+                                         float scale, long long* __restrict__ sums_u, Row row) {
+  const int lane = threadIdx.x & 31;
+  long long acc[4] = {0, 0, 0, 0};
+  int cur = -1;
+  auto flush = [&]() {
+    if (cur < 0) return;
+    long long* dst = sums_u + (size_t)cur * kD + 4 * lane;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if (acc[t]) atomicAdd(reinterpret_cast<unsigned long long*>(dst + t), (unsigned long long)acc[t]);
+      acc[t] = 0;
+    }
+  };
+  for (int base = first; base < last; base += 32) {
+    // token and list of 32 entries at once, one per lane
+    const int mine = base + lane < last ? order_u[base + lane] : -1;
+    const int my_list = mine >= 0 ? min((int)lids_u[mine], pl.n_list - 1) : -1;
+    const int cnt = min(32, last - base);
+    for (int e0 = 0; e0 < cnt; e0 += kRunBatch) {
+      float x[kRunBatch][4];
+#pragma unroll
+      for (int u = 0; u < kRunBatch; ++u) {
+        const int i = __shfl_sync(0xffffffffu, mine, e0 + u);
+        if (i >= 0) row(i, x[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kRunBatch; ++u) {
+        const int j = __shfl_sync(0xffffffffu, my_list, e0 + u);
+        if (j < 0) continue;                               // (warp-uniform)
+        if (j != cur) { flush(); cur = j; }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) acc[t] += __float2ll_rn(x[u][t] * scale);
+      }
+    }
+  }
+  flush();
+}
+
 __global__ void __launch_bounds__(kPrepThreads)
-build_accumulate_kernel(Plan pl, const float* __restrict__ U, const uint16_t* __restrict__ list_ids,
-                        const int32_t* __restrict__ seq_lens,
-                        long long* __restrict__ sums, int32_t* __restrict__ counts) {
+build_dir_sums_kernel(Plan pl, const float* __restrict__ U, const uint16_t* __restrict__ list_ids,
+                      const int32_t* __restrict__ order, const int32_t* __restrict__ seq_lens,
+                      long long* __restrict__ sums) {
   const int kv = blockIdx.y, b = blockIdx.z;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = clamp_len(seq_lens[b], pl.N_max);
   const size_t ukv = (size_t)b * pl.Hkv + kv;
-  for (int i = blockIdx.x * (kPrepThreads / 32) + warp; i < n; i += gridDim.x * (kPrepThreads / 32)) {
-    const uint32_t j = min((uint32_t)list_ids[ukv * pl.N_max + i], (uint32_t)(pl.n_list - 1));
-    const float4 u = *reinterpret_cast<const float4*>(U + (ukv * pl.N_max + i) * kD + 4 * lane);
-    long long* dst = sums + (ukv * pl.n_list + j) * kD + 4 * lane;
-    fix_add(dst, u.x, kFixDir); fix_add(dst + 1, u.y, kFixDir);
-    fix_add(dst + 2, u.z, kFixDir); fix_add(dst + 3, u.w, kFixDir);
-    if (lane == 0) atomicAdd(&counts[ukv * pl.n_list + j], 1);
-  }
+  const int first = (blockIdx.x * (kPrepThreads / 32) + warp) * kRun, last = min(n, first + kRun);
+  if (first >= n) return;
+  const float* Ub = U + ukv * pl.N_max * (size_t)kD + 4 * lane;
+  run_sums(pl, list_ids + ukv * pl.N_max, order + ukv * pl.N_max, first, last, kFixDir,
+           sums + ukv * pl.n_list * (size_t)kD, [&](int i, float (&x)[4]) {
+             *reinterpret_cast<float4*>(x) = __ldcg(reinterpret_cast<const float4*>(Ub + (size_t)i * kD));
+           });
 }
 
 // c_j <- mean of its members; an empty list keeps its centre and is counted; sums are cleared
@@ -298,89 +501,258 @@ build_reseed_kernel(Plan pl, const float* __restrict__ U, float* __restrict__ dm
   if (tid == 0) n_empty[unit] = 0;
 }
 
-// ---- product quantisation of the residuals e_i = u_i - c_{a_i}.  Codebooks [unit][M][n_code][dsub].
+// ---- residuals e_i = u_i - c_{a_i}, in place of the directions
+__global__ void __launch_bounds__(kPrepThreads)
+build_residual_kernel(Plan pl, float* __restrict__ U, const float* __restrict__ centroids,
+                      const uint16_t* __restrict__ list_ids, const int32_t* __restrict__ seq_lens) {
+  const int kv = blockIdx.y, b = blockIdx.z;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = clamp_len(seq_lens[b], pl.N_max);
+  const size_t ukv = (size_t)b * pl.Hkv + kv;
+  constexpr int kPer = 4;
+  for (int i0 = (blockIdx.x * (kPrepThreads / 32) + warp) * kPer; i0 < n; i0 += gridDim.x * (kPrepThreads / 32) * kPer) {
+    float4 u[kPer], c[kPer];
+    float4* at = reinterpret_cast<float4*>(U + (ukv * pl.N_max + i0) * kD) + lane;
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) {
+      if (i0 + t >= n) break;
+      const uint32_t a = min((uint32_t)list_ids[ukv * pl.N_max + i0 + t], (uint32_t)(pl.n_list - 1));
+      u[t] = __ldcg(at + t * (kD / 4));
+      c[t] = __ldg(reinterpret_cast<const float4*>(centroids + (ukv * pl.n_list + a) * kD) + lane);
+    }
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) {
+      if (i0 + t >= n) break;
+      at[t * (kD / 4)] = make_float4(u[t].x - c[t].x, u[t].y - c[t].y, u[t].z - c[t].z, u[t].w - c[t].w);
+    }
+  }
+}
+
+// ---- product quantisation of the residuals E.  Codebooks [unit][M][n_code][dsub].
 // Seeds: codeword z of subspace m <- residual sub-vector m of the token at seed_pos[unit][z].
 template <int DSUB>
-__global__ void build_pq_seed_kernel(Plan pl, const float* __restrict__ U,
-                                     const float* __restrict__ centroids,
-                                     const uint16_t* __restrict__ list_ids,
-                                     const int32_t* __restrict__ seed_pos,
+__global__ void build_pq_seed_kernel(Plan pl, const float* __restrict__ E, const int32_t* __restrict__ seed_pos,
                                      float* __restrict__ codebooks) {
   const size_t unit = blockIdx.y;
   const int z = blockIdx.x, d = threadIdx.x;                 // 128 threads: one per dim
   const int pos = seed_pos[unit * pl.n_code + z];
   float e = 0.f;
-  if (pos >= 0 && pos < pl.N_max) {
-    const uint32_t a = min((uint32_t)list_ids[unit * pl.N_max + pos], (uint32_t)(pl.n_list - 1));
-    e = U[(unit * pl.N_max + pos) * kD + d] - centroids[(unit * pl.n_list + a) * kD + d];
-  }
+  if (pos >= 0 && pos < pl.N_max) e = E[(unit * pl.N_max + pos) * kD + d];
   const int m = d / DSUB, t = d % DSUB;
   codebooks[((unit * pl.M + m) * pl.n_code + z) * DSUB + t] = e;
 }
 
-// Nearest codeword of every (token, subspace): CTA = 128 tokens x one group of subspaces whose
-// codebooks fit shared memory; a thread owns a token, walks the codewords (broadcast reads).
-// distance = (|e|^2 - 2 e.p) + |p|^2.  Optionally accumulates the per-codeword sums for the
-// next Lloyd step (training) or writes the final codes (encode).
-template <int DSUB>
-__global__ void __launch_bounds__(128)
-build_pq_assign_kernel(Plan pl, const float* __restrict__ U, const float* __restrict__ centroids,
-                       const uint16_t* __restrict__ list_ids, const float* __restrict__ codebooks,
-                       const int32_t* __restrict__ seq_lens, int m_per_cta,
-                       long long* __restrict__ pq_sums, int32_t* __restrict__ pq_counts,
-                       uint8_t* __restrict__ codes_out) {
-  extern __shared__ __align__(16) float s_cb[];             // [m_per_cta][n_code][DSUB + 1 (|p|^2)]
-  const int kv = blockIdx.y % pl.Hkv, b = blockIdx.y / pl.Hkv;
-  const int mg = blockIdx.z, tid = threadIdx.x;
-  const int n = clamp_len(seq_lens[b], pl.N_max);
-  const int i = blockIdx.x * 128 + tid;
-  const size_t ukv = (size_t)b * pl.Hkv + kv;
-  const int m0 = mg * m_per_cta, m1 = min(pl.M, m0 + m_per_cta);
-  if (blockIdx.x * 128 >= n) return;
-  constexpr int kW = DSUB + 1;
-  for (int idx = tid; idx < (m1 - m0) * pl.n_code; idx += 128) {
-    const float* p = codebooks + ((ukv * pl.M + m0) * pl.n_code + idx) * DSUB;
-    float pn = 0.f;
-#pragma unroll
-    for (int t = 0; t < DSUB; ++t) { const float v = p[t]; s_cb[idx * kW + t] = v; pn = fmaf(v, v, pn); }
-    s_cb[idx * kW + DSUB] = pn;
+// Nearest codeword of every (token, subspace) on the tensor cores.  A CTA keeps the codebooks of
+// kMg subspaces (64 bytes of a residual row) as tensor-core tiles and walks a range of tokens, 128 at
+// a time per warpgroup: thread = token = accumulator row.  The accumulators give the group of 8
+// codewords that holds the minimum, the codeword is decided in fp32 among those 8 (distance =
+// (|e|^2 - 2 e.p) + |p|^2, lower index on ties).  Training accumulates the codewords' sums in 64-bit
+// fixed point: two 32-bit shared-memory limbs of 21 bits and the rest (native integer atomics),
+// folded into 64 bits every kFold tokens, before a limb could overflow.
+template <int DSUB> struct PqPlan {
+  static constexpr int kMg8 = 16 / DSUB;                     // subspaces per CTA, 8-bit codes
+  static constexpr int kMg = kMg8 < 2 ? 2 : kMg8;            // (4-bit codes: whole bytes)
+  using Tile = PqTile<DSUB>;
+  static int mg(int n_code) { return n_code == 16 ? kMg : kMg8; }
+  static size_t words(int n_code) { return (size_t)mg(n_code) * n_code; }
+  static size_t smem(int n_code, bool train) {
+    return words(n_code) * (Tile::kChunks * 16 + DSUB * 4 + 4) + 4 * Tile::kChunks * 2048 +
+           (train ? words(n_code) * ((2 * DSUB + 1) * 4 + DSUB * 8) : 0);
   }
+};
+constexpr int kPqThreads = 512, kPqStep = 512;               // tokens per CTA and step
+constexpr int kFoldSteps = 3;                                // 1536 tokens: 2^21 * 1536 < 2^32, 2^20 * 1536 < 2^31
+constexpr int kLimbBits = 21;
+
+template <int DSUB, bool kTrain>
+__global__ void __launch_bounds__(kPqThreads, 1)
+build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __restrict__ codebooks,
+                       const int32_t* __restrict__ seq_lens, int mg, int range, long long* __restrict__ pq_sums,
+                       int32_t* __restrict__ pq_counts, uint8_t* __restrict__ codes_out,
+                       float* __restrict__ key_norms) {
+  using Tile = PqTile<DSUB>;
+  extern __shared__ __align__(128) unsigned char s_pq[];
+  __shared__ uint32_t s_tmem;
+  __shared__ __align__(8) uint64_t s_bar[4];
+  const int kv = blockIdx.y % pl.Hkv, b = blockIdx.y / pl.Hkv;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wg = tid >> 7, row = tid & 127;
+  const int n = clamp_len(seq_lens[b], pl.N_max);
+  const int begin = blockIdx.x * range, end = min(n, begin + range);
+  if (begin >= end) return;
+  const size_t ukv = (size_t)b * pl.Hkv + kv;
+  const int m0 = blockIdx.z * mg, nc = pl.n_code;
+  const int words = mg * nc;
+  // shared memory: codeword tiles, token tiles, fp32 codewords and |p|^2, then the training sums
+  unsigned char* s_b = s_pq;                                            // [mg][chunks][nc] x 16 bytes
+  unsigned char* s_a = s_b + (size_t)words * Tile::kChunks * 16;        // [4][chunks][128] x 16 bytes
+  long long* s_sum = reinterpret_cast<long long*>(s_a + 4 * Tile::kChunks * 2048);   // [mg][DSUB][nc] (training)
+  float* s_word = reinterpret_cast<float*>(s_sum + (kTrain ? (size_t)words * DSUB : 0));   // [mg][nc][DSUB]
+  float* s_p2 = s_word + (size_t)words * DSUB;                          // [mg][nc]
+  uint32_t* s_limb = reinterpret_cast<uint32_t*>(s_p2 + words);         // [mg][2 DSUB + 1][nc]
+  auto load_sub = [](const float* src, float (&x)[DSUB]) {
+    if constexpr (DSUB == 2) {
+      *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(src);
+    } else {
+#pragma unroll
+      for (int c4 = 0; c4 < DSUB / 4; ++c4)
+        *reinterpret_cast<float4*>(x + 4 * c4) = *reinterpret_cast<const float4*>(src + 4 * c4);
+    }
+  };
+  if (warp == 0) tmem_alloc(&s_tmem, 512);
+  if (tid < 4) mbar_init(&s_bar[tid], 1);
+  if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  const float* cb = codebooks + (ukv * pl.M + m0) * (size_t)nc * DSUB;
+  for (int w = tid; w < words; w += kPqThreads) {
+    float p[DSUB], p2 = 0.f;
+    load_sub(cb + (size_t)w * DSUB, p);
+    uint4 ch[Tile::kChunks];
+    Tile::code_row(p, ch);
+    const int mm = w / nc, z = w - mm * nc;
+#pragma unroll
+    for (int i = 0; i < Tile::kChunks; ++i)
+      *reinterpret_cast<uint4*>(s_b + (size_t)((mm * Tile::kChunks + i) * nc + z) * 16) = ch[i];
+#pragma unroll
+    for (int t = 0; t < DSUB; ++t) { s_word[(size_t)w * DSUB + t] = p[t]; p2 = fmaf(p[t], p[t], p2); }
+    s_p2[w] = p2;
+    if constexpr (kTrain) {
+#pragma unroll
+      for (int t = 0; t < DSUB; ++t) s_sum[(size_t)(mm * DSUB + t) * nc + z] = 0;
+#pragma unroll
+      for (int t = 0; t < 2 * DSUB + 1; ++t) s_limb[(size_t)(mm * (2 * DSUB + 1) + t) * nc + z] = 0u;
+    }
+  }
+  tc_fence_smem();
+  tc_fence_before();
   __syncthreads();
-  if (i >= n) return;
-  const uint32_t a = min((uint32_t)list_ids[ukv * pl.N_max + i], (uint32_t)(pl.n_list - 1));
-  const float* ur = U + (ukv * pl.N_max + i) * kD;
-  const float* cr = centroids + (ukv * pl.n_list + a) * kD;
-  for (int m = m0; m < m1; ++m) {
-    float e[DSUB], en = 0.f;
+  tc_fence_after();
+  const uint32_t d_tmem = s_tmem + (uint32_t)wg * 128u;
+  const uint32_t my_tmem = d_tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  unsigned char* pa = s_a + wg * (Tile::kChunks * 2048);
+  const uint32_t n_mma = (uint32_t)min(nc, 128);
+  uint32_t parity = 0u;
+  bool late = false;
+  // the limbs into 64 bits (every thread its own entries); all threads call
+  auto fold = [&]() {
+    __syncthreads();
+    for (int w = tid; w < words; w += kPqThreads) {
+      const int mm = w / nc, z = w - mm * nc;
 #pragma unroll
-    for (int t = 0; t < DSUB; ++t) { e[t] = ur[m * DSUB + t] - cr[m * DSUB + t]; en = fmaf(e[t], e[t], en); }
-    const float* cb = s_cb + (size_t)(m - m0) * pl.n_code * kW;
-    float bd = CUDART_INF_F;
-    int bz = 0;
-    for (int z = 0; z < pl.n_code; ++z) {
-      float dot = 0.f;
-#pragma unroll
-      for (int t = 0; t < DSUB; ++t) dot = fmaf(e[t], cb[z * kW + t], dot);
-      const float dist = (en - 2.0f * dot) + cb[z * kW + DSUB];
-      if (dist < bd) { bd = dist; bz = z; }                  // z ascends: the first minimum stays
-    }
-    if (pq_sums != nullptr) {
-      long long* dst = pq_sums + ((ukv * pl.M + m) * pl.n_code + bz) * DSUB;
-#pragma unroll
-      for (int t = 0; t < DSUB; ++t) fix_add(dst + t, e[t], kFixDir);
-      atomicAdd(&pq_counts[(ukv * pl.M + m) * pl.n_code + bz], 1);
-    }
-    if (codes_out != nullptr) {
-      if (pl.n_code == 16) {
-        // two 4-bit codes per byte, subspace 2j in the low nibble: the thread owns the token,
-        // so consecutive subspaces of one byte are written by the same thread in order
-        uint8_t* dst = codes_out + (ukv * pl.N_max + i) * pl.code_bytes + (m >> 1);
-        *dst = (m & 1) ? (uint8_t)(*dst | (bz << 4)) : (uint8_t)bz;
-      } else {
-        codes_out[(ukv * pl.N_max + i) * pl.code_bytes + m] = (uint8_t)bz;
+      for (int t = 0; t < DSUB; ++t) {
+        uint32_t* l = s_limb + (size_t)(mm * (2 * DSUB + 1) + 2 * t) * nc + z;
+        s_sum[(size_t)(mm * DSUB + t) * nc + z] += (long long)l[0] + ((long long)(int32_t)l[nc] << kLimbBits);
+        l[0] = 0u;
+        l[nc] = 0u;
       }
     }
+    __syncthreads();
+  };
+  int steps = 0;
+  for (int base = begin; base < end; base += kPqStep) {
+    const int i = base + wg * 128 + row;
+    const bool real = i < end;
+    const float* er = E + (ukv * pl.N_max + (real ? i : begin)) * (size_t)kD + m0 * DSUB;
+    float e[DSUB], e_nxt[DSUB];
+    load_sub(er, e_nxt);
+    uint32_t word = 0u;                                     // codes not yet written
+    for (int mm = 0; mm < mg; ++mm) {
+#pragma unroll
+      for (int t = 0; t < DSUB; ++t) e[t] = e_nxt[t];
+      if (mm + 1 < mg) load_sub(er + (mm + 1) * DSUB, e_nxt);
+      uint4 ch[Tile::kChunks];
+      Tile::token_row(e, ch);
+#pragma unroll
+      for (int c = 0; c < Tile::kChunks; ++c) *reinterpret_cast<uint4*>(pa + (c * 128 + row) * 16) = ch[c];
+      float bd = CUDART_INF_F;
+      int grp = 0;
+      const uint32_t sb = smem_u32(s_b + (size_t)mm * Tile::kChunks * nc * 16);
+      for (int z0 = 0; z0 < nc; z0 += 128) {
+        tc_fence_smem();
+        tc_fence_before();
+        group_sync(1 + wg);
+        if (row == 0) {
+          tc_fence_after();
+          if (nc == 16) Tile::template mma<16>(d_tmem, smem_u32(pa), sb, n_mma);
+          else Tile::template mma<256>(d_tmem, smem_u32(pa), sb + z0 * 16, n_mma);
+          tc_commit(&s_bar[wg]);
+        }
+        __syncwarp();
+        late |= !tc_wait(&s_bar[wg], parity);
+        parity ^= 1u;
+        tc_fence_after();
+        if (nc == 16) {
+          float acc[16];
+          tmem_ld16(my_tmem, acc);
+          group_minima(acc, 0, bd, grp);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 128; c += 32) {
+            float acc[32];
+            tmem_ld32(my_tmem + c, acc);
+            group_minima(acc, (z0 + c) / 8, bd, grp);
+          }
+        }
+      }
+      // the winning group in fp32; the lanes start at different codewords, so that at 16 bytes a
+      // codeword the eight lanes of an access hit eight different bank groups
+      float en = 0.f;
+#pragma unroll
+      for (int t = 0; t < DSUB; ++t) en = fmaf(e[t], e[t], en);
+      float dm = CUDART_INF_F;
+      int bz = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int z = 8 * grp + ((q + lane) & 7);
+        float w[DSUB], dot = 0.f;
+        load_sub(s_word + (size_t)(mm * nc + z) * DSUB, w);
+#pragma unroll
+        for (int t = 0; t < DSUB; ++t) dot = fmaf(e[t], w[t], dot);
+        const float dist = (en - 2.0f * dot) + s_p2[mm * nc + z];
+        if (dist < dm || (dist == dm && z < bz)) { dm = dist; bz = z; }
+      }
+      if constexpr (kTrain) {
+        if (real) {
+          uint32_t* l = s_limb + (size_t)(mm * (2 * DSUB + 1)) * nc + bz;
+#pragma unroll
+          for (int t = 0; t < DSUB; ++t) {
+            const long long q = __float2ll_rn(e[t] * kFixDir);
+            atomicAdd(l + (2 * t) * nc, (uint32_t)q & ((1u << kLimbBits) - 1u));
+            atomicAdd(l + (2 * t + 1) * nc, (uint32_t)(q >> kLimbBits));
+          }
+          atomicAdd(l + 2 * DSUB * nc, 1u);
+        }
+      } else if (real) {
+        uint8_t* dst = codes_out + (ukv * pl.N_max + i) * pl.code_bytes;
+        if (nc == 16) {
+          if (mm & 1) dst[(m0 + mm) >> 1] = (uint8_t)(word | ((uint32_t)bz << 4));
+          else word = (uint32_t)bz;
+        } else {
+          dst[m0 + mm] = (uint8_t)bz;
+        }
+      }
+    }
+    if (late && real) key_norms[ukv * pl.N_max + i] = CUDART_NAN_F;    // a bounded wait ran out
+    if constexpr (kTrain) {
+      if (++steps == kFoldSteps) { fold(); steps = 0; }
+    }
   }
+  if constexpr (kTrain) {
+    fold();
+    for (int w = tid; w < words; w += kPqThreads) {
+      const int mm = w / nc, z = w - mm * nc;
+      const size_t at = (ukv * pl.M + m0 + mm) * nc + z;
+      const uint32_t c = s_limb[(size_t)(mm * (2 * DSUB + 1) + 2 * DSUB) * nc + z];
+      if (c == 0u) continue;
+      atomicAdd(&pq_counts[at], (int32_t)c);
+#pragma unroll
+      for (int t = 0; t < DSUB; ++t)
+        atomicAdd(reinterpret_cast<unsigned long long*>(pq_sums + at * DSUB + t),
+                  (unsigned long long)s_sum[(size_t)(mm * DSUB + t) * nc + z]);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) { tc_fence_after(); tmem_free(s_tmem, 512); }
 }
 
 // codeword <- mean of its members (kept if it has none); sums and counts cleared
@@ -401,23 +773,20 @@ template <typename T>
 __global__ void __launch_bounds__(kPrepThreads)
 build_value_sums_kernel(Plan pl, const T* __restrict__ vc, long long sp, long long st, long long sh,
                         const int32_t* __restrict__ block_table, const int32_t* __restrict__ seq_lens,
-                        const uint16_t* __restrict__ list_ids, long long* __restrict__ sums,
-                        int32_t* __restrict__ counts) {
+                        const uint16_t* __restrict__ list_ids, const int32_t* __restrict__ order,
+                        long long* __restrict__ sums) {
   const int kv = blockIdx.y, b = blockIdx.z;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = clamp_len(seq_lens[b], pl.N_max);
   const Region rg = region_of(pl, n, b);
   const size_t ukv = (size_t)b * pl.Hkv + kv;
+  const int members = rg.r_end - rg.r_begin;
+  const int first = (blockIdx.x * (kPrepThreads / 32) + warp) * kRun, last = min(members, first + kRun);
+  if (first >= members) return;
   const int32_t* bt = block_table + (size_t)b * pl.max_pages;
-  for (int i = rg.r_begin + blockIdx.x * (kPrepThreads / 32) + warp; i < rg.r_end;
-       i += gridDim.x * (kPrepThreads / 32)) {
-    const uint32_t j = min((uint32_t)list_ids[ukv * pl.N_max + i], (uint32_t)(pl.n_list - 1));
-    const T* row = vc + kv_row(pl, bt, i, kv, sp, st, sh);
-    long long* dst = sums + (ukv * pl.n_list + j) * kD + 4 * lane;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) fix_add(dst + t, Unpack<T>::one(row[4 * lane + t]), kFixVal);
-    if (lane == 0) atomicAdd(&counts[ukv * pl.n_list + j], 1);
-  }
+  run_sums(pl, list_ids + ukv * pl.N_max, order + ukv * pl.N_max, first, last, kFixVal,
+           sums + ukv * pl.n_list * (size_t)kD,
+           [&](int i, float (&x)[4]) { load4<T>(vc + kv_row(pl, bt, i, kv, sp, st, sh) + 4 * lane, x); });
 }
 
 __global__ void build_value_means_kernel(Plan pl, long long* __restrict__ sums, const int32_t* __restrict__ counts,
@@ -438,7 +807,7 @@ __global__ void build_value_means_kernel(Plan pl, long long* __restrict__ sums, 
 }
 
 struct BuildWs {
-  size_t U, dmin, sums, counts, n_empty, pq_sums, pq_counts, total;
+  size_t U, dmin, images, order, cursor, sums, counts, n_empty, pq_sums, pq_counts, total;
 };
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 BuildWs build_layout(const Plan& pl) {
@@ -448,6 +817,9 @@ BuildWs build_layout(const Plan& pl) {
   const size_t units = (size_t)pl.B * pl.Hkv;
   w.U = take(units * pl.N_max * kD * 4);
   w.dmin = take(units * pl.N_max * 4);
+  w.images = take(units * ((pl.n_list + kAsgCen - 1) / kAsgCen) * (size_t)kCenTileBytes);
+  w.order = take(units * pl.N_max * 4);
+  w.cursor = take(units * pl.n_list * 4);
   w.sums = take(units * pl.n_list * kD * 8);
   w.counts = take(units * pl.n_list * 4);
   w.n_empty = take(units * 4);
@@ -476,41 +848,70 @@ cudaError_t run_build(const Plan& pl, const pqhsa_paged_kv& kv, const int32_t* s
   cudaError_t e;
 #define PQHSA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
   PQHSA_TRY(cudaMemsetAsync(ws + w.sums, 0, w.total - w.sums, st));
+  unsigned char* images = reinterpret_cast<unsigned char*>(ws + w.images);
+  int32_t* order = reinterpret_cast<int32_t*>(ws + w.order);
+  int32_t* cursor = reinterpret_cast<int32_t*>(ws + w.cursor);
   const int tok_ctas = min(1024, (pl.N_max + 7) / 8);
   build_prepare_kernel<T><<<dim3(tok_ctas, pl.Hkv, pl.B), kPrepThreads, 0, st>>>(
       pl, kc, sp, stt, sh, kv.block_table, seq_lens, U, ix.key_norms);
   build_seed_kernel<<<dim3((pl.n_list + 7) / 8, units), 256, 0, st>>>(pl, U, seed_lists, pl.n_list, ix.centroids);
   PQHSA_TRY(cudaFuncSetAttribute(build_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAsgSmemBytes));
   const dim3 asg_grid((pl.N_max + kAsgTok - 1) / kAsgTok, pl.Hkv, pl.B);
+  const dim3 split_grid((pl.n_list + kAsgCen - 1) / kAsgCen, units);
   const dim3 list_grid((pl.n_list + 7) / 8, units);
+  const dim3 sort_grid((pl.N_max + kSortChunk - 1) / kSortChunk, pl.Hkv, pl.B);
+  const dim3 run_grid((pl.N_max + kRun * (kPrepThreads / 32) - 1) / (kRun * (kPrepThreads / 32)), pl.Hkv, pl.B);
+  const size_t list_smem = (size_t)pl.n_list * 4;
+  auto assign = [&]() {
+    build_split_kernel<<<split_grid, 256, 0, st>>>(pl, ix.centroids, images);
+    build_assign_kernel<<<asg_grid, kAsgThreads, kAsgSmemBytes, st>>>(pl, U, images, ix.centroids, seq_lens, ix.list_ids, dmin, ix.key_norms);
+  };
   for (int it = 0; it < coarse_iters; ++it) {
-    build_assign_kernel<<<asg_grid, kAsgThreads, kAsgSmemBytes, st>>>(pl, U, ix.centroids, seq_lens, ix.list_ids, dmin);
+    assign();
     PQHSA_TRY(cudaMemsetAsync(counts, 0, (size_t)units * pl.n_list * 4, st));
-    build_accumulate_kernel<<<dim3(tok_ctas, pl.Hkv, pl.B), kPrepThreads, 0, st>>>(pl, U, ix.list_ids, seq_lens, sums, counts);
+    build_hist_kernel<false><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, counts);
+    build_offsets_kernel<<<units, 1024, 0, st>>>(pl, counts, cursor);
+    build_scatter_kernel<false><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, cursor, order);
+    build_dir_sums_kernel<<<run_grid, kPrepThreads, 0, st>>>(pl, U, ix.list_ids, order, seq_lens, sums);
     build_update_centroids_kernel<<<list_grid, 256, 0, st>>>(pl, sums, counts, ix.centroids, n_empty);
     build_reseed_kernel<<<units, 1024, 0, st>>>(pl, U, dmin, counts, seq_lens, n_empty, ix.centroids);
   }
-  build_assign_kernel<<<asg_grid, kAsgThreads, kAsgSmemBytes, st>>>(pl, U, ix.centroids, seq_lens, ix.list_ids, dmin);
-  // product quantisation of the residuals: as many subspaces per CTA as fit 96 KB of codebooks
-  int m_per_cta = (96 * 1024) / (pl.n_code * (DSUB + 1) * 4);
-  if (m_per_cta > pl.M) m_per_cta = pl.M;
-  if (m_per_cta < 1) return cudaErrorInvalidValue;
-  const int pq_smem = m_per_cta * pl.n_code * (DSUB + 1) * 4;
-  PQHSA_TRY(cudaFuncSetAttribute(build_pq_assign_kernel<DSUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, pq_smem));
-  const dim3 pq_grid((pl.N_max + 127) / 128, units, (pl.M + m_per_cta - 1) / m_per_cta);
+  assign();
+  build_residual_kernel<<<dim3(tok_ctas, pl.Hkv, pl.B), kPrepThreads, 0, st>>>(pl, U, ix.centroids, ix.list_ids, seq_lens);
+  // product quantisation: about three waves of CTAs, each over a range of tokens that is a multiple
+  // of a step; of the splits near that, the one whose last wave is fullest
+  const int mg = PqPlan<DSUB>::mg(pl.n_code);
+  if (pl.M % mg != 0) return cudaErrorInvalidValue;
+  const int columns = units * (pl.M / mg), total_steps = (pl.N_max + kPqStep - 1) / kPqStep;
+  int steps = total_steps, best_cost = 0x7fffffff;
+  for (int s = total_steps; s >= 1; --s) {
+    const int ranges = (total_steps + s - 1) / s;
+    const long long ctas = (long long)ranges * columns;
+    if (ctas > 8LL * pl.num_sms && best_cost != 0x7fffffff) break;
+    const int waves = (int)((ctas + pl.num_sms - 1) / pl.num_sms), cost = waves * (s + 2);    // (+ 2: start and end of a CTA)
+    if (cost < best_cost) { best_cost = cost; steps = s; }
+  }
+  const dim3 pq_grid((total_steps + steps - 1) / steps, units, pl.M / mg);
+  const int range = steps * kPqStep;
+  const int smem_train = (int)PqPlan<DSUB>::smem(pl.n_code, true), smem_code = (int)PqPlan<DSUB>::smem(pl.n_code, false);
+  PQHSA_TRY(cudaFuncSetAttribute(build_pq_assign_kernel<DSUB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_train));
+  PQHSA_TRY(cudaFuncSetAttribute(build_pq_assign_kernel<DSUB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_code));
   const size_t n_entries = (size_t)units * pl.M * pl.n_code;
-  build_pq_seed_kernel<DSUB><<<dim3(pl.n_code, units), kD, 0, st>>>(pl, U, ix.centroids, ix.list_ids, seed_codes, ix.codebooks);
+  build_pq_seed_kernel<DSUB><<<dim3(pl.n_code, units), kD, 0, st>>>(pl, U, seed_codes, ix.codebooks);
   for (int it = 0; it < pq_iters; ++it) {
-    build_pq_assign_kernel<DSUB><<<pq_grid, 128, pq_smem, st>>>(pl, U, ix.centroids, ix.list_ids, ix.codebooks,
-                                                               seq_lens, m_per_cta, pq_sums, pq_counts, nullptr);
+    build_pq_assign_kernel<DSUB, true><<<pq_grid, kPqThreads, smem_train, st>>>(
+        pl, U, ix.codebooks, seq_lens, mg, range, pq_sums, pq_counts, nullptr, ix.key_norms);
     build_pq_update_kernel<<<(unsigned)((n_entries + 255) / 256), 256, 0, st>>>(n_entries, DSUB, pq_sums, pq_counts, ix.codebooks);
   }
-  build_pq_assign_kernel<DSUB><<<pq_grid, 128, pq_smem, st>>>(pl, U, ix.centroids, ix.list_ids, ix.codebooks,
-                                                             seq_lens, m_per_cta, nullptr, nullptr, ix.codes);
+  build_pq_assign_kernel<DSUB, false><<<pq_grid, kPqThreads, smem_code, st>>>(
+      pl, U, ix.codebooks, seq_lens, mg, range, nullptr, nullptr, ix.codes, ix.key_norms);
   // list value means and member counts
   PQHSA_TRY(cudaMemsetAsync(counts, 0, (size_t)units * pl.n_list * 4, st));
-  build_value_sums_kernel<T><<<dim3(tok_ctas, pl.Hkv, pl.B), kPrepThreads, 0, st>>>(
-      pl, vc, sp, stt, sh, kv.block_table, seq_lens, ix.list_ids, sums, counts);
+  build_hist_kernel<true><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, counts);
+  build_offsets_kernel<<<units, 1024, 0, st>>>(pl, counts, cursor);
+  build_scatter_kernel<true><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, cursor, order);
+  build_value_sums_kernel<T><<<run_grid, kPrepThreads, 0, st>>>(
+      pl, vc, sp, stt, sh, kv.block_table, seq_lens, ix.list_ids, order, sums);
   build_value_means_kernel<<<list_grid, 256, 0, st>>>(pl, sums, counts, ix.list_vmeans, ix.list_counts);
 #undef PQHSA_TRY
   return cudaGetLastError();

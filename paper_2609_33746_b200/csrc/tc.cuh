@@ -206,6 +206,14 @@ template <int DSUB> struct PqTile {
 // that has it.  The codeword inside the group is found by the caller in fp32: two instructions less
 // per accumulator than carrying an index.
 __device__ __forceinline__ float min3(float a, float b, float c) { return fminf(fminf(a, b), c); }
+__device__ __forceinline__ float min32(const float (&v)[32]) {
+  float m[11];
+#pragma unroll
+  for (int i = 0; i < 10; ++i) m[i] = min3(v[3 * i], v[3 * i + 1], v[3 * i + 2]);
+  m[10] = fminf(v[30], v[31]);
+  const float a = min3(m[0], m[1], m[2]), b = min3(m[3], m[4], m[5]), c = min3(m[6], m[7], m[8]);
+  return min3(min3(a, b, c), m[9], m[10]);
+}
 template <int N> __device__ __forceinline__ void group_minima(const float (&v)[N], int grp0, float& best, int& grp) {
 #pragma unroll
   for (int g = 0; g < N / 8; ++g) {
