@@ -2,11 +2,13 @@
 // sweep (Eq. 1 with E = every cached token).  Not part of the PQ-HSA path; it exists so that
 // the operator's time can be set against a full-KV read on the same GPU and the same cache.
 //
-// Split-K flash decoding.  grid (splits, KV heads, sequences); the CTA has one warp per query
-// head of the GQA group, and all warps walk the same slice of tokens, so a K/V row comes from
-// HBM once and from L1 for the other heads.  Inside a warp: 8 lanes per 256-byte row, 16 rows
-// in flight, online softmax in base 2.  The last CTA of a (sequence, KV head) merges the
-// partial (m, Z, N) triples of its G rows (atomic ticket; nobody waits).
+// Split-K flash decoding.  grid (splits, KV heads, sequences).  A warp takes windows of 32 tokens and
+// serves up to four query heads of the GQA group from one read and one unpacking of each K/V row: 16
+// lanes per 256-byte row, 8 rows in flight, online softmax in base 2; groups of more than four heads
+// are shared out among the CTA's warps, which walk the same tokens (L1).  The last CTA of a
+// (sequence, KV head) merges the partial (m, Z, N) triples of its G rows (atomic ticket; nobody
+// waits).  What bounds it: the read of the cache.  With one warp per head the rows were unpacked
+// four times (issue bound): 394 us for 8 x 32K tokens (2.7 TB/s).
 #include "attn_common.cuh"
 #include "common.cuh"
 
@@ -15,171 +17,279 @@ namespace pqhsa {
 namespace {
 
 constexpr int kDensePart = kPartStride;
-constexpr int kMaxDenseWarps = 16;
+constexpr int kDenseThreads = 256, kDenseWarps = kDenseThreads / 32;
+constexpr int kMaxDenseHeads = 16;
 
-template <typename T, int U>
-__global__ void __launch_bounds__(32 * kMaxDenseWarps)
+__device__ __forceinline__ unsigned long long dup2(float a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mk2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void un2(unsigned long long v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+template <typename T> __device__ __forceinline__ void unpack2(const uint4& u, unsigned long long (&p)[4]) {
+  float f[8];
+  Unpack<T>::run(u, f);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) p[i] = mk2(f[2 * i], f[2 * i + 1]);
+}
+
+// Sums one value per head over the 16 lanes of a row; lane l of the 16 ends with head head_of(l)'s total.
+template <int GH> __device__ __forceinline__ int head_of(int l16) {
+  return GH == 4 ? l16 >> 2 : (GH == 2 ? l16 >> 3 : 0);
+}
+template <int GH> __device__ __forceinline__ float reduce_heads(const float (&d)[GH], int l16) {
+  float x;
+  if constexpr (GH == 4) {
+    const bool up = (l16 & 8) != 0;
+    float k0 = up ? d[2] : d[0], k1 = up ? d[3] : d[1];
+    k0 += __shfl_xor_sync(0xffffffffu, up ? d[0] : d[2], 8);
+    k1 += __shfl_xor_sync(0xffffffffu, up ? d[1] : d[3], 8);
+    const bool up4 = (l16 & 4) != 0;
+    x = up4 ? k1 : k0;
+    x += __shfl_xor_sync(0xffffffffu, up4 ? k0 : k1, 4);
+  } else if constexpr (GH == 2) {
+    const bool up = (l16 & 8) != 0;
+    x = up ? d[1] : d[0];
+    x += __shfl_xor_sync(0xffffffffu, up ? d[0] : d[1], 8);
+    x += __shfl_xor_sync(0xffffffffu, x, 4);
+  } else {
+    x = d[0];
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
+    x += __shfl_xor_sync(0xffffffffu, x, 4);
+  }
+  x += __shfl_xor_sync(0xffffffffu, x, 2);
+  x += __shfl_xor_sync(0xffffffffu, x, 1);
+  return x;
+}
+
+template <typename T, int GH>
+__global__ void __launch_bounds__(kDenseThreads, 2)
 dense_decode_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc,
                     const T* __restrict__ vc, long long stride_page, long long stride_token,
                     long long stride_head, const int32_t* __restrict__ block_table,
                     const int32_t* __restrict__ seq_lens, float* __restrict__ part,
                     uint32_t* __restrict__ tickets, T* __restrict__ out) {
+  constexpr int U = 4;                                      // row pairs in flight
   __shared__ int s_last;
+  __shared__ float s_m[kDenseWarps][GH], s_Z[kDenseWarps][GH];
+  __shared__ __align__(16) float s_N[kDenseWarps][GH][kHeadDim];
   const int split = blockIdx.x, S = gridDim.x, kv = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int row = b * pl.Hq + kv * pl.G + warp;         // one query head per warp
+  const int half = lane >> 4, l16 = lane & 15;
+  const int n_grp = (pl.G + GH - 1) / GH;                   // head groups (1, or up to 4 of four heads)
+  const int n_par = kDenseWarps / n_grp;                    // warps that share a head group's tokens
+  const int hg = warp / n_par, par = warp - hg * n_par;     // (warps past n_grp * n_par idle)
+  const int row0 = b * pl.Hq + kv * pl.G + hg * GH;         // first query head of this warp
+  const int n_heads = hg < n_grp ? min(GH, pl.G - hg * GH) : 0;
   pdl_wait();
   pdl_launch_dependents();
   const int n = clamp_len(seq_lens[b], pl.N_max);
-  const int tl = (int)((long long)split * n / S), th = (int)((long long)(split + 1) * n / S);
+  const int tl = (int)((long long)split * n / S), th = n_heads > 0 ? (int)((long long)(split + 1) * n / S) : 0;
   const int32_t* bt = block_table + (size_t)b * pl.max_pages;
 
-  const int gi = lane >> 3, gl = lane & 7;
-  float qf[16];
-  {
-    const T* qr = q + (size_t)row * kHeadDim;
-    const float sc = pl.sm_scale * kLog2e;
+  unsigned long long q2[GH][4], acc[GH][4];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      qf[t] = sc * Unpack<T>::one(qr[8 * gl + t]);
-      qf[8 + t] = sc * Unpack<T>::one(qr[64 + 8 * gl + t]);
-    }
+  for (int g = 0; g < GH; ++g) {
+    uint4 w = make_uint4(0u, 0u, 0u, 0u);
+    if (g < n_heads) w = __ldg(reinterpret_cast<const uint4*>(q + (size_t)(row0 + g) * kHeadDim) + l16);
+    unpack2<T>(w, q2[g]);
+    const unsigned long long sc = dup2(pl.sm_scale * kLog2e);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) { q2[g][t] = mul2(q2[g][t], sc); acc[g][t] = 0ull; }
   }
-  GroupState st;
-  st.m = -CUDART_INF_F;
-  st.Z = 0.f;
-#pragma unroll
-  for (int t = 0; t < 16; ++t) st.acc[t] = 0.f;
+  float m = -CUDART_INF_F, Z = 0.f;                         // of head head_of(l16), this half's rows
 
-  int my_page = (tl + lane < th) ? __ldg(bt + (tl + lane) / pl.page_size) : 0;
-  for (int base = tl; base < th; base += 32) {
+  const int first = tl + 32 * par, stride = 32 * n_par;
+  int my_page = (first + lane < th) ? __ldg(bt + (first + lane) / pl.page_size) : 0;
+  for (int base = first; base < th; base += stride) {
     const int pos = base + lane;
     long long off = 0;
     if (pos < th)
       off = (long long)my_page * stride_page + (long long)(pos % pl.page_size) * stride_token +
             (long long)kv * stride_head;
     const int nb = min(32, th - base);
-    for (int j0 = 0; j0 < nb; j0 += 4 * U) {
-      uint4 kr[U][2], vr[U][2];
-      bool ok[U];
+#pragma unroll 1
+    for (int j0 = 0; j0 < nb; j0 += 2 * U) {
+      uint4 kr[U], vr[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int tok = j0 + 4 * u + gi;
+        const int tok = j0 + 2 * u + half;
         const long long o = __shfl_sync(0xffffffffu, off, tok & 31);
-        ok[u] = tok < nb;
-        if (ok[u]) {
-          const uint4* kp = reinterpret_cast<const uint4*>(kc + o);
-          const uint4* vp = reinterpret_cast<const uint4*>(vc + o);
-          kr[u][0] = __ldg(kp + gl); kr[u][1] = __ldg(kp + 8 + gl);
-          vr[u][0] = __ldg(vp + gl); vr[u][1] = __ldg(vp + 8 + gl);
-        } else {
-          kr[u][0] = kr[u][1] = vr[u][0] = vr[u][1] = make_uint4(0u, 0u, 0u, 0u);
+        kr[u] = vr[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (tok < nb) {
+          kr[u] = __ldg(reinterpret_cast<const uint4*>(kc + o) + l16);
+          vr[u] = __ldg(reinterpret_cast<const uint4*>(vc + o) + l16);
         }
       }
-      if (j0 == 0 && base + 32 + lane < th) my_page = __ldg(bt + (base + 32 + lane) / pl.page_size);
+      if (j0 == 0 && base + stride + lane < th) my_page = __ldg(bt + (base + stride + lane) / pl.page_size);
+      float sc[U], mx = m;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        float kf[8];
-        float s = 0.f;
-        Unpack<T>::run(kr[u][0], kf);
+        unsigned long long k2[4];
+        unpack2<T>(kr[u], k2);
+        float d[GH];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) s = fmaf(qf[t], kf[t], s);
-        Unpack<T>::run(kr[u][1], kf);
+        for (int g = 0; g < GH; ++g) {
+          unsigned long long a = 0ull;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) s = fmaf(qf[8 + t], kf[t], s);
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
-        s += __shfl_xor_sync(0xffffffffu, s, 2);
-        s += __shfl_xor_sync(0xffffffffu, s, 4);
-        if (ok[u]) {
-          if (s > st.m) {
-            const float a = st.Z > 0.f ? fast_exp2(st.m - s) : 0.f;
-            st.Z *= a;
+          for (int t = 0; t < 4; ++t) a = fma2(q2[g][t], k2[t], a);
+          float x, y;
+          un2(a, x, y);
+          d[g] = x + y;
+        }
+        sc[u] = reduce_heads<GH>(d, l16);
+        if (j0 + 2 * u + half >= nb) sc[u] = -CUDART_INF_F;
+        mx = fmaxf(mx, sc[u]);
+      }
+      if (__any_sync(0xffffffffu, mx > m)) {                // some head's maximum grew
+        const float a = mx > m && m > -CUDART_INF_F ? fast_exp2(m - mx) : (mx > m ? 0.f : 1.f);
+        Z *= a;
+        m = mx;
 #pragma unroll
-            for (int t = 0; t < 16; ++t) st.acc[t] *= a;
-            st.m = s;
-          }
-          const float p = fast_exp2(s - st.m);
-          st.Z += p;
-          float vf[8];
-          Unpack<T>::run(vr[u][0], vf);
+        for (int g = 0; g < GH; ++g) {
+          const unsigned long long ag = dup2(__shfl_sync(0xffffffffu, a, (lane & 16) + g * (16 / GH)));
 #pragma unroll
-          for (int t = 0; t < 8; ++t) st.acc[t] = fmaf(p, vf[t], st.acc[t]);
-          Unpack<T>::run(vr[u][1], vf);
+          for (int t = 0; t < 4; ++t) acc[g][t] = mul2(acc[g][t], ag);
+        }
+      }
 #pragma unroll
-          for (int t = 0; t < 8; ++t) st.acc[8 + t] = fmaf(p, vf[t], st.acc[8 + t]);
+      for (int u = 0; u < U; ++u) {
+        const float p = sc[u] > -CUDART_INF_F ? fast_exp2(sc[u] - m) : 0.f;
+        Z += p;
+        unsigned long long v2[4];
+        unpack2<T>(vr[u], v2);
+#pragma unroll
+        for (int g = 0; g < GH; ++g) {
+          const unsigned long long pg = dup2(__shfl_sync(0xffffffffu, p, (lane & 16) + g * (16 / GH)));
+#pragma unroll
+          for (int t = 0; t < 4; ++t) acc[g][t] = fma2(pg, v2[t], acc[g][t]);
         }
       }
     }
   }
-  // merge the 4 lane groups of the warp
+  // the two halves of the warp, then the warps of the head group through shared memory
+  {
+    const float m_o = __shfl_xor_sync(0xffffffffu, m, 16), Z_o = __shfl_xor_sync(0xffffffffu, Z, 16);
+    const float m_n = fmaxf(m, m_o);
+    const float a = safe_scale(m, m_n, Z);
+    Z = Z * a + Z_o * safe_scale(m_o, m_n, Z_o);
+    m = m_n;
 #pragma unroll
-  for (int o = 8; o <= 16; o <<= 1) {
-    const float m_o = __shfl_xor_sync(0xffffffffu, st.m, o);
-    const float Z_o = __shfl_xor_sync(0xffffffffu, st.Z, o);
-    const float m_n = fmaxf(st.m, m_o);
-    const float a = safe_scale(st.m, m_n, st.Z), bsc = safe_scale(m_o, m_n, Z_o);
-    st.Z = st.Z * a + Z_o * bsc;
+    for (int g = 0; g < GH; ++g) {
+      const float ag = __shfl_sync(0xffffffffu, a, (lane & 16) + g * (16 / GH));
+      float f[8];
 #pragma unroll
-    for (int t = 0; t < 16; ++t) {
-      const float acc_o = __shfl_xor_sync(0xffffffffu, st.acc[t], o);
-      st.acc[t] = st.acc[t] * a + acc_o * bsc;
+      for (int t = 0; t < 4; ++t) un2(acc[g][t], f[2 * t], f[2 * t + 1]);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        f[t] *= ag;
+        f[t] += __shfl_xor_sync(0xffffffffu, f[t], 16);
+      }
+      if (half == 0) {
+        *reinterpret_cast<float4*>(&s_N[warp][g][8 * l16]) = make_float4(f[0], f[1], f[2], f[3]);
+        *reinterpret_cast<float4*>(&s_N[warp][g][8 * l16 + 4]) = make_float4(f[4], f[5], f[6], f[7]);
+      }
     }
-    st.m = m_n;
+    if (half == 0 && (l16 & (16 / GH - 1)) == 0) { s_m[warp][head_of<GH>(l16)] = m; s_Z[warp][head_of<GH>(l16)] = Z; }
   }
-  float* pr = part + ((size_t)row * S + split) * kDensePart;
-  if (gi == 0) {
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      pr[4 + 8 * gl + t] = st.acc[t];
-      pr[4 + 64 + 8 * gl + t] = st.acc[8 + t];
+  __syncthreads();
+  const int unit_row0 = b * pl.Hq + kv * pl.G;
+  for (int i = tid; i < pl.G * kHeadDim; i += kDenseThreads) {
+    const int h = i / kHeadDim, dim = i % kHeadDim, w0 = (h / GH) * n_par, g = h % GH;
+    float m_c = -CUDART_INF_F, Z_c = 0.f, N_c = 0.f;
+    for (int w = w0; w < w0 + n_par; ++w) if (s_Z[w][g] > 0.f) m_c = fmaxf(m_c, s_m[w][g]);
+    for (int w = w0; w < w0 + n_par; ++w) {
+      const float a = safe_scale(s_m[w][g], m_c, s_Z[w][g]);
+      Z_c = fmaf(s_Z[w][g], a, Z_c);
+      N_c = fmaf(s_N[w][g][dim], a, N_c);
     }
-    if (gl == 0) { pr[0] = st.m; pr[1] = st.Z; }
+    float* pr = part + ((size_t)(unit_row0 + h) * S + split) * kDensePart;
+    pr[4 + dim] = N_c;
+    if (dim == 0) { pr[0] = m_c; pr[1] = Z_c; }
   }
   if (!cta_arrived_last(&tickets[b * pl.Hkv + kv], (uint32_t)S, &s_last)) return;
-  // last CTA of this (sequence, KV head): each warp merges its row (lane t fetches (m, Z) of
-  // partials t, t + 32, ...; then every lane sums its 4 dims over the partials, 8 in flight)
-  const float* rp = part + (size_t)row * S * kDensePart;
-  float m_r = -CUDART_INF_F;
-  for (int s = lane; s < S; s += 32) {
-    const float2 mz = __ldcg(reinterpret_cast<const float2*>(rp + (size_t)s * kDensePart));
-    if (mz.y > 0.f) m_r = fmaxf(m_r, mz.x);
-  }
+  // last CTA of this (sequence, KV head): a warp merges a row (lane t fetches (m, Z) of partials
+  // t, t + 32, ...; then every lane sums its 4 dims over the partials, 8 in flight)
+  for (int h = warp; h < pl.G; h += kDenseWarps) {
+    const int row = unit_row0 + h;
+    const float* rp = part + (size_t)row * S * kDensePart;
+    float m_r = -CUDART_INF_F;
+    for (int s = lane; s < S; s += 32) {
+      const float2 mz = __ldcg(reinterpret_cast<const float2*>(rp + (size_t)s * kDensePart));
+      if (mz.y > 0.f) m_r = fmaxf(m_r, mz.x);
+    }
+    m_r = warp_max(m_r);
+    float Z_r = 0.f;
+    float4 N_r = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < S; s0 += 8) {
+      float2 mz[8];
+      float4 v[8];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m_r = fmaxf(m_r, __shfl_xor_sync(0xffffffffu, m_r, o));
-  float Z_r = 0.f;
-  float4 N_r = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s0 = 0; s0 < S; s0 += 8) {
-    float2 mz[8];
-    float4 v[8];
+      for (int u = 0; u < 8; ++u) {
+        mz[u] = make_float2(0.f, 0.f);
+        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s0 + u < S) {
+          mz[u] = __ldcg(reinterpret_cast<const float2*>(rp + (size_t)(s0 + u) * kDensePart));
+          v[u] = __ldcg(reinterpret_cast<const float4*>(rp + (size_t)(s0 + u) * kDensePart + 4) + lane);
+        }
+      }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      mz[u] = make_float2(0.f, 0.f);
-      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (s0 + u < S) {
-        mz[u] = __ldcg(reinterpret_cast<const float2*>(rp + (size_t)(s0 + u) * kDensePart));
-        v[u] = __ldcg(reinterpret_cast<const float4*>(rp + (size_t)(s0 + u) * kDensePart + 4) + lane);
+      for (int u = 0; u < 8; ++u) {
+        const float a = safe_scale(mz[u].x, m_r, mz[u].y);
+        Z_r = fmaf(mz[u].y, a, Z_r);
+        N_r.x = fmaf(v[u].x, a, N_r.x); N_r.y = fmaf(v[u].y, a, N_r.y);
+        N_r.z = fmaf(v[u].z, a, N_r.z); N_r.w = fmaf(v[u].w, a, N_r.w);
       }
     }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const float a = safe_scale(mz[u].x, m_r, mz[u].y);
-      Z_r = fmaf(mz[u].y, a, Z_r);
-      N_r.x = fmaf(v[u].x, a, N_r.x); N_r.y = fmaf(v[u].y, a, N_r.y);
-      N_r.z = fmaf(v[u].z, a, N_r.z); N_r.w = fmaf(v[u].w, a, N_r.w);
-    }
+    const float inv = Z_r > 0.f ? 1.f / Z_r : 0.f;
+    T* o = out + (size_t)row * kHeadDim + 4 * lane;
+    o[0] = Unpack<T>::pack(N_r.x * inv); o[1] = Unpack<T>::pack(N_r.y * inv);
+    o[2] = Unpack<T>::pack(N_r.z * inv); o[3] = Unpack<T>::pack(N_r.w * inv);
   }
-  const float inv = Z_r > 0.f ? 1.f / Z_r : 0.f;
-  T* o = out + (size_t)row * kHeadDim + 4 * lane;
-  o[0] = Unpack<T>::pack(N_r.x * inv); o[1] = Unpack<T>::pack(N_r.y * inv);
-  o[2] = Unpack<T>::pack(N_r.z * inv); o[3] = Unpack<T>::pack(N_r.w * inv);
 }
 
+// Splits per (sequence, KV head): whole waves of two CTAs per SM, at least 256 tokens each (more
+// pieces even out ragged lengths, but every piece leaves a partial to merge).
 int dense_splits(const Plan& pl) {
-  int s = (4 * pl.num_sms) / (pl.B * pl.Hkv);
-  const int max_s = pl.N_max / 256 > 0 ? pl.N_max / 256 : 1;
-  if (s > max_s) s = max_s;
-  if (s > 256) s = 256;
-  return s < 1 ? 1 : s;
+  const int units = pl.B * pl.Hkv, slots = 2 * pl.num_sms;
+  int max_s = pl.N_max / 256 > 0 ? pl.N_max / 256 : 1;
+  if (max_s > 256) max_s = 256;
+  int best = 1;
+  double best_cost = 1e30;
+  for (int s = 1; s <= max_s; ++s) {
+    const int waves = (units * s + slots - 1) / slots;
+    if (waves > 4 && s > 1) break;
+    const double cost = (double)waves / s + 0.002 * waves;
+    if (cost < best_cost) { best_cost = cost; best = s; }
+  }
+  return best;
+}
+
+template <typename T>
+cudaError_t launch_dense_t(const Plan& pl, const void* q, const pqhsa_paged_kv& kv, const int32_t* seq_lens,
+                           float* part, uint32_t* tickets, void* out, cudaStream_t st) {
+  auto kernel = pl.G == 1 ? dense_decode_kernel<T, 1> : pl.G == 2 ? dense_decode_kernel<T, 2> : dense_decode_kernel<T, 4>;
+  return launch_pdl(kernel, dim3(dense_splits(pl), pl.Hkv, pl.B), dim3(kDenseThreads), 0, st, pl,
+                    static_cast<const T*>(q), static_cast<const T*>(kv.k_cache), static_cast<const T*>(kv.v_cache),
+                    (long long)kv.stride_page, (long long)kv.stride_token, (long long)kv.stride_head,
+                    kv.block_table, seq_lens, part, tickets, static_cast<T*>(out));
 }
 
 size_t align256d(size_t x) { return (x + 255) / 256 * 256; }
@@ -264,7 +374,7 @@ int pqhsa_dense_decode(const pqhsa_params* params, const void* q, const pqhsa_pa
       (reinterpret_cast<uintptr_t>(ws) & 255u) != 0)
     return PQHSA_ERR_INVALID_ARG;
   if (kv->stride_page % 8 || kv->stride_token % 8 || kv->stride_head % 8) return PQHSA_ERR_UNSUPPORTED;
-  if (pl.G > kMaxDenseWarps) return PQHSA_ERR_UNSUPPORTED;
+  if (pl.G > kMaxDenseHeads) return PQHSA_ERR_UNSUPPORTED;
   if (ws_bytes < pqhsa_dense_workspace_bytes(params)) return PQHSA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
@@ -272,21 +382,9 @@ int pqhsa_dense_decode(const pqhsa_params* params, const void* q, const pqhsa_pa
   if (cudaMemsetAsync(w, 0, tick_bytes, st) != cudaSuccess) return PQHSA_ERR_CUDA;
   uint32_t* tickets = reinterpret_cast<uint32_t*>(w);
   float* part = reinterpret_cast<float*>(w + tick_bytes);
-  const dim3 grid(dense_splits(pl), pl.Hkv, pl.B), block(32 * pl.G);
-  cudaError_t e;
-  if (pl.dtype == PQHSA_F16)
-    e = launch_pdl(dense_decode_kernel<__half, 4>, grid, block, 0, st, pl,
-                   static_cast<const __half*>(q), static_cast<const __half*>(kv->k_cache),
-                   static_cast<const __half*>(kv->v_cache), (long long)kv->stride_page,
-                   (long long)kv->stride_token, (long long)kv->stride_head, kv->block_table,
-                   seq_lens, part, tickets, static_cast<__half*>(out));
-  else
-    e = launch_pdl(dense_decode_kernel<__nv_bfloat16, 4>, grid, block, 0, st, pl,
-                   static_cast<const __nv_bfloat16*>(q),
-                   static_cast<const __nv_bfloat16*>(kv->k_cache),
-                   static_cast<const __nv_bfloat16*>(kv->v_cache), (long long)kv->stride_page,
-                   (long long)kv->stride_token, (long long)kv->stride_head, kv->block_table,
-                   seq_lens, part, tickets, static_cast<__nv_bfloat16*>(out));
+  const cudaError_t e = pl.dtype == PQHSA_F16
+                            ? launch_dense_t<__half>(pl, q, *kv, seq_lens, part, tickets, out, st)
+                            : launch_dense_t<__nv_bfloat16>(pl, q, *kv, seq_lens, part, tickets, out, st);
   return e == cudaSuccess ? PQHSA_OK : PQHSA_ERR_CUDA;
 }
 
