@@ -4,13 +4,17 @@
 //
 // Split-K flash decoding.  grid (splits, KV heads, sequences).  A warp takes windows of 32 tokens and
 // serves up to four query heads of the GQA group from one read and one unpacking of each K/V row: 16
-// lanes per 256-byte row, 8 rows in flight, online softmax in base 2; groups of more than four heads
-// are shared out among the CTA's warps, which walk the same tokens (L1).  The last CTA of a
-// (sequence, KV head) merges the partial (m, Z, N) triples of its G rows (atomic ticket; nobody
-// waits).  What bounds it: the read of the cache.  With one warp per head the rows were unpacked
-// four times (issue bound): 394 us for 8 x 32K tokens (2.7 TB/s).
+// lanes per 256-byte row, online softmax in base 2; groups of more than four heads are shared out
+// among the CTA's warps, which walk the same tokens (L1).  Rows come through a per-warp ring of
+// asynchronous copies, 8 rows (4 KB) a stage and two stages ahead of the one in use; a lane copies
+// the 16 bytes that it reads itself, so the ring needs no barrier.  The last CTA of a (sequence, KV
+// head) merges the partial (m, Z, N) triples of its G rows (atomic ticket; nobody waits).
+// What bounds it: the read of the cache.  8 x 32K tokens, 32 / 8 heads: one warp per head (rows
+// unpacked four times) 394 us, four heads per warp with loads into registers 260 us (latency: 3.9
+// warps waiting per issue), with the ring 196 us (5.5 TB/s).
 #include "attn_common.cuh"
 #include "common.cuh"
+#include "scan_common.cuh"
 
 namespace pqhsa {
 
@@ -19,6 +23,8 @@ namespace {
 constexpr int kDensePart = kPartStride;
 constexpr int kDenseThreads = 256, kDenseWarps = kDenseThreads / 32;
 constexpr int kMaxDenseHeads = 16;
+constexpr int kDenseStages = 3, kStageRows = 8, kStageBytes = kStageRows * 4 * kHeadDim;
+constexpr int kDenseSmem = kDenseWarps * kDenseStages * kStageBytes;
 
 __device__ __forceinline__ unsigned long long dup2(float a) {
   unsigned long long r;
@@ -86,10 +92,10 @@ dense_decode_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc,
                     long long stride_head, const int32_t* __restrict__ block_table,
                     const int32_t* __restrict__ seq_lens, float* __restrict__ part,
                     uint32_t* __restrict__ tickets, T* __restrict__ out) {
-  constexpr int U = 4;                                      // row pairs in flight
+  constexpr int U = kStageRows / 2;                         // row pairs per stage
+  extern __shared__ __align__(128) unsigned char s_ring[];  // [warp][stage][row][K 256 bytes | V 256 bytes]
   __shared__ int s_last;
   __shared__ float s_m[kDenseWarps][GH], s_Z[kDenseWarps][GH];
-  __shared__ __align__(16) float s_N[kDenseWarps][GH][kHeadDim];
   const int split = blockIdx.x, S = gridDim.x, kv = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int half = lane >> 4, l16 = lane & 15;
@@ -116,74 +122,99 @@ dense_decode_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc,
   }
   float m = -CUDART_INF_F, Z = 0.f;                         // of head head_of(l16), this half's rows
 
+  // this warp's windows of 32 tokens: first, first + stride, ..; a stage is a quarter of a window
   const int first = tl + 32 * par, stride = 32 * n_par;
+  const int n_steps = first < th ? 4 * ((th - first + stride - 1) / stride) : 0;
+  unsigned char* ring = s_ring + warp * (kDenseStages * kStageBytes);
+  const uint32_t ring_u32 = smem_u32(ring) + half * 512 + l16 * 16;
   int my_page = (first + lane < th) ? __ldg(bt + (first + lane) / pl.page_size) : 0;
-  for (int base = first; base < th; base += stride) {
-    const int pos = base + lane;
-    long long off = 0;
-    if (pos < th)
-      off = (long long)my_page * stride_page + (long long)(pos % pl.page_size) * stride_token +
-            (long long)kv * stride_head;
-    const int nb = min(32, th - base);
+  long long off = 0;                                        // this lane's token of the window being copied
+  auto issue = [&](int st) {
+    if (st < n_steps) {
+      const int base = first + (st >> 2) * stride;
+      if ((st & 3) == 0) {
+        const int pos = base + lane;
+        off = 0;
+        if (pos < th)
+          off = (long long)my_page * stride_page + (long long)(pos % pl.page_size) * stride_token +
+                (long long)kv * stride_head;
+        if (pos + stride < th) my_page = __ldg(bt + (pos + stride) / pl.page_size);
+      }
+      const uint32_t dst = ring_u32 + (uint32_t)(st % kDenseStages) * kStageBytes;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tok = (st & 3) * kStageRows + 2 * u + half;
+        const long long o = __shfl_sync(0xffffffffu, off, tok);
+        const uint32_t bytes = base + tok < th ? 16u : 0u;  // rows past the slice are zero-filled
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + u * 1024u),
+                     "l"(reinterpret_cast<const uint4*>(kc + o) + l16), "r"(bytes) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + u * 1024u + 256u),
+                     "l"(reinterpret_cast<const uint4*>(vc + o) + l16), "r"(bytes) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto row_part = [&](uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+  };
+#pragma unroll
+  for (int st = 0; st < kDenseStages - 1; ++st) issue(st);
 #pragma unroll 1
-    for (int j0 = 0; j0 < nb; j0 += 2 * U) {
-      uint4 kr[U], vr[U];
+  for (int st = 0; st < n_steps; ++st) {
+    issue(st + kDenseStages - 1);
+    asm volatile("cp.async.wait_group %0;" ::"n"(kDenseStages - 1) : "memory");
+    const uint32_t src = ring_u32 + (uint32_t)(st % kDenseStages) * kStageBytes;
+    const int left = th - (first + (st >> 2) * stride + (st & 3) * kStageRows);   // tokens from this stage on
+    if (left <= 0) continue;                                // (warp-uniform)
+    float sc[U], mx = m;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int tok = j0 + 2 * u + half;
-        const long long o = __shfl_sync(0xffffffffu, off, tok & 31);
-        kr[u] = vr[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (tok < nb) {
-          kr[u] = __ldg(reinterpret_cast<const uint4*>(kc + o) + l16);
-          vr[u] = __ldg(reinterpret_cast<const uint4*>(vc + o) + l16);
-        }
+    for (int u = 0; u < U; ++u) {
+      unsigned long long k2[4];
+      unpack2<T>(row_part(src + u * 1024u), k2);
+      float d[GH];
+#pragma unroll
+      for (int g = 0; g < GH; ++g) {
+        unsigned long long a = 0ull;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) a = fma2(q2[g][t], k2[t], a);
+        float x, y;
+        un2(a, x, y);
+        d[g] = x + y;
       }
-      if (j0 == 0 && base + stride + lane < th) my_page = __ldg(bt + (base + stride + lane) / pl.page_size);
-      float sc[U], mx = m;
+      sc[u] = reduce_heads<GH>(d, l16);
+      if (2 * u + half >= left) sc[u] = -CUDART_INF_F;
+      mx = fmaxf(mx, sc[u]);
+    }
+    if (__any_sync(0xffffffffu, mx > m)) {                  // some head's maximum grew
+      const float a = mx > m && m > -CUDART_INF_F ? fast_exp2(m - mx) : (mx > m ? 0.f : 1.f);
+      Z *= a;
+      m = mx;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        unsigned long long k2[4];
-        unpack2<T>(kr[u], k2);
-        float d[GH];
+      for (int g = 0; g < GH; ++g) {
+        const unsigned long long ag = dup2(__shfl_sync(0xffffffffu, a, (lane & 16) + g * (16 / GH)));
 #pragma unroll
-        for (int g = 0; g < GH; ++g) {
-          unsigned long long a = 0ull;
-#pragma unroll
-          for (int t = 0; t < 4; ++t) a = fma2(q2[g][t], k2[t], a);
-          float x, y;
-          un2(a, x, y);
-          d[g] = x + y;
-        }
-        sc[u] = reduce_heads<GH>(d, l16);
-        if (j0 + 2 * u + half >= nb) sc[u] = -CUDART_INF_F;
-        mx = fmaxf(mx, sc[u]);
+        for (int t = 0; t < 4; ++t) acc[g][t] = mul2(acc[g][t], ag);
       }
-      if (__any_sync(0xffffffffu, mx > m)) {                // some head's maximum grew
-        const float a = mx > m && m > -CUDART_INF_F ? fast_exp2(m - mx) : (mx > m ? 0.f : 1.f);
-        Z *= a;
-        m = mx;
+    }
 #pragma unroll
-        for (int g = 0; g < GH; ++g) {
-          const unsigned long long ag = dup2(__shfl_sync(0xffffffffu, a, (lane & 16) + g * (16 / GH)));
+    for (int u = 0; u < U; ++u) {
+      const float p = sc[u] > -CUDART_INF_F ? fast_exp2(sc[u] - m) : 0.f;
+      Z += p;
+      unsigned long long v2[4];
+      unpack2<T>(row_part(src + u * 1024u + 256u), v2);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) acc[g][t] = mul2(acc[g][t], ag);
-        }
-      }
+      for (int g = 0; g < GH; ++g) {
+        const unsigned long long pg = dup2(__shfl_sync(0xffffffffu, p, (lane & 16) + g * (16 / GH)));
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const float p = sc[u] > -CUDART_INF_F ? fast_exp2(sc[u] - m) : 0.f;
-        Z += p;
-        unsigned long long v2[4];
-        unpack2<T>(vr[u], v2);
-#pragma unroll
-        for (int g = 0; g < GH; ++g) {
-          const unsigned long long pg = dup2(__shfl_sync(0xffffffffu, p, (lane & 16) + g * (16 / GH)));
-#pragma unroll
-          for (int t = 0; t < 4; ++t) acc[g][t] = fma2(pg, v2[t], acc[g][t]);
-        }
+        for (int t = 0; t < 4; ++t) acc[g][t] = fma2(pg, v2[t], acc[g][t]);
       }
     }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();                                             // the warp's ring now holds its partial sums
+  auto s_N = [&](int w, int g) { return reinterpret_cast<float*>(s_ring + w * (kDenseStages * kStageBytes)) + g * kHeadDim; };
   // the two halves of the warp, then the warps of the head group through shared memory
   {
     const float m_o = __shfl_xor_sync(0xffffffffu, m, 16), Z_o = __shfl_xor_sync(0xffffffffu, Z, 16);
@@ -203,8 +234,8 @@ dense_decode_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc,
         f[t] += __shfl_xor_sync(0xffffffffu, f[t], 16);
       }
       if (half == 0) {
-        *reinterpret_cast<float4*>(&s_N[warp][g][8 * l16]) = make_float4(f[0], f[1], f[2], f[3]);
-        *reinterpret_cast<float4*>(&s_N[warp][g][8 * l16 + 4]) = make_float4(f[4], f[5], f[6], f[7]);
+        *reinterpret_cast<float4*>(s_N(warp, g) + 8 * l16) = make_float4(f[0], f[1], f[2], f[3]);
+        *reinterpret_cast<float4*>(s_N(warp, g) + 8 * l16 + 4) = make_float4(f[4], f[5], f[6], f[7]);
       }
     }
     if (half == 0 && (l16 & (16 / GH - 1)) == 0) { s_m[warp][head_of<GH>(l16)] = m; s_Z[warp][head_of<GH>(l16)] = Z; }
@@ -218,7 +249,7 @@ dense_decode_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc,
     for (int w = w0; w < w0 + n_par; ++w) {
       const float a = safe_scale(s_m[w][g], m_c, s_Z[w][g]);
       Z_c = fmaf(s_Z[w][g], a, Z_c);
-      N_c = fmaf(s_N[w][g][dim], a, N_c);
+      N_c = fmaf(s_N(w, g)[dim], a, N_c);
     }
     float* pr = part + ((size_t)(unit_row0 + h) * S + split) * kDensePart;
     pr[4 + dim] = N_c;
@@ -286,7 +317,9 @@ template <typename T>
 cudaError_t launch_dense_t(const Plan& pl, const void* q, const pqhsa_paged_kv& kv, const int32_t* seq_lens,
                            float* part, uint32_t* tickets, void* out, cudaStream_t st) {
   auto kernel = pl.G == 1 ? dense_decode_kernel<T, 1> : pl.G == 2 ? dense_decode_kernel<T, 2> : dense_decode_kernel<T, 4>;
-  return launch_pdl(kernel, dim3(dense_splits(pl), pl.Hkv, pl.B), dim3(kDenseThreads), 0, st, pl,
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseSmem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kernel, dim3(dense_splits(pl), pl.Hkv, pl.B), dim3(kDenseThreads), kDenseSmem, st, pl,
                     static_cast<const T*>(q), static_cast<const T*>(kv.k_cache), static_cast<const T*>(kv.v_cache),
                     (long long)kv.stride_page, (long long)kv.stride_token, (long long)kv.stride_head,
                     kv.block_table, seq_lens, part, tickets, static_cast<T*>(out));
