@@ -1,6 +1,6 @@
 """Dense decode attention at the edges of its windows, stages and head groups (-m gpu), against
-softmax attention in float64 on the same cache values.  Tolerance: half an ulp of the output type at
-the output's magnitude (values are N(0, 1): below 4) plus fp32 sums of at most 2,000 terms."""
+softmax attention in float64 on the same cache values.  Tolerance: half an ulp of the output type
+(2^-8 of the value in bf16, 2^-11 in fp16) plus 1e-4 for the fp32 sums of at most 2,000 terms."""
 import math
 
 import pytest
@@ -11,10 +11,10 @@ from paper_2609_33746_b200 import pqhsa
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dtype,atol", [("bf16", 2.0 ** -7), ("fp16", 2.0 ** -9)])
+@pytest.mark.parametrize("dtype,half_ulp", [("bf16", 2.0 ** -8), ("fp16", 2.0 ** -11)])
 @pytest.mark.parametrize("group", [1, 2, 3, 5, 8, 12, 16])
 @pytest.mark.parametrize("lens,page", [((1, 7, 8), 16), ((9, 31, 32), 1), ((33, 255, 257), 32), ((1000, 0, 2003), 16)])
-def test_dense_at_the_edges(lens, page, group, dtype, atol):
+def test_dense_at_the_edges(lens, page, group, dtype, half_ulp):
     kv_heads, d, B = 2, 128, len(lens)
     tdt = {"bf16": torch.bfloat16, "fp16": torch.float16}[dtype]
     n_max = (max(lens) + 15) // 16 * 16
@@ -40,4 +40,4 @@ def test_dense_at_the_edges(lens, page, group, dtype, atol):
         K, V = (c[table[b, pos // page].long(), pos % page].double().transpose(0, 1) for c in cache)
         s = torch.einsum("hgd,hnd->hgn", q[b].double().view(kv_heads, group, d), K) / math.sqrt(d)
         want = torch.einsum("hgn,hnd->hgd", s.softmax(-1), V).reshape(-1, d)
-        assert float((out[b].double() - want).abs().max()) <= atol
+        assert bool(((out[b].double() - want).abs() <= half_ulp * want.abs() + 1e-4).all())
