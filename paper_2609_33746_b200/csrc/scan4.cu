@@ -3,31 +3,32 @@
 // four bits, 4 bytes of codes per token and KV head).
 //
 // A token is then 4 (M = 8) or 8 (M = 16) bytes of codes, a norm and a list id: 10 bytes read
-// and 4 * G bytes of scores written, against 8 table reads.  The kernel is laid out around that
+// and 4 * G bytes of scores written, against 4 table reads (one per byte of codes).  The kernel is laid out around that
 // record size, not around the 8-bit kernel's:
 //   * a lane owns FOUR consecutive tokens per iteration, so every global access is one 16-byte
 //     (codes, norms, one score row) or 8-byte (list ids) vector per lane, fully coalesced over
 //     the warp, and the next iteration's three loads are in flight while this one computes.
 //     No shared-memory staging of the codes at all;
-//   * the lookup table of a head group is 16 * M entries of 16 bytes (2 KB at M = 8) in the
-//     layout [z][m][g]; at step s a lane looks up subspace m = s ^ (lane & 7), so the bank group
-//     depends on m only and every 16-byte read is conflict free, as in the 8-bit kernel.  The
-//     address is formed with two instructions: a rotate that brings nibble m to the row-index
-//     bits, and one and-or with the lane's entry offset (the table is aligned to its size);
+//   * one lookup serves a whole byte, i.e. two subspaces: when a segment's tables arrive (16 * M
+//     entries, 2 KB at M = 8), the CTA forms the 256 sums of every pair of subspaces.  The pair
+//     table has one 128-byte row per byte value that holds the M / 2 pairs' entries, repeated until
+//     the row is full; at step s a lane looks up pair s ^ (lane & (pairs - 1)) in the copy given by
+//     its next lane bits, so the lanes of an access group always hit different banks: every read is
+//     conflict free.  (One lookup per nibble needed twice the reads and address instructions.)
 //   * the coarse table has one 128-byte row per list holding the entry once per lane of a
 //     quarter warp (half warp, warp for Gc = 2, 1), so the random per-token read never has a
 //     bank conflict; lists beyond what shared memory holds fall back to one entry per list;
 //   * per-list exp-sums: one vector reduction per token into the CTA's partial in global memory
 //     (L2), exactly as in the 8-bit kernel, with the same reference / rebuild rule.
-// What bounds it: the load/store data pipe again (table reads 32 wavefronts per 32 tokens, the
-// scattered reduction about 17, stores, coarse reads and loads about 14), at roughly a third
-// of the 8-bit kernel's time.
+// What bounds it: the load/store data pipe again (table reads 16 wavefronts per 32 tokens, the
+// scattered reduction about 17, stores, coarse reads and loads about 14).
 #include "scan_common.cuh"
 
 namespace pqhsa {
 
 namespace {
 
+constexpr int kPairTableBytes = 256 * 128;
 constexpr int kTok4 = 4;                         // consecutive tokens per lane and iteration
 constexpr int kWarpTok = 32 * kTok4;             // 128 tokens per warp and iteration
 constexpr int kStepTok4 = (kScanThreads / 32) * kWarpTok;
@@ -118,12 +119,11 @@ scan4_kernel(Plan pl, const uint8_t* __restrict__ codes, const uint16_t* __restr
              const float* __restrict__ coarse, const int32_t* __restrict__ seq_lens,
              float* __restrict__ scores, float* __restrict__ partials, int* __restrict__ status) {
   constexpr int kCW = M / 8;                          // 32-bit words of codes per token
-  constexpr int kLutFloats = 16 * M * GC;
+  constexpr int kLutFloats = 16 * M * GC;             // [z][m][g], as the table build leaves it
   constexpr int kEntryBytes = GC * 4;
-  constexpr int kRowBytes = M * kEntryBytes;          // stride between consecutive z
-  constexpr int kRowShift = (M == 8 ? 3 : 4) + (GC == 4 ? 4 : GC == 2 ? 3 : 2);   // log2(kRowBytes)
-  static_assert((1 << kRowShift) == kRowBytes, "row stride");
-  constexpr uint32_t kRowMask = 15u << kRowShift;
+  constexpr int kPairs = M / 2;                       // bytes of codes per token
+  constexpr int kCopies = 128 / (kPairs * kEntryBytes);      // copies of a pair's entry in a row
+  static_assert(kCopies >= 1 && kPairs * kCopies * kEntryBytes == 128, "a row is 128 bytes");
   constexpr int kRep = 128 / kEntryBytes;             // lanes of one shared-memory access group
   constexpr int kW = Packed<GC>::kW;
   constexpr int kWarps = kScanThreads / 32;
@@ -138,12 +138,11 @@ scan4_kernel(Plan pl, const uint8_t* __restrict__ codes, const uint16_t* __restr
   const int c = blockIdx.x;
   const int n_list = pl.n_list, N_max = pl.N_max, upb = pl.upb;
   const int coarse_mode = pl.coarse_in_smem;
-  // the table is addressed by or-ing the row index into the entry offset: align it to its size
-  const uint32_t raw_u32 = smem_u32(smem_raw);
-  const uint32_t lut_u32 = (raw_u32 + (kLutFloats * 4 - 1)) & ~uint32_t(kLutFloats * 4 - 1);
-  const uint32_t coarse_u32 = lut_u32 + kLutFloats * 4;
-  unsigned char* lut_ptr = smem_raw + (lut_u32 - raw_u32);
-  unsigned char* coarse_ptr = lut_ptr + kLutFloats * 4;
+  // pair table [256][kCopies][kPairs], coarse table, the nibble table as it arrives
+  unsigned char* pair_ptr = smem_raw;
+  unsigned char* coarse_ptr = pair_ptr + kPairTableBytes;
+  unsigned char* lut_ptr = coarse_ptr + (coarse_mode == 2 ? n_list * 128 : coarse_mode == 1 ? n_list * GC * 4 : 0);
+  const uint32_t pair_u32 = smem_u32(pair_ptr), coarse_u32 = smem_u32(coarse_ptr);
 
   pdl_wait();
   pdl_launch_dependents();
@@ -162,15 +161,14 @@ scan4_kernel(Plan pl, const uint8_t* __restrict__ codes, const uint16_t* __restr
   }
   uint32_t bar_parity = 0;
 
-  // per-lane constants of the skewed lookup: at step s the lane reads subspace m = s ^ (lane & 7)
-  const int lx = lane & 7;
-  uint32_t rot[8], ent[8];
+  // per-lane constants of the skewed lookup: at step s the lane reads pair s ^ lx
+  const int lx = lane & (kPairs - 1);
+  uint32_t sel[4], ent[kPairs];          // byte selector within a word, address of entry (byte 0, pair)
 #pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int m = s ^ lx;
-    rot[s] = uint32_t(4 * m - kRowShift) & 31u;          // rotate right: nibble m -> row-index bits
-    ent[s] = lut_u32 + uint32_t(m * kEntryBytes);
-  }
+  for (int s = 0; s < 4; ++s) sel[s] = 0x4440u | uint32_t(s ^ (lx & 3));
+#pragma unroll
+  for (int s = 0; s < kPairs; ++s)
+    ent[s] = pair_u32 + uint32_t(((s ^ lx) + kPairs * ((lane / kPairs) % kCopies)) * kEntryBytes);
   const uint32_t rep_off = uint32_t(lane & (kRep - 1)) * kEntryBytes;
   const unsigned long long l2e2 = pk2(kLog2e, kLog2e);
 
@@ -239,7 +237,23 @@ scan4_kernel(Plan pl, const uint8_t* __restrict__ codes, const uint16_t* __restr
     load_records<kCW>(cur, code_row, norm_row, lid_row, i4, i4 < seg_end);
     if (!mbar_wait(&s_bar, bar_parity)) atomicOr(status, kStatusCopyTimeout);
     bar_parity ^= 1u;
-    __syncthreads();   // partial zeroed, tables landed
+    // the sums of every pair of subspaces: byte = code of subspace 2 p | code of subspace 2 p + 1 << 4
+    for (int idx = tid; idx < 256 * kPairs; idx += kScanThreads) {
+      const int z = idx / kPairs, p = idx % kPairs;
+      Packed<GC> lo_e, hi_e;
+      lds_entry<GC>(lo_e, smem_u32(lut_ptr) + uint32_t(((z & 15) * M + 2 * p) * kEntryBytes));
+      lds_entry<GC>(hi_e, smem_u32(lut_ptr) + uint32_t(((z >> 4) * M + 2 * p + 1) * kEntryBytes));
+#pragma unroll
+      for (int j = 0; j < kW; ++j) lo_e.v[j] = add2(lo_e.v[j], hi_e.v[j]);
+#pragma unroll
+      for (int cp = 0; cp < kCopies; ++cp) {
+        unsigned char* dst = pair_ptr + z * 128 + (cp * kPairs + p) * kEntryBytes;
+        if constexpr (GC == 4) *reinterpret_cast<ulonglong2*>(dst) = make_ulonglong2(lo_e.v[0], lo_e.v[1]);
+        else if constexpr (GC == 2) *reinterpret_cast<unsigned long long*>(dst) = lo_e.v[0];
+        else *reinterpret_cast<uint32_t*>(dst) = (uint32_t)lo_e.v[0];
+      }
+    }
+    __syncthreads();   // partial zeroed, tables complete
 
     float mx[GC];
     unsigned long long nref2[kW];           // -(reference * log2 e) per head, packed
@@ -255,25 +269,25 @@ scan4_kernel(Plan pl, const uint8_t* __restrict__ codes, const uint16_t* __restr
       unsigned long long sc2[kTok4][kW];
 #pragma unroll
       for (int k = 0; k < kTok4; ++k) {
-        Packed<GC> acc0, acc1;
-#pragma unroll
-        for (int j = 0; j < kW; ++j) { acc0.v[j] = 0ull; acc1.v[j] = 0ull; }
+        // the lane's pairs of word cw: steps 4 cw .. 4 cw + 3 (of the words' order that the lane's
+        // bit 2 selects when there are eight pairs)
+        Packed<GC> v[kPairs];
 #pragma unroll
         for (int cw = 0; cw < kCW; ++cw) {
-          const uint32_t word = cur.code[k * kCW + cw];     // nibble m = code of subspace 8 cw + m
-          Packed<GC> v[8];
+          uint32_t word = cur.code[k * kCW + cw];
+          if constexpr (kCW == 2) { if (lx & 4) word = cur.code[k * kCW + (cw ^ 1)]; }
 #pragma unroll
-          for (int s = 0; s < 8; ++s) {
-            const uint32_t row = __funnelshift_r(word, word, rot[s]) & kRowMask;
-            lds_entry<GC>(v[s], (row | ent[s]) + uint32_t(cw * 8 * kEntryBytes));
-          }
+          for (int s = 0; s < 4; ++s)
+            lds_entry<GC>(v[4 * cw + s], ent[4 * cw + s] + (__byte_perm(word, 0u, sel[s]) << 7));
+        }
+        Packed<GC> acc0, acc1;
 #pragma unroll
-          for (int s = 0; s < 8; s += 2) {
-#pragma unroll
-            for (int j = 0; j < kW; ++j) {
-              acc0.v[j] = add2(acc0.v[j], v[s].v[j]);
-              acc1.v[j] = add2(acc1.v[j], v[s + 1].v[j]);
-            }
+        for (int j = 0; j < kW; ++j) {
+          acc0.v[j] = add2(v[0].v[j], v[1].v[j]);
+          acc1.v[j] = add2(v[2].v[j], v[3].v[j]);
+          if constexpr (kCW == 2) {
+            acc0.v[j] = add2(acc0.v[j], add2(v[4].v[j], v[5].v[j]));
+            acc1.v[j] = add2(acc1.v[j], add2(v[6].v[j], v[7].v[j]));
           }
         }
         // (a list id outside [0, n_list) is an index error, not a reason to read out of bounds)
@@ -448,14 +462,14 @@ cudaError_t launch_scan4_t(const Plan& pl, const pqhsa_index& ix, const float* l
 
 }  // namespace
 
-// Dynamic shared memory of the 4-bit scan: the table (aligned to its size inside the buffer)
-// and the coarse table in the given mode (0: none, 1: one entry per list, 2: a 128-byte row).
+// Dynamic shared memory of the 4-bit scan: the pair table, the coarse table in the given mode (0: none,
+// 1: one entry per list, 2: a 128-byte row) and the nibble table.
 size_t scan4_smem_bytes(const Plan& pl, int coarse_mode) {
   const size_t lut = (size_t)16 * pl.M * pl.Gc * 4;
   size_t co = 0;
   if (coarse_mode == 1) co = (size_t)pl.n_list * pl.Gc * 4;
   if (coarse_mode == 2) co = (size_t)pl.n_list * 128;
-  return 2 * lut + co;
+  return kPairTableBytes + co + lut;
 }
 
 cudaError_t launch_scan4(const Plan& pl, const pqhsa_index& ix, const float* lut,
