@@ -476,13 +476,16 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
   uint32_t* n_out = &counters[row * 4 + 2];
   uint32_t* n_cand = &counters[row * 4 + 3];
 
-  // Main pass.  Warps work independently: a lane marks which of its 16 scores reach the
-  // bracket and the warp packs the positions of the hits (bit 31 = certain winner) into its
-  // shared-memory buffer.  The buffer is written out when it would overflow and at the end,
-  // with one atomic per destination list, so the round trip of that atomic is paid once per
-  // warp and not once per chunk.
+  // Main pass.  Warps work independently: a lane marks which of its 16 scores reach the bracket and
+  // the warp packs the positions of the hits into its shared-memory buffer.  The buffer is written
+  // out when it would overflow and at the end, with one atomic per destination list, so the round
+  // trip of that atomic is paid once per warp and not once per chunk; only then the few hits are
+  // told apart (winner or candidate), from the score itself.
+  // What bounds the pass is instruction issue, not the read: a comparison against both edges for
+  // every score cost 22 instructions per score (44 us at 256 x 128K); the sign of the difference
+  // to the lower edge, shifted into a mask, is two.
   const int n_chunks = (n + kSelChunk - 1) / kSelChunk;
-  const bool no_winners = !(hi_f < CUDART_INF_F);   // bracket open at the top: candidates only
+  const float lo_s = lo_f == 0.f ? -0.f : lo_f;     // (so that -0 - lo is not negative)
   constexpr int kBuf = kSelChunk / 16;              // entries per warp: one chunk's worst case
   uint32_t* my_hits = s_hits + warp * kBuf;
   int buf_n = 0;                                    // warp-uniform
@@ -491,9 +494,10 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
     int nw = 0, nc = 0;
     for (int i0 = 0; i0 < buf_n; i0 += 32) {
       const bool v_ok = i0 + lane < buf_n;
-      const uint32_t ent = v_ok ? my_hits[i0 + lane] : 0u;
-      nw += __popc(__ballot_sync(0xffffffffu, v_ok && (ent >> 31)));
-      nc += __popc(__ballot_sync(0xffffffffu, v_ok && !(ent >> 31)));
+      // (from L2: this warp read it a moment ago.  NaN is neither)
+      const float sv = v_ok ? __ldcg(rs + my_hits[i0 + lane]) : CUDART_NAN_F;
+      nw += __popc(__ballot_sync(0xffffffffu, sv > hi_f));
+      nc += __popc(__ballot_sync(0xffffffffu, sv >= lo_f && sv <= hi_f));
     }
     uint32_t bw = 0, bc = 0;
     if (lane == 0) {
@@ -505,20 +509,19 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
     const unsigned lt = (1u << lane) - 1u;
     for (int i0 = 0; i0 < buf_n; i0 += 32) {
       const bool v_ok = i0 + lane < buf_n;
-      const uint32_t ent = v_ok ? my_hits[i0 + lane] : 0u;
-      const bool is_win = v_ok && (ent >> 31);
-      const bool is_cnd = v_ok && !(ent >> 31);
+      const uint32_t pos = v_ok ? my_hits[i0 + lane] : 0u;
+      const float sv = v_ok ? __ldcg(rs + pos) : CUDART_NAN_F;
+      const bool is_win = sv > hi_f, is_cnd = sv >= lo_f && sv <= hi_f;
       const unsigned mw = __ballot_sync(0xffffffffu, is_win);
       const unsigned mc = __ballot_sync(0xffffffffu, is_cnd);
       if (is_win) {
         const uint32_t p = bw + __popc(mw & lt);
-        if (p < (uint32_t)pl.k_max) out[p] = (int)(ent & 0x7fffffffu);
+        if (p < (uint32_t)pl.k_max) out[p] = (int)pos;
       }
       if (is_cnd) {
-        // the score comes back from L2 (this warp read it a moment ago), so that the row's
-        // last CTA finds key and position together and has no dependent gather to wait for
+        // key and position together: the row's last CTA has no dependent gather to wait for
         const uint32_t p = bc + __popc(mc & lt);
-        if (p < (uint32_t)pl.cand_cap) rc[p] = make_uint2(score_key(__ldcg(rs + ent)), ent);
+        if (p < (uint32_t)pl.cand_cap) rc[p] = make_uint2(score_key(sv), pos);
       }
       bw += __popc(mw);
       bc += __popc(mc);
@@ -530,18 +533,14 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
     float v[kElems];
     int pos0[4];
     load_chunk(rs, ch, n, v, pos0);
-    const bool full = (ch + 1) * kSelChunk <= n;
-    uint32_t hit = 0, win = 0;
-    if (full && no_winners) {
+    uint32_t miss = 0u;                              // bit 15 - e: score e is below the bracket
 #pragma unroll
-      for (int e = 0; e < kElems; ++e) hit |= (v[e] >= lo_f ? 1u : 0u) << e;
-    } else {
+    for (int e = 0; e < kElems; ++e) miss = __funnelshift_l(__float_as_uint(v[e] - lo_s), miss, 1);
+    uint32_t hit = ~miss & 0xffffu;
+    if ((ch + 1) * kSelChunk > n) {                  // positions past the row's end
 #pragma unroll
-      for (int e = 0; e < kElems; ++e) {
-        const bool valid = full || pos0[e >> 2] + (e & 3) < n;
-        hit |= (valid && v[e] >= lo_f ? 1u : 0u) << e;
-        win |= (valid && v[e] > hi_f ? 1u : 0u) << e;
-      }
+      for (int j = 0; j < 4; ++j)
+        hit &= ~((0xfu >> min(4, max(0, n - pos0[j]))) << (12 - 4 * j));
     }
     // exclusive scan of the per-lane hit counts over the warp
     const int mine = __popc(hit);
@@ -557,10 +556,9 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
     int slot = buf_n + inc - mine;
     const int pos_base = ch * kSelChunk + tid * 4;   // position of element e: + (e>>2)*2048 + (e&3)
     while (hit) {
-      const int e = __ffs(hit) - 1;
-      hit &= hit - 1;
-      my_hits[slot++] = (uint32_t)(pos_base + (e >> 2) * (kSelThreads * 4) + (e & 3)) |
-                        (((win >> e) & 1u) << 31);
+      const int e = __clz(hit) - 16;
+      hit ^= 0x8000u >> e;
+      my_hits[slot++] = (uint32_t)(pos_base + (e >> 2) * (kSelThreads * 4) + (e & 3));
     }
     __syncwarp();
     buf_n += total;
