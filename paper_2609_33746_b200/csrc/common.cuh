@@ -234,6 +234,18 @@ __device__ __forceinline__ bool cta_arrived_last(uint32_t* counter, uint32_t n_a
   return *s_flag != 0;
 }
 
+// Eight consecutive 16-bit elements; one 16-byte load where the address allows it (a query tensor may
+// start at any element).
+template <typename T> __device__ __forceinline__ uint4 load_eight(const T* p) {
+  static_assert(sizeof(T) == 2, "16-bit elements");
+  if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) return __ldg(reinterpret_cast<const uint4*>(p));
+  const unsigned short* h = reinterpret_cast<const unsigned short*>(p);
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w[i] = (uint32_t)__ldg(h + 2 * i) | ((uint32_t)__ldg(h + 2 * i + 1) << 16);
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));

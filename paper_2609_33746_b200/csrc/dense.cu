@@ -114,7 +114,7 @@ dense_decode_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc,
 #pragma unroll
   for (int g = 0; g < GH; ++g) {
     uint4 w = make_uint4(0u, 0u, 0u, 0u);
-    if (g < n_heads) w = __ldg(reinterpret_cast<const uint4*>(q + (size_t)(row0 + g) * kHeadDim) + l16);
+    if (g < n_heads) w = load_eight(q + (size_t)(row0 + g) * kHeadDim + 8 * l16);
     unpack2<T>(w, q2[g]);
     const unsigned long long sc = dup2(pl.sm_scale * kLog2e);
 #pragma unroll
