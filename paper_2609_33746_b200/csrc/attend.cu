@@ -544,6 +544,9 @@ cudaError_t launch_attend(const Plan& pl_in, const WsLayout& L, char* ws, const 
   float* split_part = reinterpret_cast<float*>(ws + L.split_part);
   uint32_t* tickets = reinterpret_cast<uint32_t*>(ws + L.attend_tickets);
   if (attend_parts(pl) > kMaxParts) return cudaErrorInvalidValue;
+  set_carveout<bg_prep_kernel>(kStreamCarveout);
+  set_carveout<attend_kernel<__half, 4>>(kStreamCarveout);
+  set_carveout<attend_kernel<__nv_bfloat16, 4>>(kStreamCarveout);
   cudaError_t e = cudaSuccess;
   if (!pl.bg_in_select)
     e = launch_pdl(bg_prep_kernel, dim3(pl.bg_ctas, pl.rows), dim3(kBgThreads), 0, st, pl,

@@ -7,6 +7,8 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "pqhsa.h"
 
 namespace pqhsa {
@@ -255,6 +257,24 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// Share of the SM's on-chip memory a kernel asks for as shared memory, in percent; set once per kernel
+// and device (it only steers the split, so a lost setting costs time and nothing else).  Kernels whose
+// launches overlap (programmatic dependent launch) should agree on the split: changing it drains the
+// SM.  And the L1 half has to hold the lines in flight: with 128 KB of gathers per SM a small L1
+// throttles the loads.  30 % (64 KB shared, the rest L1) for the table build, the top-k's sample, the
+// background preparation and the attention, against the driver's choice per kernel, as the decode
+// call: 128K x 8 313 -> 304 us, 512K 191 -> 181, 4-bit 128K x 8 194 -> 189; at 0 or 100 % any one
+// of them costs 5 to 25 %.
+constexpr int kStreamCarveout = 30;
+template <auto kKernel> void set_carveout(int percent) {
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+  if (done.load(std::memory_order_relaxed) >> dev & 1u) return;
+  if (cudaFuncSetAttribute(kKernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent) == cudaSuccess)
+    done.fetch_or(uint64_t(1) << dev, std::memory_order_relaxed);
 }
 
 // Launch with programmatic stream serialization allowed (see pdl_wait above).

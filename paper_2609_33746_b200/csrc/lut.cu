@@ -207,10 +207,10 @@ static cudaError_t launch_lut_t(const Plan& pl, const T* q, const pqhsa_index& i
   if (chunks < 4) chunks = 4;
   dim3 grid(chunks, pl.Hkv, pl.B);
   switch (pl.dsub) {
-    case 2: return launch_pdl(build_lut_kernel<T, 2>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
-    case 4: return launch_pdl(build_lut_kernel<T, 4>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
-    case 8: return launch_pdl(build_lut_kernel<T, 8>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
-    case 16: return launch_pdl(build_lut_kernel<T, 16>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
+    case 2: set_carveout<build_lut_kernel<T, 2>>(kStreamCarveout); return launch_pdl(build_lut_kernel<T, 2>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
+    case 4: set_carveout<build_lut_kernel<T, 4>>(kStreamCarveout); return launch_pdl(build_lut_kernel<T, 4>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
+    case 8: set_carveout<build_lut_kernel<T, 8>>(kStreamCarveout); return launch_pdl(build_lut_kernel<T, 8>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
+    case 16: set_carveout<build_lut_kernel<T, 16>>(kStreamCarveout); return launch_pdl(build_lut_kernel<T, 16>, grid, dim3(kLutThreads), 0, st, pl, q, ix.centroids, ix.codebooks, lut, coarse, zp, zn);
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

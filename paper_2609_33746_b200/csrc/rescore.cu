@@ -275,6 +275,7 @@ cudaError_t launch_rescore(const Plan& pl, const WsLayout& L, char* ws, const pq
   (void)sel_count;
   Plan plan = pl;
   plan.norm_seg = reinterpret_cast<float*>(ws + L.norm_seg);
+  set_carveout<rescore_kernel>(kStreamCarveout);
   return launch_pdl(rescore_kernel, dim3(pl.rows), dim3(kRsThreads), 0, st, plan, lut, coarse,
                     ix.codes, ix.list_ids, ix.key_norms, scores, seq_lens,
                     reinterpret_cast<const uint32_t*>(ws + L.counters),

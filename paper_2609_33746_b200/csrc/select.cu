@@ -704,6 +704,7 @@ cudaError_t launch_select(const Plan& pl, const WsLayout& L, char* ws, const flo
   int* status = reinterpret_cast<int*>(ws + L.status);
   if (pl.sel_cluster > 0)
     return launch_select_cluster(pl, scores, seq_lens, sel_idx, sel_count, kth, status, st);
+  set_carveout<sel_sample_kernel>(kStreamCarveout);
   cudaError_t e = launch_pdl(sel_sample_kernel, dim3(pl.rows), dim3(kSelThreads), 0, st, pl, scores,
                              seq_lens, rowstate, sel_count, kth);
   if (e != cudaSuccess) return e;
