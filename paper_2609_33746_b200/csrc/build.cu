@@ -86,27 +86,54 @@ __global__ void build_seed_kernel(Plan pl, const float* __restrict__ U,
   *reinterpret_cast<float4*>(dst + (unit * n_rows + j) * kD + 4 * lane) = v;
 }
 
-// ---- centroids as tensor-core tiles: 64 rows in the layout of the coarse search, the factor -2 and
+// ---- centroids as tensor-core tiles: 128 rows in the layout of the coarse search, the factor -2 and
 // |c|^2 included; rows past n_list are farther than any centroid
-constexpr int kAsgTok = 256, kAsgCen = 64, kAsgThreads = 288;
-constexpr int kCenTileBytes = kCoarseChunks * kAsgCen * 16;       // 34816
-constexpr int kTokTileBytes = kCoarseChunks * 128 * 16;           // 69632
-constexpr float kNearTie = 4e-6f * kTcScale * kTcScale;          // 4e-6 of a squared distance
-constexpr int kAsgSmemBytes = 2 * kTokTileBytes + 2 * kCenTileBytes;
+constexpr int kAsgTok = 256, kAsgCen = 128, kAsgThreads = 320;
+constexpr int kCenTileBytes = kCoarseChunks * kAsgCen * 16;       // 69632
+constexpr int kTokTileBytes = kCoarseChunks * 128 * 16;
+constexpr int kAsgSmemBytes = 2 * kTokTileBytes + kCenTileBytes;
+// A centroid tile arrives in pieces of 4 chunks (8 KB), in the order in which the MMAs want them: the lo
+// half (pieces 0-3), the hi half (4-7), the |c|^2 chunks (8).
+constexpr int kAsgPieces = 9;
+__device__ __forceinline__ constexpr uint32_t piece_chunk(int p) { return p < 4 ? 16 + 4 * p : p < 8 ? 4 * (p - 4) : 32; }
 
 // 8 rows of 128 fp32 into a tile: lane l holds row l & 7 and the chunks (l >> 3) + 4 i, so that loads
-// take whole 128-byte lines and stores have no conflicts.  Returns |row|^2 (all lanes of the row).
-__device__ __forceinline__ float split_rows(const float* __restrict__ src, bool real, float scale,
-                                            unsigned char* dst, int rows, int r, int lane) {
+// take whole 128-byte lines and stores have no conflicts.  split_rows returns |row|^2 (all lanes of the
+// row).
+// a whole 32-byte sector in one instruction (two 16-byte loads fetch it twice)
+__device__ __forceinline__ void load_sector(const float* p, float (&v)[8]) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "l"(p) : "memory");
+}
+struct RowPart {
+  float v[4][8];
+};
+// (kSectors: rows on 32-byte boundaries, the workspace's; the caller's centroids are on 16)
+template <bool kSectors>
+__device__ __forceinline__ RowPart load_rows(const float* __restrict__ src, bool real, int lane) {
+  RowPart p;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float* at = src + 8 * ((lane >> 3) + 4 * i);
+    if (real && kSectors) {
+      load_sector(at, p.v[i]);
+    } else if (real) {
+      *reinterpret_cast<float4*>(p.v[i]) = __ldcg(reinterpret_cast<const float4*>(at));
+      *reinterpret_cast<float4*>(p.v[i] + 4) = __ldcg(reinterpret_cast<const float4*>(at) + 1);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) p.v[i][t] = 0.f;
+    }
+  }
+  return p;
+}
+__device__ __forceinline__ float split_rows(const RowPart& p, float scale, unsigned char* dst, int rows, int r, int lane) {
   const int c0 = lane >> 3;
   float n2 = 0.f;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (real) {
-      *reinterpret_cast<float4*>(v) = __ldcg(reinterpret_cast<const float4*>(src) + 2 * (c0 + 4 * i));
-      *reinterpret_cast<float4*>(v + 4) = __ldcg(reinterpret_cast<const float4*>(src) + 2 * (c0 + 4 * i) + 1);
-    }
+    const float (&v)[8] = p.v[i];
     uint4 hi, lo;
     split_chunk(v, scale, hi, lo);
 #pragma unroll
@@ -119,54 +146,83 @@ __device__ __forceinline__ float split_rows(const float* __restrict__ src, bool 
   return n2;
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(4 * kAsgCen)
 build_split_kernel(Plan pl, const float* __restrict__ centroids, unsigned char* __restrict__ images) {
   const size_t unit = blockIdx.y;
   const int lane = threadIdx.x & 31, r = (threadIdx.x >> 5) * 8 + (lane & 7);
   const int j = blockIdx.x * kAsgCen + r;
   unsigned char* dst = images + (unit * gridDim.x + blockIdx.x) * (size_t)kCenTileBytes;
   const bool real = j < pl.n_list;
-  const float n2 = split_rows(centroids + (unit * pl.n_list + (real ? j : 0)) * kD, real, -2.f * kTcScale, dst,
-                              kAsgCen, r, lane);
+  const float n2 = split_rows(load_rows<false>(centroids + (unit * pl.n_list + (real ? j : 0)) * kD, real, lane),
+                              -2.f * kTcScale, dst, kAsgCen, r, lane);
   if (lane < 8) *reinterpret_cast<uint4*>(dst + (32 * kAsgCen + r) * 16) = coarse_ext_centre(n2, real);
   else if (lane < 16) *reinterpret_cast<uint4*>(dst + (33 * kAsgCen + r) * 16) = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// ---- nearest centroid.  CTA: 256 tokens of one unit as two 128-row tiles that stay in shared
-// memory, while the centroid tiles (64 rows, 34 KB, already in the tensor core's layout) stream
-// through two stages by bulk copies: 256 tokens per stage keep the L2 reads at 15 bytes per clock
-// and SM.  Warp 8 copies and issues; warpgroup w reads the accumulators of token tile w (64 columns,
-// double buffered) and keeps the minimum.  What bounds it: the MMAs (25 K-steps per tile pair at 48
-// clocks: shared-memory operand reads), then the split of the token tile at the start.
+// ---- nearest centroid.  CTA: 256 tokens of one unit as two 128-row tiles that stay in shared memory;
+// one centroid tile is resident and is replaced piece by piece: a piece is refilled as soon as its last
+// MMA is done, two thirds of a tile's time before the next tile wants it, so that 128 centroids per MMA
+// (64 clocks; 64 of them would cost 48) need no second stage.  Warp 8 issues the MMAs, warp 9 the
+// copies; warpgroup w reads the accumulators of token tile w (128 columns, double buffered).
+// What bounds it: the MMAs.  With all SMs at work they run at 108 clocks, 1.36 of the 1.63 PFLOP/s that a
+// cuBLAS GEMM reaches (64 clocks with few SMs busy): 5.4 of the 6.2 thousand clocks per tile; behind them
+// the search for the two nearest (2.4 to 3.6 thousand, overlapped) and the token tile at the start (8.1
+// thousand, 1 CTA per SM: nothing overlaps it).  1 M tokens x 1024 lists: 1231 us with 64 centroids per
+// tile, two stages and an index beside every value, 1000 us so, 940 us with whole sectors loaded.
 __global__ void __launch_bounds__(kAsgThreads, 1)
 build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* __restrict__ images,
                     const float* __restrict__ centroids, const int32_t* __restrict__ seq_lens,
                     uint16_t* __restrict__ list_ids, float* __restrict__ dmin, float* __restrict__ key_norms) {
   extern __shared__ __align__(128) unsigned char s_asg[];
   unsigned char* s_tok = s_asg;                             // two token tiles
-  unsigned char* s_cen = s_asg + 2 * kTokTileBytes;         // two centroid stages
+  unsigned char* s_cen = s_asg + 2 * kTokTileBytes;         // the centroid tile
   __shared__ float s_x2[kAsgTok];
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) uint64_t s_full[2], s_done[2], s_free[2];
+  __shared__ __align__(8) uint64_t s_full[kAsgPieces], s_used[kAsgPieces], s_done[2], s_free[2];
   const int kv = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = clamp_len(seq_lens[b], pl.N_max);
   const int t0 = blockIdx.x * kAsgTok;
-  if (t0 >= n) return;
   const size_t ukv = (size_t)b * pl.Hkv + kv;
+  // two rounds of rows in flight before anything is waited for (rows past the sequence are not used)
+  RowPart part[2];
+  auto row_of = [&](int q) { return q * 64 + warp * 8 + (lane & 7); };
+  auto load = [&](int q) {
+    const int r = row_of(q);
+    return load_rows<true>(U + (ukv * pl.N_max + t0 + r) * kD, t0 + r < pl.N_max, lane);
+  };
+  if (warp < 8) {
+    part[0] = load(0);
+    part[1] = load(1);
+  }
+  const int n = clamp_len(seq_lens[b], pl.N_max);
+  if (t0 >= n) return;
   const int n_tiles = (pl.n_list + kAsgCen - 1) / kAsgCen;
   const unsigned char* img = images + ukv * (size_t)n_tiles * kCenTileBytes;
-  if (warp == 8) tmem_alloc(&s_tmem, 256);
-  if (tid < 2) { mbar_init(&s_full[tid], 1); mbar_init(&s_done[tid], 1); mbar_init(&s_free[tid], 8); }
-  if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (warp == 8) tmem_alloc(&s_tmem, 512);
+  if (warp == 9) {
+    if (lane < kAsgPieces) { mbar_init(&s_full[lane], 1); mbar_init(&s_used[lane], 1); }
+    if (lane < 2) { mbar_init(&s_done[lane], 1); mbar_init(&s_free[lane], 8); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  auto copy = [&](int i, int p) {
+    const uint32_t bytes = (p < 8 ? 4u : 2u) * kAsgCen * 16u, at = piece_chunk(p) * kAsgCen * 16u;
+    mbar_expect_tx(&s_full[p], bytes);
+    bulk_g2s(s_cen + at, img + (size_t)i * kCenTileBytes + at, bytes, &s_full[p]);
+  };
+  if (warp == 9) {
+    __syncwarp();
+    if (lane == 0)
+      for (int p = 0; p < kAsgPieces; ++p) copy(0, p);
+  }
   // the token tiles
   if (warp < 8) {
-#pragma unroll 1
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int r = q * 64 + warp * 8 + (lane & 7);
-      const bool real = t0 + r < n;
+      const int r = row_of(q);
       unsigned char* dst = s_tok + (r >> 7) * kTokTileBytes;
-      const float x2 = split_rows(U + (ukv * pl.N_max + t0 + (real ? r : 0)) * kD, real, kTcScale, dst, 128, r & 127, lane);
+      if (t0 + r >= n) part[q & 1] = load_rows<true>(U, false, lane);         // zeros
+      const float x2 = split_rows(part[q & 1], kTcScale, dst, 128, r & 127, lane);
+      if (q < 2) part[q & 1] = load(q + 2);
       if (lane < 8) {
         s_x2[r] = x2;
         *reinterpret_cast<uint4*>(dst + (32 * 128 + (r & 127)) * 16) = coarse_ext_row();
@@ -181,70 +237,89 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   bool late = false;
-  if (warp == 8) {
+  if (warp == 9) {
     if (lane == 0) {
-      auto copy = [&](int i) {
-        mbar_expect_tx(&s_full[i & 1], kCenTileBytes);
-        bulk_g2s(s_cen + (i & 1) * kCenTileBytes, img + (size_t)i * kCenTileBytes, kCenTileBytes, &s_full[i & 1]);
-      };
-      copy(0);
-      if (n_tiles > 1) copy(1);
-      const uint32_t sa = smem_u32(s_tok);
-      for (int i = 0; i < n_tiles; ++i) {
-        const uint32_t st = i & 1, ph = (uint32_t)(i >> 1) & 1u;
-        late |= !tc_wait(&s_full[st], ph);
-        if (i >= 2) late |= !tc_wait(&s_free[st], ph ^ 1u);          // tile i - 2 has been read
-        tc_fence_after();
-        const uint32_t sb = smem_u32(s_cen + st * kCenTileBytes);
-        tc_coarse_tile<128, kAsgCen>(tmem + st * 128u, sa, sb);
-        tc_coarse_tile<128, kAsgCen>(tmem + st * 128u + 64u, sa + kTokTileBytes, sb);
-        tc_commit(&s_done[st]);
-        if (i >= 1 && i + 1 < n_tiles) {                             // the stage of tile i - 1 is free
-          late |= !tc_wait(&s_done[st ^ 1u], (uint32_t)((i - 1) >> 1) & 1u);
-          copy(i + 1);
+      for (int i = 1; i < n_tiles; ++i) {
+        for (int p = 0; p < kAsgPieces; ++p) {
+          late |= !tc_wait(&s_used[p], (uint32_t)(i - 1) & 1u);
+          copy(i, p);
         }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 8) {
+    if (lane == 0) {
+      const uint64_t a0 = tc_desc(smem_u32(s_tok), 128u * 16u), a1 = tc_desc(smem_u32(s_tok + kTokTileBytes), 128u * 16u);
+      const uint64_t bd = tc_desc(smem_u32(s_cen), kAsgCen * 16u);
+      for (int i = 0; i < n_tiles; ++i) {
+        const uint32_t st = i & 1, ph = st;
+        const uint32_t idesc = tc_idesc(pl.n_list - i * kAsgCen <= 64 ? 64u : 128u);
+        const uint32_t d0 = tmem + st * 256u, d1 = d0 + 128u;
+        if (i >= 2) late |= !tc_wait(&s_free[st], ((uint32_t)(i >> 1) & 1u) ^ 1u);   // tile i - 2 has been read
+        // one piece against 4 chunks of the token tiles (offsets in 16-byte units; all constants)
+        auto steps = [&](uint32_t a_chunk, uint32_t b_chunk, bool first) {
+#pragma unroll
+          for (uint32_t k = 0; k < 4; k += 2) {
+            tc_mma(d0, a0 + (a_chunk + k) * 128u, bd + (b_chunk + k) * kAsgCen, idesc, !first || k != 0);
+            tc_mma(d1, a1 + (a_chunk + k) * 128u, bd + (b_chunk + k) * kAsgCen, idesc, !first || k != 0);
+          }
+        };
+        // the cross terms first: they are 2^-11 of the rest, so that only nine accumulations round at
+        // full magnitude
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          late |= !tc_wait(&s_full[p], ph);
+          tc_fence_after();
+          steps(4 * p, piece_chunk(p), p == 0);
+          tc_commit(&s_used[p]);
+        }
+#pragma unroll
+        for (int p = 4; p < 8; ++p) {
+          late |= !tc_wait(&s_full[p], ph);
+          tc_fence_after();
+          steps(16 + 4 * (p - 4), piece_chunk(p), false);
+        }
+#pragma unroll
+        for (int p = 4; p < 8; ++p) {
+          steps(4 * (p - 4), piece_chunk(p), false);
+          tc_commit(&s_used[p]);
+        }
+        late |= !tc_wait(&s_full[8], ph);
+        tc_fence_after();
+        tc_mma(d0, a0 + 32u * 128u, bd + 32u * kAsgCen, idesc, true);
+        tc_mma(d1, a1 + 32u * 128u, bd + 32u * kAsgCen, idesc, true);
+        tc_commit(&s_used[8]);
+        tc_commit(&s_done[st]);
       }
     }
     __syncwarp();
   } else {
     const int wg = warp >> 2;
     const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
-    float best = CUDART_INF_F, second = CUDART_INF_F;
-    int near = 0, next = 0;                                 // nearest and second nearest so far
+    Nearest2 nn;
+    nn.clear();
     for (int i = 0; i < n_tiles; ++i) {
       const uint32_t st = i & 1;
       late |= !tc_wait(&s_done[st], (uint32_t)(i >> 1) & 1u);
       tc_fence_after();
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      const int n_cols = min(pl.n_list - i * kAsgCen, kAsgCen);
+#pragma unroll 1
+      for (int c = 0; c < n_cols; c += 32) {
         float acc[32];
-        tmem_ld32(tmem + st * 128u + wg * 64u + h * 32u + lanes, acc);
-        if (h == 1) {
-          tc_fence_before();
-          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&s_free[st])) : "memory");
-        }
-        // the minimum of the 32 first (three inputs per instruction); one by one only where it could
-        // become the nearest or a near-tie of it
-        const float m = min32(acc);
-        if (m < best + kNearTie) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {                             // ascending: the first minimum stays
-            const int cj = i * kAsgCen + h * 32 + j;
-            const bool first = acc[j] < best;
-            const float other = fmaxf(acc[j], best);
-            if (other < second) next = first ? near : cj;
-            second = fminf(second, other);
-            if (first) near = cj;
-            best = fminf(best, acc[j]);
-          }
-        }
+        tmem_ld32(tmem + st * 256u + wg * 128u + c + lanes, acc);
+        nn.take(acc, i * (kAsgCen / 32) + (c >> 5));
       }
+      tc_fence_before();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&s_free[st])) : "memory");
+      __syncwarp();
     }
+    int near = nn.near();
+    const int next = nn.next();
     const int r = wg * 128 + (warp & 3) * 32 + lane;
     if (t0 + r < n) {
       const size_t at = ukv * pl.N_max + t0 + r;
-      float d = s_x2[r] + best * kTcUnscale;
-      if (second < best + kNearTie && max(near, next) < pl.n_list) {
+      float d = s_x2[r] + nn.low * kTcUnscale;
+      if (nn.tie() && max(near, next) < pl.n_list) {
         // the two are within the rounding of either arithmetic: decided in plain fp32, every sum one
         // chain over the dims (a few tokens in a thousand)
         const float4* u = reinterpret_cast<const float4*>(U + at * kD);
@@ -271,7 +346,7 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) { tc_fence_after(); tmem_free(tmem, 256); }
+  if (warp == 8) { tc_fence_after(); tmem_free(tmem, 512); }
 }
 
 // ---- tokens grouped by list.  hist: members per list; offsets: exclusive prefix (and a running
@@ -863,7 +938,7 @@ cudaError_t run_build(const Plan& pl, const pqhsa_paged_kv& kv, const int32_t* s
   const dim3 run_grid((pl.N_max + kRun * (kPrepThreads / 32) - 1) / (kRun * (kPrepThreads / 32)), pl.Hkv, pl.B);
   const size_t list_smem = (size_t)pl.n_list * 4;
   auto assign = [&]() {
-    build_split_kernel<<<split_grid, 256, 0, st>>>(pl, ix.centroids, images);
+    build_split_kernel<<<split_grid, 4 * kAsgCen, 0, st>>>(pl, ix.centroids, images);
     build_assign_kernel<<<asg_grid, kAsgThreads, kAsgSmemBytes, st>>>(pl, U, images, ix.centroids, seq_lens, ix.list_ids, dmin, ix.key_norms);
   };
   for (int it = 0; it < coarse_iters; ++it) {

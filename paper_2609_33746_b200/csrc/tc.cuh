@@ -214,6 +214,60 @@ __device__ __forceinline__ float min32(const float (&v)[32]) {
   const float a = min3(m[0], m[1], m[2]), b = min3(m[3], m[4], m[5]), c = min3(m[6], m[7], m[8]);
   return min3(min3(a, b, c), m[9], m[10]);
 }
+
+// The two nearest centroids of a token, 32 accumulators at a time.  Their column's low 5 bits travel in
+// the mantissa, so that a column costs 4 instructions (an index carried beside each value: 7 to 8), and
+// only where the 32 hold something near enough to matter.  Two that are nearer than kNearTie to each
+// other are a tie of the split arithmetic (4e-6 of a squared distance; 2^-19 for the 5 bits): the
+// caller decides it in fp32, so that the lists do not depend on how the search was split.
+constexpr uint32_t kColBits = 31u;
+constexpr float kNearTie = 6e-6f * kTcScale * kTcScale;
+struct Nearest2 {
+  float low, best, second;                               // exact minimum; with column bits
+  int best_at, second_at;                                // which 32 columns
+  __device__ __forceinline__ void clear() {
+    low = best = second = CUDART_INF_F;
+    best_at = second_at = 0;
+  }
+  // (column bits: the value's own, or infinity's zeros)
+  static __device__ __forceinline__ int column(float v, int at) { return at * 32 + (int)(__float_as_uint(v) & kColBits); }
+  __device__ __forceinline__ int near() const { return column(best, best_at); }
+  __device__ __forceinline__ int next() const { return column(second, second_at); }
+  __device__ __forceinline__ bool tie() const { return second < best + kNearTie; }
+  // b <= s: the two nearest of another set
+  __device__ __forceinline__ void merge(float b, int b_at, float s, int s_at) {
+    const bool first = b < best;
+    const float other = fmaxf(best, b);
+    const int other_at = first ? best_at : b_at;
+    if (other < second) { second = other; second_at = other_at; }
+    if (s < second) { second = s; second_at = s_at; }
+    if (first) { best = b; best_at = b_at; }
+  }
+  __device__ __forceinline__ void take(const float (&acc)[32], int at) {
+    const float m = min32(acc);
+    if (m < low + kNearTie) {
+      low = fminf(low, m);
+      float b2[16], s2[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float x = __uint_as_float((__float_as_uint(acc[2 * j]) & ~kColBits) | (2 * j));
+        const float y = __uint_as_float((__float_as_uint(acc[2 * j + 1]) & ~kColBits) | (2 * j + 1));
+        b2[j] = fminf(x, y);
+        s2[j] = fmaxf(x, y);
+      }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+          s2[j] = min3(s2[j], s2[j + o], fmaxf(b2[j], b2[j + o]));
+          b2[j] = fminf(b2[j], b2[j + o]);
+        }
+      }
+      merge(b2[0], at, s2[0], at);
+    }
+  }
+};
+
 template <int N> __device__ __forceinline__ void group_minima(const float (&v)[N], int grp0, float& best, int& grp) {
 #pragma unroll
   for (int g = 0; g < N / 8; ++g) {

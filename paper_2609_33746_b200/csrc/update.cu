@@ -11,8 +11,10 @@
 //   index_refresh_means_kernel  groups the new tokens by list (first occurrence = leader), sums
 //       each group's value rows in token order and sets vbar_j = (n_j vbar_j + sum) / (n_j + new_j),
 //       n_j += new_j; a warp per leader.
-// What bounds the encoding: per CTA the centroids (512 KB at 1024 lists) pass through registers once
-// to be split, and the tensor core re-reads the token tile for every 32 centroids.
+// What bounds the encoding: latency.  Of 102 thousand clocks per CTA the rows' first loads take 11, the
+// centroids (512 KB at 1024 lists, through registers once to be split) 46, the codes 39: short steps
+// of store, MMA, wait and search per subspace.  8 requests x 8 KV heads x 128 new tokens: 778 us with
+// fp32 FMAs and a serial grouping of the means, 75 us so.
 #include "attn_common.cuh"
 #include "common.cuh"
 #include "tc.cuh"
@@ -62,8 +64,9 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
   extern __shared__ __align__(128) unsigned char s_dyn[];
   unsigned char* s_a = s_dyn;
   unsigned char* s_b = s_a + kUpdA;
-  __shared__ float s_best[kUpdGroups][kUpdTok];
-  __shared__ uint16_t s_near[kUpdGroups][kUpdTok];
+  __shared__ float s_best[2][kUpdGroups][kUpdTok];               // the groups' two nearest
+  __shared__ uint16_t s_at[2][kUpdGroups][kUpdTok];
+  __shared__ uint16_t s_near[2][kUpdTok];                        // the two that tie, or the nearest twice
   __shared__ __align__(16) uint8_t s_code[kUpdTok][64];
   __shared__ uint32_t s_tmem;
   __shared__ __align__(8) uint64_t s_bar[2 + kUpdGroups];        // centroid tiles, codeword tiles
@@ -176,8 +179,8 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
   };
   const uint32_t my_lanes = (uint32_t)(wq * 32) << 16;      // this warp's TMEM lanes
   const int n_tiles = (pl.n_list + kUpdCen - 1) / kUpdCen;
-  float best = CUDART_INF_F;
-  int near = 0;
+  Nearest2 nn;
+  nn.clear();
   bool late = false;
   for (int i = -1; i < n_tiles; ++i) {
     if (i + 1 < n_tiles) {
@@ -199,40 +202,57 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
     tc_fence_after();
     float acc[32];
     tmem_ld32(tmem + (i & 1) * kUpdCen + 32 * wg + my_lanes, acc);
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-      if (acc[j] < best) { best = acc[j]; near = i * kUpdCen + 32 * wg + j; }     // ascending: the first minimum stays
+    nn.take(acc, i * (kUpdCen / 32) + wg);
   }
-  s_best[wg][row] = best;
-  s_near[wg][row] = (uint16_t)min(near, pl.n_list - 1);
+  s_best[0][wg][row] = nn.best;
+  s_best[1][wg][row] = nn.second;
+  s_at[0][wg][row] = (uint16_t)nn.best_at;
+  s_at[1][wg][row] = (uint16_t)nn.second_at;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  {
-    // the groups' minima (equal distances: lower index)
-    float d = s_best[0][row];
-    int j = s_near[0][row];
-#pragma unroll
-    for (int g = 1; g < kUpdGroups; ++g) {
-      const float od = s_best[g][row];
-      const int oj = s_near[g][row];
-      if (od < d || (od == d && oj < j)) { d = od; j = oj; }
-    }
-    near = j;
-  }
-  __syncthreads();
   if (wg == 0) {
-    s_near[0][row] = (uint16_t)near;
-    if (ok(row)) list_ids[ukv * pl.N_max + p0 + row] = (uint16_t)near;
+#pragma unroll
+    for (int g = 1; g < kUpdGroups; ++g) nn.merge(s_best[0][g][row], s_at[0][g][row], s_best[1][g][row], s_at[1][g][row]);
+    const int near = nn.near(), next = nn.next();
+    s_near[0][row] = (uint16_t)min(near, pl.n_list - 1);
+    s_near[1][row] = (uint16_t)(nn.tie() && max(near, next) < pl.n_list ? next : min(near, pl.n_list - 1));
   }
   __syncthreads();
+  // ---- ties in fp32, every sum one chain over the dims (a few tokens in a thousand); a warp per token
+  int list[kPer];
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    const int t = r * kUpdWarps + warp;
+    list[r] = s_near[0][t];
+    const int alt = s_near[1][t];
+    if (alt != list[r]) {
+      const int lo = min(list[r], alt), hi = max(list[r], alt);
+      const float4* c0 = reinterpret_cast<const float4*>(cbase + (size_t)lo * kHeadDim);
+      const float4* c1 = reinterpret_cast<const float4*>(cbase + (size_t)hi * kHeadDim);
+      float x[4], a0 = 0.f, a1 = 0.f, n0 = 0.f, n1 = 0.f;
+      direction(r, x);
+#pragma unroll 4
+      for (int k = 0; k < kHeadDim / 4; ++k) {
+        const float4 y = __ldg(c0 + k), z = __ldg(c1 + k);
+        const float u0 = __shfl_sync(0xffffffffu, x[0], k), u1 = __shfl_sync(0xffffffffu, x[1], k);
+        const float u2 = __shfl_sync(0xffffffffu, x[2], k), u3 = __shfl_sync(0xffffffffu, x[3], k);
+        a0 = fmaf(u0, y.x, a0); a0 = fmaf(u1, y.y, a0); a0 = fmaf(u2, y.z, a0); a0 = fmaf(u3, y.w, a0);
+        n0 = fmaf(y.x, y.x, n0); n0 = fmaf(y.y, y.y, n0); n0 = fmaf(y.z, y.z, n0); n0 = fmaf(y.w, y.w, n0);
+        a1 = fmaf(u0, z.x, a1); a1 = fmaf(u1, z.y, a1); a1 = fmaf(u2, z.z, a1); a1 = fmaf(u3, z.w, a1);
+        n1 = fmaf(z.x, z.x, n1); n1 = fmaf(z.y, z.y, n1); n1 = fmaf(z.z, z.z, n1); n1 = fmaf(z.w, z.w, n1);
+      }
+      list[r] = fmaf(-2.f, a1, n1) < fmaf(-2.f, a0, n0) ? hi : lo;
+    }
+    if (lane == 0 && ok(t)) list_ids[ukv * pl.N_max + p0 + t] = (uint16_t)list[r];
+  }
   // ---- residuals
   float* s_u = reinterpret_cast<float*>(s_dyn);
   {
     float4 c[kPer];
 #pragma unroll
     for (int r = 0; r < kPer; ++r)
-      c[r] = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)s_near[0][r * kUpdWarps + warp] * kHeadDim) + lane);
+      c[r] = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)list[r] * kHeadDim) + lane);
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
       float x[4];
