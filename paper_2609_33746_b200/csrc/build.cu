@@ -623,29 +623,46 @@ __global__ void build_pq_seed_kernel(Plan pl, const float* __restrict__ E, const
 // codewords that holds the minimum, the codeword is decided in fp32 among those 8 (distance =
 // (|e|^2 - 2 e.p) + |p|^2, lower index on ties).  Training accumulates the codewords' sums in 64-bit
 // fixed point: two 32-bit shared-memory limbs of 21 bits and the rest (native integer atomics),
-// folded into 64 bits every kFold tokens, before a limb could overflow.
-template <int DSUB> struct PqPlan {
-  static constexpr int kMg8 = 16 / DSUB;                     // subspaces per CTA, 8-bit codes
-  static constexpr int kMg = kMg8 < 2 ? 2 : kMg8;            // (4-bit codes: whole bytes)
+// folded into 64 bits every kFoldSteps steps, before a limb could overflow.
+// What bounds it: the integer pipe (minima, comparisons, selects: 69 % of its cycles at 340 of 550
+// instructions per token and subspace) and, with one warp of each group per scheduler, the 650 clocks
+// from an MMA's issue to its mbarrier.  1 M tokens x 32 subspaces x 256 codewords: 1190 us a training
+// pass and 1050 us for the codes with run-time sizes, the codewords decided before the next MMA and codes
+// stored byte by byte; 1036 and 913 us so.  MMAs of 64 codewords into two accumulators: 1505 and 1395.
+template <int DSUB, int NC> struct PqPlan {
   using Tile = PqTile<DSUB>;
-  static int mg(int n_code) { return n_code == 16 ? kMg : kMg8; }
-  static size_t words(int n_code) { return (size_t)mg(n_code) * n_code; }
-  static size_t smem(int n_code, bool train) {
-    return words(n_code) * (Tile::kChunks * 16 + DSUB * 4 + 4) + 4 * Tile::kChunks * 2048 +
-           (train ? words(n_code) * ((2 * DSUB + 1) * 4 + DSUB * 8) : 0);
+  static constexpr int kMg8 = 16 / DSUB;                     // subspaces per CTA, 8-bit codes
+  static constexpr int kMg = NC == 16 && kMg8 < 2 ? 2 : kMg8;   // (4-bit codes: whole bytes)
+  static constexpr int kWords = kMg * NC;
+  static constexpr int kBits = NC == 16 ? 4 : 8, kBytes = kMg * kBits / 8;      // codes of one token
+  static constexpr size_t smem(bool train) {
+    return (size_t)kWords * (Tile::kChunks * 16 + DSUB * 4) + 4 * Tile::kChunks * 2048 +
+           (train ? (size_t)kWords * ((2 * DSUB + 1) * 4 + DSUB * 8) : 0);
   }
 };
 constexpr int kPqThreads = 512, kPqStep = 512;               // tokens per CTA and step
 constexpr int kFoldSteps = 3;                                // 1536 tokens: 2^21 * 1536 < 2^32, 2^20 * 1536 < 2^31
 constexpr int kLimbBits = 21;
+constexpr int kPqCols = 128;                                 // codewords per MMA step
+// x * kFixDir to the nearest integer as hi * 2^21 + lo, |lo| <= 2^20, for |x| < 8: rounded by the adder
+// (1.5 * 2^23 in, its bits out), the conversion instruction being an eighth as fast
+__device__ __forceinline__ void limbs(float x, int& hi, int& lo) {
+  constexpr float kMagic = 12582912.f;
+  const float y = x * (kFixDir / (float)(1 << kLimbBits)), h = y + kMagic;
+  const float l = fmaf(y - (h - kMagic), (float)(1 << kLimbBits), kMagic);
+  hi = __float_as_int(h) - __float_as_int(kMagic);
+  lo = __float_as_int(l) - __float_as_int(kMagic);
+}
 
-template <int DSUB, bool kTrain>
+template <int DSUB, int NC, bool kTrain>
 __global__ void __launch_bounds__(kPqThreads, 1)
 build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __restrict__ codebooks,
-                       const int32_t* __restrict__ seq_lens, int mg, int range, long long* __restrict__ pq_sums,
+                       const int32_t* __restrict__ seq_lens, int range, long long* __restrict__ pq_sums,
                        int32_t* __restrict__ pq_counts, uint8_t* __restrict__ codes_out,
                        float* __restrict__ key_norms) {
   using Tile = PqTile<DSUB>;
+  using P = PqPlan<DSUB, NC>;
+  constexpr int mg = P::kMg, nc = NC, words = P::kWords;
   extern __shared__ __align__(128) unsigned char s_pq[];
   __shared__ uint32_t s_tmem;
   __shared__ __align__(8) uint64_t s_bar[4];
@@ -656,15 +673,13 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
   const int begin = blockIdx.x * range, end = min(n, begin + range);
   if (begin >= end) return;
   const size_t ukv = (size_t)b * pl.Hkv + kv;
-  const int m0 = blockIdx.z * mg, nc = pl.n_code;
-  const int words = mg * nc;
-  // shared memory: codeword tiles, token tiles, fp32 codewords and |p|^2, then the training sums
+  const int m0 = blockIdx.z * mg;
+  // shared memory: codeword tiles, token tiles, fp32 codewords, then the training sums
   unsigned char* s_b = s_pq;                                            // [mg][chunks][nc] x 16 bytes
   unsigned char* s_a = s_b + (size_t)words * Tile::kChunks * 16;        // [4][chunks][128] x 16 bytes
   long long* s_sum = reinterpret_cast<long long*>(s_a + 4 * Tile::kChunks * 2048);   // [mg][DSUB][nc] (training)
   float* s_word = reinterpret_cast<float*>(s_sum + (kTrain ? (size_t)words * DSUB : 0));   // [mg][nc][DSUB]
-  float* s_p2 = s_word + (size_t)words * DSUB;                          // [mg][nc]
-  uint32_t* s_limb = reinterpret_cast<uint32_t*>(s_p2 + words);         // [mg][2 DSUB + 1][nc]
+  uint32_t* s_limb = reinterpret_cast<uint32_t*>(s_word + (size_t)words * DSUB);   // [mg][2 DSUB + 1][nc]
   auto load_sub = [](const float* src, float (&x)[DSUB]) {
     if constexpr (DSUB == 2) {
       *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(src);
@@ -679,7 +694,7 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
   if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   const float* cb = codebooks + (ukv * pl.M + m0) * (size_t)nc * DSUB;
   for (int w = tid; w < words; w += kPqThreads) {
-    float p[DSUB], p2 = 0.f;
+    float p[DSUB];
     load_sub(cb + (size_t)w * DSUB, p);
     uint4 ch[Tile::kChunks];
     Tile::code_row(p, ch);
@@ -688,8 +703,7 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
     for (int i = 0; i < Tile::kChunks; ++i)
       *reinterpret_cast<uint4*>(s_b + (size_t)((mm * Tile::kChunks + i) * nc + z) * 16) = ch[i];
 #pragma unroll
-    for (int t = 0; t < DSUB; ++t) { s_word[(size_t)w * DSUB + t] = p[t]; p2 = fmaf(p[t], p[t], p2); }
-    s_p2[w] = p2;
+    for (int t = 0; t < DSUB; ++t) s_word[(size_t)w * DSUB + t] = p[t];
     if constexpr (kTrain) {
 #pragma unroll
       for (int t = 0; t < DSUB; ++t) s_sum[(size_t)(mm * DSUB + t) * nc + z] = 0;
@@ -704,8 +718,7 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
   const uint32_t d_tmem = s_tmem + (uint32_t)wg * 128u;
   const uint32_t my_tmem = d_tmem + ((uint32_t)((warp & 3) * 32) << 16);
   unsigned char* pa = s_a + wg * (Tile::kChunks * 2048);
-  const uint32_t n_mma = (uint32_t)min(nc, 128);
-  uint32_t parity = 0u;
+  constexpr int kCols = nc < kPqCols ? nc : kPqCols, per = nc / kCols;   // MMA steps per subspace
   bool late = false;
   // the limbs into 64 bits (every thread its own entries); all threads call
   auto fold = [&]() {
@@ -715,98 +728,133 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
 #pragma unroll
       for (int t = 0; t < DSUB; ++t) {
         uint32_t* l = s_limb + (size_t)(mm * (2 * DSUB + 1) + 2 * t) * nc + z;
-        s_sum[(size_t)(mm * DSUB + t) * nc + z] += (long long)l[0] + ((long long)(int32_t)l[nc] << kLimbBits);
+        s_sum[(size_t)(mm * DSUB + t) * nc + z] += (long long)(int32_t)l[0] + ((long long)(int32_t)l[nc] << kLimbBits);
         l[0] = 0u;
         l[nc] = 0u;
       }
     }
     __syncthreads();
   };
+  // Items: (512 tokens, subspace), subspaces innermost.  The next MMA of a warpgroup is issued as soon as
+  // its accumulators have been read: the first of an item therefore before the last item's codewords are
+  // decided in fp32, which covers its latency (about 650 clocks from issue to the mbarrier).
+  auto put_row = [&](const float (&x)[DSUB]) {
+    uint4 ch[Tile::kChunks];
+    Tile::token_row(x, ch);
+#pragma unroll
+    for (int c = 0; c < Tile::kChunks; ++c) *reinterpret_cast<uint4*>(pa + (c * 128 + row) * 16) = ch[c];
+    tc_fence_smem();
+  };
+  // codewords c * kPqCols .. of subspace mm against the group's token tile
+  const uint64_t a_desc = tc_desc(smem_u32(pa), 128u * 16u), b_desc = tc_desc(smem_u32(s_b), (uint32_t)nc * 16u);
+  constexpr uint32_t idesc = tc_idesc((uint32_t)kCols);
+  auto issue = [&](int mm, int c) {
+    tc_fence_before();
+    group_sync(1 + wg);
+    if (row == 0) {
+      tc_fence_after();
+      const uint64_t bw = b_desc + (uint32_t)(mm * Tile::kChunks * nc + c * kCols);        // (16-byte units)
+#pragma unroll
+      for (int s = 0; s < Tile::kChunks; s += 2) tc_mma(d_tmem, a_desc + s * 128, bw + (uint32_t)(s * nc), idesc, s != 0);
+      tc_commit(&s_bar[wg]);
+    }
+    __syncwarp();
+  };
+  auto row_of = [&](int base) {
+    return E + (ukv * pl.N_max + min(base + wg * 128 + row, end - 1)) * (size_t)kD + m0 * DSUB;
+  };
+  constexpr uint32_t kRow = DSUB * 4;                       // bytes of a codeword
+  const uint32_t rot = (uint32_t)(lane & 7) * kRow;
+  float e[DSUB], e_nxt[DSUB];
+  const float* er = row_of(begin);
+  load_sub(er, e_nxt);
+  put_row(e_nxt);
+  issue(0, 0);
+  uint32_t parity = 0u;
   int steps = 0;
   for (int base = begin; base < end; base += kPqStep) {
+    const bool more = base + kPqStep < end;
+    const float* er_next = more ? row_of(base + kPqStep) : er;
     const int i = base + wg * 128 + row;
     const bool real = i < end;
-    const float* er = E + (ukv * pl.N_max + (real ? i : begin)) * (size_t)kD + m0 * DSUB;
-    float e[DSUB], e_nxt[DSUB];
-    load_sub(er, e_nxt);
-    uint32_t word = 0u;                                     // codes not yet written
+    unsigned long long code = 0ull;
+#pragma unroll 1
     for (int mm = 0; mm < mg; ++mm) {
 #pragma unroll
       for (int t = 0; t < DSUB; ++t) e[t] = e_nxt[t];
-      if (mm + 1 < mg) load_sub(er + (mm + 1) * DSUB, e_nxt);
-      uint4 ch[Tile::kChunks];
-      Tile::token_row(e, ch);
-#pragma unroll
-      for (int c = 0; c < Tile::kChunks; ++c) *reinterpret_cast<uint4*>(pa + (c * 128 + row) * 16) = ch[c];
+      const bool next = mm + 1 < mg || more;
+      load_sub(mm + 1 < mg ? er + (mm + 1) * DSUB : er_next, e_nxt);
       float bd = CUDART_INF_F;
       int grp = 0;
-      const uint32_t sb = smem_u32(s_b + (size_t)mm * Tile::kChunks * nc * 16);
-      for (int z0 = 0; z0 < nc; z0 += 128) {
-        tc_fence_smem();
-        tc_fence_before();
-        group_sync(1 + wg);
-        if (row == 0) {
-          tc_fence_after();
-          if (nc == 16) Tile::template mma<16>(d_tmem, smem_u32(pa), sb, n_mma);
-          else Tile::template mma<256>(d_tmem, smem_u32(pa), sb + z0 * 16, n_mma);
-          tc_commit(&s_bar[wg]);
-        }
-        __syncwarp();
+#pragma unroll
+      for (int c = 0; c < per; ++c) {
         late |= !tc_wait(&s_bar[wg], parity);
         parity ^= 1u;
         tc_fence_after();
-        if (nc == 16) {
+        if (c + 1 == per && next) put_row(e_nxt);           // (the item's last MMA is done)
+        if constexpr (nc == 16) {
           float acc[16];
           tmem_ld16(my_tmem, acc);
-          group_minima(acc, 0, bd, grp);
+          group_minima<true>(acc, 0, bd, grp);
         } else {
 #pragma unroll
-          for (int c = 0; c < 128; c += 32) {
+          for (int h = 0; h < kCols; h += 32) {
             float acc[32];
-            tmem_ld32(my_tmem + c, acc);
-            group_minima(acc, (z0 + c) / 8, bd, grp);
+            tmem_ld32(my_tmem + h, acc);
+            group_minima<true>(acc, (c * kCols + h) / 8, bd, grp);
           }
         }
+        if (c + 1 < per) issue(mm, c + 1);
+        else if (next) issue(mm + 1 < mg ? mm + 1 : 0, 0);
       }
-      // the winning group in fp32; the lanes start at different codewords, so that at 16 bytes a
-      // codeword the eight lanes of an access hit eight different bank groups
-      float en = 0.f;
+      // the winning group in fp32, lower index on ties; the lanes start at different codewords, so that
+      // at 16 bytes a codeword the eight lanes of an access hit eight different bank groups
+      float en = 0.f, dist[8];
 #pragma unroll
       for (int t = 0; t < DSUB; ++t) en = fmaf(e[t], e[t], en);
-      float dm = CUDART_INF_F;
-      int bz = 0;
+      const uint32_t at = (uint32_t)(8 * grp) * kRow + rot;
+      const unsigned char* s_sub = reinterpret_cast<const unsigned char*>(s_word) + (size_t)mm * nc * kRow;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const int z = 8 * grp + ((q + lane) & 7);
-        float w[DSUB], dot = 0.f;
-        load_sub(s_word + (size_t)(mm * nc + z) * DSUB, w);
+        float w[DSUB], dot = 0.f, p2 = 0.f;
+        load_sub(reinterpret_cast<const float*>(s_sub + (at ^ (q * kRow))), w);
 #pragma unroll
-        for (int t = 0; t < DSUB; ++t) dot = fmaf(e[t], w[t], dot);
-        const float dist = (en - 2.0f * dot) + s_p2[mm * nc + z];
-        if (dist < dm || (dist == dm && z < bz)) { dm = dist; bz = z; }
+        for (int t = 0; t < DSUB; ++t) { dot = fmaf(e[t], w[t], dot); p2 = fmaf(w[t], w[t], p2); }
+        dist[q] = (en - 2.0f * dot) + p2;
       }
+      const float dm = min3(min3(dist[0], dist[1], dist[2]), min3(dist[3], dist[4], dist[5]), fminf(dist[6], dist[7]));
+      uint32_t first = nc * kRow;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (dist[q] == dm) first = min(first, at ^ (q * kRow));
+      const uint32_t bz = first < nc * kRow ? first / kRow : 0u;         // (not a number: 0)
       if constexpr (kTrain) {
         if (real) {
-          uint32_t* l = s_limb + (size_t)(mm * (2 * DSUB + 1)) * nc + bz;
+          uint32_t* l = s_limb + mm * (2 * DSUB + 1) * nc + bz;
 #pragma unroll
           for (int t = 0; t < DSUB; ++t) {
-            const long long q = __float2ll_rn(e[t] * kFixDir);
-            atomicAdd(l + (2 * t) * nc, (uint32_t)q & ((1u << kLimbBits) - 1u));
-            atomicAdd(l + (2 * t + 1) * nc, (uint32_t)(q >> kLimbBits));
+            int hi, lo;
+            limbs(e[t], hi, lo);
+            atomicAdd(l + (2 * t) * nc, (uint32_t)lo);
+            atomicAdd(l + (2 * t + 1) * nc, (uint32_t)hi);
           }
           atomicAdd(l + 2 * DSUB * nc, 1u);
         }
-      } else if (real) {
-        uint8_t* dst = codes_out + (ukv * pl.N_max + i) * pl.code_bytes;
-        if (nc == 16) {
-          if (mm & 1) dst[(m0 + mm) >> 1] = (uint8_t)(word | ((uint32_t)bz << 4));
-          else word = (uint32_t)bz;
-        } else {
-          dst[m0 + mm] = (uint8_t)bz;
-        }
+      } else {
+        code |= (unsigned long long)bz << (mm * P::kBits);
+      }
+    }
+    if constexpr (!kTrain) {
+      if (real) {
+        uint8_t* dst = codes_out + (ukv * pl.N_max + i) * pl.code_bytes + m0 * P::kBits / 8;
+        if constexpr (P::kBytes == 8) *reinterpret_cast<unsigned long long*>(dst) = code;
+        else if constexpr (P::kBytes == 4) *reinterpret_cast<uint32_t*>(dst) = (uint32_t)code;
+        else if constexpr (P::kBytes == 2) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)code;
+        else *dst = (uint8_t)code;
       }
     }
     if (late && real) key_norms[ukv * pl.N_max + i] = CUDART_NAN_F;    // a bounded wait ran out
+    er = er_next;
     if constexpr (kTrain) {
       if (++steps == kFoldSteps) { fold(); steps = 0; }
     }
@@ -904,6 +952,43 @@ BuildWs build_layout(const Plan& pl) {
   return w;
 }
 
+#define PQHSA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
+
+// codebooks (pq_iters rounds of k-means from the seeded residuals U), then the codes
+template <int DSUB, int NC>
+cudaError_t pq_build(const Plan& pl, const float* U, const int32_t* seq_lens, const int32_t* seed_codes, int pq_iters,
+                     long long* pq_sums, int32_t* pq_counts, const pqhsa_index_out& ix, cudaStream_t st) {
+  using P = PqPlan<DSUB, NC>;
+  const int units = pl.B * pl.Hkv;
+  if (pl.M % P::kMg != 0) return cudaErrorInvalidValue;
+  // about three waves of CTAs, each over a range of tokens that is a multiple of a step; of the splits
+  // near that, the one whose last wave is fullest
+  const int columns = units * (pl.M / P::kMg), total_steps = (pl.N_max + kPqStep - 1) / kPqStep;
+  int steps = total_steps, best_cost = 0x7fffffff;
+  for (int s = total_steps; s >= 1; --s) {
+    const int ranges = (total_steps + s - 1) / s;
+    const long long ctas = (long long)ranges * columns;
+    if (ctas > 8LL * pl.num_sms && best_cost != 0x7fffffff) break;
+    const int waves = (int)((ctas + pl.num_sms - 1) / pl.num_sms), cost = waves * (s + 2);    // (+ 2: start and end of a CTA)
+    if (cost < best_cost) { best_cost = cost; steps = s; }
+  }
+  const dim3 grid((total_steps + steps - 1) / steps, units, pl.M / P::kMg);
+  cudaError_t e;
+  const int range = steps * kPqStep, smem_train = (int)P::smem(true), smem_code = (int)P::smem(false);
+  PQHSA_TRY(cudaFuncSetAttribute(build_pq_assign_kernel<DSUB, NC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_train));
+  PQHSA_TRY(cudaFuncSetAttribute(build_pq_assign_kernel<DSUB, NC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_code));
+  const size_t n_entries = (size_t)units * pl.M * NC;
+  build_pq_seed_kernel<DSUB><<<dim3(NC, units), kD, 0, st>>>(pl, U, seed_codes, ix.codebooks);
+  for (int it = 0; it < pq_iters; ++it) {
+    build_pq_assign_kernel<DSUB, NC, true><<<grid, kPqThreads, smem_train, st>>>(
+        pl, U, ix.codebooks, seq_lens, range, pq_sums, pq_counts, nullptr, ix.key_norms);
+    build_pq_update_kernel<<<(unsigned)((n_entries + 255) / 256), 256, 0, st>>>(n_entries, DSUB, pq_sums, pq_counts, ix.codebooks);
+  }
+  build_pq_assign_kernel<DSUB, NC, false><<<grid, kPqThreads, smem_code, st>>>(
+      pl, U, ix.codebooks, seq_lens, range, nullptr, nullptr, ix.codes, ix.key_norms);
+  return cudaSuccess;
+}
+
 template <typename T, int DSUB>
 cudaError_t run_build(const Plan& pl, const pqhsa_paged_kv& kv, const int32_t* seq_lens,
                       const int32_t* seed_lists, const int32_t* seed_codes, int coarse_iters,
@@ -921,7 +1006,6 @@ cudaError_t run_build(const Plan& pl, const pqhsa_paged_kv& kv, const int32_t* s
   const T* vc = static_cast<const T*>(kv.v_cache);
   const long long sp = kv.stride_page, stt = kv.stride_token, sh = kv.stride_head;
   cudaError_t e;
-#define PQHSA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
   PQHSA_TRY(cudaMemsetAsync(ws + w.sums, 0, w.total - w.sums, st));
   unsigned char* images = reinterpret_cast<unsigned char*>(ws + w.images);
   int32_t* order = reinterpret_cast<int32_t*>(ws + w.order);
@@ -953,33 +1037,9 @@ cudaError_t run_build(const Plan& pl, const pqhsa_paged_kv& kv, const int32_t* s
   }
   assign();
   build_residual_kernel<<<dim3(tok_ctas, pl.Hkv, pl.B), kPrepThreads, 0, st>>>(pl, U, ix.centroids, ix.list_ids, seq_lens);
-  // product quantisation: about three waves of CTAs, each over a range of tokens that is a multiple
-  // of a step; of the splits near that, the one whose last wave is fullest
-  const int mg = PqPlan<DSUB>::mg(pl.n_code);
-  if (pl.M % mg != 0) return cudaErrorInvalidValue;
-  const int columns = units * (pl.M / mg), total_steps = (pl.N_max + kPqStep - 1) / kPqStep;
-  int steps = total_steps, best_cost = 0x7fffffff;
-  for (int s = total_steps; s >= 1; --s) {
-    const int ranges = (total_steps + s - 1) / s;
-    const long long ctas = (long long)ranges * columns;
-    if (ctas > 8LL * pl.num_sms && best_cost != 0x7fffffff) break;
-    const int waves = (int)((ctas + pl.num_sms - 1) / pl.num_sms), cost = waves * (s + 2);    // (+ 2: start and end of a CTA)
-    if (cost < best_cost) { best_cost = cost; steps = s; }
-  }
-  const dim3 pq_grid((total_steps + steps - 1) / steps, units, pl.M / mg);
-  const int range = steps * kPqStep;
-  const int smem_train = (int)PqPlan<DSUB>::smem(pl.n_code, true), smem_code = (int)PqPlan<DSUB>::smem(pl.n_code, false);
-  PQHSA_TRY(cudaFuncSetAttribute(build_pq_assign_kernel<DSUB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_train));
-  PQHSA_TRY(cudaFuncSetAttribute(build_pq_assign_kernel<DSUB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_code));
-  const size_t n_entries = (size_t)units * pl.M * pl.n_code;
-  build_pq_seed_kernel<DSUB><<<dim3(pl.n_code, units), kD, 0, st>>>(pl, U, seed_codes, ix.codebooks);
-  for (int it = 0; it < pq_iters; ++it) {
-    build_pq_assign_kernel<DSUB, true><<<pq_grid, kPqThreads, smem_train, st>>>(
-        pl, U, ix.codebooks, seq_lens, mg, range, pq_sums, pq_counts, nullptr, ix.key_norms);
-    build_pq_update_kernel<<<(unsigned)((n_entries + 255) / 256), 256, 0, st>>>(n_entries, DSUB, pq_sums, pq_counts, ix.codebooks);
-  }
-  build_pq_assign_kernel<DSUB, false><<<pq_grid, kPqThreads, smem_code, st>>>(
-      pl, U, ix.codebooks, seq_lens, mg, range, nullptr, nullptr, ix.codes, ix.key_norms);
+  const cudaError_t e_pq = pl.n_code == 16 ? pq_build<DSUB, 16>(pl, U, seq_lens, seed_codes, pq_iters, pq_sums, pq_counts, ix, st)
+                                           : pq_build<DSUB, 256>(pl, U, seq_lens, seed_codes, pq_iters, pq_sums, pq_counts, ix, st);
+  if (e_pq != cudaSuccess) return e_pq;
   // list value means and member counts
   PQHSA_TRY(cudaMemsetAsync(counts, 0, (size_t)units * pl.n_list * 4, st));
   build_hist_kernel<true><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, counts);

@@ -205,7 +205,11 @@ template <int DSUB> struct PqTile {
 // Smallest of groups of 8 accumulators; `best` / `grp` keep the smallest group and the first one
 // that has it.  The codeword inside the group is found by the caller in fp32: two instructions less
 // per accumulator than carrying an index.
-__device__ __forceinline__ float min3(float a, float b, float c) { return fminf(fminf(a, b), c); }
+__device__ __forceinline__ float min3(float a, float b, float c) {      // one instruction
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
 __device__ __forceinline__ float min32(const float (&v)[32]) {
   float m[11];
 #pragma unroll
@@ -268,12 +272,27 @@ struct Nearest2 {
   }
 };
 
-template <int N> __device__ __forceinline__ void group_minima(const float (&v)[N], int grp0, float& best, int& grp) {
+// (kTree: merged pairwise, the shorter chain; one after the other, the fewer registers.  1 M tokens x 32
+// subspaces, encode: 961 us in a row, 916 as a tree; the update, with 128 registers full: 74.6 and 80.6.)
+template <bool kTree, int N>
+__device__ __forceinline__ void group_minima(const float (&v)[N], int grp0, float& best, int& grp) {
+  float m[N / 8];
+  int at[N / 8];
 #pragma unroll
   for (int g = 0; g < N / 8; ++g) {
     const float* w = v + 8 * g;
-    const float m = min3(min3(w[0], w[1], w[2]), min3(w[3], w[4], w[5]), fminf(w[6], w[7]));
-    if (m < best) { best = m; grp = grp0 + g; }
+    m[g] = min3(min3(w[0], w[1], w[2]), min3(w[3], w[4], w[5]), fminf(w[6], w[7]));
+    at[g] = grp0 + g;
+    if (!kTree && m[g] < best) { best = m[g]; grp = at[g]; }
+  }
+  if constexpr (kTree) {                                    // the lower group on ties
+#pragma unroll
+    for (int o = 1; o < N / 8; o *= 2) {
+#pragma unroll
+      for (int g = 0; g + o < N / 8; g += 2 * o)
+        if (m[g + o] < m[g]) { m[g] = m[g + o]; at[g] = at[g + o]; }
+    }
+    if (m[0] < best) { best = m[0]; grp = at[0]; }
   }
 }
 

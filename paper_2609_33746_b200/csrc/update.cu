@@ -324,13 +324,13 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
       if (pl.n_code == 16) {
         float acc[16];
         tmem_ld16(my_tmem, acc);
-        group_minima(acc, 0, bd, grp);
+        group_minima<false>(acc, 0, bd, grp);
       } else {
 #pragma unroll
         for (int c = 0; c < kUpdWords; c += 32) {
           float acc[32];
           tmem_ld32(my_tmem + c, acc);
-          group_minima(acc, (z0 + c) / 8, bd, grp);
+          group_minima<false>(acc, (z0 + c) / 8, bd, grp);
         }
       }
     }
