@@ -587,9 +587,17 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
       for (int w = 0; w < kSelThreads / 32; ++w) kstar = min(kstar, (uint32_t)s_scan[w]);
       __syncthreads();
     } else {
-      int src = kFromList;
-      uint32_t kmin = 0xffffffffu, kmax = 0u;                  // range of the finite staged keys
-      if (C <= kStashCap) {
+      // the first kStashCap candidates are staged; the rest, if any, is read from the list each time (a
+      // bracket 1 % of 512K scores wide holds about 5200: with all of them left to the radix select,
+      // whose passes reread the list, the finish took 17 us instead of 5)
+      uint32_t kmin = 0xffffffffu, kmax = 0u;                  // range of the finite keys
+      auto widen = [&](uint32_t key) {
+        if (fabsf(key_score(key)) < CUDART_INF_F) {
+          kmin = min(kmin, key);
+          kmax = max(kmax, key);
+        }
+      };
+      {
         constexpr int kPer = kStashCap / kSelThreads;          // 10: all loads issued together
         uint2 it[kPer];
 #pragma unroll
@@ -602,12 +610,10 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
           const int i = u * kSelThreads + tid;
           if (i < C) {
             s_stash[i] = it[u];
-            if (fabsf(key_score(it[u].x)) < CUDART_INF_F) {
-              kmin = min(kmin, it[u].x);
-              kmax = max(kmax, it[u].x);
-            }
+            widen(it[u].x);
           }
         }
+        for (int i = kStashCap + tid; i < C; i += kSelThreads) widen(__ldcg(rc + i).x);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
@@ -621,11 +627,12 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
           kmax = max(kmax, (uint32_t)s_scan[16 + w]);
         }
         __syncthreads();                                       // s_scan is reused below
-        src = kFromStash;
       }
+      const int src = C <= kStashCap ? kFromStash : kFromList;
+      auto item = [&](int i) { return i < kStashCap ? s_stash[i] : __ldcg(rc + i); };
       bool done = false;
-      if (src == kFromStash && kmax > kmin) {
-        // Fast finish.  ONE histogram of the staged candidates over 4096 equal buckets of the
+      if (kmax > kmin) {
+        // Fast finish.  ONE histogram of the candidates over 4096 equal buckets of the
         // range of their finite scores (candidates at -inf, the sink and window positions of a
         // row that was not bracketed from below, fall into the bottom bucket) finds the bucket of
         // the r-th largest; everything in a higher bucket is taken at once, and the few items of
@@ -636,7 +643,7 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
         for (int i = tid; i < kHistBins; i += kSelThreads) s_hist[i] = 0u;
         __syncthreads();
         for (int i = tid; i < C; i += kSelThreads)
-          atomicAdd(&s_hist[linear_bucket(key_score(s_stash[i].x), lo_h, scale)], 1u);
+          atomicAdd(&s_hist[linear_bucket(key_score(item(i).x), lo_h, scale)], 1u);
         __syncthreads();
         int d, above;
         find_digit(s_hist, kHistBins, r, s_scan, d, above);
@@ -650,7 +657,7 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
           for (int base = 0; base < C; base += kSelThreads) {
             const int i = base + tid;
             const bool v = i < C;
-            const uint2 it = v ? s_stash[i] : make_uint2(0u, 0u);
+            const uint2 it = v ? item(i) : make_uint2(0u, 0u);
             const int bk = v ? linear_bucket(key_score(it.x), lo_h, scale) : -1;
             const int p = warp_append(v && bk > d, &s_emit);
             if (p >= 0 && (uint32_t)W + p < (uint32_t)pl.k_max) out[W + p] = (int)it.y;
