@@ -473,8 +473,8 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
   const float* rs = scores + (size_t)row * pl.N_max;
   int32_t* out = sel_idx + (size_t)row * pl.k_max;
   uint2* rc = cand + (size_t)row * pl.cand_cap;          // (key, position) pairs
-  uint32_t* n_out = &counters[row * 4 + 2];
-  uint32_t* n_cand = &counters[row * 4 + 3];
+  // winners (low half) and candidates so far, moved by one atomic
+  unsigned long long* n_both = reinterpret_cast<unsigned long long*>(&counters[row * 4 + 2]);
 
   // Main pass.  Warps work independently: a lane marks which of its 16 scores reach the bracket and
   // the warp packs the positions of the hits into its shared-memory buffer.  The buffer is written
@@ -491,40 +491,45 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
   int buf_n = 0;                                    // warp-uniform
   auto flush = [&]() {
     if (buf_n == 0) return;
-    int nw = 0, nc = 0;
-    for (int i0 = 0; i0 < buf_n; i0 += 32) {
-      const bool v_ok = i0 + lane < buf_n;
-      // (from L2: this warp read it a moment ago.  NaN is neither)
-      const float sv = v_ok ? __ldcg(rs + my_hits[i0 + lane]) : CUDART_NAN_F;
-      nw += __popc(__ballot_sync(0xffffffffu, sv > hi_f));
-      nc += __popc(__ballot_sync(0xffffffffu, sv >= lo_f && sv <= hi_f));
-    }
-    uint32_t bw = 0, bc = 0;
-    if (lane == 0) {
-      if (nw) bw = atomicAdd(n_out, (uint32_t)nw);
-      if (nc) bc = atomicAdd(n_cand, (uint32_t)nc);
-    }
-    bw = __shfl_sync(0xffffffffu, bw, 0);
-    bc = __shfl_sync(0xffffffffu, bc, 0);
+    constexpr int kKeep = 4;                        // 128 hits at once: their scores are read together
     const unsigned lt = (1u << lane) - 1u;
-    for (int i0 = 0; i0 < buf_n; i0 += 32) {
-      const bool v_ok = i0 + lane < buf_n;
-      const uint32_t pos = v_ok ? my_hits[i0 + lane] : 0u;
-      const float sv = v_ok ? __ldcg(rs + pos) : CUDART_NAN_F;
-      const bool is_win = sv > hi_f, is_cnd = sv >= lo_f && sv <= hi_f;
-      const unsigned mw = __ballot_sync(0xffffffffu, is_win);
-      const unsigned mc = __ballot_sync(0xffffffffu, is_cnd);
-      if (is_win) {
-        const uint32_t p = bw + __popc(mw & lt);
-        if (p < (uint32_t)pl.k_max) out[p] = (int)pos;
+    for (int i0 = 0; i0 < buf_n; i0 += 32 * kKeep) {
+      float sv[kKeep];
+      uint32_t pos[kKeep];
+      int nw = 0, nc = 0;
+#pragma unroll
+      for (int u = 0; u < kKeep; ++u) {
+        const int i = i0 + 32 * u + lane;
+        pos[u] = i < buf_n ? my_hits[i] : 0u;
+        // (from L2: this warp read it a moment ago.  NaN is neither)
+        sv[u] = i < buf_n ? __ldcg(rs + pos[u]) : CUDART_NAN_F;
       }
-      if (is_cnd) {
-        // key and position together: the row's last CTA has no dependent gather to wait for
-        const uint32_t p = bc + __popc(mc & lt);
-        if (p < (uint32_t)pl.cand_cap) rc[p] = make_uint2(score_key(sv), pos);
+#pragma unroll
+      for (int u = 0; u < kKeep; ++u) {
+        nw += __popc(__ballot_sync(0xffffffffu, sv[u] > hi_f));
+        nc += __popc(__ballot_sync(0xffffffffu, sv[u] >= lo_f && sv[u] <= hi_f));
       }
-      bw += __popc(mw);
-      bc += __popc(mc);
+      unsigned long long at = 0ull;                 // winners and candidates before these
+      if (lane == 0) at = atomicAdd(n_both, ((unsigned long long)nc << 32) | (unsigned long long)nw);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      uint32_t bw = (uint32_t)at, bc = (uint32_t)(at >> 32);
+#pragma unroll
+      for (int u = 0; u < kKeep; ++u) {
+        const bool is_win = sv[u] > hi_f, is_cnd = sv[u] >= lo_f && sv[u] <= hi_f;
+        const unsigned mw = __ballot_sync(0xffffffffu, is_win);
+        const unsigned mc = __ballot_sync(0xffffffffu, is_cnd);
+        if (is_win) {
+          const uint32_t p = bw + __popc(mw & lt);
+          if (p < (uint32_t)pl.k_max) out[p] = (int)pos[u];
+        }
+        if (is_cnd) {
+          // key and position together: the row's last CTA has no dependent gather to wait for
+          const uint32_t p = bc + __popc(mc & lt);
+          if (p < (uint32_t)pl.cand_cap) rc[p] = make_uint2(score_key(sv[u]), pos[u]);
+        }
+        bw += __popc(mw);
+        bc += __popc(mc);
+      }
     }
     __syncwarp();
     buf_n = 0;
@@ -567,7 +572,8 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
   if (!cta_arrived_last(&counters[row * 4 + 1], gridDim.x, &s_last)) return;
 
   // ---- last CTA of the row: check the bracket by counting, then select among the candidates
-  const int W = (int)__ldcg(n_out), C = (int)__ldcg(n_cand);
+  const unsigned long long both = __ldcg(n_both);
+  const int W = (int)(uint32_t)both, C = (int)(both >> 32);
   if (tid == 0) s_emit = 0u;
   __syncthreads();
   uint32_t kstar;
