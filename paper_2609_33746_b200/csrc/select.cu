@@ -596,30 +596,33 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
       // the first kStashCap candidates are staged; the rest, if any, is read from the list each time (a
       // bracket 1 % of 512K scores wide holds about 5200: with all of them left to the radix select,
       // whose passes reread the list, the finish took 17 us instead of 5)
-      uint32_t kmin = 0xffffffffu, kmax = 0u;                  // range of the finite keys
-      auto widen = [&](uint32_t key) {
-        if (fabsf(key_score(key)) < CUDART_INF_F) {
-          kmin = min(kmin, key);
-          kmax = max(kmax, key);
-        }
-      };
-      {
-        constexpr int kPer = kStashCap / kSelThreads;          // 10: all loads issued together
-        uint2 it[kPer];
+      constexpr int kPer = kStashCap / kSelThreads;            // 10: all loads issued together
+      uint2 it[kPer];
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-          const int i = u * kSelThreads + tid;
-          it[u] = i < C ? __ldcg(rc + i) : make_uint2(0x80000000u, 0u);
-        }
+      for (int u = 0; u < kPer; ++u) {
+        const int i = u * kSelThreads + tid;
+        it[u] = i < C ? __ldcg(rc + i) : make_uint2(0x80000000u, 0u);
+      }
+      for (int i = tid; i < kHistBins; i += kSelThreads) s_hist[i] = 0u;
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-          const int i = u * kSelThreads + tid;
-          if (i < C) {
-            s_stash[i] = it[u];
-            widen(it[u].x);
+      for (int u = 0; u < kPer; ++u) {
+        const int i = u * kSelThreads + tid;
+        if (i < C) s_stash[i] = it[u];
+      }
+      const int src = C <= kStashCap ? kFromStash : kFromList;
+      auto item = [&](int i) { return i < kStashCap ? s_stash[i] : __ldcg(rc + i); };
+      __syncthreads();
+      // range of the candidates: the bracket, or, where it is open, their finite scores
+      float lo_h = lo_f, hi_h = hi_f;
+      if (!(lo_f > -CUDART_INF_F && hi_f < CUDART_INF_F)) {
+        uint32_t kmin = 0xffffffffu, kmax = 0u;
+        for (int i = tid; i < C; i += kSelThreads) {
+          const uint32_t key = item(i).x;
+          if (fabsf(key_score(key)) < CUDART_INF_F) {
+            kmin = min(kmin, key);
+            kmax = max(kmax, key);
           }
         }
-        for (int i = kStashCap + tid; i < C; i += kSelThreads) widen(__ldcg(rc + i).x);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
@@ -633,21 +636,17 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
           kmax = max(kmax, (uint32_t)s_scan[16 + w]);
         }
         __syncthreads();                                       // s_scan is reused below
+        lo_h = kmin < kmax ? key_score(kmin) : 0.f;
+        hi_h = kmin < kmax ? key_score(kmax) : 0.f;
       }
-      const int src = C <= kStashCap ? kFromStash : kFromList;
-      auto item = [&](int i) { return i < kStashCap ? s_stash[i] : __ldcg(rc + i); };
       bool done = false;
-      if (kmax > kmin) {
-        // Fast finish.  ONE histogram of the candidates over 4096 equal buckets of the
-        // range of their finite scores (candidates at -inf, the sink and window positions of a
-        // row that was not bracketed from below, fall into the bottom bucket) finds the bucket of
-        // the r-th largest; everything in a higher bucket is taken at once, and the few items of
-        // that bucket are ranked against each other (larger score first, then lower position:
-        // the stable rule).
-        const float lo_h = key_score(kmin);
-        const float scale = (float)kHistBins / (key_score(kmax) - lo_h);
-        for (int i = tid; i < kHistBins; i += kSelThreads) s_hist[i] = 0u;
-        __syncthreads();
+      if (hi_h > lo_h) {
+        // Fast finish.  ONE histogram of the candidates over 4096 equal buckets of their range
+        // (candidates at -inf, the sink and window positions of a row that was not bracketed from
+        // below, fall into the bottom bucket) finds the bucket of the r-th largest; everything in a
+        // higher bucket is taken at once, and the few items of that bucket are ranked against each
+        // other (larger score first, then lower position: the stable rule).
+        const float scale = (float)kHistBins / (hi_h - lo_h);
         for (int i = tid; i < C; i += kSelThreads)
           atomicAdd(&s_hist[linear_bucket(key_score(item(i).x), lo_h, scale)], 1u);
         __syncthreads();
@@ -660,14 +659,30 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
           uint2* tie = reinterpret_cast<uint2*>(s_hist);
           if (tid == 0) s_tie = 0u;
           __syncthreads();
-          for (int base = 0; base < C; base += kSelThreads) {
-            const int i = base + tid;
-            const bool v = i < C;
-            const uint2 it = v ? item(i) : make_uint2(0u, 0u);
-            const int bk = v ? linear_bucket(key_score(it.x), lo_h, scale) : -1;
-            const int p = warp_append(v && bk > d, &s_emit);
-            if (p >= 0 && (uint32_t)W + p < (uint32_t)pl.k_max) out[W + p] = (int)it.y;
-            if (v && bk == d) tie[atomicAdd(&s_tie, 1u)] = it;
+          // 32 items per thread and append
+          for (int base = 0; base < C; base += 32 * kSelThreads) {
+            uint32_t take = 0u;
+            for (int u = 0; u < 32 && base + u * kSelThreads < C; ++u) {
+              const int i = base + u * kSelThreads + tid;
+              if (i >= C) break;
+              const uint2 x = item(i);
+              const int bk = linear_bucket(key_score(x.x), lo_h, scale);
+              if (bk > d) take |= 1u << u;
+              if (bk == d) tie[atomicAdd(&s_tie, 1u)] = x;
+            }
+            __syncwarp();
+            const int mine = __popc(take);
+            int inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const int v = __shfl_up_sync(0xffffffffu, inc, o);
+              if (lane >= o) inc += v;
+            }
+            uint32_t p = 0u;
+            if (lane == 31 && inc > 0) p = atomicAdd(&s_emit, (uint32_t)inc);
+            p = (uint32_t)W + __shfl_sync(0xffffffffu, p, 31) + (uint32_t)(inc - mine);
+            for (; take != 0u; take &= take - 1u, ++p)
+              if (p < (uint32_t)pl.k_max) out[p] = (int)item(base + (__ffs(take) - 1) * kSelThreads + tid).y;
           }
           __syncthreads();
           for (int base = 0; base < m; base += kSelThreads) {
