@@ -2,7 +2,7 @@
 // T(q) = TopK_{k, i in R} l~_i with k = ceil(rho |R|).
 //
 // One pass over the scores instead of a multi-pass radix sort of the whole row:
-//   sample kernel  one CTA per row reads up to 16384 scores (1024 groups of 16 at a jittered
+//   sample kernel  one CTA per row reads up to 8192 or 16384 scores (groups of 16 at a jittered
 //                  stride; never more than a quarter of the row) and takes two order
 //                  statistics of the sample that bracket the k-th largest score of the row
 //                  with a 6-sigma margin: lo <= s_k <= hi (one histogram of the sample over
@@ -29,9 +29,12 @@ namespace {
 constexpr int kElems = kSelChunk / kSelThreads;   // scores per thread per chunk (16)
 constexpr int kStashCap = 5120;                   // candidates resolved from shared memory
 constexpr int kFilterSmemBytes = kHistBins * 4 + kStashCap * 8;   // dynamic: above the 48 KB static limit
-constexpr int kSample = 16384;                    // sampled scores per row (at most a quarter of it)
-constexpr int kSamplePer = kSample / kSelThreads; // per thread (32)
-constexpr int kSampleGroups = kSample / 16;       // groups of 16 consecutive scores (64 bytes)
+// Sampled scores per row, in groups of 16 consecutive ones (64 bytes): 16 or 32 per thread, at most a
+// quarter of the row.  A larger sample brackets tighter, a smaller one is read sooner and leaves room
+// for three rows per SM.  Decode step, 32 -> 16 per thread, us: 8 x 128K 300.0 -> 299.3, 4-bit codes
+// 185.2 -> 184.3, 16 ragged up to 128K 516.0 -> 510.2; but 2 x 256K 167.8 -> 170.9, one of 512K
+// 173.1 -> 178.6.
+constexpr int kSampleLong = 131072;               // rows with room for more than this take 32
 constexpr float kBracketSigmas = 6.0f;
 
 // rowstate: [0] lo, [1] hi (float bits), [2] k, [3] n
@@ -202,10 +205,12 @@ __device__ void find_two_buckets(const uint32_t* hist, int rank_a, int rank_b, i
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSelThreads, 2)     // two rows per SM: 64 registers
+template <int kSamplePer>
+__global__ void __launch_bounds__(kSelThreads, kSamplePer > 16 ? 2 : 3)
 sel_sample_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __restrict__ seq_lens,
                   int32_t* __restrict__ rowstate, int32_t* __restrict__ sel_count,
                   float* __restrict__ kth) {
+  constexpr int kSampleGroups = kSamplePer * kSelThreads / 16;
   __shared__ __align__(16) uint32_t s_hist[kHistBins];
   __shared__ int s_scan[36];
   __shared__ float s_mm[2][kSelThreads / 32];
@@ -216,7 +221,7 @@ sel_sample_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __re
   const int n = clamp_len(seq_lens[b], pl.N_max);
   const int k = region_budget(pl, n, b);
   const Region rg = region_of(pl, n, b);
-  // n_groups aligned groups of 16 consecutive scores (1024 of them on a long row, never more
+  // n_groups aligned groups of 16 consecutive scores (kSampleGroups of them on a long row, never more
   // than a quarter of the row); group g sits in the g-th of n_groups equal strides of the
   // row at a hashed offset, and four neighbouring threads read its 64 bytes
   const int n_groups = min(kSampleGroups, n / 64);
@@ -732,9 +737,17 @@ cudaError_t launch_select(const Plan& pl, const WsLayout& L, char* ws, const flo
   int* status = reinterpret_cast<int*>(ws + L.status);
   if (pl.sel_cluster > 0)
     return launch_select_cluster(pl, scores, seq_lens, sel_idx, sel_count, kth, status, st);
-  set_carveout<sel_sample_kernel>(kStreamCarveout);
-  cudaError_t e = launch_pdl(sel_sample_kernel, dim3(pl.rows), dim3(kSelThreads), 0, st, pl, scores,
-                             seq_lens, rowstate, sel_count, kth);
+  auto sample = [&](auto kernel) {
+    return launch_pdl(kernel, dim3(pl.rows), dim3(kSelThreads), 0, st, pl, scores, seq_lens, rowstate, sel_count, kth);
+  };
+  cudaError_t e;
+  if (pl.N_max > kSampleLong) {
+    set_carveout<sel_sample_kernel<32>>(kStreamCarveout);
+    e = sample(sel_sample_kernel<32>);
+  } else {
+    set_carveout<sel_sample_kernel<16>>(kStreamCarveout);
+    e = sample(sel_sample_kernel<16>);
+  }
   if (e != cudaSuccess) return e;
   // more than 48 KB of dynamic shared memory needs an opt-in (per device, so set every time)
   e = cudaFuncSetAttribute(sel_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
