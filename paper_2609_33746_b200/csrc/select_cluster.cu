@@ -17,7 +17,8 @@
 //      over the positions of equal scores;
 //   3. everything above the range is emitted to slots from a prefix sum over the cluster; the items
 //      inside it are ranked by (score, lower position first) in CTA 0.
-// The result is the exact top-k with the stable tie rule for every input.
+// The result is the exact top-k with the stable tie rule for every input; a score that is not a number
+// (the token's cached key has one) ranks below -inf.
 //
 // What bounds it: latency.  A cluster barrier costs 600 to 1000 clocks, and the kernel runs through
 // its code once, so that instruction fetches are the largest stall (4.4 warps per issue of 16).
@@ -40,6 +41,7 @@ constexpr int kClTies = 1024;           // items CTA 0 ranks at the end
 constexpr int kClList = 3072;           // scores at or above the bound that a CTA lists
 constexpr int kClMax = 8;               // largest cluster
 constexpr int kOctaveShift = 19;        // step 1: 16 ranges per power of two
+constexpr uint32_t kNanKey = 1u;        // NaN ranks below -inf: taken only when nothing else is left
 
 // ---- cluster primitives
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -185,7 +187,8 @@ struct Slice {
         const int e = __clz(hit);
         hit ^= 0x80000000u >> e;
         const int p = 4 * (i0 + (e >> 2) * kClThreads) + (e & 3);
-        f(max(score_key(reinterpret_cast<const float*>(s)[p]), 1u), begin + p, slot++);
+        const float v = reinterpret_cast<const float*>(s)[p];
+        f(v == v ? score_key(v) : kNanKey, begin + p, slot++);
       }
     }
   }
