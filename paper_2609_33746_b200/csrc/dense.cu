@@ -200,7 +200,7 @@ dense_decode_kernel(Plan pl, const T* __restrict__ q, const T* __restrict__ kc,
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float p = sc[u] > -CUDART_INF_F ? fast_exp2(sc[u] - m) : 0.f;
+      const float p = sc[u] == -CUDART_INF_F ? 0.f : fast_exp2(sc[u] - m);      // (not a number: shows in the output)
       Z += p;
       unsigned long long v2[4];
       unpack2<T>(row_part(src + u * 1024u + 256u), v2);
