@@ -11,13 +11,15 @@
 //   build_prepare_kernel     norms and unit directions U (fp32, workspace) from the paged cache
 //   build_seed_kernel        centroids <- U rows at the given positions
 //   build_split_kernel       centroids as split fp16 tensor-core tiles (tc.cuh), once per iteration
-//   build_assign_kernel      nearest centroid of 256 tokens per CTA on the tensor cores
+//   build_assign_kernel      nearest centroid of 256 tokens per CTA on the tensor cores; what comes within
+//                            the rounding of the nearest is compared in fp32 (tc.cuh): the lists, and
+//                            with them everything that follows, are those of an fp32 search
 //   build_hist / _offsets / _scatter   the tokens of a unit grouped by list (counting sort)
 //   build_dir_sums_kernel    per-list sums of the member directions (64-bit fixed point, so the
 //                            result does not depend on the order of the atomics): a warp sums the
 //                            rows of consecutive grouped tokens and adds once per list it meets
-//   build_update_centroids_kernel   takes the mean; build_reseed_kernel: empty lists take the
-//                            farthest points (rare)
+//   build_update_centroids_kernel   takes the mean; build_distance_kernel, build_reseed_kernel: empty
+//                            lists take the farthest points (rare)
 //   build_residual_kernel    U <- U - c_a, in place
 //   build_pq_* kernels       the same steps for the residual sub-vectors, also on the tensor cores
 //   build_value_* kernels    list value means and member counts from the paged values, in list order
@@ -168,15 +170,19 @@ build_split_kernel(Plan pl, const float* __restrict__ centroids, unsigned char* 
 // cuBLAS GEMM reaches (64 clocks with few SMs busy): 5.4 of the 6.2 thousand clocks per tile; behind them
 // the search for the two nearest (2.4 to 3.6 thousand, overlapped) and the token tile at the start (8.1
 // thousand, 1 CTA per SM: nothing overlaps it).  1 M tokens x 1024 lists: 1231 us with 64 centroids per
-// tile, two stages and an index beside every value, 1000 us so, 940 us with whole sectors loaded.
+// tile, two stages and an index beside every value, 1000 us so, 940 us with whole sectors loaded, 970 us
+// with what fp32 decides.
 __global__ void __launch_bounds__(kAsgThreads, 1)
 build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* __restrict__ images,
                     const float* __restrict__ centroids, const int32_t* __restrict__ seq_lens,
-                    uint16_t* __restrict__ list_ids, float* __restrict__ dmin, float* __restrict__ key_norms) {
+                    uint16_t* __restrict__ list_ids, float* __restrict__ key_norms) {
   extern __shared__ __align__(128) unsigned char s_asg[];
   unsigned char* s_tok = s_asg;                             // two token tiles
   unsigned char* s_cen = s_asg + 2 * kTokTileBytes;         // the centroid tile
   __shared__ float s_x2[kAsgTok];
+  __shared__ uint8_t s_crowd[kAsgTok];                      // tokens that fp32 searches for
+  __shared__ int s_n_crowd;
+  __shared__ Found s_found[8][kCrowd];
   __shared__ uint32_t s_tmem;
   __shared__ __align__(8) uint64_t s_full[kAsgPieces], s_used[kAsgPieces], s_done[2], s_free[2];
   const int kv = blockIdx.y, b = blockIdx.z;
@@ -198,6 +204,7 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
   if (t0 >= n) return;
   const int n_tiles = (pl.n_list + kAsgCen - 1) / kAsgCen;
   const unsigned char* img = images + ukv * (size_t)n_tiles * kCenTileBytes;
+  if (tid == 0) s_n_crowd = 0;
   if (warp == 8) tmem_alloc(&s_tmem, 512);
   if (warp == 9) {
     if (lane < kAsgPieces) { mbar_init(&s_full[lane], 1); mbar_init(&s_used[lane], 1); }
@@ -296,6 +303,8 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
   } else {
     const int wg = warp >> 2;
     const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+    const int r = wg * 128 + (warp & 3) * 32 + lane;
+    const TieLimit lim(s_x2[r]);
     Nearest2 nn;
     nn.clear();
     for (int i = 0; i < n_tiles; ++i) {
@@ -307,46 +316,69 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
       for (int c = 0; c < n_cols; c += 32) {
         float acc[32];
         tmem_ld32(tmem + st * 256u + wg * 128u + c + lanes, acc);
-        nn.take(acc, i * (kAsgCen / 32) + (c >> 5));
+        nn.take(acc, i * (kAsgCen / 32) + (c >> 5), lim);
       }
       tc_fence_before();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&s_free[st])) : "memory");
       __syncwarp();
     }
-    int near = nn.near();
-    const int next = nn.next();
-    const int r = wg * 128 + (warp & 3) * 32 + lane;
-    if (t0 + r < n) {
-      const size_t at = ukv * pl.N_max + t0 + r;
-      float d = s_x2[r] + nn.low * kTcUnscale;
-      if (nn.tie() && max(near, next) < pl.n_list) {
-        // the two are within the rounding of either arithmetic: decided in plain fp32, every sum one
-        // chain over the dims (a few tokens in a thousand)
-        const float4* u = reinterpret_cast<const float4*>(U + at * kD);
-        const float4* c0 = reinterpret_cast<const float4*>(centroids + (ukv * pl.n_list + min(near, next)) * kD);
-        const float4* c1 = reinterpret_cast<const float4*>(centroids + (ukv * pl.n_list + max(near, next)) * kD);
-        float xx = 0.f, a0 = 0.f, a1 = 0.f, n0 = 0.f, n1 = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < kD / 4; ++k) {
-          const float4 x = __ldcg(u + k), y = __ldcg(c0 + k), z = __ldcg(c1 + k);
-          xx = fmaf(x.x, x.x, xx); xx = fmaf(x.y, x.y, xx); xx = fmaf(x.z, x.z, xx); xx = fmaf(x.w, x.w, xx);
-          a0 = fmaf(x.x, y.x, a0); a0 = fmaf(x.y, y.y, a0); a0 = fmaf(x.z, y.z, a0); a0 = fmaf(x.w, y.w, a0);
-          n0 = fmaf(y.x, y.x, n0); n0 = fmaf(y.y, y.y, n0); n0 = fmaf(y.z, y.z, n0); n0 = fmaf(y.w, y.w, n0);
-          a1 = fmaf(x.x, z.x, a1); a1 = fmaf(x.y, z.y, a1); a1 = fmaf(x.z, z.z, a1); a1 = fmaf(x.w, z.w, a1);
-          n1 = fmaf(z.x, z.x, n1); n1 = fmaf(z.y, z.y, n1); n1 = fmaf(z.z, z.z, n1); n1 = fmaf(z.w, z.w, n1);
-        }
-        const float d0 = (xx - 2.0f * a0) + n0, d1 = (xx - 2.0f * a1) + n1;
-        near = d1 < d0 ? max(near, next) : min(near, next);
-        d = fminf(d0, d1);
-      }
-      list_ids[at] = (uint16_t)min(near, pl.n_list - 1);
-      dmin[at] = d;
-      if (late) key_norms[at] = CUDART_NAN_F;              // a bounded wait ran out: the norms say so
+    // between the centroids of one or two blocks fp32 decides (a few tokens in a hundred), a warp per token
+    int near = min(nn.near(), pl.n_list - 1);
+    const bool real = t0 + r < n, crowd = real && nn.crowded();
+    const int block1 = nn.second_near(lim) ? nn.second_at : nn.best_at;
+    unsigned ties = __ballot_sync(0xffffffffu, real && !crowd && nn.tie(lim));
+    while (ties) {
+      const int src = __ffs(ties) - 1;
+      ties &= ties - 1u;
+      const int at = nearest_of_blocks<true>(U + (ukv * pl.N_max + t0 + r - lane + src) * kD, centroids + ukv * pl.n_list * (size_t)kD,
+                                             pl.n_list, __shfl_sync(0xffffffffu, nn.best_at, src), __shfl_sync(0xffffffffu, block1, src));
+      if (lane == src) near = at;
+    }
+    if (crowd) s_crowd[atomicAdd(&s_n_crowd, 1)] = (uint8_t)r;
+    if (real) {
+      list_ids[ukv * pl.N_max + t0 + r] = (uint16_t)near;
+      if (late) key_norms[ukv * pl.N_max + t0 + r] = CUDART_NAN_F;      // a bounded wait ran out: the norms say so
     }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 8) { tc_fence_after(); tmem_free(tmem, 512); }
+  // between more of them over all centroids, by eight warps
+  const int n_crowd = s_n_crowd;
+  const int n_search = n_crowd > kCrowd ? kCrowd : 1;       // for together
+#pragma unroll 1
+  for (int c = 0; c < n_crowd; c += n_search) {
+    const float* rows = U + (ukv * pl.N_max + t0) * kD;
+    const float* cen = centroids + ukv * pl.n_list * (size_t)kD;
+    if (warp < 8) {
+      if (n_search == 1) nearest_of_all<true, 1>(rows, kD, s_crowd, c, n_crowd, cen, pl.n_list, tid, 256, s_found[warp]);
+      else nearest_of_all<true, kCrowd>(rows, kD, s_crowd, c, n_crowd, cen, pl.n_list, tid, 256, s_found[warp]);
+    }
+    __syncthreads();
+    if (tid < n_search && c + tid < n_crowd) {
+      Found f = s_found[0][tid];
+      for (int w = 1; w < 8; ++w) nearer(f.d, f.at, s_found[w][tid].d, s_found[w][tid].at);
+      list_ids[ukv * pl.N_max + t0 + s_crowd[c + tid]] = (uint16_t)f.at;
+    }
+    __syncthreads();
+  }
+}
+
+// Squared distance of every token to its list's centroid, in fp32, one chain per sum; only for units with
+// an empty list (they take the farthest points), infinite where it is not a number
+__global__ void __launch_bounds__(kPrepThreads)
+build_distance_kernel(Plan pl, const float* __restrict__ U, const float* __restrict__ centroids,
+                      const int32_t* __restrict__ seq_lens, const uint16_t* __restrict__ list_ids,
+                      const int32_t* __restrict__ n_empty, float* __restrict__ dmin) {
+  const int kv = blockIdx.y, b = blockIdx.z;
+  const int n = clamp_len(seq_lens[b], pl.N_max);
+  const size_t ukv = (size_t)b * pl.Hkv + kv;
+  if (n_empty[ukv] == 0 || n <= pl.n_list) return;
+  for (int i = blockIdx.x * kPrepThreads + threadIdx.x; i < n; i += gridDim.x * kPrepThreads) {
+    const size_t at = ukv * pl.N_max + i;
+    const float d = distance_fp32<true>(U + at * kD, centroids + (ukv * pl.n_list + min((int)list_ids[at], pl.n_list - 1)) * (size_t)kD);
+    dmin[at] = d == d ? d : CUDART_INF_F;
+  }
 }
 
 // ---- tokens grouped by list.  hist: members per list; offsets: exclusive prefix (and a running
@@ -381,17 +413,20 @@ build_hist_kernel(Plan pl, const uint16_t* __restrict__ list_ids, const int32_t*
 }
 
 __global__ void __launch_bounds__(1024)
-build_offsets_kernel(Plan pl, const int32_t* __restrict__ counts, int32_t* __restrict__ cursor) {
+build_offsets_kernel(Plan pl, const int32_t* __restrict__ counts, int32_t* __restrict__ cursor,
+                     int32_t* __restrict__ n_empty) {
   __shared__ int s_warp[32];
   const size_t unit = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int v[4], local = 0;                                      // n_list <= 4096: 4 lists per thread
+  int v[4], local = 0, empty = 0;                           // n_list <= 4096: 4 lists per thread
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int j = 4 * tid + u;
     v[u] = j < pl.n_list ? counts[unit * pl.n_list + j] : 0;
     local += v[u];
+    empty += j < pl.n_list && v[u] == 0 ? 1 : 0;
   }
+  if (empty != 0 && n_empty != nullptr) atomicAdd(&n_empty[unit], empty);
   int inc = local;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -506,11 +541,10 @@ build_dir_sums_kernel(Plan pl, const float* __restrict__ U, const uint16_t* __re
            });
 }
 
-// c_j <- mean of its members; an empty list keeps its centre and is counted; sums are cleared
+// c_j <- mean of its members; an empty list keeps its centre; sums are cleared
 __global__ void build_update_centroids_kernel(Plan pl, long long* __restrict__ sums,
                                               const int32_t* __restrict__ counts,
-                                              float* __restrict__ centroids,
-                                              int32_t* __restrict__ n_empty) {
+                                              float* __restrict__ centroids) {
   const size_t unit = blockIdx.y;
   const int j = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (j >= pl.n_list) return;
@@ -520,8 +554,6 @@ __global__ void build_update_centroids_kernel(Plan pl, long long* __restrict__ s
     *reinterpret_cast<float4*>(centroids + at) =
         make_float4(fix_mean(sums[at], c, kFixDir), fix_mean(sums[at + 1], c, kFixDir),
                     fix_mean(sums[at + 2], c, kFixDir), fix_mean(sums[at + 3], c, kFixDir));
-  } else if (lane == 0) {
-    atomicAdd(&n_empty[unit], 1);
   }
 #pragma unroll
   for (int t = 0; t < 4; ++t) sums[at + t] = 0;
@@ -626,14 +658,16 @@ __global__ void build_pq_seed_kernel(Plan pl, const float* __restrict__ E, const
 // kMg subspaces (64 bytes of a residual row) as tensor-core tiles and walks a range of tokens, 128 at
 // a time per warpgroup: thread = token = accumulator row.  The accumulators give the group of 8
 // codewords that holds the minimum, the codeword is decided in fp32 among those 8 (distance =
-// (|e|^2 - 2 e.p) + |p|^2, lower index on ties).  Training accumulates the codewords' sums in 64-bit
-// fixed point: two 32-bit shared-memory limbs of 21 bits and the rest (native integer atomics),
-// folded into 64 bits every kFoldSteps steps, before a limb could overflow.
-// What bounds it: the integer pipe (minima, comparisons, selects: 69 % of its cycles at 340 of 550
-// instructions per token and subspace) and, with one warp of each group per scheduler, the 650 clocks
-// from an MMA's issue to its mbarrier.  1 M tokens x 32 subspaces x 256 codewords: 1190 us a training
-// pass and 1050 us for the codes with run-time sizes, the codewords decided before the next MMA and codes
-// stored byte by byte; 1036 and 913 us so.  MMAs of 64 codewords into two accumulators: 1505 and 1395.
+// (|e|^2 - 2 e.p) + |p|^2, lower index on ties); where a second group comes within the rounding, or two
+// of the 8 are equal, all codewords are compared in fp32 (one sub-vector in some thousand).  Training
+// accumulates the codewords' sums in 64-bit fixed point: two 32-bit shared-memory limbs of 21 bits and
+// the rest (native integer atomics), folded into 64 bits every kFoldSteps steps, before a limb could
+// overflow.
+// What bounds it: the integer pipe (minima, comparisons, selects) and, with one warp of each group per
+// scheduler, the 650 clocks from an MMA's issue to its mbarrier.  1 M tokens x 32 subspaces x 256
+// codewords: 1190 us a training pass and 1050 us for the codes with run-time sizes, the codewords decided
+// before the next MMA and codes stored byte by byte; 1037 and 914 us so; 1170 and 1034 us with the second
+// group kept beside the first.  MMAs of 64 codewords into two accumulators: 1505 and 1395.
 template <int DSUB, int NC> struct PqPlan {
   using Tile = PqTile<DSUB>;
   static constexpr int kMg8 = 16 / DSUB;                     // subspaces per CTA, 8-bit codes
@@ -658,6 +692,46 @@ __device__ __forceinline__ void limbs(float x, int& hi, int& lo) {
   hi = __float_as_int(h) - __float_as_int(kMagic);
   lo = __float_as_int(l) - __float_as_int(kMagic);
 }
+
+// a sub-vector into the sums of codeword z of subspace mm
+template <int DSUB, int NC>
+__device__ __forceinline__ void add_member(uint32_t* s_limb, int mm, const float (&x)[DSUB], uint32_t z) {
+  uint32_t* l = s_limb + mm * (2 * DSUB + 1) * NC + z;
+#pragma unroll
+  for (int t = 0; t < DSUB; ++t) {
+    int hi, lo;
+    limbs(x[t], hi, lo);
+    atomicAdd(l + (2 * t) * NC, (uint32_t)lo);
+    atomicAdd(l + (2 * t + 1) * NC, (uint32_t)hi);
+  }
+  atomicAdd(l + 2 * DSUB * NC, 1u);
+}
+// (see settle_codewords; item mm is subspace m0 + mm)
+template <int DSUB, int NC, bool kTrain> struct PqSettle {
+  const float* rows;                                        // residuals of the warp's tokens, first subspace
+  int last;                                                 // last of them inside the range
+  const float* s_word;
+  uint32_t* s_limb;
+  unsigned long long result;                                // codes of this lane's token
+  __device__ __forceinline__ void load(int lane, int mm, float (&x)[DSUB]) const {
+    load_sub<DSUB>(rows + (long long)min(lane, last) * kD + mm * DSUB, x);
+  }
+  __device__ __forceinline__ float distance(int mm, const float (&x)[DSUB], int z) const {
+    float w[DSUB], x2 = 0.f, dot = 0.f, p2 = 0.f;
+    load_sub<DSUB>(s_word + (mm * NC + z) * DSUB, w);
+#pragma unroll
+    for (int t = 0; t < DSUB; ++t) { x2 = fmaf(x[t], x[t], x2); dot = fmaf(x[t], w[t], dot); p2 = fmaf(w[t], w[t], p2); }
+    return (x2 - 2.0f * dot) + p2;
+  }
+  __device__ __forceinline__ void done(int mm, const float (&x)[DSUB], int z) {
+    if constexpr (kTrain) {
+      add_member<DSUB, NC>(s_limb, mm, x, (uint32_t)z);
+    } else {
+      constexpr int kBits = PqPlan<DSUB, NC>::kBits;
+      result = (result & ~((unsigned long long)(NC - 1) << (mm * kBits))) | ((unsigned long long)z << (mm * kBits));
+    }
+  }
+};
 
 template <int DSUB, int NC, bool kTrain>
 __global__ void __launch_bounds__(kPqThreads, 1)
@@ -685,22 +759,13 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
   long long* s_sum = reinterpret_cast<long long*>(s_a + 4 * Tile::kChunks * 2048);   // [mg][DSUB][nc] (training)
   float* s_word = reinterpret_cast<float*>(s_sum + (kTrain ? (size_t)words * DSUB : 0));   // [mg][nc][DSUB]
   uint32_t* s_limb = reinterpret_cast<uint32_t*>(s_word + (size_t)words * DSUB);   // [mg][2 DSUB + 1][nc]
-  auto load_sub = [](const float* src, float (&x)[DSUB]) {
-    if constexpr (DSUB == 2) {
-      *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(src);
-    } else {
-#pragma unroll
-      for (int c4 = 0; c4 < DSUB / 4; ++c4)
-        *reinterpret_cast<float4*>(x + 4 * c4) = *reinterpret_cast<const float4*>(src + 4 * c4);
-    }
-  };
   if (warp == 0) tmem_alloc(&s_tmem, 512);
   if (tid < 4) mbar_init(&s_bar[tid], 1);
   if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   const float* cb = codebooks + (ukv * pl.M + m0) * (size_t)nc * DSUB;
   for (int w = tid; w < words; w += kPqThreads) {
     float p[DSUB];
-    load_sub(cb + (size_t)w * DSUB, p);
+    load_sub<DSUB>(cb + (size_t)w * DSUB, p);
     uint4 ch[Tile::kChunks];
     Tile::code_row(p, ch);
     const int mm = w / nc, z = w - mm * nc;
@@ -772,7 +837,7 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
   const uint32_t rot = (uint32_t)(lane & 7) * kRow;
   float e[DSUB], e_nxt[DSUB];
   const float* er = row_of(begin);
-  load_sub(er, e_nxt);
+  load_sub<DSUB>(er, e_nxt);
   put_row(e_nxt);
   issue(0, 0);
   uint32_t parity = 0u;
@@ -783,14 +848,15 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
     const int i = base + wg * 128 + row;
     const bool real = i < end;
     unsigned long long code = 0ull;
+    unsigned ties = 0u;                                     // bit mm: decided after the others
 #pragma unroll 1
     for (int mm = 0; mm < mg; ++mm) {
 #pragma unroll
       for (int t = 0; t < DSUB; ++t) e[t] = e_nxt[t];
       const bool next = mm + 1 < mg || more;
-      load_sub(mm + 1 < mg ? er + (mm + 1) * DSUB : er_next, e_nxt);
-      float bd = CUDART_INF_F;
-      int grp = 0;
+      load_sub<DSUB>(mm + 1 < mg ? er + (mm + 1) * DSUB : er_next, e_nxt);
+      NearestGroup ng;
+      ng.clear();
 #pragma unroll
       for (int c = 0; c < per; ++c) {
         late |= !tc_wait(&s_bar[wg], parity);
@@ -800,13 +866,13 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
         if constexpr (nc == 16) {
           float acc[16];
           tmem_ld16(my_tmem, acc);
-          group_minima<true>(acc, 0, bd, grp);
+          ng.take(acc, 0u);
         } else {
 #pragma unroll
           for (int h = 0; h < kCols; h += 32) {
             float acc[32];
             tmem_ld32(my_tmem + h, acc);
-            group_minima<true>(acc, (c * kCols + h) / 8, bd, grp);
+            ng.take(acc, (uint32_t)(c * kCols + h) / 8u);
           }
         }
         if (c + 1 < per) issue(mm, c + 1);
@@ -817,37 +883,34 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
       float en = 0.f, dist[8];
 #pragma unroll
       for (int t = 0; t < DSUB; ++t) en = fmaf(e[t], e[t], en);
-      const uint32_t at = (uint32_t)(8 * grp) * kRow + rot;
+      const uint32_t at = (uint32_t)(8 * ng.group()) * kRow + rot;
       const unsigned char* s_sub = reinterpret_cast<const unsigned char*>(s_word) + (size_t)mm * nc * kRow;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         float w[DSUB], dot = 0.f, p2 = 0.f;
-        load_sub(reinterpret_cast<const float*>(s_sub + (at ^ (q * kRow))), w);
+        load_sub<DSUB>(reinterpret_cast<const float*>(s_sub + (at ^ (q * kRow))), w);
 #pragma unroll
         for (int t = 0; t < DSUB; ++t) { dot = fmaf(e[t], w[t], dot); p2 = fmaf(w[t], w[t], p2); }
         dist[q] = (en - 2.0f * dot) + p2;
       }
       const float dm = min3(min3(dist[0], dist[1], dist[2]), min3(dist[3], dist[4], dist[5]), fminf(dist[6], dist[7]));
-      uint32_t first = nc * kRow;
+      uint32_t above = 0u;                                  // bit 7 - q: codeword q of the lane's order is farther
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (dist[q] == dm) first = min(first, at ^ (q * kRow));
-      const uint32_t bz = first < nc * kRow ? first / kRow : 0u;         // (not a number: 0)
+      for (int q = 0; q < 8; ++q) above = __funnelshift_l(__float_as_uint(dm - dist[q]), above, 1);
+      const uint32_t equal = ~above << 24;                  // (not a number: all)
+      const uint32_t bz = (at ^ ((uint32_t)__clz(equal) * kRow)) / kRow;
+      const bool tie = pq_tie(ng, en) || (equal & (equal - 1u)) != 0u;      // (equal distances: the lower index)
+      if (tie) ties |= 1u << mm;
       if constexpr (kTrain) {
-        if (real) {
-          uint32_t* l = s_limb + mm * (2 * DSUB + 1) * nc + bz;
-#pragma unroll
-          for (int t = 0; t < DSUB; ++t) {
-            int hi, lo;
-            limbs(e[t], hi, lo);
-            atomicAdd(l + (2 * t) * nc, (uint32_t)lo);
-            atomicAdd(l + (2 * t + 1) * nc, (uint32_t)hi);
-          }
-          atomicAdd(l + 2 * DSUB * nc, 1u);
-        }
+        if (real && !tie) add_member<DSUB, NC>(s_limb, mm, e, bz);
       } else {
         code |= (unsigned long long)bz << (mm * P::kBits);
       }
+    }
+    // where another group may hold a codeword as near: all of them
+    if (__any_sync(0xffffffffu, real && ties != 0u)) {
+      const PqSettle<DSUB, NC, kTrain> st = {E + (ukv * pl.N_max + i - lane) * (size_t)kD + m0 * DSUB, end - 1 - (i - lane), s_word, s_limb, code};
+      code = settle_codewords<DSUB, NC>(real ? ties : 0u, mg, st);
     }
     if constexpr (!kTrain) {
       if (real) {
@@ -1029,16 +1092,18 @@ cudaError_t run_build(const Plan& pl, const pqhsa_paged_kv& kv, const int32_t* s
   const size_t list_smem = (size_t)pl.n_list * 4;
   auto assign = [&]() {
     build_split_kernel<<<split_grid, 4 * kAsgCen, 0, st>>>(pl, ix.centroids, images);
-    build_assign_kernel<<<asg_grid, kAsgThreads, kAsgSmemBytes, st>>>(pl, U, images, ix.centroids, seq_lens, ix.list_ids, dmin, ix.key_norms);
+    build_assign_kernel<<<asg_grid, kAsgThreads, kAsgSmemBytes, st>>>(pl, U, images, ix.centroids, seq_lens, ix.list_ids, ix.key_norms);
   };
   for (int it = 0; it < coarse_iters; ++it) {
     assign();
     PQHSA_TRY(cudaMemsetAsync(counts, 0, (size_t)units * pl.n_list * 4, st));
     build_hist_kernel<false><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, counts);
-    build_offsets_kernel<<<units, 1024, 0, st>>>(pl, counts, cursor);
+    build_offsets_kernel<<<units, 1024, 0, st>>>(pl, counts, cursor, n_empty);
+    build_distance_kernel<<<dim3(min(64, (pl.N_max + kPrepThreads - 1) / kPrepThreads), pl.Hkv, pl.B), kPrepThreads, 0, st>>>(
+        pl, U, ix.centroids, seq_lens, ix.list_ids, n_empty, dmin);
     build_scatter_kernel<false><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, cursor, order);
     build_dir_sums_kernel<<<run_grid, kPrepThreads, 0, st>>>(pl, U, ix.list_ids, order, seq_lens, sums);
-    build_update_centroids_kernel<<<list_grid, 256, 0, st>>>(pl, sums, counts, ix.centroids, n_empty);
+    build_update_centroids_kernel<<<list_grid, 256, 0, st>>>(pl, sums, counts, ix.centroids);
     build_reseed_kernel<<<units, 1024, 0, st>>>(pl, U, dmin, counts, seq_lens, n_empty, ix.centroids);
   }
   assign();
@@ -1049,7 +1114,7 @@ cudaError_t run_build(const Plan& pl, const pqhsa_paged_kv& kv, const int32_t* s
   // list value means and member counts
   PQHSA_TRY(cudaMemsetAsync(counts, 0, (size_t)units * pl.n_list * 4, st));
   build_hist_kernel<true><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, counts);
-  build_offsets_kernel<<<units, 1024, 0, st>>>(pl, counts, cursor);
+  build_offsets_kernel<<<units, 1024, 0, st>>>(pl, counts, cursor, nullptr);
   build_scatter_kernel<true><<<sort_grid, kSortThreads, list_smem, st>>>(pl, ix.list_ids, seq_lens, cursor, order);
   build_value_sums_kernel<T><<<run_grid, kPrepThreads, 0, st>>>(
       pl, vc, sp, stt, sh, kv.block_table, seq_lens, ix.list_ids, order, sums);

@@ -173,7 +173,8 @@ template <int DSUB> struct PqTile {
     w[3 * DSUB / 2 + 1] = bits16(__floats2half2_rn(kTcScale, 0.f));
     pack(w, c);
   }
-  static __device__ __forceinline__ void code_row(const float (&p)[DSUB], uint4 (&c)[kChunks]) {
+  // (returns |p|^2)
+  static __device__ __forceinline__ float code_row(const float (&p)[DSUB], uint4 (&c)[kChunks]) {
     uint32_t w[kK / 2];
 #pragma unroll
     for (int i = 0; i < kK / 2; ++i) w[i] = 0u;
@@ -187,6 +188,7 @@ template <int DSUB> struct PqTile {
     for (int t = 0; t < DSUB; ++t) n2 = fmaf(p[t], p[t], n2);
     split_norm(n2, w[3 * DSUB / 2], w[3 * DSUB / 2 + 1]);
     pack(w, c);
+    return n2;
   }
   static __device__ __forceinline__ void pack(const uint32_t (&w)[kK / 2], uint4 (&c)[kChunks]) {
 #pragma unroll
@@ -202,9 +204,6 @@ template <int DSUB> struct PqTile {
   }
 };
 
-// Smallest of groups of 8 accumulators; `best` / `grp` keep the smallest group and the first one
-// that has it.  The codeword inside the group is found by the caller in fp32: two instructions less
-// per accumulator than carrying an index.
 __device__ __forceinline__ float min3(float a, float b, float c) {      // one instruction
   float d;
   asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -219,37 +218,60 @@ __device__ __forceinline__ float min32(const float (&v)[32]) {
   return min3(min3(a, b, c), m[9], m[10]);
 }
 
-// The two nearest centroids of a token, 32 accumulators at a time.  Their column's low 5 bits travel in
-// the mantissa, so that a column costs 4 instructions (an index carried beside each value: 7 to 8), and
-// only where the 32 hold something near enough to matter.  Two that are nearer than kNearTie to each
-// other are a tie of the split arithmetic (4e-6 of a squared distance; 2^-19 for the 5 bits): the
-// caller decides it in fp32, so that the lists do not depend on how the search was split.
+// ---- When is the smallest accumulator the nearest centre?  The split arithmetic and fp32 each round, so
+// a search is trusted only where no other centre comes within the sum of both errors of the smallest;
+// everything else is decided in plain fp32, every sum one chain over the dims, lower index on ties.
+// The result is then that of an fp32 search over all centres, whatever the split.
+//
+// For a row x and a centre at distance d, |centre| <= |x| + d: the partial sums are of the size of |x|^2
+// and of the accumulated value v = d^2 - |x|^2.  The errors, per unit of those: nine accumulations at
+// full magnitude, truncated (4e-6 of the squared distance of unit vectors, the largest error
+// seen); the column's bits in the mantissa (2^-18 of |v| for each of the two compared); the fp32 chain.
+// kTieFloor: the fp16 terms have an absolute resolution of 2^-32.  Beyond kTieRange (|.|^2 of a row or
+// centre) they could overflow: fp32 decides.
+constexpr float kTieX2 = 6e-6f, kTieV = 8e-6f;
+constexpr float kTieFloor = kTcScale * kTcScale / 536870912.f;      // 2^-29
+constexpr float kTieRange = 100.f;
+struct TieLimit {
+  float k0;
+  __device__ __forceinline__ explicit TieLimit(float x2) : k0(fmaf(kTieX2 * kTcScale * kTcScale, x2, kTieFloor)) {}
+  // values below this may be as near as the one that gave `low`
+  __device__ __forceinline__ float operator()(float low) const { return low + fmaf(kTieV, fabsf(low), k0); }
+};
+
+// The nearest centroids of a token, a block of 32 accumulators at a time.  Their column's low 5 bits
+// travel in the mantissa, so that a column costs 4 instructions (an index carried beside each value: 7 to
+// 8), and only where the 32 hold something near enough to matter.  What is kept: the nearest of the two
+// best blocks, and how many blocks hold a centroid within reach of the nearest, or one of them two.
+// One or two such blocks are searched in fp32 by the caller, more of them (crowded) mean a search over all.
 constexpr uint32_t kColBits = 31u;
-constexpr float kNearTie = 6e-6f * kTcScale * kTcScale;
 struct Nearest2 {
   float low, best, second;                               // exact minimum; with column bits
   int best_at, second_at;                                // which 32 columns
+  int blocks;                                            // within reach of `low` (at most so many)
+  bool pair;                                             // two in one block
   __device__ __forceinline__ void clear() {
     low = best = second = CUDART_INF_F;
-    best_at = second_at = 0;
+    best_at = second_at = blocks = 0;
+    pair = false;
   }
   // (column bits: the value's own, or infinity's zeros)
-  static __device__ __forceinline__ int column(float v, int at) { return at * 32 + (int)(__float_as_uint(v) & kColBits); }
-  __device__ __forceinline__ int near() const { return column(best, best_at); }
-  __device__ __forceinline__ int next() const { return column(second, second_at); }
-  __device__ __forceinline__ bool tie() const { return second < best + kNearTie; }
-  // b <= s: the two nearest of another set
-  __device__ __forceinline__ void merge(float b, int b_at, float s, int s_at) {
+  __device__ __forceinline__ int near() const { return best_at * 32 + (int)(__float_as_uint(best) & kColBits); }
+  __device__ __forceinline__ bool second_near(const TieLimit& lim) const { return second < lim(best); }
+  __device__ __forceinline__ bool tie(const TieLimit& lim) const { return pair || second_near(lim); }
+  __device__ __forceinline__ bool crowded() const { return blocks > 2; }
+  // the best of another block
+  __device__ __forceinline__ void merge(float b, int b_at) {
     const bool first = b < best;
     const float other = fmaxf(best, b);
     const int other_at = first ? best_at : b_at;
     if (other < second) { second = other; second_at = other_at; }
-    if (s < second) { second = s; second_at = s_at; }
     if (first) { best = b; best_at = b_at; }
   }
-  __device__ __forceinline__ void take(const float (&acc)[32], int at) {
+  __device__ __forceinline__ void take(const float (&acc)[32], int at, const TieLimit& lim) {
     const float m = min32(acc);
-    if (m < low + kNearTie) {
+    if (m < lim(low)) {
+      if (lim(m) <= low) { blocks = 0; pair = false; }   // all that came before is out of reach
       low = fminf(low, m);
       float b2[16], s2[16];
 #pragma unroll
@@ -267,33 +289,193 @@ struct Nearest2 {
           b2[j] = fminf(b2[j], b2[j + o]);
         }
       }
-      merge(b2[0], at, s2[0], at);
+      ++blocks;
+      pair |= s2[0] < lim(low);
+      merge(b2[0], at);
     }
   }
 };
 
-// (kTree: merged pairwise, the shorter chain; one after the other, the fewer registers.  1 M tokens x 32
-// subspaces, encode: 961 us in a row, 916 as a tree; the update, with 128 registers full: 74.6 and 80.6.)
-template <bool kTree, int N>
-__device__ __forceinline__ void group_minima(const float (&v)[N], int grp0, float& best, int& grp) {
-  float m[N / 8];
-  int at[N / 8];
+// Squared distances of kT rows and a centroid in fp32, every sum one chain over the dims, up to |x|^2
+// where kX2 is false.
+template <bool kX2, int kT, class Row>
+__device__ __forceinline__ void distances_fp32(Row row, const float* __restrict__ c, float (&d)[kT]) {
+  const float4* cp = reinterpret_cast<const float4*>(c);
+  float xx[kT], a[kT], n = 0.f;
 #pragma unroll
-  for (int g = 0; g < N / 8; ++g) {
-    const float* w = v + 8 * g;
-    m[g] = min3(min3(w[0], w[1], w[2]), min3(w[3], w[4], w[5]), fminf(w[6], w[7]));
-    at[g] = grp0 + g;
-    if (!kTree && m[g] < best) { best = m[g]; grp = at[g]; }
-  }
-  if constexpr (kTree) {                                    // the lower group on ties
+  for (int t = 0; t < kT; ++t) xx[t] = a[t] = 0.f;
+#pragma unroll(kT == 1 ? 16 : 8)
+  for (int k = 0; k < kHeadDim / 4; ++k) {
+    const float4 y = __ldg(cp + k);
+    n = fmaf(y.x, y.x, n); n = fmaf(y.y, y.y, n); n = fmaf(y.z, y.z, n); n = fmaf(y.w, y.w, n);
 #pragma unroll
-    for (int o = 1; o < N / 8; o *= 2) {
-#pragma unroll
-      for (int g = 0; g + o < N / 8; g += 2 * o)
-        if (m[g + o] < m[g]) { m[g] = m[g + o]; at[g] = at[g + o]; }
+    for (int t = 0; t < kT; ++t) {
+      const float4 u = reinterpret_cast<const float4*>(row(t))[k];
+      a[t] = fmaf(u.x, y.x, a[t]); a[t] = fmaf(u.y, y.y, a[t]); a[t] = fmaf(u.z, y.z, a[t]); a[t] = fmaf(u.w, y.w, a[t]);
+      if constexpr (kX2) {
+        xx[t] = fmaf(u.x, u.x, xx[t]); xx[t] = fmaf(u.y, u.y, xx[t]); xx[t] = fmaf(u.z, u.z, xx[t]); xx[t] = fmaf(u.w, u.w, xx[t]);
+      }
     }
-    if (m[0] < best) { best = m[0]; grp = at[0]; }
   }
+#pragma unroll
+  for (int t = 0; t < kT; ++t) d[t] = kX2 ? (xx[t] - 2.0f * a[t]) + n : fmaf(-2.f, a[t], n);
+}
+template <bool kX2> __device__ __forceinline__ float distance_fp32(const float* x, const float* __restrict__ c) {
+  float d[1];
+  distances_fp32<kX2, 1>([&](int) { return x; }, c, d);
+  return d[0];
+}
+// the smaller of two (distance, index), the lower index on ties
+__device__ __forceinline__ void nearer(float& d, int& at, float od, int oat) {
+  if (od < d || (od == d && oat < at)) { d = od; at = oat; }
+}
+__device__ __forceinline__ void warp_nearest(float& d, int& at) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float od = __shfl_xor_sync(0xffffffffu, d, o);
+    const int oat = __shfl_xor_sync(0xffffffffu, at, o);
+    nearer(d, at, od, oat);
+  }
+}
+
+// The nearest centroid of a row among those of up to two blocks of 32, by a warp.  (A call: rare, and long
+// where it would stand.)
+template <bool kX2>
+__device__ __noinline__ int nearest_of_blocks(const float* x, const float* __restrict__ centroids, int n_list, int block0, int block1) {
+  float d = CUDART_INF_F;
+  int at = 0;
+#pragma unroll 1
+  for (int blk = block0;; blk = block1) {
+    const int j = 32 * blk + (threadIdx.x & 31);
+    if (j < n_list) nearer(d, at, distance_fp32<kX2>(x, centroids + (size_t)j * kHeadDim), j);
+    if (blk == block1) break;
+  }
+  warp_nearest(d, at);
+  return at;
+}
+// ... of kT rows (index[c], index[c + 1], .., at most n of them) among all centroids, by the threads first,
+// first + step, .. ; leaves each warp's result at found[0 .. kT).  (One row: the loads run ahead of the
+// chains; four share every centroid's load, for data where all is equally near.)
+struct Found {
+  float d;
+  int at;
+};
+template <bool kX2, int kT>
+__device__ __noinline__ void nearest_of_all(const float* rows, int stride, const uint8_t* index, int c, int n,
+                                            const float* __restrict__ centroids, int n_list, int first, int step, Found* found) {
+  const float* row[kT];
+  float d[kT];
+  int at[kT];
+#pragma unroll
+  for (int t = 0; t < kT; ++t) {
+    row[t] = rows + (int)index[min(c + t, n - 1)] * stride;
+    d[t] = CUDART_INF_F;
+    at[t] = 0;
+  }
+#pragma unroll 1
+  for (int j = first; j < n_list; j += step) {
+    float dist[kT];
+    distances_fp32<kX2, kT>([&](int t) { return row[t]; }, centroids + (size_t)j * kHeadDim, dist);
+#pragma unroll
+    for (int t = 0; t < kT; ++t) nearer(d[t], at[t], dist[t], j);
+  }
+#pragma unroll
+  for (int t = 0; t < kT; ++t) {
+    warp_nearest(d[t], at[t]);
+    if ((threadIdx.x & 31) == 0) { found[t].d = d[t]; found[t].at = at[t]; }
+  }
+}
+constexpr int kCrowd = 4;                                  // rows searched for together
+
+// ---- codewords: the smallest of every group of 8 accumulators with the group's number (at most 32 of
+// them) in the mantissa's low 5 bits, the nearest group and the second's value.  The codeword inside
+// the group is found by the caller in fp32; where the second group may hold one as near, the
+// caller searches them all.
+struct NearestGroup {
+  float best, second;
+  __device__ __forceinline__ void clear() { best = second = CUDART_INF_F; }
+  __device__ __forceinline__ int group() const { return (int)(__float_as_uint(best) & 31u); }
+  template <int N> __device__ __forceinline__ void take(const float (&v)[N], uint32_t grp0) {
+    float b[N / 8];
+#pragma unroll
+    for (int g = 0; g < N / 8; ++g) {
+      const float* w = v + 8 * g;
+      const float m = min3(min3(w[0], w[1], w[2]), min3(w[3], w[4], w[5]), fminf(w[6], w[7]));
+      b[g] = __uint_as_float((__float_as_uint(m) & ~31u) | (grp0 + g));
+    }
+#pragma unroll
+    for (int g = 0; g < N / 8; ++g) {
+      // (the larger of the two, as their sum without the smaller: the integer pipe, which does minima, is
+      // what bounds the search)
+      const float sum = best + b[g];
+      best = fminf(best, b[g]);
+      second = fminf(second, sum - best);
+    }
+  }
+};
+// Is the second group within the errors of both arithmetics of the best?  (e2 = |e|^2 of the sub-vector;
+// at most four accumulations, the group's bits the larger part: 2^-18 of each value.  Generous: a search
+// that was not needed costs less than a hundredth.)
+constexpr float kPqTieE2 = 4e-5f, kPqTieV = 1.6e-5f;
+__device__ __forceinline__ bool pq_tie(const NearestGroup& g, float e2) {
+  const float reach = fmaf(kPqTieE2 * kTcScale * kTcScale, e2, fmaf(kPqTieV, fabsf(g.best), 2.f * kTieFloor));
+  return !(g.second >= g.best + reach);
+}
+template <int DSUB> __device__ __forceinline__ void load_sub(const float* src, float (&x)[DSUB]) {
+  if constexpr (DSUB == 2) {
+    *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(src);
+  } else {
+#pragma unroll
+    for (int c4 = 0; c4 < DSUB / 4; ++c4)
+      *reinterpret_cast<float4*>(x + 4 * c4) = *reinterpret_cast<const float4*>(src + 4 * c4);
+  }
+}
+// Sub-vectors that have to be compared with all codewords: bit i of `mine` is this lane's i-th.
+// s.load(lane, i, x) reads one, s.distance(i, x, z) compares it as the caller does, s.done(i, x, z) takes
+// the nearest codeword (lower index on ties) in the lane it belongs to.  A few: one after the other, the
+// warp's lanes over the codewords; many (equal keys, all zeros): every lane its own.  All lanes call.
+// (A call of its own: inlined, it took registers from the search before it, 4 us of an update.)
+template <int DSUB, int kCodes, class S>
+__device__ __noinline__ unsigned long long settle_codewords(unsigned mine, int n_items, S s) {
+  constexpr int kAhead = kCodes < 32 ? 1 : DSUB <= 4 ? 8 : 32 / DSUB;      // codewords in flight (they may be in global memory)
+  const int lane = threadIdx.x & 31;
+  const int n_lanes = __popc(__ballot_sync(0xffffffffu, mine != 0u));
+#pragma unroll 1
+  for (int i = 0; i < n_items; ++i) {
+    const unsigned who = __ballot_sync(0xffffffffu, (mine >> i) & 1u);
+    float x[DSUB];
+    if (n_lanes > 8 && who) {
+      float d = CUDART_INF_F;
+      int at = 0;
+      s.load(lane, i, x);
+#pragma unroll 2
+      for (int z = 0; z < kCodes; ++z) {
+        const float dist = s.distance(i, x, z);
+        if (dist < d) { d = dist; at = z; }
+      }
+      if ((who >> lane) & 1u) s.done(i, x, at);
+    } else {
+#pragma unroll 1
+      for (unsigned left = who; left; left &= left - 1u) {
+        const int src = __ffs(left) - 1;
+        float d = CUDART_INF_F;
+        int at = 0;
+        s.load(src, i, x);
+#pragma unroll 1
+        for (int z0 = lane; z0 < kCodes; z0 += 32 * kAhead) {
+          float dist[kAhead];
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u) dist[u] = s.distance(i, x, z0 + 32 * u);
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u)
+            if (dist[u] < d) { d = dist[u]; at = z0 + 32 * u; }
+        }
+        warp_nearest(d, at);
+        if (lane == src) s.done(i, x, at);
+      }
+    }
+  }
+  return s.result;
 }
 
 }  // namespace

@@ -6,15 +6,16 @@
 //
 //   index_encode_kernel         128 new tokens of one (sequence, KV head) per CTA.  Both searches
 //       are contractions and run on the tensor cores with split fp16 operands (tc.cuh): tiles of 128
-//       centroids, then every warpgroup takes every fourth subspace.
-//       The codeword is decided in fp32 among the 8 of the winning group.
+//       centroids, then every warpgroup takes every fourth subspace.  What comes within the rounding of
+//       the nearest, and centres too far out for fp16, are compared in fp32: lists and codes are those of
+//       an fp32 search.  The codeword is decided in fp32 among the 8 of the winning group.
 //   index_refresh_means_kernel  groups the new tokens by list (first occurrence = leader), sums
 //       each group's value rows in token order and sets vbar_j = (n_j vbar_j + sum) / (n_j + new_j),
 //       n_j += new_j; a warp per leader.
-// What bounds the encoding: latency.  Of 102 thousand clocks per CTA the rows' first loads take 11, the
-// centroids (512 KB at 1024 lists, through registers once to be split) 46, the codes 39: short steps
-// of store, MMA, wait and search per subspace.  8 requests x 8 KV heads x 128 new tokens: 778 us with
-// fp32 FMAs and a serial grouping of the means, 75 us so.
+// What bounds the encoding: latency.  The rows' first loads, the centroids (512 KB at 1024 lists, through
+// registers once to be split), then the codes: short steps of store, MMA, wait and search per subspace.
+// 8 requests x 8 KV heads x 256 new tokens: 779 us with fp32 FMAs and a serial grouping of the means, 74
+// with the split searches alone, 80 with what fp32 decides.
 #include "attn_common.cuh"
 #include "common.cuh"
 #include "tc.cuh"
@@ -53,6 +54,30 @@ __device__ __forceinline__ long long row_offset(const Plan& pl, const int32_t* _
          (long long)kv * stride_head;
 }
 
+// |x - word|^2, one chain over the dims
+template <int DSUB> __device__ __forceinline__ float word_distance(const float (&x)[DSUB], const float* word) {
+  float w[DSUB], dist = 0.f;
+  load_sub<DSUB>(word, w);
+#pragma unroll
+  for (int t = 0; t < DSUB; ++t) dist = fmaf(x[t] - w[t], x[t] - w[t], dist);
+  return dist;
+}
+// (see settle_codewords; item i is subspace wg + 4 i)
+template <int DSUB> struct UpdateSettle {
+  const float* rows;                                        // residuals of the warp's tokens, first subspace
+  const float* words;                                       // its codebook
+  size_t item_words;                                        // floats to the next item's
+  uint8_t* code;                                            // this lane's
+  unsigned long long result;
+  __device__ __forceinline__ void load(int lane, int i, float (&x)[DSUB]) const {
+    load_sub<DSUB>(rows + lane * kUStride + i * kUpdGroups * DSUB, x);
+  }
+  __device__ __forceinline__ float distance(int i, const float (&x)[DSUB], int z) const {
+    return word_distance<DSUB>(x, words + i * item_words + z * DSUB);
+  }
+  __device__ __forceinline__ void done(int i, const float (&)[DSUB], int z) { code[i * kUpdGroups] = (uint8_t)z; }
+};
+
 template <typename T, int DSUB>
 __global__ void __launch_bounds__(kUpdThreads, 1)
 index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, long long stride_token,
@@ -64,9 +89,14 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
   extern __shared__ __align__(128) unsigned char s_dyn[];
   unsigned char* s_a = s_dyn;
   unsigned char* s_b = s_a + kUpdA;
-  __shared__ float s_best[2][kUpdGroups][kUpdTok];               // the groups' two nearest
+  __shared__ float s_best[2][kUpdGroups][kUpdTok];               // the groups' two nearest blocks
   __shared__ uint16_t s_at[2][kUpdGroups][kUpdTok];
-  __shared__ uint16_t s_near[2][kUpdTok];                        // the two that tie, or the nearest twice
+  __shared__ uint8_t s_blocks[kUpdGroups][kUpdTok];              // how many within reach, 128: a pair
+  __shared__ uint16_t s_near[kUpdTok], s_tie[2][kUpdTok];        // the nearest; blocks to search in fp32, or none
+  __shared__ float s_x2[kUpdTok];                                // |u|^2
+  __shared__ uint8_t s_crowd[kUpdTok];                           // tokens that fp32 searches for
+  __shared__ int s_n_crowd, s_wild, s_wild_words[kUpdGroups];
+  __shared__ Found s_found[kUpdWarps][kCrowd];
   __shared__ __align__(16) uint8_t s_code[kUpdTok][64];
   __shared__ uint32_t s_tmem;
   __shared__ __align__(8) uint64_t s_bar[2 + kUpdGroups];        // centroid tiles, codeword tiles
@@ -87,6 +117,8 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
 
   if (warp == 0) tmem_alloc(&s_tmem, 512);
   if (tid < 2 + kUpdGroups) mbar_init(&s_bar[tid], 1);
+  if (tid < kUpdGroups) s_wild_words[tid] = -1;
+  if (tid == 0) { s_n_crowd = 0; s_wild = 0; }
   if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 
   // ---- norms and directions: a warp per token, a lane holds 4 of the 128 dims
@@ -119,6 +151,8 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
       inv[r] = nr > 0.f ? 1.f / nr : 0.f;
       direction(r, x);
       *reinterpret_cast<float4*>(s_u + t * kUStride + 4 * lane) = make_float4(x[0], x[1], x[2], x[3]);
+      // (|u|^2 = 1; less sure where the squares underflow.  0 and not-a-number stay themselves)
+      if (lane == 0) s_x2[t] = nr > 1e-18f ? 1.f : nr > 0.f ? (float)kHeadDim : nr;
       if (lane == 0 && ok(t)) key_norms[ukv * pl.N_max + p0 + t] = nr;
     }
   }
@@ -175,10 +209,12 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
     n2 += __shfl_xor_sync(0xffffffffu, n2, 8);
     n2 += __shfl_xor_sync(0xffffffffu, n2, 16);
     if (bc == 0) *reinterpret_cast<uint4*>(dst + (32 * kUpdCen + br) * 16) = coarse_ext_centre(n2, c0 + br < pl.n_list);
+    if (!(n2 < kTieRange)) s_wild = 1;                      // (the caller's centroids: any numbers)
     if (bc == 1) *reinterpret_cast<uint4*>(dst + (33 * kUpdCen + br) * 16) = make_uint4(0u, 0u, 0u, 0u);
   };
   const uint32_t my_lanes = (uint32_t)(wq * 32) << 16;      // this warp's TMEM lanes
   const int n_tiles = (pl.n_list + kUpdCen - 1) / kUpdCen;
+  const TieLimit lim(s_x2[row]);
   Nearest2 nn;
   nn.clear();
   bool late = false;
@@ -202,52 +238,70 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
     tc_fence_after();
     float acc[32];
     tmem_ld32(tmem + (i & 1) * kUpdCen + 32 * wg + my_lanes, acc);
-    nn.take(acc, i * (kUpdCen / 32) + wg);
+    nn.take(acc, i * (kUpdCen / 32) + wg, lim);
   }
   s_best[0][wg][row] = nn.best;
   s_best[1][wg][row] = nn.second;
   s_at[0][wg][row] = (uint16_t)nn.best_at;
   s_at[1][wg][row] = (uint16_t)nn.second_at;
+  s_blocks[wg][row] = (uint8_t)(min(nn.blocks, 3) | (nn.pair ? 128 : 0));
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   if (wg == 0) {
 #pragma unroll
-    for (int g = 1; g < kUpdGroups; ++g) nn.merge(s_best[0][g][row], s_at[0][g][row], s_best[1][g][row], s_at[1][g][row]);
-    const int near = nn.near(), next = nn.next();
-    s_near[0][row] = (uint16_t)min(near, pl.n_list - 1);
-    s_near[1][row] = (uint16_t)(nn.tie() && max(near, next) < pl.n_list ? next : min(near, pl.n_list - 1));
+    for (int g = 1; g < kUpdGroups; ++g) {
+      const float b = s_best[0][g][row];
+      if (lim(b) <= nn.best) { nn.blocks = 0; nn.pair = false; }      // (as within a group)
+      if (b < lim(nn.best)) {
+        nn.blocks += s_blocks[g][row] & 127;
+        nn.pair |= s_blocks[g][row] >> 7;
+      }
+      nn.merge(b, s_at[0][g][row]);
+      nn.merge(s_best[1][g][row], s_at[1][g][row]);
+    }
+    const bool crowd = nn.crowded() || s_wild;
+    s_near[row] = (uint16_t)min(nn.near(), pl.n_list - 1);
+    s_tie[0][row] = (uint16_t)(nn.tie(lim) && !crowd ? nn.best_at : 0xffff);
+    s_tie[1][row] = (uint16_t)(nn.second_near(lim) ? nn.second_at : nn.best_at);
+    if (ok(row) && crowd) s_crowd[atomicAdd(&s_n_crowd, 1)] = (uint8_t)row;
   }
   __syncthreads();
-  // ---- ties in fp32, every sum one chain over the dims (a few tokens in a thousand); a warp per token
+  // ---- what fp32 decides: a few tokens in a hundred between the centroids of one or two blocks, by the
+  // token's warp; hardly any over all centroids, by the whole CTA
+  float* s_u = reinterpret_cast<float*>(s_dyn);             // (the tiles are done)
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    float x[4];
+    direction(r, x);
+    *reinterpret_cast<float4*>(s_u + (r * kUpdWarps + warp) * kUStride + 4 * lane) = make_float4(x[0], x[1], x[2], x[3]);
+  }
+  const int n_crowd = s_n_crowd;
+  if (n_crowd != 0) __syncthreads(); else __syncwarp();     // (uniform)
+  const int n_search = n_crowd > kCrowd ? kCrowd : 1;       // for together
+#pragma unroll 1
+  for (int c = 0; c < n_crowd; c += n_search) {
+    if (n_search == 1) nearest_of_all<false, 1>(s_u, kUStride, s_crowd, c, n_crowd, cbase, pl.n_list, tid, kUpdThreads, s_found[warp]);
+    else nearest_of_all<false, kCrowd>(s_u, kUStride, s_crowd, c, n_crowd, cbase, pl.n_list, tid, kUpdThreads, s_found[warp]);
+    __syncthreads();
+    if (tid < n_search && c + tid < n_crowd) {
+      Found f = s_found[0][tid];
+      for (int w = 1; w < kUpdWarps; ++w) nearer(f.d, f.at, s_found[w][tid].d, s_found[w][tid].at);
+      s_near[s_crowd[c + tid]] = (uint16_t)f.at;
+    }
+    __syncthreads();
+  }
   int list[kPer];
 #pragma unroll
   for (int r = 0; r < kPer; ++r) {
     const int t = r * kUpdWarps + warp;
-    list[r] = s_near[0][t];
-    const int alt = s_near[1][t];
-    if (alt != list[r]) {
-      const int lo = min(list[r], alt), hi = max(list[r], alt);
-      const float4* c0 = reinterpret_cast<const float4*>(cbase + (size_t)lo * kHeadDim);
-      const float4* c1 = reinterpret_cast<const float4*>(cbase + (size_t)hi * kHeadDim);
-      float x[4], a0 = 0.f, a1 = 0.f, n0 = 0.f, n1 = 0.f;
-      direction(r, x);
-#pragma unroll 4
-      for (int k = 0; k < kHeadDim / 4; ++k) {
-        const float4 y = __ldg(c0 + k), z = __ldg(c1 + k);
-        const float u0 = __shfl_sync(0xffffffffu, x[0], k), u1 = __shfl_sync(0xffffffffu, x[1], k);
-        const float u2 = __shfl_sync(0xffffffffu, x[2], k), u3 = __shfl_sync(0xffffffffu, x[3], k);
-        a0 = fmaf(u0, y.x, a0); a0 = fmaf(u1, y.y, a0); a0 = fmaf(u2, y.z, a0); a0 = fmaf(u3, y.w, a0);
-        n0 = fmaf(y.x, y.x, n0); n0 = fmaf(y.y, y.y, n0); n0 = fmaf(y.z, y.z, n0); n0 = fmaf(y.w, y.w, n0);
-        a1 = fmaf(u0, z.x, a1); a1 = fmaf(u1, z.y, a1); a1 = fmaf(u2, z.z, a1); a1 = fmaf(u3, z.w, a1);
-        n1 = fmaf(z.x, z.x, n1); n1 = fmaf(z.y, z.y, n1); n1 = fmaf(z.z, z.z, n1); n1 = fmaf(z.w, z.w, n1);
-      }
-      list[r] = fmaf(-2.f, a1, n1) < fmaf(-2.f, a0, n0) ? hi : lo;
-    }
+    list[r] = s_near[t];
+    if (s_tie[0][t] != 0xffff && ok(t))                     // (warp-uniform)
+      list[r] = nearest_of_blocks<false>(s_u + t * kUStride, cbase, pl.n_list, s_tie[0][t], s_tie[1][t]);
     if (lane == 0 && ok(t)) list_ids[ukv * pl.N_max + p0 + t] = (uint16_t)list[r];
   }
+  __syncthreads();                                          // (the directions have been read)
   // ---- residuals
-  float* s_u = reinterpret_cast<float*>(s_dyn);
   {
     float4 c[kPer];
 #pragma unroll
@@ -273,34 +327,26 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
   // the subspace's codewords in fp32 for the final decision, where they fit
   float* s_word = reinterpret_cast<float*>(pb + Tile::kChunks * 2048);
   const bool staged = 2 * Tile::kChunks * 2048 + pl.n_code * DSUB * 4 <= kUpdPq;
-  auto load_sub = [](const float* src, float (&x)[DSUB]) {
-    if constexpr (DSUB == 2) {
-      *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(src);
-    } else {
-#pragma unroll
-      for (int c4 = 0; c4 < DSUB / 4; ++c4)
-        *reinterpret_cast<float4*>(x + 4 * c4) = *reinterpret_cast<const float4*>(src + 4 * c4);
-    }
-  };
   const int words = min(kUpdWords, pl.n_code);
   float p[DSUB];                                            // this thread's codeword, one tile ahead
   auto fetch_word = [&](int m, int z0) {
-    if (row < words && m < pl.M) load_sub(codebooks + ((ukv * pl.M + m) * (size_t)pl.n_code + z0 + row) * DSUB, p);
+    if (row < words && m < pl.M) load_sub<DSUB>(codebooks + ((ukv * pl.M + m) * (size_t)pl.n_code + z0 + row) * DSUB, p);
   };
+      unsigned ties = 0u;                                       // bit i: this token's subspace wg + 4 i
   fetch_word(wg, 0);
   for (int m = wg; m < pl.M; m += kUpdGroups) {
     const float* cb = codebooks + (ukv * pl.M + m) * (size_t)pl.n_code * DSUB;
     float e[DSUB];
-    load_sub(s_u + row * kUStride + m * DSUB, e);
+    load_sub<DSUB>(s_u + row * kUStride + m * DSUB, e);
     uint4 ch[Tile::kChunks];
     Tile::token_row(e, ch);
 #pragma unroll
     for (int i = 0; i < Tile::kChunks; ++i) *reinterpret_cast<uint4*>(pa + (i * 128 + row) * 16) = ch[i];
-    float bd = CUDART_INF_F;
-    int grp = 0;
+    NearestGroup ng;
+    ng.clear();
     for (int z0 = 0; z0 < pl.n_code; z0 += kUpdWords) {
       if (row < words) {
-        Tile::code_row(p, ch);
+        if (!(Tile::code_row(p, ch) < kTieRange)) s_wild_words[wg] = m;      // (the caller's codebook: any numbers)
         if (staged) {
 #pragma unroll
           for (int t = 0; t < DSUB; ++t) s_word[(z0 + row) * DSUB + t] = p[t];
@@ -324,38 +370,43 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
       if (pl.n_code == 16) {
         float acc[16];
         tmem_ld16(my_tmem, acc);
-        group_minima<false>(acc, 0, bd, grp);
+        ng.take(acc, 0u);
       } else {
 #pragma unroll
         for (int c = 0; c < kUpdWords; c += 32) {
           float acc[32];
           tmem_ld32(my_tmem + c, acc);
-          group_minima<false>(acc, (z0 + c) / 8, bd, grp);
+          ng.take(acc, (uint32_t)(z0 + c) / 8u);
         }
       }
     }
     // the winning group's codewords in fp32, first minimum.  The lanes start at different codewords:
     // at 16 bytes a codeword the eight lanes of an access then hit eight different bank groups
-    float dm = CUDART_INF_F;
+    float dm = CUDART_INF_F, e2 = 0.f;
     int bz = 0;
     auto decide = [&](const float* words_of_m) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const int z = 8 * grp + ((i + lane) & 7);
-        float w[DSUB];
-        load_sub(words_of_m + z * DSUB, w);
-        float dist = 0.f;
-#pragma unroll
-        for (int dd = 0; dd < DSUB; ++dd) {
-          const float x = e[dd] - w[dd];
-          dist = fmaf(x, x, dist);
-        }
+        const int z = 8 * ng.group() + ((i + lane) & 7);
+        const float dist = word_distance<DSUB>(e, words_of_m + z * DSUB);
         if (dist < dm || (dist == dm && z < bz)) { dm = dist; bz = z; }
       }
     };
     if (staged) decide(s_word); else decide(cb);
+#pragma unroll
+    for (int t = 0; t < DSUB; ++t) e2 = fmaf(e[t], e[t], e2);
+    if (pq_tie(ng, e2) || !(e2 < kTieRange) || s_wild_words[wg] == m) ties |= 1u << (m / kUpdGroups);
     group_sync(1 + wg);                              // (the codewords are overwritten next)
     s_code[row][m] = (uint8_t)bz;
+  }
+  // where another group may hold a codeword as near: all of them
+  if (__any_sync(0xffffffffu, ok(row) && ties != 0u)) {
+    const UpdateSettle<DSUB> st = {s_u + (row & ~31) * kUStride + wg * DSUB,
+                                   codebooks + (ukv * pl.M + wg) * (size_t)pl.n_code * DSUB,
+                                   (size_t)kUpdGroups * pl.n_code * DSUB, s_code[row] + wg, 0ull};
+    const unsigned mine = ok(row) ? ties : 0u;
+    if (pl.n_code == 16) settle_codewords<DSUB, 16>(mine, pl.M / kUpdGroups, st);
+    else settle_codewords<DSUB, 256>(mine, pl.M / kUpdGroups, st);
   }
   tc_fence_before();
   __syncthreads();

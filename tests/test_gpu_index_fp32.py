@@ -1,0 +1,156 @@
+"""Lists and codes of the index build and update are those of a plain fp32 search over all centres
+(-m gpu), lower index on ties, whatever arithmetic the search itself runs in: with centres that are
+close to one another, equal, far outside the unit ball, not numbers, or residuals near zero.
+
+Exact: the fp32 chains (one per sum, over the dims in order, fused multiply-adds) are formed here step
+by step in float64 and rounded after each."""
+import pytest
+import torch
+
+from paper_2609_33746_b200 import pqhsa
+
+pytestmark = pytest.mark.gpu
+
+
+def fma(a, b, c):
+    return (a.double() * b.double() + c.double()).float()
+
+
+def chain(terms, shape):
+    acc = torch.zeros(shape, device="cuda")
+    for a, b in terms:
+        acc = fma(a, b, acc)
+    return acc
+
+
+def first_argmin(d):                                     # not a number: never the nearest; none: 0
+    d = torch.where(d.isnan(), float("inf"), d)
+    low = d.min(dim=-1, keepdim=True).values
+    return torch.where(d == low, 1, 0).argmax(dim=-1) * (low[..., 0] < float("inf"))
+
+
+def nearest_lists(u, c, with_x2):
+    n, L = u.shape[0], c.shape[0]
+    dot = chain(((u[:, None, k], c[None, :, k]) for k in range(128)), (n, L))
+    cc = chain(((c[:, k], c[:, k]) for k in range(128)), (L,))
+    if not with_x2:
+        return first_argmin(fma(torch.full_like(dot, -2.0), dot, cc.expand(n, L)))
+    xx = chain(((u[:, k], u[:, k]) for k in range(128)), (n,))
+    return first_argmin(fma(torch.full_like(dot, -2.0), dot, xx[:, None].expand(n, L)) + cc)
+
+
+def nearest_codes(e, books, expanded):
+    n, (m, z, ds) = e.shape[0], books.shape
+    out = []
+    for j in range(m):
+        x, p = e[:, None, j * ds:(j + 1) * ds], books[None, j]
+        if expanded:
+            dot = chain(((x[..., t], p[..., t]) for t in range(ds)), (n, z))
+            xx = chain(((x[..., t], x[..., t]) for t in range(ds)), (n, 1))
+            pp = chain(((p[..., t], p[..., t]) for t in range(ds)), (1, z))
+            d = fma(torch.full_like(dot, -2.0), dot, xx.expand(n, z)) + pp
+        else:
+            d = chain(((x[..., t] - p[..., t], x[..., t] - p[..., t]) for t in range(ds)), (n, z))
+        out.append(first_argmin(d))
+    return torch.stack(out, dim=1)
+
+
+def keys_of(kind, n, g):
+    k = torch.randn((n, 128), generator=g, device="cuda")
+    if kind == "mean":                                   # a large common part: centroids close to one another
+        k = 5 * torch.randn((1, 128), generator=g, device="cuda") + k
+    elif kind == "tight":                                # residuals near zero
+        k = torch.randn((50, 128), generator=g, device="cuda")[torch.randint(0, 50, (n,), generator=g, device="cuda")]
+        k = k + 2e-3 * torch.randn((n, 128), generator=g, device="cuda")
+    elif kind == "repeats":                              # equal keys: equal seeds, equal centroids
+        k = k[torch.randint(0, 97, (n,), generator=g, device="cuda")]
+    elif kind == "zeros":
+        k[::3] = 0
+    return k.bfloat16()
+
+
+class Index:
+    def __init__(self, kind, n, n_list, m, ncode, seed):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        self.n, self.n_list, self.m, self.ncode = n, n_list, m, ncode
+        self.n_max = nm = (n + 15) // 16 * 16
+        self.k = torch.zeros((nm, 128), dtype=torch.bfloat16, device="cuda")
+        self.k[:n] = keys_of(kind, n, g)
+        self.v = torch.randn((nm, 128), generator=g, device="cuda").bfloat16()
+        self.table = torch.arange(nm // 16, dtype=torch.int32, device="cuda").view(1, -1)
+        self.params = pqhsa.make_params(batch=1, n_q_heads=1, n_kv_heads=1, n_list=n_list, pq_m=m, pq_ncode=ncode,
+                                        max_seq_len=nm, max_pages_per_seq=nm // 16, budget_ppm=10000, dtype="bf16")
+        self.kv = pqhsa.make_paged_kv(self.k, self.v, 16 * 128, 128, 128, self.table)
+        self.centroids = torch.zeros((n_list, 128), device="cuda")
+        self.books = torch.zeros((m, ncode, 128 // m), device="cuda")
+        self.seq = torch.tensor([n], dtype=torch.int32, device="cuda")
+        self.seeds = [torch.randint(0, n, (c,), generator=g, device="cuda").int() for c in (n_list, ncode)]
+        self.clear()
+
+    def clear(self):
+        z = lambda *s, dtype=torch.float32: torch.zeros(s, dtype=dtype, device="cuda")
+        self.codes = z(self.n_max, self.m if self.ncode == 256 else self.m // 2, dtype=torch.uint8)
+        self.ids, self.norms = z(self.n_max, dtype=torch.int16), z(self.n_max)
+        self.vmeans, self.counts = z(self.n_list, 128), z(self.n_list, dtype=torch.int32)
+
+    def build(self, coarse_iters, pq_iters):
+        ws = torch.empty(pqhsa.index_build_workspace_bytes(self.params), dtype=torch.uint8, device="cuda")
+        pqhsa.index_build(self.params, self.kv, self.seq, *self.seeds, coarse_iters, pq_iters, self.centroids,
+                          self.books, self.codes, self.ids, self.norms, self.vmeans, self.counts, ws)
+
+    def update(self, n_new):
+        self.clear()
+        rw = pqhsa.make_index_rw(self.centroids, self.books, self.codes, self.ids, self.norms, self.vmeans, self.counts)
+        first = torch.zeros(1, dtype=torch.int32, device="cuda")
+        pqhsa.index_update(self.params, rw, self.kv, first, torch.tensor([n_new], dtype=torch.int32, device="cuda"), n_new)
+
+    def check(self, n, build):
+        r = self.norms[:n]
+        u = self.k[:n].float() * torch.where(r > 0, 1.0 / r, 0.0)[:, None]
+        a = self.ids[:n].long() & 0xffff
+        assert torch.equal(a, nearest_lists(u, self.centroids, build)), "lists"
+        z = self.codes[:n].long()
+        if self.ncode == 16:
+            z = torch.stack((z & 15, z >> 4), dim=2).view(n, self.m)
+        assert torch.equal(z, nearest_codes(u - self.centroids[a], self.books, build)), "codes"
+
+
+SHAPES = [(193, 32, 256), (600, 16, 256), (40, 8, 16), (129, 64, 256), (1000, 8, 256), (65, 16, 16)]
+
+
+@pytest.mark.parametrize("n_list,m,ncode", SHAPES)
+@pytest.mark.parametrize("kind", ["normal", "mean", "tight", "repeats", "zeros"])
+def test_lists_and_codes_are_those_of_an_fp32_search(kind, n_list, m, ncode):
+    ix = Index(kind, 3001, n_list, m, ncode, seed=n_list + m)
+    ix.build(1, 1)
+    ix.check(ix.n, build=True)
+    ix.update(700)
+    ix.check(700, build=False)
+
+
+@pytest.mark.parametrize("n_list,m,ncode", SHAPES[:3])
+@pytest.mark.parametrize("centroids,books", [(1e-3, 1.0), (20.0, 1.0), (300.0, 1.0), (1.0, 1e-3), (1.0, 20.0), (1.0, 3000.0)])
+def test_update_takes_any_centroids_and_codebooks(centroids, books, n_list, m, ncode):
+    ix = Index("normal", 1500, n_list, m, ncode, seed=3)
+    ix.build(1, 1)
+    ix.centroids *= centroids
+    ix.books *= books
+    ix.update(300)
+    ix.check(300, build=False)
+    ix.centroids[5, 7], ix.centroids[17, 3] = float("nan"), float("inf")
+    ix.books[:, 3, 0], ix.books[:, 9, 1] = float("nan"), -float("inf")
+    ix.update(300)
+    ix.check(300, build=False)
+
+
+def test_the_lowest_of_equal_centroids():
+    ix = Index("normal", 512, 193, 32, 256, seed=9)
+    for token, columns in ((0, (3, 7, 9)), (1, (40, 75, 130)), (2, (20, 21, 22, 150)), (3, (190, 191, 192))):
+        ix.seeds[0][list(columns)] = token               # in one block of columns and across blocks
+    keep = torch.ones(193, dtype=torch.bool, device="cuda")
+    keep[[3, 7, 9, 40, 75, 130, 20, 21, 22, 150, 190, 191, 192]] = False
+    ix.seeds[0][keep & (ix.seeds[0] < 4)] = 100
+    ix.build(0, 0)
+    assert ix.ids[:4].tolist() == [3, 40, 20, 190]
+    ix.update(4)
+    assert ix.ids[:4].tolist() == [3, 40, 20, 190]
