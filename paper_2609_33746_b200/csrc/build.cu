@@ -602,10 +602,14 @@ build_reseed_kernel(Plan pl, const float* __restrict__ U, float* __restrict__ dm
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (od > bd || (od == bd && oi < bi)) { bd = od; bi = oi; }
       }
-      if (tid == 0) { s_pick = bi; d[bi] = -CUDART_INF_F; }      // taken: not picked again
+      if (tid == 0) {
+        s_pick = bi;
+        if (bi < n) d[bi] = -CUDART_INF_F;                       // taken: not picked again
+      }
     }
     __syncthreads();
     const int pick = s_pick;
+    if (pick >= n) break;                                        // (uniform; no distance is a number)
     if (tid < kD) centroids[((size_t)unit * pl.n_list + j) * kD + tid] = U[((size_t)unit * pl.N_max + pick) * kD + tid];
     ++j;
     __syncthreads();

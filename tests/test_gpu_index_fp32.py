@@ -154,3 +154,13 @@ def test_the_lowest_of_equal_centroids():
     assert ix.ids[:4].tolist() == [3, 40, 20, 190]
     ix.update(4)
     assert ix.ids[:4].tolist() == [3, 40, 20, 190]
+
+
+@pytest.mark.parametrize("n,n_list", [(500, 40), (1025, 256), (40, 64)])
+def test_a_cache_without_a_number(n, n_list):
+    """Every key is NaN: no distance is a number, and there are empty lists to re-seed."""
+    ix = Index("normal", n, n_list, 16, 256, seed=4)
+    ix.k[:n] = float("nan")
+    ix.build(2, 1)
+    assert bool((ix.ids[:n] == 0).all()) and bool((ix.codes[:n] == 0).all()) and bool(ix.norms[:n].isnan().all())
+    assert ix.counts[0] == n and ix.counts.sum() == n
