@@ -686,6 +686,7 @@ template <int DSUB, int NC> struct PqPlan {
 constexpr int kPqThreads = 512, kPqStep = 512;               // tokens per CTA and step
 constexpr int kFoldSteps = 3;                                // 1536 tokens: 2^21 * 1536 < 2^32, 2^20 * 1536 < 2^31
 constexpr int kLimbBits = 21;
+constexpr float kLimbRange = 7.f;                            // |e|^2 below it: 2^19 |e_t| * 1536 < 2^31
 constexpr int kPqCols = 128;                                 // codewords per MMA step
 // x * kFixDir to the nearest integer as hi * 2^21 + lo, |lo| <= 2^20, for |x| < 8: rounded by the adder
 // (1.5 * 2^23 in, its bits out), the conversion instruction being an eighth as fast
@@ -716,6 +717,7 @@ template <int DSUB, int NC, bool kTrain> struct PqSettle {
   int last;                                                 // last of them inside the range
   const float* s_word;
   uint32_t* s_limb;
+  long long* s_sum;
   unsigned long long result;                                // codes of this lane's token
   __device__ __forceinline__ void load(int lane, int mm, float (&x)[DSUB]) const {
     load_sub<DSUB>(rows + (long long)min(lane, last) * kD + mm * DSUB, x);
@@ -729,7 +731,17 @@ template <int DSUB, int NC, bool kTrain> struct PqSettle {
   }
   __device__ __forceinline__ void done(int mm, const float (&x)[DSUB], int z) {
     if constexpr (kTrain) {
-      add_member<DSUB, NC>(s_limb, mm, x, (uint32_t)z);
+      float x2 = 0.f;
+#pragma unroll
+      for (int t = 0; t < DSUB; ++t) x2 = fmaf(x[t], x[t], x2);
+      if (x2 < kLimbRange) {
+        add_member<DSUB, NC>(s_limb, mm, x, (uint32_t)z);
+      } else {                                              // (not a number: as the conversion has it)
+#pragma unroll
+        for (int t = 0; t < DSUB; ++t)
+          atomicAdd(reinterpret_cast<unsigned long long*>(s_sum + (mm * DSUB + t) * NC + z), (unsigned long long)__float2ll_rn(x[t] * kFixDir));
+        atomicAdd(s_limb + (mm * (2 * DSUB + 1) + 2 * DSUB) * NC + z, 1u);
+      }
     } else {
       constexpr int kBits = PqPlan<DSUB, NC>::kBits;
       result = (result & ~((unsigned long long)(NC - 1) << (mm * kBits))) | ((unsigned long long)z << (mm * kBits));
@@ -903,7 +915,9 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
       for (int q = 0; q < 8; ++q) above = __funnelshift_l(__float_as_uint(dm - dist[q]), above, 1);
       const uint32_t equal = ~above << 24;                  // (not a number: all)
       const uint32_t bz = (at ^ ((uint32_t)__clz(equal) * kRow)) / kRow;
-      const bool tie = pq_tie(ng, en) || (equal & (equal - 1u)) != 0u;      // (equal distances: the lower index)
+      // (equal distances: the lower index; beyond the range of limbs and fp16 terms, as next to a centroid
+      // with a member that is not a number: see PqSettle)
+      const bool tie = pq_tie(ng, en) || (equal & (equal - 1u)) != 0u || !(en < kLimbRange);
       if (tie) ties |= 1u << mm;
       if constexpr (kTrain) {
         if (real && !tie) add_member<DSUB, NC>(s_limb, mm, e, bz);
@@ -913,7 +927,7 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
     }
     // where another group may hold a codeword as near: all of them
     if (__any_sync(0xffffffffu, real && ties != 0u)) {
-      const PqSettle<DSUB, NC, kTrain> st = {E + (ukv * pl.N_max + i - lane) * (size_t)kD + m0 * DSUB, end - 1 - (i - lane), s_word, s_limb, code};
+      const PqSettle<DSUB, NC, kTrain> st = {E + (ukv * pl.N_max + i - lane) * (size_t)kD + m0 * DSUB, end - 1 - (i - lane), s_word, s_limb, s_sum, code};
       code = settle_codewords<DSUB, NC>(real ? ties : 0u, mg, st);
     }
     if constexpr (!kTrain) {

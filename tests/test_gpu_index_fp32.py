@@ -66,6 +66,9 @@ def keys_of(kind, n, g):
         k = k[torch.randint(0, 97, (n,), generator=g, device="cuda")]
     elif kind == "zeros":
         k[::3] = 0
+    elif kind == "nan":                                  # (list 0, and its centroid is no direction any more)
+        k[5::501] = float("nan")
+        k[11::777, 3] = float("inf")
     return k.bfloat16()
 
 
@@ -119,7 +122,7 @@ SHAPES = [(193, 32, 256), (600, 16, 256), (40, 8, 16), (129, 64, 256), (1000, 8,
 
 
 @pytest.mark.parametrize("n_list,m,ncode", SHAPES)
-@pytest.mark.parametrize("kind", ["normal", "mean", "tight", "repeats", "zeros"])
+@pytest.mark.parametrize("kind", ["normal", "mean", "tight", "repeats", "zeros", "nan"])
 def test_lists_and_codes_are_those_of_an_fp32_search(kind, n_list, m, ncode):
     ix = Index(kind, 3001, n_list, m, ncode, seed=n_list + m)
     ix.build(1, 1)
@@ -164,3 +167,29 @@ def test_a_cache_without_a_number(n, n_list):
     ix.build(2, 1)
     assert bool((ix.ids[:n] == 0).all()) and bool((ix.codes[:n] == 0).all()) and bool(ix.norms[:n].isnan().all())
     assert ix.counts[0] == n and ix.counts.sum() == n
+
+
+@pytest.mark.parametrize("n_nan", [2, 3])
+@pytest.mark.parametrize("m,ncode", [(32, 256), (64, 256), (16, 256), (8, 16)])
+def test_codewords_are_the_fixed_point_means_of_their_members(m, ncode, n_nan):
+    """One training pass from known codewords.  A component that is not a number enters the 64-bit sums
+    as the conversion to integers has it (-2^63), and no other codeword changes."""
+    n, n_list, ds = 1700, 40, 128 // m
+    ix = Index("normal", n, n_list, m, ncode, seed=m)
+    ix.k[[1600, 77, 1699][:n_nan]] = float("nan")
+    ix.seeds = [torch.arange(100, 100 + n_list, device="cuda").int(), torch.arange(200, 200 + ncode, device="cuda").int()]
+    ix.build(0, 0)
+    r = ix.norms[:n]
+    e = ix.k[:n].float() * torch.where(r > 0, 1.0 / r, 0.0)[:, None] - ix.centroids[ix.ids[:n].long() & 0xffff]
+    z = ix.codes[:n].long()
+    if ncode == 16:
+        z = torch.stack((z & 15, z >> 4), dim=2).view(n, m)
+    before = ix.books.clone()
+    ix.build(0, 1)
+    fixed = torch.round((e * 2.0 ** 40).double()).nan_to_num(0).long()
+    fixed = torch.where(e.isnan(), torch.iinfo(torch.int64).min, fixed).view(n, m, ds)
+    for j in range(m):
+        sums = torch.zeros((ncode, ds), dtype=torch.int64, device="cuda").index_add_(0, z[:, j], fixed[:, j])
+        count = torch.bincount(z[:, j], minlength=ncode)
+        mean = (sums.double() / 2.0 ** 40 / count.clamp(min=1)[:, None]).float()
+        assert torch.equal(ix.books[j], torch.where(count[:, None] > 0, mean, before[j])), j
