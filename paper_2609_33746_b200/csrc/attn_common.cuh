@@ -33,14 +33,29 @@ template <> struct Unpack<__half> {
   static __device__ __forceinline__ __half pack(float v) { return __float2half_rn(v); }
 };
 
-// Four consecutive cache elements (rows are 16-byte aligned: one 8-byte load).
-template <typename T> __device__ __forceinline__ void load4(const T* p, float (&x)[4]) {
-  const uint2 w = __ldg(reinterpret_cast<const uint2*>(p));
+// Four consecutive cache elements: as they lie there, and as fp32.  Build and update take a cache that
+// starts at any element (rows are multiples of 8 apart, so all are alike): kWhole, one 8-byte load.
+template <bool kWhole, typename T> __device__ __forceinline__ uint2 load_four(const T* p) {
+  if constexpr (kWhole) {
+    return __ldg(reinterpret_cast<const uint2*>(p));
+  } else {
+    const unsigned short* h = reinterpret_cast<const unsigned short*>(p);
+    return make_uint2((uint32_t)__ldg(h) | ((uint32_t)__ldg(h + 1) << 16), (uint32_t)__ldg(h + 2) | ((uint32_t)__ldg(h + 3) << 16));
+  }
+}
+template <typename T> __device__ __forceinline__ bool whole_rows(const T* cache) {
+  return (reinterpret_cast<uintptr_t>(cache) & 7u) == 0;
+}
+template <typename T> __device__ __forceinline__ uint2 load_four(const T* p) {
+  return whole_rows(p) ? load_four<true>(p) : load_four<false>(p);
+}
+template <typename T> __device__ __forceinline__ void to_fp32(const uint2& w, float (&x)[4]) {
   float f[8];
   Unpack<T>::run(make_uint4(w.x, w.y, 0u, 0u), f);
 #pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = f[i];
 }
+template <typename T> __device__ __forceinline__ void load4(const T* p, float (&x)[4]) { to_fp32<T>(load_four(p), x); }
 
 // Online-softmax state of a lane group: running max m (log2 units), normaliser Z and the 16
 // output dims the lane owns.

@@ -781,7 +781,8 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
   const float* cb = codebooks + (ukv * pl.M + m0) * (size_t)nc * DSUB;
   for (int w = tid; w < words; w += kPqThreads) {
     float p[DSUB];
-    load_sub<DSUB>(cb + (size_t)w * DSUB, p);
+#pragma unroll
+    for (int t = 0; t < DSUB; ++t) p[t] = __ldg(cb + (size_t)w * DSUB + t);      // (the caller's: aligned to an element)
     uint4 ch[Tile::kChunks];
     Tile::code_row(p, ch);
     const int mm = w / nc, z = w - mm * nc;
@@ -933,7 +934,10 @@ build_pq_assign_kernel(Plan pl, const float* __restrict__ E, const float* __rest
     if constexpr (!kTrain) {
       if (real) {
         uint8_t* dst = codes_out + (ukv * pl.N_max + i) * pl.code_bytes + m0 * P::kBits / 8;
-        if constexpr (P::kBytes == 8) *reinterpret_cast<unsigned long long*>(dst) = code;
+        if ((reinterpret_cast<uintptr_t>(dst) & (P::kBytes - 1)) != 0) {      // (the caller's array starts anywhere)
+#pragma unroll
+          for (int t = 0; t < P::kBytes; ++t) dst[t] = (uint8_t)(code >> (8 * t));
+        } else if constexpr (P::kBytes == 8) *reinterpret_cast<unsigned long long*>(dst) = code;
         else if constexpr (P::kBytes == 4) *reinterpret_cast<uint32_t*>(dst) = (uint32_t)code;
         else if constexpr (P::kBytes == 2) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)code;
         else *dst = (uint8_t)code;
@@ -993,10 +997,13 @@ build_value_sums_kernel(Plan pl, const T* __restrict__ vc, long long sp, long lo
   const int first = (blockIdx.x * (kPrepThreads / 32) + warp) * kRun, last = min(members, first + kRun);
   if (first >= members) return;
   const int32_t* bt = block_table + (size_t)b * pl.max_pages;
-  run_sums(pl, list_ids + ukv * pl.N_max, order + ukv * pl.N_max, first, last, kFixVal,
-           sums + ukv * pl.n_list * (size_t)kD,
-           [&](int i) { return kv_row(pl, bt, i, kv, sp, st, sh); },
-           [&](long long at, float (&x)[4]) { load4<T>(vc + at + 4 * lane, x); });
+  auto sum = [&](auto row) {
+    run_sums(pl, list_ids + ukv * pl.N_max, order + ukv * pl.N_max, first, last, kFixVal, sums + ukv * pl.n_list * (size_t)kD,
+             [&](int i) { return kv_row(pl, bt, i, kv, sp, st, sh); }, row);
+  };
+  // (asked once: a question per row kept its loads from being issued together, 156 -> 214 us)
+  if (whole_rows(vc)) sum([&](long long at, float (&x)[4]) { to_fp32<T>(load_four<true>(vc + at + 4 * lane), x); });
+  else sum([&](long long at, float (&x)[4]) { to_fp32<T>(load_four<false>(vc + at + 4 * lane), x); });
 }
 
 __global__ void build_value_means_kernel(Plan pl, long long* __restrict__ sums, const int32_t* __restrict__ counts,

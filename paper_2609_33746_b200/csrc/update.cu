@@ -130,7 +130,7 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
     const int t = r * kUpdWarps + warp;
     raw[r] = make_uint2(0u, 0u);
     if (ok(t))
-      raw[r] = __ldg(reinterpret_cast<const uint2*>(kc + row_offset(pl, bt, p0 + t, kv, stride_page, stride_token, stride_head)) + lane);
+      raw[r] = load_four(kc + row_offset(pl, bt, p0 + t, kv, stride_page, stride_token, stride_head) + 4 * lane);
   }
   auto direction = [&](int r, float (&x)[4]) {
     float f[8];
