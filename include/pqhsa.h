@@ -297,8 +297,10 @@ int pqhsa_decode_events(const pqhsa_params* params, const void* q, const pqhsa_i
  * positions, and every list that received tokens gets vbar_j = (n_j vbar_j + sum of the new
  * members' values) / (n_j + new_j), n_j += new_j.  first_pos / n_new: device int32 [B];
  * positions outside [0, max_seq_len) are skipped.  centroids, codebooks and list_vmeans 16-byte
- * aligned; the caches and the other arrays may start at any element.  Two launches on `stream`, no
- * workspace, no synchronisation; must not overlap a decode call that reads the same index. */
+ * aligned; the caches and the other arrays may start at any element.  A wait inside the kernel that
+ * runs out (all are bounded; none does on a working GPU) leaves NaN in the key_norms of the tokens
+ * whose lists and codes are then not to be trusted.  Two launches on `stream`, no workspace, no
+ * synchronisation; must not overlap a decode call that reads the same index. */
 int pqhsa_index_update(const pqhsa_params* params, const pqhsa_index_rw* index,
                        const pqhsa_paged_kv* kv, const int32_t* first_pos, const int32_t* n_new,
                        int32_t max_new, void* stream);
@@ -316,7 +318,8 @@ int pqhsa_index_update(const pqhsa_params* params, const pqhsa_index_rw* index,
  * int32 [B][H_kv][n_list] and [B][H_kv][pq_ncode].  All arrays of `index` are outputs.
  * ws: pqhsa_index_build_workspace_bytes(params) bytes (it holds the fp32 directions: 512 bytes
  * per token and KV head), 256-byte aligned.  centroids and list_vmeans 16-byte aligned; the caches and
- * the other arrays may start at any element.  Launches only; no synchronisation. */
+ * the other arrays may start at any element.  NaN in key_norms where a key is finite: as for
+ * pqhsa_index_update.  Launches only; no synchronisation. */
 typedef struct {
   float* centroids;           /* [B][H_kv][n_list][d]                                        */
   float* codebooks;           /* [B][H_kv][M][pq_ncode][dsub]                                */

@@ -181,10 +181,10 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
   unsigned char* s_cen = s_asg + 2 * kTokTileBytes;         // the centroid tile
   __shared__ float s_x2[kAsgTok];
   __shared__ uint8_t s_crowd[kAsgTok];                      // tokens that fp32 searches for
-  __shared__ int s_n_crowd;
+  __shared__ int s_n_crowd, s_late;
   __shared__ Found s_found[8][kCrowd];
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) uint64_t s_full[kAsgPieces], s_used[kAsgPieces], s_done[2], s_free[2];
+  __shared__ __align__(8) uint64_t s_full[kAsgPieces], s_used[kAsgPieces], s_done[2], s_free[2], s_end;
   const int kv = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t0 = blockIdx.x * kAsgTok;
@@ -204,11 +204,12 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
   if (t0 >= n) return;
   const int n_tiles = (pl.n_list + kAsgCen - 1) / kAsgCen;
   const unsigned char* img = images + ukv * (size_t)n_tiles * kCenTileBytes;
-  if (tid == 0) s_n_crowd = 0;
+  if (tid == 0) { s_n_crowd = 0; s_late = 0; }
   if (warp == 8) tmem_alloc(&s_tmem, 512);
   if (warp == 9) {
     if (lane < kAsgPieces) { mbar_init(&s_full[lane], 1); mbar_init(&s_used[lane], 1); }
     if (lane < 2) { mbar_init(&s_done[lane], 1); mbar_init(&s_free[lane], 8); }
+    if (lane == 2) mbar_init(&s_end, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   auto copy = [&](int i, int p) {
@@ -243,15 +244,28 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
+  // A wait that runs out (none does while the GPU works) ends its role's loop, so that nothing in use is
+  // overwritten, and is told through s_late: the lists of the CTA's tokens are then not to be trusted.
   bool late = false;
+  auto ready = [&](uint64_t* bar, uint32_t parity) {
+    if (!late) late = !tc_wait(bar, parity);
+    return !late;
+  };
   if (warp == 9) {
     if (lane == 0) {
-      for (int i = 1; i < n_tiles; ++i) {
+      uint32_t last[kAsgPieces] = {};                       // parity of each piece's last copy
+      for (int i = 1; i < n_tiles && !late; ++i) {
+#pragma unroll
         for (int p = 0; p < kAsgPieces; ++p) {
-          late |= !tc_wait(&s_used[p], (uint32_t)(i - 1) & 1u);
+          if (!ready(&s_used[p], (uint32_t)(i - 1) & 1u)) break;
           copy(i, p);
+          last[p] = (uint32_t)i & 1u;
         }
       }
+#pragma unroll
+      for (int p = 0; p < kAsgPieces; ++p)                  // (no copy outlives the CTA)
+        if (!tc_wait(&s_full[p], last[p])) late = true;
+      if (late) s_late = 1;
     }
     __syncwarp();
   } else if (warp == 8) {
@@ -262,7 +276,7 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
         const uint32_t st = i & 1, ph = st;
         const uint32_t idesc = tc_idesc(pl.n_list - i * kAsgCen <= 64 ? 64u : 128u);
         const uint32_t d0 = tmem + st * 256u, d1 = d0 + 128u;
-        if (i >= 2) late |= !tc_wait(&s_free[st], ((uint32_t)(i >> 1) & 1u) ^ 1u);   // tile i - 2 has been read
+        if (i >= 2 && !ready(&s_free[st], ((uint32_t)(i >> 1) & 1u) ^ 1u)) break;   // tile i - 2 has been read
         // one piece against 4 chunks of the token tiles (offsets in 16-byte units; all constants)
         auto steps = [&](uint32_t a_chunk, uint32_t b_chunk, bool first) {
 #pragma unroll
@@ -275,29 +289,33 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
         // full magnitude
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
-          late |= !tc_wait(&s_full[p], ph);
+          if (!ready(&s_full[p], ph)) break;
           tc_fence_after();
           steps(4 * p, piece_chunk(p), p == 0);
           tc_commit(&s_used[p]);
         }
 #pragma unroll
         for (int p = 4; p < 8; ++p) {
-          late |= !tc_wait(&s_full[p], ph);
+          if (!ready(&s_full[p], ph)) break;
           tc_fence_after();
           steps(16 + 4 * (p - 4), piece_chunk(p), false);
         }
+        if (late) break;
 #pragma unroll
         for (int p = 4; p < 8; ++p) {
           steps(4 * (p - 4), piece_chunk(p), false);
           tc_commit(&s_used[p]);
         }
-        late |= !tc_wait(&s_full[8], ph);
+        if (!ready(&s_full[8], ph)) break;
         tc_fence_after();
         tc_mma(d0, a0 + 32u * 128u, bd + 32u * kAsgCen, idesc, true);
         tc_mma(d1, a1 + 32u * 128u, bd + 32u * kAsgCen, idesc, true);
         tc_commit(&s_used[8]);
         tc_commit(&s_done[st]);
       }
+      tc_commit(&s_end);                                    // (nor does an MMA)
+      if (!tc_wait(&s_end, 0u)) late = true;
+      if (late) s_late = 1;
     }
     __syncwarp();
   } else {
@@ -309,7 +327,7 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
     nn.clear();
     for (int i = 0; i < n_tiles; ++i) {
       const uint32_t st = i & 1;
-      late |= !tc_wait(&s_done[st], (uint32_t)(i >> 1) & 1u);
+      if (__any_sync(0xffffffffu, !ready(&s_done[st], (uint32_t)(i >> 1) & 1u))) { s_late = 1; break; }
       tc_fence_after();
       const int n_cols = min(pl.n_list - i * kAsgCen, kAsgCen);
 #pragma unroll 1
@@ -335,14 +353,12 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
       if (lane == src) near = at;
     }
     if (crowd) s_crowd[atomicAdd(&s_n_crowd, 1)] = (uint8_t)r;
-    if (real) {
-      list_ids[ukv * pl.N_max + t0 + r] = (uint16_t)near;
-      if (late) key_norms[ukv * pl.N_max + t0 + r] = CUDART_NAN_F;      // a bounded wait ran out: the norms say so
-    }
+    if (real) list_ids[ukv * pl.N_max + t0 + r] = (uint16_t)near;
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 8) { tc_fence_after(); tmem_free(tmem, 512); }
+  if (s_late != 0 && t0 + tid < min(n, t0 + kAsgTok)) key_norms[ukv * pl.N_max + t0 + tid] = CUDART_NAN_F;
   // between more of them over all centroids, by eight warps
   const int n_crowd = s_n_crowd;
   const int n_search = n_crowd > kCrowd ? kCrowd : 1;       // for together
