@@ -10,7 +10,7 @@ namespace pqhsa {
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr size_t kMaxSmemPerCta = 227 * 1024 - 1024;   // opt-in limit minus static shared memory
+constexpr size_t kMaxSmemPerCta = kMaxDynamicSmem;     // opt-in limit minus static shared memory
 constexpr int kDefaultSms = 148;                        // B200
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }

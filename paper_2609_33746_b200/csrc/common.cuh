@@ -277,6 +277,16 @@ template <auto kKernel> void set_carveout(int percent) {
     done.fetch_or(uint64_t(1) << dev, std::memory_order_relaxed);
 }
 
+// Dynamic shared memory of kernels whose need depends on the call's shape.  The opt-in is one setting per
+// kernel and device for all host threads: it is set to the most that a CTA may have and not to a call's
+// own size, which another thread's smaller call could put in place between setting and launch.
+// (kStaticSmem: an upper bound of those kernels' static shared memory.)
+constexpr int kStaticSmem = 1024;
+constexpr int kMaxDynamicSmem = 227 * 1024 - kStaticSmem;
+template <typename K> cudaError_t allow_max_smem(K* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
+}
+
 // Launch with programmatic stream serialization allowed (see pdl_wait above).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,

@@ -532,8 +532,7 @@ static cudaError_t launch_scan_t(const Plan& pl, const pqhsa_index& ix, const fl
                                  const float* coarse, const int32_t* seq_lens, float* scores,
                                  float* partials, int* status, cudaStream_t st) {
   const size_t smem = scan_smem_bytes(pl, pl.coarse_in_smem != 0, S);
-  cudaError_t e = cudaFuncSetAttribute(scan_kernel<M, GC, S, kHalf>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_max_smem(scan_kernel<M, GC, S, kHalf>);
   if (e != cudaSuccess) return e;
   return launch_pdl(scan_kernel<M, GC, S, kHalf>, dim3(pl.scan_ctas), dim3(kScanThreads), smem, st, pl,
                     ix.codes, ix.list_ids, ix.key_norms, lut, coarse, seq_lens, scores, partials,

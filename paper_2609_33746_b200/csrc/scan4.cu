@@ -452,8 +452,7 @@ cudaError_t launch_scan4_t(const Plan& pl, const pqhsa_index& ix, const float* l
                            const float* coarse, const int32_t* seq_lens, float* scores,
                            float* partials, int* status, cudaStream_t st) {
   const size_t smem = scan4_smem_bytes(pl, pl.coarse_in_smem);
-  cudaError_t e = cudaFuncSetAttribute(scan4_kernel<M, GC>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_max_smem(scan4_kernel<M, GC>);
   if (e != cudaSuccess) return e;
   return launch_pdl(scan4_kernel<M, GC>, dim3(pl.scan_ctas), dim3(kScanThreads), smem, st, pl,
                     ix.codes, ix.list_ids, ix.key_norms, lut, coarse, seq_lens, scores, partials,

@@ -530,7 +530,7 @@ select_cluster_kernel(Plan pl, const float* __restrict__ scores, const int32_t* 
 }
 
 constexpr size_t kClHead = (sizeof(ClShared) + 127) & ~size_t(127);
-constexpr int kClSlice = (int)((227 * 1024 - 1024 - kClHead) / 16 * 4);       // scores a CTA can hold
+constexpr int kClSlice = (int)((kMaxDynamicSmem - kClHead) / 16 * 4);       // scores a CTA can hold
 
 int slice_of(const Plan& pl, int cs) { return (pl.N_max + 4 * cs - 1) / (4 * cs) * 4; }
 size_t smem_of(const Plan& pl, int cs) { return kClHead + (size_t)slice_of(pl, cs) * 4; }
@@ -543,7 +543,7 @@ cudaError_t launch_t(const Plan& pl, const float* scores, const int32_t* seq_len
                      const uint16_t* lids, float* bg_mass, float* bg_max, cudaStream_t st) {
   const size_t smem = smem_of(pl, pl.sel_cluster);
   auto kernel = select_cluster_kernel<kBg, kPerSm>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_max_smem(kernel);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(pl.rows * pl.sel_cluster));
