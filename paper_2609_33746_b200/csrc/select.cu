@@ -600,7 +600,8 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
     } else {
       // the first kStashCap candidates are staged; the rest, if any, is read from the list each time (a
       // bracket 1 % of 512K scores wide holds about 5200: with all of them left to the radix select,
-      // whose passes reread the list, the finish took 17 us instead of 5)
+      // whose passes reread the list, the finish took 17 us instead of 5), four loads at a time: 32 x
+      // 512K, half of each row selected, top-k alone 134 us one by one, 110 so
       constexpr int kPer = kStashCap / kSelThreads;            // 10: all loads issued together
       uint2 it[kPer];
 #pragma unroll
@@ -615,19 +616,32 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
         if (i < C) s_stash[i] = it[u];
       }
       const int src = C <= kStashCap ? kFromStash : kFromList;
-      auto item = [&](int i) { return i < kStashCap ? s_stash[i] : __ldcg(rc + i); };
+      // f(i, candidate i) for this thread's candidates from `base` on, kAhead * kSelThreads of them: the loads
+      // of those that are not staged go out together
+      constexpr int kAhead = 4;
+      auto some_items = [&](int base, auto f) {
+        uint2 x[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+          const int i = base + u * kSelThreads + tid;
+          if (i < C) x[u] = i < kStashCap ? s_stash[i] : __ldcg(rc + i);
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+          if (base + u * kSelThreads + tid < C) f(u, x[u]);
+      };
       __syncthreads();
       // range of the candidates: the bracket, or, where it is open, their finite scores
       float lo_h = lo_f, hi_h = hi_f;
       if (!(lo_f > -CUDART_INF_F && hi_f < CUDART_INF_F)) {
         uint32_t kmin = 0xffffffffu, kmax = 0u;
-        for (int i = tid; i < C; i += kSelThreads) {
-          const uint32_t key = item(i).x;
-          if (fabsf(key_score(key)) < CUDART_INF_F) {
-            kmin = min(kmin, key);
-            kmax = max(kmax, key);
-          }
-        }
+        for (int base = 0; base < C; base += kAhead * kSelThreads)
+          some_items(base, [&](int, uint2 x) {
+            if (fabsf(key_score(x.x)) < CUDART_INF_F) {
+              kmin = min(kmin, x.x);
+              kmax = max(kmax, x.x);
+            }
+          });
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
@@ -652,8 +666,8 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
         // higher bucket is taken at once, and the few items of that bucket are ranked against each
         // other (larger score first, then lower position: the stable rule).
         const float scale = (float)kHistBins / (hi_h - lo_h);
-        for (int i = tid; i < C; i += kSelThreads)
-          atomicAdd(&s_hist[linear_bucket(key_score(item(i).x), lo_h, scale)], 1u);
+        for (int base = 0; base < C; base += kAhead * kSelThreads)
+          some_items(base, [&](int, uint2 x) { atomicAdd(&s_hist[linear_bucket(key_score(x.x), lo_h, scale)], 1u); });
         __syncthreads();
         int d, above;
         find_digit(s_hist, kHistBins, r, s_scan, d, above);
@@ -667,14 +681,12 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
           // 32 items per thread and append
           for (int base = 0; base < C; base += 32 * kSelThreads) {
             uint32_t take = 0u;
-            for (int u = 0; u < 32 && base + u * kSelThreads < C; ++u) {
-              const int i = base + u * kSelThreads + tid;
-              if (i >= C) break;
-              const uint2 x = item(i);
-              const int bk = linear_bucket(key_score(x.x), lo_h, scale);
-              if (bk > d) take |= 1u << u;
-              if (bk == d) tie[atomicAdd(&s_tie, 1u)] = x;
-            }
+            for (int u0 = 0; u0 < 32 && base + u0 * kSelThreads < C; u0 += kAhead)
+              some_items(base + u0 * kSelThreads, [&](int u, uint2 x) {
+                const int bk = linear_bucket(key_score(x.x), lo_h, scale);
+                if (bk > d) take |= 1u << (u0 + u);
+                if (bk == d) tie[atomicAdd(&s_tie, 1u)] = x;
+              });
             __syncwarp();
             const int mine = __popc(take);
             int inc = mine;
@@ -686,8 +698,13 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
             uint32_t p = 0u;
             if (lane == 31 && inc > 0) p = atomicAdd(&s_emit, (uint32_t)inc);
             p = (uint32_t)W + __shfl_sync(0xffffffffu, p, 31) + (uint32_t)(inc - mine);
-            for (; take != 0u; take &= take - 1u, ++p)
-              if (p < (uint32_t)pl.k_max) out[p] = (int)item(base + (__ffs(take) - 1) * kSelThreads + tid).y;
+            for (int u0 = 0; u0 < 32 && base + u0 * kSelThreads < C; u0 += kAhead)
+              some_items(base + u0 * kSelThreads, [&](int u, uint2 x) {
+                if ((take >> (u0 + u)) & 1u) {
+                  if (p < (uint32_t)pl.k_max) out[p] = (int)x.y;
+                  ++p;
+                }
+              });
           }
           __syncthreads();
           for (int base = 0; base < m; base += kSelThreads) {
