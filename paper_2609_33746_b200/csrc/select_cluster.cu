@@ -573,8 +573,10 @@ cudaError_t launch_t(const Plan& pl, const float* scores, const int32_t* seq_len
 //   one CTA per SM and row, up to three waves: 8 x 32K 122 -> 114, 12 x 32K 163 -> 157, but
 //   16 x 24K 173 -> 173 at three and a half;
 //   several CTAs per row, up to two waves: 2 x 128K 111 -> 108, 4 x 64K 114 -> 112, but 4 x 128K
-//   181 -> 193; of clusters of eight a GPC holds two at most, and 16 rows do not fit at once (top-k alone
-//   of 256K at 0.1 %: 16 rows 28 -> 33, 14 rows of 200K 0.74 times the sampled path's time).
+//   181 -> 193; of clusters of eight a GPC holds two at most, and 16 rows do not run at once: a row is then
+//   cut in four where that is enough (16 rows of 30K 53 -> 45, of 100K 56 -> 45 against eight), in eight
+//   while the slices are short (16 rows of 200K, sampled -> cluster: 73 -> 66; of 256K 117 -> 117, and the
+//   top-k alone 28 -> 33).
 // And only while most of what is selected is listed: passes over the whole slice for every step cost more
 // than the sampled path's.  1 x 128K (4 CTAs a row): budget 4 % 0.90 times the sampled path's time, 6 %
 // 1.02, 8 % 1.10; 1 x 64K: 12.5 % 0.91, 20 % 1.01; 8 x 32K: 4 % 1.00, 8 % 1.12.  Short slices bear it:
@@ -582,17 +584,18 @@ cudaError_t launch_t(const Plan& pl, const float* scores, const int32_t* seq_len
 // first bound is no bound: 1 x 8K: 40 % 0.76, 50 % 1.12, 70 % 1.38.
 constexpr int kClListed = 2048;          // selected scores per CTA that still leave room in its list
 constexpr int kClShort = 8192;           // a slice that may be passed over instead
+constexpr int kClTurns = 28672;          // longest slice of clusters of eight that take turns
 constexpr uint32_t kClMaxPpm = 400000u;
 void plan_select_cluster(Plan* pl) {
   pl->sel_cluster = 0;
   if (pl->rescore) return;                 // the re-score reads the sampled path's candidate lists
   int cs = 1;
-  while (cs < kClMax && pl->rows * cs * 2 <= pl->num_sms && pl->N_max / cs > 4096) cs *= 2;
+  const int most = 5 * pl->rows * kClMax <= 4 * pl->num_sms ? kClMax : kClMax / 2;
+  while (cs < most && pl->rows * cs * 2 <= pl->num_sms && pl->N_max / cs > 4096) cs *= 2;
   while (cs < kClMax && slice_of(*pl, cs) > kClSlice) cs *= 2;
-  if (slice_of(*pl, cs) > kClSlice) return;
+  if (slice_of(*pl, cs) > (cs > most ? kClTurns : kClSlice)) return;
   const int waves = cs > 1 ? 2 : 3;
   if (!(cs == 1 && two_per_sm(*pl, 1)) && pl->rows * cs > waves * pl->num_sms) return;
-  if (cs == kClMax && 5 * pl->rows * cs > 4 * pl->num_sms) return;
   if (pl->ppm > kClMaxPpm) return;
   const long long k = ((long long)pl->N_max * pl->ppm + 999999LL) / 1000000LL;
   if (k > (long long)kClListed * cs && slice_of(*pl, cs) > kClShort) return;
