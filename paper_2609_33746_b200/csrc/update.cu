@@ -9,6 +9,7 @@
 //       centroids, then every warpgroup takes every fourth subspace.  What comes within the rounding of
 //       the nearest, and centres too far out for fp16, are compared in fp32: lists and codes are those of
 //       an fp32 search.  The codeword is decided in fp32 among the 8 of the winning group.
+//   index_encode_few_kernel     the same with fp32 FMAs, 8 tokens per CTA: few tokens against few lists.
 //   index_refresh_means_kernel  groups the new tokens by list (first occurrence = leader), sums
 //       each group's value rows in token order and sets vbar_j = (n_j vbar_j + sum) / (n_j + new_j),
 //       n_j += new_j; a warp per leader.
@@ -423,6 +424,128 @@ index_encode_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, lo
   }
 }
 
+// The same for few tokens against few lists: 8 tokens per CTA, all of it in fp32.  Centroids pass through
+// shared memory in tiles of 32 rows (a lane owns a centroid, a warp a token); for the codes a warp owns
+// subspaces and a lane codewords, so a codebook row is read once for all 8 tokens.
+constexpr int kFewTok = 8;              // tokens per CTA = warps per CTA
+constexpr int kFewThreads = 32 * kFewTok;
+constexpr int kFewCen = 32;             // centroid rows per tile
+
+template <typename T, int DSUB>
+__global__ void __launch_bounds__(kFewThreads)
+index_encode_few_kernel(Plan pl, const T* __restrict__ kc, long long stride_page, long long stride_token,
+                        long long stride_head, const int32_t* __restrict__ block_table,
+                        const int32_t* __restrict__ first_pos, const int32_t* __restrict__ n_new,
+                        int max_new, const float* __restrict__ centroids,
+                        const float* __restrict__ codebooks, uint8_t* __restrict__ codes,
+                        uint16_t* __restrict__ list_ids, float* __restrict__ key_norms) {
+  __shared__ float s_u[kFewTok][kHeadDim];                  // direction, later the residual
+  __shared__ float s_c[kFewCen][kHeadDim + 1];              // (padded: lane j reads row j without conflicts)
+  __shared__ uint8_t s_code[kFewTok][64];
+  const int kv = blockIdx.y, b = blockIdx.z;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const size_t ukv = (size_t)b * pl.Hkv + kv;
+  pdl_wait();
+  pdl_launch_dependents();
+  const int nb = min(max(n_new[b], 0), max_new);
+  const int t0 = blockIdx.x * kFewTok;
+  if (t0 >= nb) return;
+  const int ntok = min(kFewTok, nb - t0);
+  const int p0 = first_pos[b] + t0;                 // position of this CTA's first token
+  const int32_t* bt = block_table + (size_t)b * pl.max_pages;
+  // tokens whose position falls outside the index rows are left alone
+  const bool mine_ok = warp < ntok && p0 + warp >= 0 && p0 + warp < pl.N_max;
+  // ---- norm and direction: warp w <-> token w, a lane holds 4 of the 128 dims
+  {
+    float x[4] = {0.f, 0.f, 0.f, 0.f};
+    if (mine_ok) load4<T>(kc + row_offset(pl, bt, p0 + warp, kv, stride_page, stride_token, stride_head) + 4 * lane, x);
+    const float ss = warp_sum(x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3]);
+    const float r = sqrtf(ss);
+    const float inv = r > 0.f ? 1.f / r : 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s_u[warp][4 * lane + i] = x[i] * inv;
+    if (mine_ok && lane == 0) key_norms[ukv * pl.N_max + p0 + warp] = r;
+  }
+  // ---- nearest centroid: |u - c|^2 = |u|^2 - 2 u.c + |c|^2, the first term is common
+  float best_d = CUDART_INF_F;
+  int best_j = 0;
+  const float* cbase = centroids + ukv * (size_t)pl.n_list * kHeadDim;
+  for (int c0 = 0; c0 < pl.n_list; c0 += kFewCen) {
+    __syncthreads();                                // previous tile consumed, s_u complete
+    for (int i = tid; i < kFewCen * (kHeadDim / 4); i += kFewThreads) {
+      const int rr = i / (kHeadDim / 4), c4 = i % (kHeadDim / 4);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c0 + rr < pl.n_list) v = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)(c0 + rr) * kHeadDim) + c4);
+      s_c[rr][4 * c4] = v.x; s_c[rr][4 * c4 + 1] = v.y;
+      s_c[rr][4 * c4 + 2] = v.z; s_c[rr][4 * c4 + 3] = v.w;
+    }
+    __syncthreads();
+    float dot = 0.f, cn = 0.f;
+#pragma unroll 8
+    for (int d = 0; d < kHeadDim; ++d) {
+      const float c = s_c[lane][d];
+      dot = fmaf(s_u[warp][d], c, dot);
+      cn = fmaf(c, c, cn);
+    }
+    const float dist = fmaf(-2.f, dot, cn);
+    if (c0 + lane < pl.n_list && dist < best_d) { best_d = dist; best_j = c0 + lane; }
+  }
+  warp_nearest(best_d, best_j);
+  if (mine_ok && lane == 0) list_ids[ukv * pl.N_max + p0 + warp] = (uint16_t)best_j;
+  // ---- residual, in place
+  {
+    const float4 c = __ldg(reinterpret_cast<const float4*>(cbase + (size_t)best_j * kHeadDim) + lane);
+    s_u[warp][4 * lane] -= c.x; s_u[warp][4 * lane + 1] -= c.y;
+    s_u[warp][4 * lane + 2] -= c.z; s_u[warp][4 * lane + 3] -= c.w;
+  }
+  __syncthreads();
+  // ---- codes: warp <-> subspaces m = warp, warp + 8, ...; lane <-> codewords lane + 32 i
+  for (int m = warp; m < pl.M; m += kFewTok) {
+    float bd[kFewTok];
+    int bz[kFewTok];
+#pragma unroll
+    for (int t = 0; t < kFewTok; ++t) { bd[t] = CUDART_INF_F; bz[t] = 0; }
+    const float* cb = codebooks + (ukv * pl.M + m) * (size_t)pl.n_code * DSUB;
+    for (int z0 = 0; z0 < pl.n_code; z0 += 32) {
+      const int z = min(z0 + lane, pl.n_code - 1);      // lanes past the codebook repeat its last word
+      float p[DSUB];
+      if constexpr (DSUB == 2) {
+        const float2 v = __ldg(reinterpret_cast<const float2*>(cb + (size_t)z * DSUB));
+        p[0] = v.x; p[1] = v.y;
+      } else {
+#pragma unroll
+        for (int c4 = 0; c4 < DSUB / 4; ++c4) {
+          const float4 v = __ldg(reinterpret_cast<const float4*>(cb + (size_t)z * DSUB) + c4);
+          p[4 * c4] = v.x; p[4 * c4 + 1] = v.y; p[4 * c4 + 2] = v.z; p[4 * c4 + 3] = v.w;
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < kFewTok; ++t) {
+        float dist = 0.f;
+#pragma unroll
+        for (int dd = 0; dd < DSUB; ++dd) {
+          const float e = s_u[t][m * DSUB + dd] - p[dd];
+          dist = fmaf(e, e, dist);
+        }
+        if (dist < bd[t]) { bd[t] = dist; bz[t] = z; }      // z ascends: first minimum stays
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < kFewTok; ++t) {
+      warp_nearest(bd[t], bz[t]);
+      if (lane == 0) s_code[t][m] = (uint8_t)bz[t];
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < ntok * pl.code_bytes; i += kFewThreads) {
+    const int t = i / pl.code_bytes, j = i - t * pl.code_bytes;
+    const int pos = p0 + t;
+    const uint8_t byte = pl.n_code == 16 ? (uint8_t)(s_code[t][2 * j] | (s_code[t][2 * j + 1] << 4))
+                                         : s_code[t][j];
+    if (pos >= 0 && pos < pl.N_max) codes[(ukv * pl.N_max + pos) * pl.code_bytes + j] = byte;
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kMeanThreads)
 index_refresh_means_kernel(Plan pl, const T* __restrict__ vc, long long stride_page,
@@ -430,7 +553,7 @@ index_refresh_means_kernel(Plan pl, const T* __restrict__ vc, long long stride_p
                            const int32_t* __restrict__ block_table,
                            const int32_t* __restrict__ first_pos, const int32_t* __restrict__ n_new,
                            int max_new, const uint16_t* __restrict__ list_ids,
-                           float* __restrict__ list_vmeans, int32_t* __restrict__ list_counts) {
+                           float* __restrict__ list_vmeans, int32_t* __restrict__ list_counts, int early) {
   extern __shared__ int s_first[];                   // [n_list] first new token of every list
   __shared__ uint16_t s_lid[kMaxNew];
   const int kv = blockIdx.y, b = blockIdx.z;
@@ -443,7 +566,9 @@ index_refresh_means_kernel(Plan pl, const T* __restrict__ vc, long long stride_p
   nb = min(nb, pl.N_max - p0);                       // same positions as the encode kernel
   const int t_begin = blockIdx.x * kMeanTok, t_end = min(nb, t_begin + kMeanTok);
   pdl_wait();                                        // the list ids come from the encode kernel
-  pdl_launch_dependents();
+  // (not beside the small encode kernel of a next call: between these CTAs its own land unevenly, 50 -> 70 us
+  // at 256 units x 512 lists)
+  if (early) pdl_launch_dependents();
   if (t_begin >= nb) return;
   const int32_t* bt = block_table + (size_t)b * pl.max_pages;
   __syncthreads();
@@ -482,23 +607,48 @@ index_refresh_means_kernel(Plan pl, const T* __restrict__ vc, long long stride_p
   }
 }
 
+// Which of the two encodes.  Both times fitted, in us of a whole call: a fixed part, the codes, a part that
+// grows with the lists, and the CTAs per SM.  Measured, fp32 kernel / tensor cores, 32 one-byte codes: one
+// unit, 8 tokens, 16 lists 17 / 37, 128 23 / 38, 384 39 / 45, 512 47 / 47, 1024 78 / 59; 64 units x 32
+// tokens, 16 lists 36 / 45, 128 44 / 44, 384 52 / 50.  Eight 4-bit codes: 64 units x 64 tokens, 16 lists
+// 23 / 37, 64 27 / 37; 256 units x 16 tokens, 128 lists 36 / 57, 256 52 / 64.
+bool few_tokens(const Plan& pl, int max_new) {
+  const int units = pl.B * pl.Hkv;
+  auto ctas = [&](int tokens) { return units * ((max_new + tokens - 1) / tokens); };
+  const bool bytes = pl.n_code == 256;
+  const float codes_few = !bytes ? 2.f : pl.M == 8 ? 5.f : pl.M == 16 ? 8.f : pl.M == 32 ? 11.f : 19.f;
+  const float codes_tc = !bytes ? 2.f : pl.M == 8 ? 8.f : pl.M == 16 ? 6.f : pl.M == 32 ? 12.f : 31.f;
+  const float r = (float)ctas(kFewTok) / (float)pl.num_sms;
+  const float few = (8.f + codes_few) * (r > 1.f ? 0.6f + 0.4f * r : 1.f) + 0.061f * pl.n_list * (r > 1.25f ? 0.8f * r : 1.f);
+  const int waves = (ctas(kUpdTok) + pl.num_sms - 1) / pl.num_sms;
+  return few < (24.f + codes_tc + 0.022f * pl.n_list) * waves;
+}
+
 template <typename T>
 cudaError_t launch_update_t(const Plan& pl, const pqhsa_index_rw& ix, const pqhsa_paged_kv& kv,
                             const int32_t* first_pos, const int32_t* n_new, int max_new,
                             cudaStream_t st) {
-  const dim3 grid((max_new + kUpdTok - 1) / kUpdTok, pl.Hkv, pl.B), block(kUpdThreads);
   const T* kc = static_cast<const T*>(kv.k_cache);
   const T* vc = static_cast<const T*>(kv.v_cache);
+  const bool few = few_tokens(pl, max_new);
+  const int per_cta = few ? kFewTok : kUpdTok;
+  const dim3 grid((max_new + per_cta - 1) / per_cta, pl.Hkv, pl.B);
   cudaError_t e;
+  auto encode = [&](auto kernel, int threads, size_t smem) {
+    return launch_pdl(kernel, grid, dim3(threads), smem, st, pl, kc, (long long)kv.stride_page,
+                      (long long)kv.stride_token, (long long)kv.stride_head, kv.block_table, first_pos, n_new,
+                      max_new, ix.centroids, ix.codebooks, ix.codes, ix.list_ids, ix.key_norms);
+  };
 #define PQHSA_UPD_CASE(D)                                                                       \
   case D:                                                                                       \
+    if (few) {                                                                                  \
+      e = encode(index_encode_few_kernel<T, D>, kFewThreads, 0);                                \
+      break;                                                                                    \
+    }                                                                                           \
     e = cudaFuncSetAttribute(index_encode_kernel<T, D>,                                         \
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kUpdSmem);            \
     if (e != cudaSuccess) return e;                                                             \
-    e = launch_pdl(index_encode_kernel<T, D>, grid, block, kUpdSmem, st, pl, kc,                \
-                   (long long)kv.stride_page, (long long)kv.stride_token,                       \
-                   (long long)kv.stride_head, kv.block_table, first_pos, n_new, max_new,        \
-                   ix.centroids, ix.codebooks, ix.codes, ix.list_ids, ix.key_norms);            \
+    e = encode(index_encode_kernel<T, D>, kUpdThreads, kUpdSmem);                               \
     break;
   switch (pl.dsub) {
     PQHSA_UPD_CASE(2) PQHSA_UPD_CASE(4) PQHSA_UPD_CASE(8) PQHSA_UPD_CASE(16)
@@ -510,7 +660,7 @@ cudaError_t launch_update_t(const Plan& pl, const pqhsa_index_rw& ix, const pqhs
                     dim3(kMeanThreads), (size_t)pl.n_list * 4, st, pl, vc,
                     (long long)kv.stride_page, (long long)kv.stride_token,
                     (long long)kv.stride_head, kv.block_table, first_pos, n_new, max_new,
-                    static_cast<const uint16_t*>(ix.list_ids), ix.list_vmeans, ix.list_counts);
+                    static_cast<const uint16_t*>(ix.list_ids), ix.list_vmeans, ix.list_counts, few ? 0 : 1);
 }
 
 }  // namespace
