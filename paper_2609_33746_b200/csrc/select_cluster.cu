@@ -575,8 +575,8 @@ cudaError_t launch_t(const Plan& pl, const float* scores, const int32_t* seq_len
 //   several CTAs per row, up to two waves: 2 x 128K 111 -> 108, 4 x 64K 114 -> 112, but 4 x 128K
 //   181 -> 193; of clusters of eight a GPC holds two at most, and 16 rows do not run at once: a row is then
 //   cut in four where that is enough (16 rows of 30K 53 -> 45, of 100K 56 -> 45 against eight), in eight
-//   while the slices are short (16 rows of 200K, sampled -> cluster: 73 -> 66; of 256K 117 -> 117, and the
-//   top-k alone 28 -> 33).
+//   while the slices are short and the rows few (16 rows of 200K, sampled -> cluster: 73 -> 66; of 256K
+//   117 -> 117, and the top-k alone 28 -> 33; 32 rows of 190K 174 -> 187).
 // And only while most of what is selected is listed: passes over the whole slice for every step cost more
 // than the sampled path's.  1 x 128K (4 CTAs a row): budget 4 % 0.90 times the sampled path's time, 6 %
 // 1.02, 8 % 1.10; 1 x 64K: 12.5 % 0.91, 20 % 1.01; 8 x 32K: 4 % 1.00, 8 % 1.12.  Short slices bear it:
@@ -594,6 +594,7 @@ void plan_select_cluster(Plan* pl) {
   while (cs < most && pl->rows * cs * 2 <= pl->num_sms && pl->N_max / cs > 4096) cs *= 2;
   while (cs < kClMax && slice_of(*pl, cs) > kClSlice) cs *= 2;
   if (slice_of(*pl, cs) > (cs > most ? kClTurns : kClSlice)) return;
+  if (cs > most && pl->rows * cs > pl->num_sms) return;
   const int waves = cs > 1 ? 2 : 3;
   if (!(cs == 1 && two_per_sm(*pl, 1)) && pl->rows * cs > waves * pl->num_sms) return;
   if (pl->ppm > kClMaxPpm) return;
