@@ -570,13 +570,14 @@ cudaError_t launch_t(const Plan& pl, const float* scores, const int32_t* seq_len
 // requires.  Whole decode call, 32 rows per sequence, sampled -> cluster, us:
 //   slices that leave room for two CTAs per SM win with any number of rows: 16 x 8K 135 -> 92,
 //   32 x 8K 225 -> 165, 32 x 4K 155 -> 136, 16 x 16K 139 -> 127, 32 x 16K 241 -> 229;
-//   one CTA per SM and row, up to three waves: 8 x 32K 122 -> 114, 12 x 32K 163 -> 157, but
-//   16 x 24K 173 -> 173 at three and a half;
-//   several CTAs per row, up to two waves: 2 x 128K 111 -> 108, 4 x 64K 114 -> 112, but 4 x 128K
-//   181 -> 193; of clusters of eight a GPC holds two at most, and 16 rows do not run at once: a row is then
-//   cut in four where that is enough (16 rows of 30K 53 -> 45, of 100K 56 -> 45 against eight), in eight
-//   while the slices are short and the rows few (16 rows of 200K, sampled -> cluster: 73 -> 66; of 256K
-//   117 -> 117, and the top-k alone 28 -> 33; 32 rows of 190K 174 -> 187).
+//   one CTA per SM and row, several waves: 8 x 20K 92 -> 88, 13 x 20K 123 -> 123; longer slices up to two
+//   waves, the last at least half full: 8 x 32K 116 -> 111, 8 x 45K 144 -> 141, but 5 x 32K (1.1 waves)
+//   85 -> 89, 6 x 45K (1.3) 114 -> 122, 12 x 45K (2.6) 189 -> 197;
+//   several CTAs per row while all run at once: 1 x 92K of 64 heads 91 -> 81, but 3 x 92K 112 -> 124,
+//   4 x 92K 136 -> 144.  Of clusters of eight a GPC holds two at most, and 16 rows do not run at once: a row
+//   is then cut in four where that is enough (16 rows of 30K 53 -> 45, of 100K 56 -> 45 against eight), in
+//   eight while the slices are short and the rows few (16 rows of 200K, sampled -> cluster: 73 -> 66; of
+//   256K 117 -> 117, and the top-k alone 28 -> 33; 32 rows of 190K 174 -> 187).
 // And only while most of what is selected is listed: passes over the whole slice for every step cost more
 // than the sampled path's.  1 x 128K (4 CTAs a row): budget 4 % 0.90 times the sampled path's time, 6 %
 // 1.02, 8 % 1.10; 1 x 64K: 12.5 % 0.91, 20 % 1.01; 8 x 32K: 4 % 1.00, 8 % 1.12.  Short slices bear it:
@@ -584,6 +585,7 @@ cudaError_t launch_t(const Plan& pl, const float* scores, const int32_t* seq_len
 // first bound is no bound: 1 x 8K: 40 % 0.76, 50 % 1.12, 70 % 1.38.
 constexpr int kClListed = 2048;          // selected scores per CTA that still leave room in its list
 constexpr int kClShort = 8192;           // a slice that may be passed over instead
+constexpr int kClFill = 24576;           // longest slice whose last wave may be nearly empty
 constexpr int kClTurns = 28672;          // longest slice of clusters of eight that take turns
 constexpr uint32_t kClMaxPpm = 400000u;
 void plan_select_cluster(Plan* pl) {
@@ -595,8 +597,12 @@ void plan_select_cluster(Plan* pl) {
   while (cs < kClMax && slice_of(*pl, cs) > kClSlice) cs *= 2;
   if (slice_of(*pl, cs) > (cs > most ? kClTurns : kClSlice)) return;
   if (cs > most && pl->rows * cs > pl->num_sms) return;
-  const int waves = cs > 1 ? 2 : 3;
-  if (!(cs == 1 && two_per_sm(*pl, 1)) && pl->rows * cs > waves * pl->num_sms) return;
+  const int waves = (pl->rows * cs + pl->num_sms - 1) / pl->num_sms;
+  if (cs > 1 && waves > 1) return;
+  if (cs == 1 && waves > 1 && !two_per_sm(*pl, 1)) {
+    if (waves > 3) return;
+    if (pl->N_max > kClFill && (waves > 2 || 4 * pl->rows < 3 * waves * pl->num_sms)) return;
+  }
   if (pl->ppm > kClMaxPpm) return;
   const long long k = ((long long)pl->N_max * pl->ppm + 999999LL) / 1000000LL;
   if (k > (long long)kClListed * cs && slice_of(*pl, cs) > kClShort) return;
