@@ -367,8 +367,8 @@ build_assign_kernel(Plan pl, const float* __restrict__ U, const unsigned char* _
     const float* rows = U + (ukv * pl.N_max + t0) * kD;
     const float* cen = centroids + ukv * pl.n_list * (size_t)kD;
     if (warp < 8) {
-      if (n_search == 1) nearest_of_all<true, 1>(rows, kD, s_crowd, c, n_crowd, cen, pl.n_list, tid, 256, s_found[warp]);
-      else nearest_of_all<true, kCrowd>(rows, kD, s_crowd, c, n_crowd, cen, pl.n_list, tid, 256, s_found[warp]);
+      if (n_search == 1) nearest_of_all<true, 1>(rows, kD, s_crowd, c, n_crowd, cen, pl.n_list, tid, 256, ~0u, s_found[warp]);
+      else nearest_of_all<true, kCrowd>(rows, kD, s_crowd, c, n_crowd, cen, pl.n_list, tid, 256, ~0u, s_found[warp]);
     }
     __syncthreads();
     if (tid < n_search && c + tid < n_crowd) {

@@ -250,9 +250,11 @@ struct Nearest2 {
   int best_at, second_at;                                // which 32 columns
   int blocks;                                            // within reach of `low` (at most so many)
   bool pair;                                             // two in one block
+  uint32_t seen;                                         // the blocks counted, a bit for each four (at / 4)
   __device__ __forceinline__ void clear() {
     low = best = second = CUDART_INF_F;
     best_at = second_at = blocks = 0;
+    seen = 0u;
     pair = false;
   }
   // (column bits: the value's own, or infinity's zeros)
@@ -271,7 +273,7 @@ struct Nearest2 {
   __device__ __forceinline__ void take(const float (&acc)[32], int at, const TieLimit& lim) {
     const float m = min32(acc);
     if (m < lim(low)) {
-      if (lim(m) <= low) { blocks = 0; pair = false; }   // all that came before is out of reach
+      if (lim(m) <= low) { blocks = 0; pair = false; seen = 0u; }      // all that came before is out of reach
       low = fminf(low, m);
       float b2[16], s2[16];
 #pragma unroll
@@ -290,6 +292,7 @@ struct Nearest2 {
         }
       }
       ++blocks;
+      seen |= 1u << (at >> 2);
       pair |= s2[0] < lim(low);
       merge(b2[0], at);
     }
@@ -354,15 +357,18 @@ __device__ __noinline__ int nearest_of_blocks(const float* x, const float* __res
   return at;
 }
 // ... of kT rows (index[c], index[c + 1], .., at most n of them) among all centroids, by the threads first,
-// first + step, .. ; leaves each warp's result at found[0 .. kT).  (One row: the loads run ahead of the
-// chains; four share every centroid's load, for data where all is equally near.)
+// first + step, .. (step a multiple of 128); leaves each warp's result at found[0 .. kT).  (One row: the
+// loads run ahead of the chains; four share every centroid's load, for data where all is equally near.)
+// near_by: bit i tells whether the row's block of 32 centroids at the thread's place of every 128 has to be
+// looked at in the i-th 128.
 struct Found {
   float d;
   int at;
 };
 template <bool kX2, int kT>
 __device__ __noinline__ void nearest_of_all(const float* rows, int stride, const uint8_t* index, int c, int n,
-                                            const float* __restrict__ centroids, int n_list, int first, int step, Found* found) {
+                                            const float* __restrict__ centroids, int n_list, int first, int step, uint32_t near_by,
+                                            Found* found) {
   const float* row[kT];
   float d[kT];
   int at[kT];
@@ -374,6 +380,7 @@ __device__ __noinline__ void nearest_of_all(const float* rows, int stride, const
   }
 #pragma unroll 1
   for (int j = first; j < n_list; j += step) {
+    if (!((near_by >> (j >> 7)) & 1u)) continue;          // (warp-uniform)
     float dist[kT];
     distances_fp32<kX2, kT>([&](int t) { return row[t]; }, centroids + (size_t)j * kHeadDim, dist);
 #pragma unroll
