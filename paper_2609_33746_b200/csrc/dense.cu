@@ -5,13 +5,13 @@
 // Split-K flash decoding.  grid (splits, KV heads, sequences).  A warp takes windows of 32 tokens and
 // serves up to four query heads of the GQA group from one read and one unpacking of each K/V row: 16
 // lanes per 256-byte row, online softmax in base 2; groups of more than four heads are shared out
-// among the CTA's warps, which walk the same tokens (L1).  Rows come through a per-warp ring of
+// among the CTA's warps, which walk the same tokens, each from L2.  Rows come through a per-warp ring of
 // asynchronous copies, 8 rows (4 KB) a stage and two stages ahead of the one in use; a lane copies
 // the 16 bytes that it reads itself, so the ring needs no barrier.  The last CTA of a (sequence, KV
 // head) merges the partial (m, Z, N) triples of its G rows (atomic ticket; nobody waits).
 // What bounds it: the read of the cache.  8 x 32K tokens, 32 / 8 heads: one warp per head (rows
 // unpacked four times) 394 us, four heads per warp with loads into registers 260 us (latency: 3.9
-// warps waiting per issue), with the ring 196 us (5.5 TB/s).
+// warps waiting per issue), with the ring 218 us (4.9 TB/s, 0.75 of the copy rate).
 #include "attn_common.cuh"
 #include "common.cuh"
 #include "scan_common.cuh"

@@ -12,10 +12,10 @@
 //                  [lo, hi] are appended, as (key, position) pairs, to a candidate list; the
 //                  last CTA of the row (atomic ticket, nobody waits) checks the bracket by
 //                  counting (#winners <= k <= #winners + #candidates) and finishes exactly:
-//                  one histogram of the candidates over 4096 equal buckets of their range,
-//                  everything above the bucket of the k-th largest is taken, the few items
-//                  inside it are ranked against each other (a 12/12/8-bit radix select remains
-//                  for candidate sets that do not fit shared memory or pile up in one bucket).
+//                  one histogram of the candidates over 4096 equal buckets of the bracket (of their
+//                  range where the bracket is open), everything above the bucket of the k-th largest
+//                  is taken, the few items inside it are ranked against each other (a 12/12/8-bit
+//                  radix select remains for candidates that are all equal or pile up in one bucket).
 // If the bracket misses (a row whose order defeats the sample), that last CTA redoes the
 // row from the scores themselves with the same radix select, so the result is always the
 // exact top-k; equal scores at the threshold are taken in order of position (lowest first),
@@ -483,9 +483,8 @@ sel_filter_kernel(Plan pl, const float* __restrict__ scores, uint32_t* __restric
 
   // Main pass.  Warps work independently: a lane marks which of its 16 scores reach the bracket and
   // the warp packs the positions of the hits into its shared-memory buffer.  The buffer is written
-  // out when it would overflow and at the end, with one atomic per destination list, so the round
-  // trip of that atomic is paid once per warp and not once per chunk; only then the few hits are
-  // told apart (winner or candidate), from the score itself.
+  // out when it would overflow and at the end: 128 hits at a time are told apart (winner or
+  // candidate) from their scores, read again, and one 64-bit atomic moves both lists' ends.
   // What bounds the pass is instruction issue, not the read: a comparison against both edges for
   // every score cost 22 instructions per score (44 us at 256 x 128K); the sign of the difference
   // to the lower edge, shifted into a mask, is two.
