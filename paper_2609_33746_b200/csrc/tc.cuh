@@ -439,19 +439,20 @@ template <int DSUB> __device__ __forceinline__ void load_sub(const float* src, f
 }
 // Sub-vectors that have to be compared with all codewords: bit i of `mine` is this lane's i-th.
 // s.load(lane, i, x) reads one, s.distance(i, x, z) compares it as the caller does, s.done(i, x, z) takes
-// the nearest codeword (lower index on ties) in the lane it belongs to.  A few: one after the other, the
-// warp's lanes over the codewords; many (equal keys, all zeros): every lane its own.  All lanes call.
+// the nearest codeword (lower index on ties) in the lane it belongs to.  One after the other, the warp's
+// lanes over the codewords, unless most lanes have one (equal keys, all zeros): then every lane its own.
+// That is told for each i: codebooks with a dozen equal words tie for a few lanes at every i, and 8 x 256
+// tokens took 281 us with the lanes counted over all i, 103 so.  All lanes call.
 // (A call of its own: inlined, it took registers from the search before it, 4 us of an update.)
 template <int DSUB, int kCodes, class S>
 __device__ __noinline__ unsigned long long settle_codewords(unsigned mine, int n_items, S s) {
   constexpr int kAhead = kCodes < 32 ? 1 : DSUB <= 4 ? 8 : 32 / DSUB;      // codewords in flight (they may be in global memory)
   const int lane = threadIdx.x & 31;
-  const int n_lanes = __popc(__ballot_sync(0xffffffffu, mine != 0u));
 #pragma unroll 1
   for (int i = 0; i < n_items; ++i) {
     const unsigned who = __ballot_sync(0xffffffffu, (mine >> i) & 1u);
     float x[DSUB];
-    if (n_lanes > 8 && who) {
+    if (__popc(who) > 16) {
       float d = CUDART_INF_F;
       int at = 0;
       s.load(lane, i, x);
