@@ -249,6 +249,7 @@ __device__ __noinline__ uint32_t walk_row(TsShared& sh, uint32_t k, int32_t* out
     if (!by_pos && lo == hi) by_pos = true;
     __syncthreads();
   }
+  __syncthreads();                                      // (every thread has read what find_range left)
   if (tid == 0) { sh.n_tie = 0u; sh.n_emit = 0u; sh.found_bin = 0u; }
   __syncthreads();
   for (int i = tid; i < r.n; i += kTsThreads) {
