@@ -445,8 +445,10 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
     const uint32_t lk = sh.min_key, hk = sh.max_key;
     if (rank <= (uint32_t)((n + kTile - 1) / kTile)) {  // (more: the maxima give no bound)
       const float mn = key_score(lk), range = key_score(hk) - mn;      // (-inf where no maximum is finite)
-      const bool spread = range > 0.f && range < CUDART_INF_F;
-      const float scale = spread ? __fdividef((float)kTsBins, range) : 0.f, width = spread ? range * (1.f / (float)kTsBins) : 0.f;
+      // (maxima that span less than 1.5e-36 have no finite scale: like equal ones, they bound by the smallest)
+      const float per_range = __fdividef((float)kTsBins, range);
+      const bool spread = range > 0.f && range < CUDART_INF_F && per_range < CUDART_INF_F;
+      const float scale = spread ? per_range : 0.f, width = spread ? range * (1.f / (float)kTsBins) : 0.f;
       constexpr float kLast = (float)(kTsBins - 1);
       auto bucket = [&](float v) { return fminf(fmaxf(truncf((v - mn) * scale), 0.f), kLast); };
       for (int i = tid; i < n_mx; i += kTsThreads) {
@@ -517,9 +519,10 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
   const uint32_t first_lo = lo_key;
   bool whole_list = true, fits;
   for (int attempt = 0;; ++attempt) {
-    fits = sh.n_list <= r.list_cap;
+    // (fewer than k: no bound of the k-th score, which no arithmetic above should give; the row is walked then)
+    fits = sh.n_list <= r.list_cap && sh.n_list >= (uint32_t)k;
     if (attempt == 0) whole_list = fits;
-    if (fits || attempt == 1) break;
+    if (fits || attempt == 1 || sh.n_list < (uint32_t)k) break;
     // once more from a tighter bound: the lower edge of the key range that holds the k-th largest score
     const int shift = max(0, 32 - __clz(hi_key - lo_key) - 9);
     hist = next_hist();

@@ -14,7 +14,7 @@ from paper_2609_33746_b200.index_builder import build_index
 
 pytestmark = pytest.mark.gpu
 
-PATTERNS = ("normal", "equal", "two_values", "sorted", "runs", "outliers", "narrow", "infinite", "nan", "negative")
+PATTERNS = ("normal", "equal", "two_values", "sorted", "runs", "outliers", "narrow", "infinite", "nan", "negative", "tiny")
 
 
 def norms_of(pattern, n, g):
@@ -40,6 +40,8 @@ def norms_of(pattern, n, g):
         x[64:128] = float("nan")
     elif pattern == "negative":
         x -= 100.0
+    elif pattern == "tiny":                              # 512 over the range of the scores is no number
+        x = torch.rand(n, generator=g, device="cuda") * 6e-38
     return x
 
 
