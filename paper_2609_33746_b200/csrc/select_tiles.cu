@@ -668,7 +668,10 @@ cudaError_t launch_t(const Plan& pl, const float* scores, const int32_t* seq_len
 void plan_select_tiles(Plan* pl) {
   pl->sel_tiles = 0;
   pl->n_tile = (pl->N_max + 4 * kTile - 1) / (4 * kTile) * 4;
-  const long long k = ((long long)pl->N_max * pl->ppm + 999999LL) / 1000000LL;
+  // (most that a row selects: the exact set may be rounded up to a multiple; 8 x 128K, multiples of 4096: 883 us in lists
+  // sized without it, which no row fitted into, 373 by the sampled top-k)
+  long long k = ((long long)pl->N_max * pl->ppm + 999999LL) / 1000000LL + (pl->exact_multiple > 1 ? pl->exact_multiple - 1 : 0);
+  if (k > pl->N_max) k = pl->N_max;
   if (4 * (k + (pl->rescore ? k / 4 + 64 : 0)) > 3LL * pl->n_tile) return;
   if (4 * pl->rows < 3 * pl->num_sms || pl->N_max <= 16384 || pl->n_tile > kTsTiles || k > 3072) return;
   pl->sel_tiles = 1;
