@@ -10,9 +10,13 @@
 //   3. a histogram of the listed keys finds the range of the k-th largest, everything above it is taken and
 //      the few items inside it are compared with each other (larger score, then lower position: the stable
 //      rule).
-// A list that overflows (scores that crowd in few tiles) is made again from a tighter bound, taken from a
-// histogram of all scores that reach the first; rows with more equal scores at the threshold than fit are
-// walked as a whole.  The result is exact for every input; a score that is not a number ranks below -inf.
+// A list that is full (scores that crowd in few tiles, or tie) is cut: it keeps the k largest and up to 128 more, what
+// it takes from there on has to reach the cut (by position, where too many scores are equal), and the warps go on
+// where they were.  The warps start at sixteen places of the row, so that the first cut is near the last one
+// also where scores rise along it.  The result is exact for every input; a score that is not a number ranks below -inf.
+// (8 x 128K, 2 %, made again from a tighter bound -> cut -> the other top-k, us: scores that crowd in runs of 40
+// neighbours 347 -> 315 -> 317, of 300 381 -> 348 -> 350, rising 385 -> 350 -> 344; 1 %, rising 311 -> 295 -> 310, all
+// equal 1331 -> 377 -> 1135.)
 //
 // What bounds it: the reads of the tiles, 128 bytes each in random order beside the write-back of the scan's
 // lines (2.2 to 2.6 TB/s, whatever the loop around them), 17 of its 38 us at 256 rows of 128K; then chains of
@@ -32,6 +36,7 @@ constexpr int kTsThreads = 512;
 constexpr int kTsWarps = kTsThreads / 32;
 constexpr int kTsBins = 512;            // histogram ranges, the largest first
 constexpr int kTsTies = 512;            // items ranked one by one
+constexpr int kTsSlack = 128;           // items that a cut of the full list may keep beyond the k-th
 constexpr uint32_t kNanKey = 1u;        // NaN ranks below -inf: taken only when nothing else is left
 constexpr int kTsTiles = 32 * kTsThreads;      // tiles of the longest row (a bit each of a thread's mask)
 
@@ -48,9 +53,11 @@ struct TsShared {
   alignas(16) uint32_t hist[kTsBins];
   uint2 ties[kTsTies];                  // (key, position)
   uint32_t warp_n[kTsWarps];
-  uint32_t n_list, n_tiles, n_tie, n_emit;
+  int next[kTsWarps], end[kTsWarps];            // of the listed tiles, those that a warp has still to read
+  uint32_t n_list, n_tie, n_emit;
   uint32_t found_bin, found_above, found_count;
   uint32_t min_key, max_key, top_key, m_key;    // finite maxima; all maxima; the scan's segments
+  uint32_t cut_key, cut_pos;                    // what the list takes: keys above, or equal and before the position
   int n, k;
   Row row;
   BgRow bg;
@@ -108,12 +115,18 @@ __device__ __noinline__ void find_range(TsShared& sh, const uint32_t* hist, uint
 __device__ __forceinline__ float floor_of(uint32_t key) { return key > kNanKey ? key_score(key) : -CUDART_INF_F; }
 __device__ __forceinline__ uint32_t ranked_key(float x) { return x == x ? score_key(x) : kNanKey; }
 
+// The tiles that reach lo_f, in order of position (a thread looks at neighbouring ones), shared out among the warps;
+// empties the list.
 __device__ __noinline__ void list_tiles(TsShared& sh, float lo_f) {
   const Row& r = sh.row;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = (r.n_tiles / 4 + kTsThreads - 1) / kTsThreads * 4;
+  const int first = tid * per;
   uint32_t hit = 0u;
-  for (int o = tid, u = 0; o < r.n_tiles; o += kTsThreads, ++u)
-    if (!(r.mx[o] < lo_f)) hit |= 1u << u;
+  for (int u = 0; u < per && first + u < r.n_tiles; u += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(r.mx + first + u);
+    hit |= ((v.x < lo_f ? 0u : 1u) | (v.y < lo_f ? 0u : 2u) | (v.z < lo_f ? 0u : 4u) | (v.w < lo_f ? 0u : 8u)) << u;
+  }
   const uint32_t mine = (uint32_t)__popc(hit);
   uint32_t inc = mine;
 #pragma unroll
@@ -126,55 +139,60 @@ __device__ __noinline__ void list_tiles(TsShared& sh, float lo_f) {
   const uint32_t w = lane < kTsWarps ? sh.warp_n[lane] : 0u;
   uint32_t at = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + inc - mine;
   if (warp == 0) {
-    const uint32_t all = __reduce_add_sync(0xffffffffu, w);
-    if (lane == 0) { sh.n_tiles = all; sh.n_list = 0u; }
+    const int all = (int)__reduce_add_sync(0xffffffffu, w);
+    if (lane < kTsWarps) { sh.next[lane] = all * lane / kTsWarps; sh.end[lane] = all * (lane + 1) / kTsWarps; }
+    if (lane == 0) sh.n_list = 0u;
   }
   while (hit) {
     const int u = __ffs(hit) - 1;
     hit &= hit - 1u;
-    r.ids[at++] = (uint16_t)(tid + u * kTsThreads);
+    r.ids[at++] = (uint16_t)(first + u);
   }
   __syncthreads();
 }
 
-// The scores of the listed tiles that reach lo_f, into the list, or, where hist is given, only counted by
-// range of their keys below hi_key.  A warp takes 16 tiles at a time: copied to its 2 KB of shared memory
-// whole lines at a time, then two lanes a tile, so that a score costs two instructions (the sign of the
-// difference to the number below the bound, into a mask) and what follows is per hit.  (A ballot per score instead: 50
-// instructions a tile, and 40 thousand clocks for 1344 tiles of two CTAs per SM.)
+// The scores of the warp's listed tiles that reach the cut (a larger key, or an equal one before a position), into
+// the list.  A warp takes 16 tiles at a time: copied to its 2 KB of shared memory whole lines at a time, then two
+// lanes a tile, so that a score costs two instructions (the sign of the difference to the number below the cut,
+// into a mask) and what follows is per hit.  (A ballot per score instead: 50 instructions a tile.)
+// Ends early when the list is full (n_list beyond its capacity); the warp's next tile is then the first not listed.
 // 16-byte chunk c of tile t sits at c ^ (t & 7): the lanes' reads then have no bank conflicts.
 constexpr int kBatch = 16;
 constexpr int kStageBytes = kTsWarps * kBatch * kTile * 4;
-__device__ __noinline__ void gather(TsShared& sh, uint32_t lo_key, uint32_t* hist, uint32_t hi_key, int shift) {
+__device__ __noinline__ void gather(TsShared& sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const Row& r = sh.row;
-  const int m = (int)sh.n_tiles, n = r.n;
+  const int n = r.n;
   const uint32_t cap = r.list_cap;
   const float* rs = r.rs;
   const uint16_t* ids = r.ids;
   unsigned char* stage = r.stage + warp * (kBatch * kTile * 4);
   const int t = lane >> 1, half = lane & 1;
   const unsigned char* mine = stage + t * 128;
-  const float lo_f = floor_of(lo_key);
+  const uint32_t cut_key = sh.cut_key, cut_pos = sh.cut_pos;
+  const float lo_f = floor_of(cut_key);
   const bool all = !(lo_f > -CUDART_INF_F);             // (at or below -inf: every position counts)
-  // the next number below the bound: what reaches the bound is above it, and what is no number is not
+  // the next number below the cut: what reaches the cut is above it, and what is no number is not
   const float under = lo_f == 0.f ? -__uint_as_float(1u) : key_score(score_key(lo_f) - 1u);
+  int e0 = sh.next[warp];
+  const int e1 = sh.end[warp];
 #pragma unroll 1
-  for (int e0 = warp * kBatch; e0 < m; e0 += kTsWarps * kBatch) {
+  for (; e0 < e1; e0 += kBatch) {
+    if (__any_sync(0xffffffffu, *const_cast<volatile uint32_t*>(&sh.n_list) > cap)) break;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int tt = 4 * i + (lane >> 3), c = lane & 7;
-      const int p = e0 + tt < m ? (int)ids[e0 + tt] * kTile + 4 * c : n;
+      const int p = e0 + tt < e1 ? (int)ids[e0 + tt] * kTile + 4 * c : n;
       // (the row stride is a multiple of 4 scores: a partial group of four stays inside the row)
       if (p < n)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
                      ::"r"(smem_u32(stage) + (uint32_t)(tt * 128 + ((c ^ (tt & 7)) << 4))), "l"(rs + p) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const int p0 = e0 + t < m ? (int)ids[e0 + t] * kTile + 16 * half : n;
+    const int p0 = e0 + t < e1 ? (int)ids[e0 + t] * kTile + 16 * half : n;
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
-    uint32_t reach = 0u;                                // bit 15 - e: score e of this lane reaches the bound
+    uint32_t reach = 0u;                                // bit 15 - e: score e of this lane reaches the cut
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float4 v = *reinterpret_cast<const float4*>(mine + (((4 * half + j) ^ (t & 7)) << 4));
@@ -183,102 +201,43 @@ __device__ __noinline__ void gather(TsShared& sh, uint32_t lo_key, uint32_t* his
       reach = __funnelshift_l(__float_as_uint(under - v.z), reach, 1);
       reach = __funnelshift_l(__float_as_uint(under - v.w), reach, 1);
     }
+    auto key_at = [&](int e) {
+      return ranked_key(*reinterpret_cast<const float*>(mine + (((4 * half + (e >> 2)) ^ (t & 7)) << 4) + (e & 3) * 4));
+    };
     const uint32_t valid = 0xffffu & ~(0xffffu >> min(16, max(0, n - p0)));      // (what was not copied is stale)
     uint32_t hit = (all ? valid : reach & valid) << 16;
-    uint32_t slot = 0u;
-    if (hist == nullptr) {
-      const uint32_t cnt = (uint32_t)__popc(hit);
-      uint32_t inc = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += u;
+    if (all || cut_pos != 0xffffffffu) {                // equal keys count by position
+      for (uint32_t left = hit; left;) {
+        const int e = __clz(left);
+        left ^= 0x80000000u >> e;
+        const uint32_t key = key_at(e);
+        if (key < cut_key || (key == cut_key && (uint32_t)(p0 + e) >= cut_pos)) hit ^= 0x80000000u >> e;
       }
-      if (lane == 31) slot = atomicAdd(&sh.n_list, inc);
-      slot = __shfl_sync(0xffffffffu, slot, 31) + inc - cnt;
     }
+    const uint32_t cnt = (uint32_t)__popc(hit);
+    uint32_t inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += u;
+    }
+    uint32_t slot = 0u;
+    if (lane == 31) slot = atomicAdd(&sh.n_list, inc);
+    slot = __shfl_sync(0xffffffffu, slot, 31);
+    const uint32_t sum = __shfl_sync(0xffffffffu, inc, 31);
+    if (slot + sum > cap) {                             // full: these tiles once more after the next cut
+      for (uint32_t i = slot + lane; i < cap; i += 32) r.list[i] = make_uint2(0u, 0u);     // (below every key)
+      break;
+    }
+    slot += inc - cnt;
     while (hit) {
       const int e = __clz(hit);
       hit ^= 0x80000000u >> e;
-      const uint32_t key = ranked_key(*reinterpret_cast<const float*>(mine + (((4 * half + (e >> 2)) ^ (t & 7)) << 4) + (e & 3) * 4));
-      if (hist != nullptr) {
-        if (key >= lo_key && key <= hi_key) atomicAdd(&hist[(hi_key - key) >> shift], 1u);
-      } else if (slot < cap) {
-        r.list[slot] = make_uint2(key, (uint32_t)(p0 + e));
-      }
-      ++slot;
+      r.list[slot++] = make_uint2(key_at(e), (uint32_t)(p0 + e));
     }
     __syncwarp();
   }
-  __syncthreads();
-}
-
-// One CTA walks the whole row: the key's range (then, among equal keys, the position's) that holds the k-th
-// largest is narrowed 512-fold until what is inside can be ranked.
-__device__ __noinline__ uint32_t walk_row(TsShared& sh, uint32_t k, int32_t* out, const uint16_t* lids, int n_list, float* mass) {
-  const int tid = threadIdx.x;
-  const Row r = sh.row;
-  auto take = [&](int pos, uint32_t key) {              // (mass: null where there is no background to take it out of)
-    if (mass != nullptr) bg_take_out(sh.bg, sh.seg, pos, key_score(key), min((uint32_t)lids[pos], (uint32_t)(n_list - 1)), mass);
-  };
-  uint32_t lo = kNanKey, hi = 0xffffffffu, above = 0u, inside = 0u;
-  int p_lo = 0, p_hi = r.n - 1;
-  bool by_pos = false;
-  for (;;) {
-    for (int i = tid; i < kTsBins; i += kTsThreads) sh.hist[i] = 0u;
-    __syncthreads();
-    const uint32_t span = by_pos ? (uint32_t)(p_hi - p_lo) : hi - lo;
-    const int shift = max(0, 32 - __clz(span) - 9);
-    for (int i = tid; i < r.n; i += kTsThreads) {
-      const uint32_t key = ranked_key(__ldcg(r.rs + i));
-      if (by_pos ? key == lo && i >= p_lo && i <= p_hi : key >= lo && key <= hi)
-        atomicAdd(&sh.hist[(by_pos ? (uint32_t)(i - p_lo) : hi - key) >> shift], 1u);
-    }
-    find_range(sh, sh.hist, k - above);
-    above += sh.found_above;
-    inside = sh.found_count;
-    const uint32_t bin = sh.found_bin;
-    if (by_pos) {
-      p_lo += (int)(bin << shift);
-      p_hi = min(p_hi, p_lo + (int)((1u << shift) - 1u));
-    } else {
-      hi -= bin << shift;
-      lo = hi - min(hi - lo, (1u << shift) - 1u);
-    }
-    if (inside <= (uint32_t)kTsTies) break;
-    if (!by_pos && lo == hi) by_pos = true;
-    __syncthreads();
-  }
-  __syncthreads();                                      // (every thread has read what find_range left)
-  if (tid == 0) { sh.n_tie = 0u; sh.n_emit = 0u; sh.found_bin = 0u; }
-  __syncthreads();
-  for (int i = tid; i < r.n; i += kTsThreads) {
-    const uint32_t key = ranked_key(__ldcg(r.rs + i));
-    if (key > hi || (by_pos && key == lo && i < p_lo)) {
-      const uint32_t at = atomicAdd(&sh.n_emit, 1u);
-      if (at < k) out[at] = i;
-      take(i, key);
-    } else if (key >= lo && (!by_pos || i <= p_hi)) {
-      const uint32_t at = atomicAdd(&sh.n_tie, 1u);
-      if (at < (uint32_t)kTsTies) sh.ties[at] = make_uint2(key, (uint32_t)i);
-    }
-  }
-  __syncthreads();
-  for (uint32_t i = tid; i < inside; i += kTsThreads) {
-    const uint2 it = sh.ties[i];
-    uint32_t rank = 0u;
-    for (uint32_t j = 0; j < inside; ++j) {
-      const uint2 o = sh.ties[j];
-      rank += (o.x > it.x || (o.x == it.x && o.y < it.y)) ? 1u : 0u;
-    }
-    if (above + rank < k) {
-      out[above + rank] = (int)it.y;
-      take((int)it.y, it.x);
-      if (above + rank == k - 1u) sh.found_bin = it.x;
-    }
-  }
-  __syncthreads();
-  return sh.found_bin;
+  if (lane == 0) sh.next[warp] = e0;
 }
 
 // What the re-score wants to know of the top-k (fp16 tables): the listed scores, their bound and number.
@@ -306,6 +265,8 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
     sh.min_key = 0xffffffffu;
     sh.max_key = sh.top_key = sh.m_key = 0u;
     sh.n_tie = sh.n_emit = 0u;
+    sh.cut_key = kNanKey;
+    sh.cut_pos = 0xffffffffu;
     Row& r = sh.row;
     r.rs = scores + (size_t)row * pl.N_max;
     r.list = reinterpret_cast<uint2*>(s_dyn + kTsHead);
@@ -328,13 +289,12 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
   const int n_mx = r.n_tiles;
   if constexpr (kBg) bg_segment_ends(bg, seg, kTsThreads);
   // The steps' instructions are fetched while the scan still runs (a first call costs 1 to 4 thousand clocks
-  // more than the next): one tile that nothing reaches.
-  if (tid == 0) { sh.n_tiles = 0u; sh.n_list = 0u; }
+  // more than the next): no tile is listed.
   {
     for (int o = tid; o < n_mx; o += kTsThreads) r.mx[o] = -1.f;
     __syncthreads();
     list_tiles(sh, 0.f);
-    gather(sh, score_key(0.f), nullptr, 0u, 0);
+    gather(sh);
     find_range(sh, sh.hist, 1u);
   }
   pdl_wait();
@@ -479,6 +439,7 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
     }
     lo_key = min(lo_key, hi_key);
   }
+  if (tid == 0) sh.cut_key = lo_key;
   list_tiles(sh, floor_of(lo_key));
 
   // ---- the lists' totals (stored, not added: the selected tokens are taken out with atomics after barriers)
@@ -514,29 +475,112 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
     }
   }
 
-  // ---- 2. what reaches the bound
-  gather(sh, lo_key, nullptr, 0u, 0);
-  const uint32_t first_lo = lo_key;
-  bool whole_list = true, fits;
-  for (int attempt = 0;; ++attempt) {
-    // (fewer than k: no bound of the k-th score, which no arithmetic above should give; the row is walked then)
-    fits = sh.n_list <= r.list_cap && sh.n_list >= (uint32_t)k;
-    if (attempt == 0) whole_list = fits;
-    if (fits || attempt == 1 || sh.n_list < (uint32_t)k) break;
-    // once more from a tighter bound: the lower edge of the key range that holds the k-th largest score
-    const int shift = max(0, 32 - __clz(hi_key - lo_key) - 9);
-    hist = next_hist();
-    gather(sh, lo_key, hist, hi_key, shift);
-    find_range(sh, hist, (uint32_t)k);
-    const uint32_t below = (sh.found_bin + 1u) << shift;
-    if (sh.found_count > 0u && below - 1u < hi_key - lo_key) lo_key = hi_key - (below - 1u);
-    list_tiles(sh, floor_of(lo_key));
-    gather(sh, lo_key, nullptr, 0u, 0);
+  int32_t* out = sel_idx + (size_t)row * pl.k_max;
+  [[maybe_unused]] auto take_out = [&](int pos, uint32_t key, uint32_t lid) {
+    if (has_bg) bg_take_out(bg, seg, pos, key_score(key), min(lid, (uint32_t)(pl.n_list - 1)), mass);
+  };
+  [[maybe_unused]] const uint16_t* row_lids = lids;
+  if constexpr (kBg) row_lids = lids + bg.lid_base;
+  constexpr int kPreLids = 4;
+  [[maybe_unused]] uint32_t my_lid[kPreLids] = {};      // list ids of this thread's first listed scores
+
+  // ---- 2. what reaches the bound, 3. the range of the k-th largest of what is listed: of keys [lo, hi] and, where
+  // too many share one key, of positions [p_lo, p_hi].  A list that is full is cut there and goes on.
+  uint32_t lo, hi, p_lo, p_hi, above, inside, n_mine;
+  bool first_cut = true;                                // all that reaches the first bound is listed
+#pragma unroll 1
+  for (;;) {
+    gather(sh);
+    __syncthreads();
+    const bool full = sh.n_list > r.list_cap;
+    n_mine = min(sh.n_list, r.list_cap);
+    if (n_mine < (uint32_t)k && sh.cut_key != kNanKey) {
+      // no bound of the k-th score (no arithmetic above should give one): all scores
+      __syncthreads();
+      if (tid == 0) { sh.cut_key = kNanKey; sh.cut_pos = 0xffffffffu; }
+      list_tiles(sh, -CUDART_INF_F);
+      first_cut = false;
+      continue;
+    }
+    if constexpr (kBg) {
+      if (!full) {
+#pragma unroll
+        for (int u = 0; u < kPreLids; ++u)
+          if (u * kTsThreads + tid < (int)n_mine) my_lid[u] = (uint32_t)row_lids[r.list[u * kTsThreads + tid].y];
+      }
+    }
+    lo = sh.cut_key, hi = hi_key, p_lo = 0u, p_hi = (uint32_t)n - 1u;
+    above = 0u;
+    bool by_pos = false;
+#pragma unroll 1
+    for (;;) {
+      const uint32_t span = by_pos ? p_hi - p_lo : hi - lo;
+      const int shift = max(0, 32 - __clz(span) - 9);
+      hist = next_hist();
+#pragma unroll 1
+      for (uint32_t i = tid; i < n_mine; i += kTsThreads) {
+        const uint2 it = r.list[i];
+        if (it.x >= lo && it.x <= hi && it.y >= p_lo && it.y <= p_hi)
+          atomicAdd(&hist[(by_pos ? it.y - p_lo : hi - it.x) >> shift], 1u);
+      }
+      find_range(sh, hist, (uint32_t)k - above);
+      above += sh.found_above;
+      inside = sh.found_count;
+      const uint32_t down = sh.found_bin << shift, width = (1u << shift) - 1u;
+      if (by_pos) {
+        p_lo += down;
+        p_hi = p_lo + min(p_hi - p_lo, width);
+      } else {
+        hi -= down;
+        lo = hi - min(hi - lo, width);
+      }
+      if (inside <= (uint32_t)(full ? kTsSlack : kTsTies)) break;
+      if (lo == hi) by_pos = true;
+    }
+    if (!full) break;
+    // the list keeps what is in the range or above it
+    const uint32_t cut_pos = by_pos ? p_hi + 1u : 0xffffffffu;
+    if (tid == 0) { sh.n_list = 0u; sh.cut_key = lo; sh.cut_pos = cut_pos; }
+    constexpr int kMove = 4;
+#pragma unroll 1
+    for (uint32_t i0 = 0; i0 < n_mine; i0 += kMove * kTsThreads) {
+      uint2 it[kMove];
+#pragma unroll
+      for (int u = 0; u < kMove; ++u) {
+        const uint32_t i = i0 + u * kTsThreads + tid;
+        it[u] = i < n_mine ? r.list[i] : make_uint2(0u, 0u);
+      }
+      __syncthreads();                                  // (what is kept lands before what has been read)
+#pragma unroll
+      for (int u = 0; u < kMove; ++u) {
+        const bool keep = it[u].x > lo || (it[u].x == lo && it[u].y < cut_pos);
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        uint32_t at = 0u;
+        if (lane == 0 && m) at = atomicAdd(&sh.n_list, (uint32_t)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+        if (keep) r.list[at] = it[u];
+      }
+    }
+    // and of its other tiles a warp keeps those that reach the cut
+    const float lo_f = floor_of(lo);
+    const int warp = tid >> 5, e0 = sh.next[warp], e1 = sh.end[warp];
+    int e_end = e0;
+#pragma unroll 1
+    for (int i0 = e0; i0 < e1; i0 += 32) {
+      const uint16_t tile = r.ids[min(i0 + lane, e1 - 1)];
+      const bool keep = i0 + lane < e1 && !(r.mx[tile] < lo_f);
+      const unsigned m = __ballot_sync(0xffffffffu, keep);
+      if (keep) r.ids[e_end + __popc(m & ((1u << lane) - 1u))] = tile;
+      e_end += __popc(m);
+      __syncwarp();
+    }
+    if (lane == 0) sh.end[warp] = e_end;
+    __syncthreads();
+    first_cut = false;
   }
-  const uint32_t n_mine = min(sh.n_list, r.list_cap);
   if (cand.cand != nullptr) {
     // (the re-score trusts the list only where it reaches down to the first bound: counter 0)
-    if (whole_list) {
+    if (first_cut) {
       uint2* dst = cand.cand + (size_t)row * pl.cand_cap;
       for (uint32_t i = tid; i < n_mine; i += kTsThreads)
         if (i < (uint32_t)pl.cand_cap) dst[i] = r.list[i];
@@ -545,103 +589,65 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
       cand.counters[row * 4 + 0] = 1u;
     }
     if (tid == 0) {
-      cand.rowstate[row * 4 + 0] = __float_as_int(floor_of(first_lo));
+      cand.rowstate[row * 4 + 0] = __float_as_int(floor_of(lo_key));
       cand.rowstate[row * 4 + 1] = __float_as_int(CUDART_INF_F);
       cand.rowstate[row * 4 + 2] = k;
       cand.rowstate[row * 4 + 3] = n;
     }
   }
-  int32_t* out = sel_idx + (size_t)row * pl.k_max;
-  [[maybe_unused]] auto take_out = [&](int pos, uint32_t key, uint32_t lid) {
-    if (has_bg) bg_take_out(bg, seg, pos, key_score(key), min(lid, (uint32_t)(pl.n_list - 1)), mass);
-  };
-  [[maybe_unused]] const uint16_t* row_lids = lids;
-  if constexpr (kBg) row_lids = lids + bg.lid_base;
 
-  // ---- 3. the k-th largest of what is listed
-  constexpr int kPreLids = 4;
-  [[maybe_unused]] uint32_t my_lid[kPreLids] = {};      // list ids of this thread's first listed scores
-  if constexpr (kBg) {
-#pragma unroll
-    for (int u = 0; u < kPreLids; ++u)
-      if (u * kTsThreads + tid < (int)n_mine) my_lid[u] = (uint32_t)row_lids[r.list[u * kTsThreads + tid].y];
+  // ---- everything above the range, and the best of what is inside (larger score, then lower position)
+#pragma unroll 1
+  for (uint32_t i = tid; i < n_mine; i += kTsThreads) {
+    const uint2 it = r.list[i];
+    if (it.x >= lo && it.x <= hi && it.y >= p_lo && it.y <= p_hi)
+      sh.ties[min(atomicAdd(&sh.n_tie, 1u), (uint32_t)kTsTies - 1u)] = it;
   }
-  auto for_all_items = [&](auto f) {                    // f(key, position)
+  __syncthreads();
+  const uint32_t need = (uint32_t)k - above;
+  int u = 0;
 #pragma unroll 1
-    for (uint32_t i = tid; i < n_mine; i += kTsThreads) f(r.list[i].x, r.list[i].y);
-  };
-  uint32_t above = 0u, inside = 0u;
-  if (fits) {
-    uint32_t lo = lo_key, hi = hi_key;
-#pragma unroll 1
-    for (;;) {
-      const int shift = max(0, 32 - __clz(hi - lo) - 9);
-      hist = next_hist();
-      for_all_items([&](uint32_t key, uint32_t) {
-        if (key >= lo && key <= hi) atomicAdd(&hist[(hi - key) >> shift], 1u);
-      });
-      find_range(sh, hist, (uint32_t)k - above);
-      above += sh.found_above;
-      inside = sh.found_count;
-      hi -= sh.found_bin << shift;
-      lo = hi - min(hi - lo, (1u << shift) - 1u);
-      if (inside <= (uint32_t)kTsTies || lo == hi) break;
-    }
-    fits = inside <= (uint32_t)kTsTies;
-    if (fits) {
-      for_all_items([&](uint32_t key, uint32_t pos) {
-        if (key >= lo && key <= hi) sh.ties[min(atomicAdd(&sh.n_tie, 1u), (uint32_t)kTsTies - 1u)] = make_uint2(key, pos);
-      });
-      __syncthreads();
-      const uint32_t need = (uint32_t)k - above;
-      int u = 0;
-#pragma unroll 1
-      for (uint32_t i0 = tid & ~31; i0 < n_mine; i0 += kTsThreads, ++u) {
-        const uint32_t i = i0 + lane;
-        const uint32_t key = i < n_mine ? r.list[i].x : 0u, pos = i < n_mine ? r.list[i].y : 0u;
-        bool take = i < n_mine && key > hi;
-        const unsigned m = __ballot_sync(0xffffffffu, take);
-        uint32_t at = 0u;
-        if (lane == 0 && m) at = atomicAdd(&sh.n_emit, (uint32_t)__popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-        if (take) {
-          if (at < (uint32_t)k) out[at] = (int)pos;
-        } else if (i < n_mine && key >= lo) {
-          uint32_t better = 0u;
-          for (uint32_t j = 0; j < inside; ++j) {
-            const uint2 o = sh.ties[j];
-            better += (o.x > key || (o.x == key && o.y < pos)) ? 1u : 0u;
-          }
-          if (better < need) {
-            out[above + better] = (int)pos;
-            take = true;
-            if (better == need - 1u) {
-              sel_count[row] = k;
-              kth[row] = key_score(key);
-            }
-          }
-        }
-        if constexpr (kBg) {
-          if (take) {
-            uint32_t lid = u == 0 ? my_lid[0] : u == 1 ? my_lid[1] : u == 2 ? my_lid[2] : my_lid[3];
-            if (u >= kPreLids) lid = (uint32_t)row_lids[pos];
-            take_out((int)pos, key, lid);
-          }
+  for (uint32_t i0 = tid & ~31; i0 < n_mine; i0 += kTsThreads, ++u) {
+    const uint32_t i = i0 + lane;
+    const uint32_t key = i < n_mine ? r.list[i].x : 0u, pos = i < n_mine ? r.list[i].y : 0u;
+    bool take = key > hi || (key == lo && pos < p_lo);
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    uint32_t at = 0u;
+    if (lane == 0 && m) at = atomicAdd(&sh.n_emit, (uint32_t)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+    if (take) {
+      if (at < (uint32_t)k) out[at] = (int)pos;
+    } else if (key >= lo && pos <= p_hi) {
+      uint32_t better = 0u;
+      for (uint32_t j = 0; j < inside; ++j) {
+        const uint2 o = sh.ties[j];
+        better += (o.x > key || (o.x == key && o.y < pos)) ? 1u : 0u;
+      }
+      if (better < need) {
+        out[above + better] = (int)pos;
+        take = true;
+        if (better == need - 1u) {
+          sel_count[row] = k;
+          kth[row] = key_score(key);
         }
       }
-      if (tid == 0 && (need == 0u || inside < need)) atomicOr(status, kStatusCountMismatch);
-      return;
+    }
+    if constexpr (kBg) {
+      if (take) {
+        uint32_t lid = u == 0 ? my_lid[0] : u == 1 ? my_lid[1] : u == 2 ? my_lid[2] : my_lid[3];
+        if (u >= kPreLids) lid = (uint32_t)row_lids[pos];
+        take_out((int)pos, key, lid);
+      }
     }
   }
-  // ---- too many for the list: walk the row
-  __syncthreads();
-  const uint32_t kstar = walk_row(sh, (uint32_t)k, out, row_lids, pl.n_list, has_bg ? mass : nullptr);
-  if (tid == 0) {
-    sel_count[row] = k;
-    kth[row] = key_score(kstar);
+  if (tid == 0 && (need == 0u || inside < need)) {      // (never: the list holds the k largest)
+    sel_count[row] = 0;
+    kth[row] = CUDART_NAN_F;
+    atomicOr(status, kStatusCountMismatch);
   }
 }
 
+constexpr size_t kSmemSplits[] = {100 * 1024, 132 * 1024, 164 * 1024, 196 * 1024, 228 * 1024};     // shared, the rest L1
 size_t smem_bytes(const Plan& pl) {
   return kTsHead + (size_t)pl.sel_list * 8 + kStageBytes + (size_t)pl.n_tile * 6;
 }
@@ -675,7 +681,18 @@ void plan_select_tiles(Plan* pl) {
   if (4 * (k + (pl->rescore ? k / 4 + 64 : 0)) > 3LL * pl->n_tile) return;
   if (4 * pl->rows < 3 * pl->num_sms || pl->N_max <= 16384 || pl->n_tile > kTsTiles || k > 3072) return;
   pl->sel_tiles = 1;
-  pl->sel_list = (int)((7 * k / 4 + 512 + 15) / 16 * 16);
+  // A full list keeps k + 128 scores at most and a warp brings up to 512 at a time.  What the split of the SM's memory
+  // that holds these CTAs has left goes to the list too (fewer cuts where scores crowd); a larger split would be
+  // taken from L1 (8 x 128K, 1 %: lists of 5.9 K scores 279 us, of 2.8 K 275).
+  const long long most = 7 * k / 4 > k + kTsSlack ? 7 * k / 4 : k + kTsSlack;
+  pl->sel_list = (int)((most + 32 * 16 + 15) / 16 * 16);
+  const size_t need = smem_bytes(*pl) + 1024;           // (1 KB per CTA is the system's)
+  const size_t ctas = 2 * need <= kSmemSplits[4] ? 2 : 1;
+  for (size_t split : kSmemSplits)
+    if (ctas * need <= split) {
+      pl->sel_list += (int)((split / ctas - need) / 128 * 16);
+      break;
+    }
 }
 
 cudaError_t launch_select_tiles(const Plan& pl, const WsLayout& L, char* ws, const float* scores, const int32_t* seq_lens,
