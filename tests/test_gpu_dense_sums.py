@@ -71,3 +71,56 @@ def test_an_infinite_value_stays_one(group, dtype):
     keep[5] = keep[90] = False
     torch.testing.assert_close(out[:group, keep], clean[:group, keep], rtol=2.0 ** -7, atol=2.0 ** -12)
     assert torch.equal(out[group:], clean[group:])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("group,n", [(1, 31), (4, 700), (8, 700), (16, 3000)])
+def test_infinite_values_in_many_places(group, n, dtype):
+    """Infinite values of either sign and values that are no numbers, several in a dim and in a stage of 16 tokens:
+    infinite, no number and finite where the weighted sum in float64 is."""
+    g = torch.Generator(device="cuda").manual_seed(group)
+    q, k, v = (torch.randn(s, generator=g, device="cuda").to(dtype) for s in ((2 * group, D), (2, n, D), (2, n, D)))
+    bad = torch.tensor([float("inf"), -float("inf"), float("nan")], device="cuda", dtype=dtype)
+    at, dim, what = (torch.randint(0, m, (40,), generator=g, device="cuda") for m in (n, 100, 3))
+    v[0, at, dim] = bad[what]
+    v[0, :, 127] = float("inf")
+    out = run(q, k, v, n, dtype, 2).double()
+    w = (q.double().view(2, group, D) / math.sqrt(D) @ k.double().transpose(1, 2)).softmax(-1)
+    want = (w @ v.double()).view(-1, D)
+    assert torch.equal(out.isnan(), want.isnan()) and torch.equal(out.isinf(), want.isinf())
+    assert torch.equal(out[want.isinf()], want[want.isinf()])
+    size = (w @ v.double().abs()).view(-1, D)
+    fine = want.isfinite()
+    assert bool(((out - want).abs() <= 2.0 ** -7 * want.abs() + 2.0 ** -12 * size)[fine].all())
+
+
+@pytest.mark.parametrize("group", [4, 8])
+def test_an_infinite_value_costs_no_time(group):
+    """The 16 tokens around it are taken again, nothing else (13 times the call when a warp repeated all of its tokens)."""
+    n, kv_heads = 65536, 4
+    g = torch.Generator(device="cuda").manual_seed(group)
+    q, k, v = (torch.randn(s, generator=g, device="cuda").bfloat16() for s in ((kv_heads * group, D), (kv_heads, n, D), (kv_heads, n, D)))
+    pages = n // PAGE
+    table = torch.arange(pages, dtype=torch.int32, device="cuda").view(1, pages)
+    kc, vc = (x.transpose(0, 1).contiguous() for x in (k, v))
+    kv = pqhsa.make_paged_kv(kc, vc, PAGE * kv_heads * D, kv_heads * D, D, table)
+    p = pqhsa.make_params(batch=1, n_q_heads=q.shape[0], n_kv_heads=kv_heads, n_list=16, pq_m=8, max_seq_len=n,
+                          max_pages_per_seq=pages, budget_ppm=10000, dtype="bf16", page_size=PAGE)
+    ws = torch.empty(pqhsa.dense_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    out, seq = torch.zeros_like(q), torch.tensor([n], dtype=torch.int32, device="cuda")
+
+    def time_of():
+        best = float("inf")
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(4):
+                pqhsa.dense_decode(p, q, kv, seq, out, ws)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    clean = time_of()
+    vc.view(-1)[n * kv_heads * D // 2 + 77] = float("inf")
+    assert time_of() <= 1.5 * clean
