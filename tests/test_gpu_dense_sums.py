@@ -57,6 +57,52 @@ def test_weights_of_every_size(group, n, spread, dtype):
     assert bool(((out - want).abs() <= ulp * want.abs() + bound).all())
 
 
+def cancelling(group, n, head, dtype, seed, device="cuda"):
+    """Queries and keys of one dim, so that dot products are exact; values whose sum weighted for one head of each
+    KV head is next to nothing: the last three take back what the others leave."""
+    g = torch.Generator().manual_seed(seed)
+    q, k = torch.zeros(2, group, D), torch.zeros(2, n, D)
+    q[..., 0], k[..., 0] = 1 + 3 * torch.rand(2, group, generator=g), 6 * torch.rand(2, n, generator=g)
+    q, k, v = q.to(dtype).view(-1, D), k.to(dtype), torch.randn(2, n, D, generator=g).to(dtype)
+    w = (q.double().view(2, group, D)[:, head:head + 1] / math.sqrt(D) @ k.double().transpose(1, 2)).softmax(-1)[:, 0, :, None]
+    left = (w * v.double())[:, :-3].sum(1)
+    for j in (-3, -2, -1):
+        v[:, j] = (-left / w[:, j]).to(dtype)
+        left = left + w[:, j] * v[:, j].double()
+    return [x.to(device) for x in (q, k, v, left, (w * v.double().abs()).sum(1))]
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("group", [1, 4, 8, 16])
+@pytest.mark.parametrize("n", [5, 8, 16, 21])
+def test_sums_that_cancel(group, n, dtype):
+    """What is left of values that cancel shows the bits of the weights, not the output's rounding.  Tolerance, of the
+    weighted magnitudes: exponentials to 2 ulp (2^-22), their argument of at most 3 rounded once (2^-22.5 times ln 2), a few
+    fp32 additions (2^-24 each): 2^-20.  (Without the third bf16 number of a weight the errors reach 2^-18.9 and more in
+    every case, without the second fp16 one 2^-12.5; the third fp16 number is below the exponential's error.)"""
+    for seed in range(4):
+        head = seed % group
+        q, k, v, want, size = cancelling(group, n, head, dtype, 100 * n + seed)
+        out = run(q, k, v, n, dtype, 2).double().view(2, group, D)[:, head]
+        assert bool(((out - want).abs() <= 2.0 ** -20 * size + 2.0 ** -11 * want.abs()).all()), float(((out - want).abs() / size).max())
+
+
+@pytest.mark.parametrize("dtype,half_ulp", [(torch.bfloat16, 2.0 ** -9), (torch.float16, 2.0 ** -12)])
+@pytest.mark.parametrize("group", [4, 8])
+@pytest.mark.parametrize("log2_weight", [24, 41, 48])
+def test_many_small_weights_beside_a_large_one(log2_weight, group, dtype, half_ulp):
+    """60 thousand weights far below that of a token whose values are zero: the output is theirs alone."""
+    n = 60001
+    q, k, v = torch.zeros((2 * group, D)), torch.zeros((2, n, D)), torch.full((2, n, D), 60000.0)
+    q[:, 0], k[:, n // 2, 0], v[:, n // 2] = 16.0, log2_weight * math.log(2) * math.sqrt(D) / 16, 0.0
+    q, k, v = (x.cuda().to(dtype) for x in (q, k, v))
+    out = run(q, k, v, n, dtype, 2).double()
+    w = (q.double().view(2, group, D) / math.sqrt(D) @ k.double().transpose(1, 2)).softmax(-1)
+    want = (w @ v.double()).view(-1, D)
+    # (fp32: 2^-24 of the exponent's argument, 48, and of some ten thousand additions in a chain; fp16 below 2^-14: 2^-25)
+    assert bool(((out - want).abs() <= (half_ulp + 2.0 ** -11) * want + 2.0 ** -25).all()), (float(out[0, 0]), float(want[0, 0]))
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
 @pytest.mark.parametrize("group", [2, 8])
 def test_an_infinite_value_stays_one(group, dtype):
