@@ -46,6 +46,9 @@ def test_selected_tokens_leave_the_background(q_heads, kv_heads, codes, lens, pp
     assert torch.equal(scores[0, :lens[0]], op.scores.view(rows, n_max)[0, :lens[0]])
     sel = op.decode_buffer(pqhsa.BUF_SEL_IDX, torch.int32).view(rows, op.params.k_max)
     count = op.decode_buffer(pqhsa.BUF_SEL_COUNT, torch.int32).tolist()
+    assert count == op.sel_count.tolist()
+    for row in range(rows):
+        assert torch.equal(sel[row, :count[row]].sort().values, op.sel_idx.view(rows, -1)[row, :count[row]].sort().values), row
     mass = op.decode_buffer(pqhsa.BUF_BG_MASS).view(rows, cfg.n_list).double()
     top = op.decode_buffer(pqhsa.BUF_BG_MAX)
     passes = 2 if q_heads // kv_heads == 8 else 1        # (of up to four heads)
