@@ -18,10 +18,12 @@
 // neighbours 347 -> 315 -> 317, of 300 381 -> 348 -> 350, rising 385 -> 350 -> 344; 1 %, rising 311 -> 295 -> 310, all
 // equal 1331 -> 377 -> 1135.)
 //
-// What bounds it: the reads of the tiles, 128 bytes each in random order beside the write-back of the scan's
-// lines (2.2 to 2.6 TB/s, whatever the loop around them), 17 of its 38 us at 256 rows of 128K; then chains of
-// short steps.  Whole decode call, sampled top-k (select.cu) and background kernel -> this one, us: 8 x 128K
-// 299 -> 278 (budget 0.5 % 286 -> 260, 2 % 339 -> 332), 16 x 64K 314 -> 296, 8 x 32K 110 -> 97.
+// What bounds it: a chain of short steps around the reads of the tiles, 128 bytes each in random order beside the
+// write-back of the scan's lines.  256 rows of 128K: 37 us; of a CTA's 45 to 55 K clocks after the scan, the tiles' maxima
+// and the bound take 9 to 12 K, the lists' sums 1 to 3 K, the tiles 17 to 29 K, the range of the k-th 7 to 15 K, writing the
+// selection and taking it out of the sums 6 to 9 K.
+// Whole decode call, sampled top-k (select.cu) and background kernel -> this one, us: 8 x 128K 299 -> 278 (budget 0.5 %
+// 286 -> 260, 2 % 328 -> 319), 16 x 64K 314 -> 297, 8 x 32K 110 -> 97.
 #include <cstddef>
 
 #include "background.cuh"
