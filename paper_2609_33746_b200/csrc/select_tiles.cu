@@ -15,7 +15,7 @@
 // where they were.  The warps start at sixteen places of the row, so that the first cut is near the last one
 // also where scores rise along it.  The result is exact for every input; a score that is not a number ranks below -inf.
 // (8 x 128K, 2 %, made again from a tighter bound -> cut -> the other top-k, us: scores that crowd in runs of 40
-// neighbours 347 -> 315 -> 317, of 300 381 -> 348 -> 350, rising 385 -> 350 -> 344; 1 %, rising 311 -> 295 -> 310, all
+// neighbours 347 -> 315 -> 317, of 300 381 -> 348 -> 350, rising 385 -> 348 -> 346; 1 %, rising 311 -> 295 -> 310, all
 // equal 1331 -> 377 -> 1135.)
 //
 // What bounds it: a chain of short steps around the reads of the tiles, 128 bytes each in random order beside the
@@ -240,6 +240,50 @@ __device__ __noinline__ void gather(TsShared& sh) {
     __syncwarp();
   }
   if (lane == 0) sh.next[warp] = e0;
+}
+
+// The list keeps what is above (lo, cut_pos), which is the cut from here on; of its other tiles a warp keeps those that
+// reach it.  Called between barriers; ends with the CTA in step.  (A function of its own: what most rows skip would lie
+// between steps that are fetched once per CTA, 1.2 to 2 us of a call: 8 x 32K 102.5 -> 101.1, 8 x 128K 275.0 -> 273.3.)
+__device__ __noinline__ void cut_list(TsShared& sh, uint32_t n_mine, uint32_t lo, uint32_t cut_pos) {
+  const Row& r = sh.row;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) { sh.n_list = 0u; sh.cut_key = lo; sh.cut_pos = cut_pos; }
+  constexpr int kMove = 4;
+#pragma unroll 1
+  for (uint32_t i0 = 0; i0 < n_mine; i0 += kMove * kTsThreads) {
+    uint2 it[kMove];
+#pragma unroll
+    for (int u = 0; u < kMove; ++u) {
+      const uint32_t i = i0 + u * kTsThreads + tid;
+      it[u] = i < n_mine ? r.list[i] : make_uint2(0u, 0u);
+    }
+    __syncthreads();                                    // (what is kept lands before what has been read)
+#pragma unroll
+    for (int u = 0; u < kMove; ++u) {
+      const bool keep = it[u].x > lo || (it[u].x == lo && it[u].y < cut_pos);
+      const unsigned m = __ballot_sync(0xffffffffu, keep);
+      uint32_t at = 0u;
+      if (lane == 0 && m) at = atomicAdd(&sh.n_list, (uint32_t)__popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (keep) r.list[at] = it[u];
+    }
+  }
+  const float lo_f = floor_of(lo);
+  const int e0 = sh.next[warp], e1 = sh.end[warp];
+  int e_end = e0;
+#pragma unroll 1
+  for (int i0 = e0; i0 < e1; i0 += 32) {
+    const uint16_t tile = r.ids[min(i0 + lane, e1 - 1)];
+    const bool keep = i0 + lane < e1 && !(r.mx[tile] < lo_f);
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (keep) r.ids[e_end + __popc(m & ((1u << lane) - 1u))] = tile;
+    e_end += __popc(m);
+    __syncwarp();
+  }
+  __syncwarp();
+  if (lane == 0) sh.end[warp] = e_end;
+  __syncthreads();
 }
 
 // What the re-score wants to know of the top-k (fp16 tables): the listed scores, their bound and number.
@@ -540,44 +584,7 @@ select_tiles_kernel(Plan pl, const float* __restrict__ scores, const int32_t* __
       if (lo == hi) by_pos = true;
     }
     if (!full) break;
-    // the list keeps what is in the range or above it
-    const uint32_t cut_pos = by_pos ? p_hi + 1u : 0xffffffffu;
-    if (tid == 0) { sh.n_list = 0u; sh.cut_key = lo; sh.cut_pos = cut_pos; }
-    constexpr int kMove = 4;
-#pragma unroll 1
-    for (uint32_t i0 = 0; i0 < n_mine; i0 += kMove * kTsThreads) {
-      uint2 it[kMove];
-#pragma unroll
-      for (int u = 0; u < kMove; ++u) {
-        const uint32_t i = i0 + u * kTsThreads + tid;
-        it[u] = i < n_mine ? r.list[i] : make_uint2(0u, 0u);
-      }
-      __syncthreads();                                  // (what is kept lands before what has been read)
-#pragma unroll
-      for (int u = 0; u < kMove; ++u) {
-        const bool keep = it[u].x > lo || (it[u].x == lo && it[u].y < cut_pos);
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        uint32_t at = 0u;
-        if (lane == 0 && m) at = atomicAdd(&sh.n_list, (uint32_t)__popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-        if (keep) r.list[at] = it[u];
-      }
-    }
-    // and of its other tiles a warp keeps those that reach the cut
-    const float lo_f = floor_of(lo);
-    const int warp = tid >> 5, e0 = sh.next[warp], e1 = sh.end[warp];
-    int e_end = e0;
-#pragma unroll 1
-    for (int i0 = e0; i0 < e1; i0 += 32) {
-      const uint16_t tile = r.ids[min(i0 + lane, e1 - 1)];
-      const bool keep = i0 + lane < e1 && !(r.mx[tile] < lo_f);
-      const unsigned m = __ballot_sync(0xffffffffu, keep);
-      if (keep) r.ids[e_end + __popc(m & ((1u << lane) - 1u))] = tile;
-      e_end += __popc(m);
-      __syncwarp();
-    }
-    if (lane == 0) sh.end[warp] = e_end;
-    __syncthreads();
+    cut_list(sh, n_mine, lo, by_pos ? p_hi + 1u : 0xffffffffu);
     first_cut = false;
   }
   if (cand.cand != nullptr) {
